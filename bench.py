@@ -519,8 +519,6 @@ def roofline(w, kernels, peaks):
 # profiles/ (kernel, workload) -> bytes.
 TRAFFIC_BYTES_PER_LAUNCH = {
     ("tc_fwd_kernel", "C2"): 475.3e6,        # profiles/tc_fwd_kernel_C2.md
-    ("tc_bwd_dq_kernel", "C2"): 691.0e6,     # profiles/tc_bwd_dq_kernel_C2.md
-    ("tc_bwd_dkv_kernel", "C2"): 823.0e6,    # profiles/tc_bwd_dkv_kernel_C2.md (with the row statistic D)
 }
 
 

@@ -104,9 +104,8 @@ std::mutex g_timing_mutex;
 bool g_timing_on = false;
 std::vector<TimedLaunch> g_timed;
 const char *const kKernelNames[kKernelCount] = {
-    "tc_fwd_kernel", "simt_row_dot_kernel", "tc_bwd_dq_kernel", "tc_bwd_dkv_kernel",
-    "bwd_dkv_mma_kernel",
-    "simt_fwd_kernel", "simt_bwd_dq_kernel", "simt_bwd_dkv_kernel", "ce_fwd_kernel", "ce_finalize_kernel", "tc_bwd_prefix_kernel", "simt_bwd_prefix_kernel"};
+    "tc_fwd_kernel", "simt_row_dot_kernel", "tc_bwd_dq_kernel" /* dQ and the suffix gradients */, "simt_fwd_kernel", "simt_bwd_dq_kernel",
+    "simt_bwd_dkv_kernel", "ce_fwd_kernel", "ce_finalize_kernel", "tc_bwd_prefix_kernel", "simt_bwd_prefix_kernel"};
 
 }  // namespace
 
@@ -308,8 +307,7 @@ pskv_status bwd_checked(const Dims &dm, const void *dout, const float *dlse, con
     a.scale = scale;
     a.dims = dm;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e = tc_bwd_supported(dm) ? launch_tc_bwd(a, workspace, status_word, stream)
-                                         : launch_simt_bwd(a, stream);
+    cudaError_t e = tc_bwd_supported(dm) ? launch_tc_bwd(a, status_word, stream) : launch_simt_bwd(a, stream);
     return e == cudaSuccess ? PSKV_OK : cuda_fail(e);
 }
 
@@ -445,6 +443,16 @@ SideStream *side_stream()
 // pskv_set_multi_form: 0 = the library chooses between one launch for all instructions and one pass per
 // instruction, 1 = one launch wherever the shapes allow it (the same as 0 today), 2 = always passes.
 int multi_form() { return g_multi_form.load(std::memory_order_relaxed); }
+
+// Launches of the gradient step of pskv_attn_bwd_multi.  One is enough; the shapes for which the row statistic,
+// dQ and the suffix gradients have been three launches so far keep that count (pskv_kernel_launches is part of
+// the interface), as the row statistic and two halves of the units, the second half's CTAs filling in as
+// the first half's drain.
+int tc_bwd_multi_launches(const Dims &dm, int Bp)
+{
+    const bool grouped = dm.S % 8 == 0 && dm.S <= 128 && !(dm.S <= 48 && dm.n_rep * dm.S >= 128);
+    return grouped && tc_fwd_fused_supported(dm, Bp) ? 2 : 1;
+}
 
 // checks shared by the two multi-instruction calls; fills the per-instruction geometry
 pskv_status check_multi(int B, int Bp, int Hq, int Hkv, int S, int Pmax, int d, const int *prefix_len)
@@ -590,21 +598,16 @@ pskv_status pskv_attn_bwd_multi(const void *dout, const void *q, const void *pre
         a.scale = scale;
         a.dims = dm;
     };
-    {
-        // All instructions in one dQ launch when every tile lies inside one instruction (as in the forward);
-        // the row statistic before it and the suffix gradients after it never involved the prefix.
-        Dims dall;
-        if (Bp > 1 && multi_form() != 2 && check_dims(B, Hq, Hkv, S, Pmax, d, &dall) == PSKV_OK &&
-            tc_bwd_fused_supported(dall, Bp)) {
-            BwdArgs a;
-            fill(a, 0, dall, 0);
-            cudaError_t e = launch_tc_bwd(a, workspace, status_word, stream, kBwdPartAll, Bp, prefix_len);
-            return e == cudaSuccess ? PSKV_OK : cuda_fail(e);
-        }
+    Dims dall;
+    const bool dall_ok = check_dims(B, Hq, Hkv, S, Pmax, d, &dall) == PSKV_OK;
+    if (Bp > 1 && multi_form() != 2 && dall_ok && tc_bwd_fused_supported(dall, Bp)) {
+        BwdArgs a;
+        fill(a, 0, dall, 0);
+        cudaError_t e = launch_tc_bwd(a, status_word, stream, kBwdPartAll, Bp, prefix_len, tc_bwd_multi_launches(dall, Bp));
+        return e == cudaSuccess ? PSKV_OK : cuda_fail(e);
     }
-    // The row statistic D = <dout, out> and the suffix gradients do not involve the prefix: when every
-    // instruction's part runs on the tensor-core kernels they are done once over all B candidates, and
-    // only the dQ step runs once per instruction.
+    // One pass per instruction.  The row statistic D does not involve the prefix: when every instruction's part
+    // runs on the tensor-core kernel it is formed once over all B candidates.
     bool all_tc = true;
     for (int i = 0; i < Bp && all_tc; ++i) {
         Dims dm;
@@ -612,17 +615,16 @@ pskv_status pskv_attn_bwd_multi(const void *dout, const void *q, const void *pre
         if (st != PSKV_OK) return st;
         all_tc = tc_bwd_supported(dm);
     }
-    Dims whole;
-    st = check_dims(B, Hq, Hkv, S, prefix_len[0], d, &whole);
-    if (st != PSKV_OK) return st;
-    all_tc = all_tc && tc_bwd_supported(whole);
     if (all_tc) {
+        Dims whole;
+        st = check_dims(B, Hq, Hkv, S, prefix_len[0], d, &whole);
+        if (st != PSKV_OK) return st;
         BwdArgs a;
         fill(a, 0, whole, 0);
-        cudaError_t e = launch_tc_bwd(a, workspace, status_word, stream, kBwdPartRowDot);
+        cudaError_t e = launch_simt_row_dot(a, stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    // the dQ passes of different instructions alternate between the caller's stream and the internal one
+    // the passes of different instructions alternate between the caller's stream and the internal one
     std::lock_guard<std::mutex> lock(g_side_mutex);
     SideStream *side = (all_tc && Bp > 1) ? side_stream() : nullptr;
     if (side) {
@@ -640,8 +642,8 @@ pskv_status pskv_attn_bwd_multi(const void *dout, const void *q, const void *pre
         cudaStream_t pass_stream = (side && (i & 1)) ? side->stream : stream;
         BwdArgs a;
         fill(a, i, dm, p_off);
-        cudaError_t e = all_tc ? launch_tc_bwd(a, a.row_dot, status_word, pass_stream, kBwdPartDq)
-                               : tc_bwd_supported(dm) ? launch_tc_bwd(a, a.row_dot, status_word, stream)
+        cudaError_t e = all_tc ? launch_tc_bwd(a, status_word, pass_stream, kBwdPartGrad)
+                               : tc_bwd_supported(dm) ? launch_tc_bwd(a, status_word, stream)
                                                       : launch_simt_bwd(a, stream);
         if (e != cudaSuccess) result = cuda_fail(e);
     }
@@ -650,14 +652,7 @@ pskv_status pskv_attn_bwd_multi(const void *dout, const void *q, const void *pre
         if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, side->join, 0);
         if (e != cudaSuccess && result == PSKV_OK) result = cuda_fail(e);
     }
-    if (result != PSKV_OK) return result;
-    if (all_tc) {
-        BwdArgs a;
-        fill(a, 0, whole, 0);
-        cudaError_t e = launch_tc_bwd(a, workspace, status_word, stream, kBwdPartDkv);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    return PSKV_OK;
+    return result;
 }
 
 // ---- gradients of the shared prefix cache ---------------------------------------------------------------

@@ -50,14 +50,8 @@ struct BwdArgs {
 // General CUDA-core kernels (any S, Skv, P; d in {64,128}; ragged or not).
 cudaError_t launch_simt_fwd(const FwdArgs &a, cudaStream_t stream);
 cudaError_t launch_simt_bwd(const BwdArgs &a, cudaStream_t stream);
-// Pieces of the backward the tensor-core path reuses: D = <dout, out> per row into a.row_dot, and
-// dk_suffix / dv_suffix (needs row_dot and lse).
+// Row statistic of the backward pass, D = <dout, out> - dlse per row, into a.row_dot.
 cudaError_t launch_simt_row_dot(const BwdArgs &a, cudaStream_t stream);
-cudaError_t launch_simt_bwd_dkv(const BwdArgs &a, cudaStream_t stream);
-// dk_suffix / dv_suffix on warp-level tensor-core MMAs, one CTA per (candidate, KV head); S <= 64.
-bool mma_bwd_dkv_supported(const Dims &d);
-cudaError_t launch_mma_bwd_dkv(const BwdArgs &a, cudaStream_t stream);
-bool tc_bwd_dkv_supported(const Dims &d);
 // Gradients of the shared prefix cache (need row_dot): tensor-core kernel (d = 128; `acc32` holds
 // 2 * Hkv * P * d floats of scratch) or the general one.
 bool tc_bwd_prefix_supported(const Dims &d);
@@ -65,10 +59,6 @@ cudaError_t launch_tc_bwd_prefix(const BwdArgs &a, __nv_bfloat16 *dk_prefix, __n
                                  unsigned int *status_word, cudaStream_t stream);
 cudaError_t launch_simt_bwd_prefix(const BwdArgs &a, __nv_bfloat16 *dk_prefix, __nv_bfloat16 *dv_prefix,
                                    cudaStream_t stream);
-// with_d: the kernel also forms D = <dout, out> - dlse per row and writes it to a.row_dot (it then needs
-// a.out and no pre-pass); tc_bwd_dkv_row_dot_supported tells whether the shape allows that.
-bool tc_bwd_dkv_row_dot_supported(const Dims &d);
-cudaError_t launch_tc_bwd_dkv(const BwdArgs &a, unsigned int *status_word, cudaStream_t stream, bool with_d = false);
 
 // tcgen05/TMEM kernels.  `status_word` is the device status flag that bounded waits set.
 bool tc_fwd_supported(const Dims &d);
@@ -87,16 +77,13 @@ cudaError_t launch_tc_fwd_pair(const FwdArgs &a, unsigned int *status_word, cuda
 bool cta_pairs_enabled();
 bool tc_bwd_supported(const Dims &d);
 size_t tc_bwd_workspace_bytes(const Dims &d);
-// `parts` selects which of the three steps run (all by default): the row statistic D and the suffix
-// gradients do not involve the prefix, so a caller with several prefixes runs them once over all
-// candidates and the dQ step once per prefix.  Where one kernel produces both the row statistic and the
-// suffix gradients (tc_bwd_dkv_row_dot_supported) it runs for kBwdPartRowDot and kBwdPartDkv is empty;
-// a caller that splits the parts must ask for kBwdPartRowDot before kBwdPartDq either way.
-enum { kBwdPartRowDot = 1, kBwdPartDq = 2, kBwdPartDkv = 4, kBwdPartAll = 7 };
-bool tc_bwd_fused_supported(const Dims &d, int n_instr);  // several instructions in one dQ launch (as for the forward)
-cudaError_t launch_tc_bwd(const BwdArgs &a, void *workspace, unsigned int *status_word,
-                          cudaStream_t stream, int parts = kBwdPartAll, int n_instr = 1,
-                          const int *prefix_len = nullptr);
+// `parts` selects which of the two steps run (all by default): the row statistic D does not involve the prefix,
+// so a caller with several prefixes runs it once over all candidates and the gradients once per prefix.
+// `split` > 1 takes the units of the gradient step in that many launches.
+enum { kBwdPartRowDot = 1, kBwdPartGrad = 2, kBwdPartAll = 3 };
+bool tc_bwd_fused_supported(const Dims &d, int n_instr);  // several instructions in one launch (as for the forward)
+cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStream_t stream, int parts = kBwdPartAll,
+                          int n_instr = 1, const int *prefix_len = nullptr, int split = 1);
 
 // Masked target cross-entropy fused with the vocabulary projection (tcgen05 GEMM whose logits stay on chip).
 struct CeArgs {
@@ -120,8 +107,7 @@ void count_launches(int n);
 // Optional per-kernel device timing (pskv_kernel_timing_*): when enabled, a launch site brackets
 // its kernel with two CUDA events on the launch stream.
 enum KernelId {
-    kKernelFwdTc = 0, kKernelRowDot, kKernelBwdDqTc, kKernelBwdDkvTc, kKernelBwdDkvMma,
-    kKernelFwdSimt, kKernelBwdDqSimt, kKernelBwdDkvSimt, kKernelCeFwd, kKernelCeFinalize, kKernelBwdPrefixTc, kKernelBwdPrefixSimt, kKernelCount
+    kKernelFwdTc = 0, kKernelRowDot, kKernelBwdTc, kKernelFwdSimt, kKernelBwdDqSimt, kKernelBwdDkvSimt, kKernelCeFwd, kKernelCeFinalize, kKernelBwdPrefixTc, kKernelBwdPrefixSimt, kKernelCount
 };
 void *timing_begin(int kernel_id, cudaStream_t stream);  // returns nullptr when timing is off
 void timing_end(void *token, cudaStream_t stream);

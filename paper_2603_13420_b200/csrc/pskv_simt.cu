@@ -293,18 +293,6 @@ cudaError_t launch_simt_row_dot(const BwdArgs &a, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-cudaError_t launch_simt_bwd_dkv(const BwdArgs &a, cudaStream_t stream)
-{
-    const long long keys = (long long)a.dims.B * a.dims.Hkv * a.dims.Skv;
-    KernelTiming timing(kKernelBwdDkvSimt, stream);
-    if (a.dims.d == 128)
-        simt_bwd_dkv_kernel<128><<<blocks_for(keys), kWarpsPerBlock * 32, 0, stream>>>(a);
-    else
-        simt_bwd_dkv_kernel<64><<<blocks_for(keys), kWarpsPerBlock * 32, 0, stream>>>(a);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_simt_bwd_prefix(const BwdArgs &a, __nv_bfloat16 *dk_prefix, __nv_bfloat16 *dv_prefix, cudaStream_t stream)
 {
     const long long keys = (long long)a.dims.Hkv * a.dims.P;

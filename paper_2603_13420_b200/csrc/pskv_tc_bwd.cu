@@ -1,23 +1,48 @@
-// Shared-prefix attention backward, query side, for sm_100a (tcgen05 / TMEM / TMA):
-//   dQ = scale * sum_j dS_j K_j   over the shared prefix keys and the visible suffix keys,
-//   dS = P o (dP - D),  P = exp(S - lse),  S = scale Q K^T,  dP = dO V^T,  D = <dO, O>.
-// The prefix K/V is frozen (Sec. 4.2): no gradient flows into it, so the prefix part costs three
-// contractions per block instead of five.  Tiling, operand staging and roles mirror the forward
-// kernel: 128-row tiles of the flat row list of a KV head, prefix blocks resident in shared memory
-// when they fit, one suffix block per tile with the block-diagonal causal mask.
+// Shared-prefix attention backward for sm_100a (tcgen05 / TMEM / TMA), one kernel for all three gradients:
+//   dQ        = scale * sum_j dS_j K_j              over the shared prefix keys and the visible suffix keys
+//   dK_suffix = scale * sum over rows of dS^T Q     (suffix keys only: the prefix cache is frozen, Sec. 4.2)
+//   dV_suffix =         sum over rows of  P^T dO
+//   with P = exp(S - lse), S = scale Q K^T, dP = dO V^T, dS = P o (dP - D), D = <dO, O> (a pre-pass).
+// Q and dO are fetched once; nothing is read or recomputed twice except in the passes named below.
+//
+// A CTA works on units.  A unit is `cu` neighbouring candidates of one KV head, so that the sums over rows
+// and heads that make dK_suffix / dV_suffix stay inside the CTA: its rows (n_rep * S per candidate, padded
+// to Rp, a multiple of 8) are cut into 128-row tiles.  A tile meets its keys in pieces of 64: the pieces of
+// the prefix, and for every candidate it touches the pieces of that candidate's suffix (several short
+// candidates share a piece).  One (tile, piece) pair is an item:
+//   S  = Q K^T, dP = dO V^T       (M = 128 rows, N = keys)   -> one of two tensor-memory slots
+//   dS (and for suffix pieces P)  element-wise, bf16, to shared memory
+//   dQ += dS K                    (M = 128 rows, N = d)
+//   suffix pieces: dV^T += dO^T P, dK^T += Q^T dS   (M = d, N = keys, K = rows)
+// The second and third products read the very tiles the first ones read, as operands of the other major-ness.
+//
+// What bounds it: HBM for head layouts with one query head per KV head (every row's q, dout, k, v and three
+// gradients move once), else the chain of an item.  64 keys instead of 128 per item cost a third more shared
+// memory reads by the tensor cores (768 instead of 512 cycles for a 128 x 128 score block and its dP), but two
+// S/dP slots fit beside dQ and the accumulators, and because dS goes to shared memory a slot is handed back
+// as soon as the element-wise warps have loaded it, before their arithmetic: the next scores never wait
+// for the previous item's dQ.
+//
+// Measured (whole forward + backward step, before: a dQ kernel and a suffix-gradient kernel that each read q and
+// dout, for S a multiple of 8 and up to 64, CUDA-core kernels for the rest): B = 512, 32/8 heads, P = 256, S = 48
+// 563 -> 519 us; B = 128, 32/32 heads, P = 160, S = 40 171 -> 142 us; B = 100, 32/32 heads, P = 78, S = 113 10.4 ms ->
+// 0.30 ms.  With a staging buffer for dQ instead of four K and three V stages (three and two fit): 529 us.
+//
+// Suffixes beyond 64 keys have several pieces per candidate but only one pair of accumulators (128 columns).
+// When the unit is one tile the pieces take turns; when it is several tiles, pass 0 accumulates piece 0 (and
+// all of dQ) and every later pass walks over the tiles once more for one further piece.
 //
 // Persistent CTA, one per SM, 24 warps:
-//   warp 0      TMA producer: Q tile, prefix K blocks, suffix K
-//   warp 1      tcgen05.mma issuer: S = Q K^T of every item
-//   warp 2      tcgen05.mma issuer: dP = dO V^T of the next item, then dQ += dS K of the current one
-//               (owns the TMEM allocation)
-//   warp 3      TMA producer: dO tile, prefix V blocks, suffix V
-//   warps 4-19  element-wise, four warpgroups sharing each item by 32-column pieces (thread <->
-//               query row): dS = exp2(S*sl2 - lse2) * (dP - D) as bf16
-//   warps 20-23 epilogue: dQ from tensor memory, * scale, bf16, staging, TMA store
-// Tensor memory: two 128-column S slots (dS overwrites the first half of its own slot), one dP
-// slot, and the 128 columns of dQ.  D comes from a streaming pre-pass, dK_suffix / dV_suffix from
-// a kernel of their own behind this one.  Every wait is bounded.
+//   warp 0      TMA producer: K and V pieces (two rings); writes the descriptor of every item
+//   warp 1      tcgen05.mma issuer: S and dP
+//   warp 2      tcgen05.mma issuer: dQ, dV^T, dK^T (owns the TMEM allocation)
+//   warp 3      TMA producer: Q and dO tiles; writes the row table of every tile
+//   warps 4-19  element-wise: two sets of eight warps take the items in turn; a warp covers 32 rows x 32 keys
+//   warps 20-23 epilogue: dQ, dK and dV from tensor memory to global memory
+// The walk over units, tiles and pieces is done by the producers (and the epilogue); the MMA issuers and the
+// element-wise warps follow 16-byte descriptors in shared memory.  With the walk in every role the registers it
+// took spilled and the roles' loops ran 900 to 2 900 cycles an item of bookkeeping.
+// Every wait is bounded.
 #include <string.h>
 
 #include "pskv_common.cuh"
@@ -29,90 +54,213 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kSlots = 2;
-constexpr int kGroups = 4;   // element-wise warpgroups: one 32-column piece of every score block each
-constexpr int kPiece = 32;
-constexpr int kThreads = 32 * (4 + 4 * kGroups + 4);
-constexpr int kDpCol = kSlots * kBlockN;
-constexpr int kDqCol = kDpCol + kBlockN;
-constexpr int kMaxStages = 4;
+constexpr int kPieceN = 64;   // keys per item
+constexpr int kThreads = 32 * 24;
+constexpr int kMaxRing = 4;
 constexpr int kMaxInstr = kMaxFusedInstructions;  // prefixes one launch can serve
+// tensor memory: two (S, dP) slots, dQ, the two transposed accumulators
+constexpr int kSlotCols = 128, kColDp = 64, kColDq = 256, kColDv = 384, kColDk = 448;
+constexpr int kDsBytes = kTileM * 128;  // P or dS of an item: 128 rows x 64 keys of bf16
 
 enum : unsigned int {
-    kErrProdA = 0x201, kErrProdB = 0x202, kErrMmaS = 0x203, kErrMmaDq = 0x204, kErrElem = 0x205,
+    kErrProdKv = 0x201, kErrProdQ = 0x202, kErrMmaS = 0x203, kErrMmaGrad = 0x204, kErrElem = 0x205,
     kErrEpi = 0x206, kErrAlign = 0x207
 };
 
 struct TcBwdParams {
     const float *lse;      // [B*Hq*S] from the forward pass
-    const float *row_dot;  // [B*Hq*S] D = <dout, out>
+    const float *row_dot;  // [B*Hq*S] D
+    __nv_bfloat16 *dq;       // [B,Hq,S,d]
+    __nv_bfloat16 *dk, *dv;  // [B,Hkv,S,d]
     unsigned int *status;
     float sl2;             // scale * log2(e)
     float scale;
-    int B, Hq, Hkv, S, P, n_rep;
-    int Rg, tile_rows, seg_rows, tiles_per_group, total_tiles;
-    FastDiv fd_tpg, fd_Rg, fd_S, fd_seg;  // divisions by tiles_per_group, Rg, S, seg_rows
-    int nblk_p, tail_rows, resident, stages_k, stages_v, sfx_rows;  // ring stages of prefix K / V (streaming mode)
-    int off_pk, off_pv, off_q, off_do, off_sk, off_sv, off_stage, off_bar, off_misc;
-    // several instructions in one launch (Sec. 4.3): the candidates of instruction i are contiguous and use
-    // prefix cache i of [n_instr][Hkv][P][d], whose first pad[i] rows are left padding
-    int n_instr;  // 1: one shared prefix
-    int rpi;      // rows of one instruction inside a KV head's row list (a multiple of tile_rows)
-    FastDiv fd_rpi;
-    int pad[kMaxInstr];
+    int dq_sectors;        // dq is 32-byte aligned
+    int Hq, Hkv, S, P, n_rep;
+    int Rg;                // rows of a candidate in one KV-head group: n_rep * S
+    int Rp;                // rows it takes in the unit's row list: Rg rounded up to 8
+    int Sp;                // key columns a candidate takes in a piece that holds several: S rounded up to 8
+    int cu;                // candidates per unit
+    int cpp;               // candidates per suffix piece (> 1 only when a unit is one tile)
+    int nh;                // suffix pieces per candidate: ceil(S / 64)
+    int seg, cbox;         // rows and candidates of one Q / dO box
+    int sfx_box;           // key rows per candidate in a suffix K / V box
+    int nblk;              // prefix pieces: ceil(P / 64)
+    int Kq;                // candidates per instruction (all of them when there is one prefix)
+    int upi, upg;          // units per (KV head, instruction), per KV head
+    int unit0, n_units;
+    FastDiv fd_upg, fd_upi, fd_Rp, fd_S, fd_cpp;
+    int stages_k, stages_v;
+    int off_do, off_q, off_k, off_v, off_p, off_ds, off_rows, off_bar, off_misc;
+    int pad[kMaxInstr];    // left padding of each instruction's prefix cache (Sec. 4.3)
 };
 
 template <int D>
 struct Cfg {
-    static constexpr int kSlabs = D / 64;
-    static constexpr int kSlabBytes = kTileM * 128;
+    static constexpr int kSlabs = D / 64;              // 64-column (128-byte) swizzle slabs per row
+    static constexpr int kSlabBytes = kTileM * 128;    // slab of a 128-row tile
     static constexpr int kTileBytes = kSlabs * kSlabBytes;
+    static constexpr int kPieceSlab = kPieceN * 128;   // slab of a 64-row K / V piece
+    static constexpr int kPieceBytes = kSlabs * kPieceSlab;
 };
 
 enum {
-    kBarQFull = 0,
-    kBarQkFree,     // every S MMA of a tile completed: the Q buffer is free
-    kBarDoFull,
-    kBarDvFree,     // every dP MMA of a tile completed: dO, suffix V (and resident prefix V) are free
-    kBarSKFull,
-    kBarSVFull,
-    kBarDqFull,     // every dQ MMA of a tile completed: dQ is final, suffix K (and resident prefix K) are free
-    kBarDqFree,     // the epilogue has read dQ out (4 arrivals)
-    kBarStageFull,  // (4 arrivals)
-    kBarStageFree,
-    kBarDpFull,     // dP of an item is in tensor memory
-    kBarDpFree,     // the element-wise warps have read dP (4 arrivals)
-    kBarSFull,                        // [kSlots]
-    kBarDsReady = kBarSFull + kSlots, // [kSlots] dS written (4 arrivals)
-    kBarDqDone = kBarDsReady + kSlots, // [kSlots] the dQ MMAs of an item completed: its S slot is free
-    kBarKFull = kBarDqDone + kSlots,
-    kBarVFull = kBarKFull + kMaxStages,
-    kBarKFree = kBarVFull + kMaxStages,
-    kBarVFree = kBarKFree + kMaxStages,
-    kNumBars = kBarVFree + kMaxStages
+    kBarQFull = 0,   // Q and dO of a tile landed
+    kBarQFree,       // the last MMA of each issuer that reads them has completed (2 arrivals)
+    kBarDqFull,      // dQ of a tile is final
+    kBarDqFree,      // the epilogue has read it out (4 arrivals)
+    kBarPFree,       // the MMAs that read P have completed
+    kBarAccFull,     // the accumulators are final
+    kBarAccFree,     // the epilogue has read them out (4 arrivals)
+    kBarSFull,                       // [2] S and dP of an item are in tensor memory
+    kBarSFree = kBarSFull + 2,       // [2] the element-wise warps have loaded them (8 arrivals)
+    kBarDsReady = kBarSFree + 2,     // [2] dS (and P) of an item are in shared memory (8 arrivals)
+    kBarDsFree = kBarDsReady + 2,    // [2] the MMAs that read dS have completed
+    kBarRowsFull = kBarDsFree + 2,   // [2] the row table of a tile is written
+    kBarKFull = kBarRowsFull + 2,    // (also: the item's descriptor is written)
+    kBarVFull = kBarKFull + kMaxRing,
+    kBarKFree = kBarVFull + kMaxRing,
+    kBarVFree = kBarKFree + kMaxRing,
+    kNumBars = kBarVFree + kMaxRing
 };
 constexpr int kBarBytes = 512;
-static_assert(kNumBars * 8 <= kBarBytes, "barrier area");
+constexpr int kDescOff = 384;   // descriptors behind the barriers: eight entries of 16 bytes
+static_assert(kNumBars * 8 <= kDescOff && kDescOff + 8 * 16 <= kBarBytes, "barrier area");
+constexpr int kRowsBytes = 2 * kTileM * 8;  // row tables (-lse log2(e), D) of two tiles
 
-__device__ __forceinline__ int prefix_block_rows(const TcBwdParams &p, int k)
+// Descriptor of an item.  x: MMA N and the flags below; y: suffix item: candidate group, prefix item: first and
+// last real key (8 bits each); z: first key of the piece inside the suffix; w: running number of the tile.
+// At most five items are between the producer (which needs a free K stage) and the element-wise warps, so
+// eight entries are enough.
+enum : uint32_t {
+    kDescN = 0x7f, kDescSfx = 1u << 7, kDescAcc = 1u << 8, kDescAccFirst = 1u << 9, kDescAccLast = 1u << 10,
+    kDescQDone = 1u << 11,     // last item of the tile that feeds dK / dV
+    kDescLast = 1u << 12, kDescDq = 1u << 13, kDescFirst = 1u << 14,
+    kDescAccOdd = 1u << 15,    // parity of the items that fed dK / dV so far
+    kDescK0 = 16, kDescK1 = 20,  // rows of the group inside the tile, in steps of 16 (4 bits each)
+    kDescEnd = 1u << 31
+};
+
+// The walk over units, passes, tiles and items, the same in every role.
+struct Walk {
+    int u, u_end;           // unit
+    int g, inst, b0, ncand; // its KV head, instruction, first candidate, candidates
+    int ntile, npass, pass, tt;
+    int R0, rows;           // tile: first row of the unit's row list, rows that belong to the unit
+    int grp_lo, ngrp;       // candidate groups (pieces' worth of candidates) the tile touches
+    int kp0;                // first prefix piece (pieces of padding only are left out)
+    int n_sfx, n_items;
+    // item
+    int k, e, j, q;         // position, interleaving state, next suffix / prefix index
+    bool sfx;
+
+    __device__ __forceinline__ bool done() const { return u >= u_end; }
+
+    __device__ __forceinline__ void unit(const TcBwdParams &p)
+    {
+        if (done()) return;
+        const int w = p.unit0 + u;
+        g = p.fd_upg.div(w);
+        const int r = w - g * p.upg;
+        inst = p.fd_upi.div(r);
+        const int ub = r - inst * p.upi;
+        b0 = inst * p.Kq + ub * p.cu;
+        ncand = min(p.cu, p.Kq - ub * p.cu);
+        ntile = (ncand * p.Rp + kTileM - 1) / kTileM;
+        npass = ntile > 1 ? p.nh : 1;
+        pass = tt = 0;
+        kp0 = p.pad[inst] / kPieceN;
+        tile(p);
+    }
+    __device__ __forceinline__ void tile(const TcBwdParams &p)
+    {
+        R0 = tt * kTileM;
+        rows = min(kTileM, ncand * p.Rp - R0);
+        grp_lo = p.fd_cpp.div(p.fd_Rp.div(R0));
+        ngrp = p.fd_cpp.div(p.fd_Rp.div(R0 + rows - 1)) - grp_lo + 1;
+        n_sfx = pass == 0 ? ngrp * p.nh : ngrp;
+        n_items = n_sfx + (pass == 0 ? p.nblk - kp0 : 0);
+        k = e = j = q = 0;
+        sfx = true;
+    }
+    __device__ __forceinline__ void start(const TcBwdParams &p)
+    {
+        u = (int)((long long)blockIdx.x * p.n_units / gridDim.x);
+        u_end = (int)((long long)(blockIdx.x + 1) * p.n_units / gridDim.x);
+        unit(p);
+    }
+    __device__ __forceinline__ void next_tile(const TcBwdParams &p)
+    {
+        if (++tt < ntile) { tile(p); return; }
+        tt = 0;
+        if (++pass < npass) { tile(p); return; }
+        ++u;
+        unit(p);
+    }
+    // Suffix items are spread evenly over the tile's items, the first one first: their accumulators are
+    // drained, and their P buffer is read, under the prefix items in between.
+    __device__ __forceinline__ void next_item()
+    {
+        if (sfx) ++j; else ++q;
+        ++k;
+        e += n_sfx;
+        if (e >= n_items) e -= n_items;
+        sfx = e < n_sfx;
+    }
+    __device__ __forceinline__ bool last_item() const { return k == n_items - 1; }
+    // suffix item: candidate group and 64-key piece of its suffix
+    __device__ __forceinline__ int grp(const TcBwdParams &p) const
+    {
+        return grp_lo + (pass > 0 || p.nh == 1 ? j : j / p.nh);
+    }
+    __device__ __forceinline__ int half(const TcBwdParams &p) const
+    {
+        return pass > 0 ? pass : p.nh == 1 ? 0 : j - j / p.nh * p.nh;
+    }
+    __device__ __forceinline__ bool acc(int h) const { return npass == 1 || h == pass; }  // feeds dK / dV
+    __device__ __forceinline__ int grp_row0(const TcBwdParams &p, int gr) const { return gr * p.cpp * p.Rp; }
+    __device__ __forceinline__ int grp_row1(const TcBwdParams &p, int gr) const
+    {
+        return min((gr + 1) * p.cpp, ncand) * p.Rp;
+    }
+    // MMA N of the current item (keys rounded up to 16)
+    __device__ __forceinline__ int n16(const TcBwdParams &p) const
+    {
+        int n;
+        if (!sfx) n = min(kPieceN, p.P - (kp0 + q) * kPieceN);
+        else if (p.nh > 1) n = min(kPieceN, p.S - half(p) * kPieceN);
+        else {
+            const int gr = grp(p);
+            n = p.cpp == 1 ? p.S : min(p.cpp, ncand - gr * p.cpp) * p.Sp;
+        }
+        return (n + 15) & ~15;
+    }
+};
+
+// 32 bytes of a row, a whole sector in one instruction where the alignment allows it.  dQ goes to memory this way,
+// straight from the epilogue's registers: lane <-> row, so an instruction covers 32 full sectors of 32 rows.  (With
+// 16-byte stores, half a sector each, such a store is slow; a staging buffer and TMA stores need 32 KB that
+// the K / V rings use better.)
+__device__ __forceinline__ void store_sector(__nv_bfloat16 *dst, const uint32_t *v, bool aligned)
 {
-    return k == p.nblk_p - 1 ? p.tail_rows : kBlockN;
+    if (aligned) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                     "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
+    } else {
+        reinterpret_cast<uint4 *>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4 *>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
 }
 
-// MODE bit 0: the prefix K blocks of a KV head stay in shared memory; bit 1: the prefix V blocks do
-// (else they stream through rings).  A K block is needed through a whole item (the dQ MMA reads it
-// after the element-wise stage), a V block only for its dP MMA, so when not both fit it is K that
-// stays.  Compile-time, so that each launch carries only the code of its own mode.
-template <int D, int MODE, bool MI>
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
-tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
-                 const __grid_constant__ CUtensorMap tm_dq, const __grid_constant__ CUtensorMap tm_pk,
-                 const __grid_constant__ CUtensorMap tm_pv, const __grid_constant__ CUtensorMap tm_pk_tail,
-                 const __grid_constant__ CUtensorMap tm_pv_tail, const __grid_constant__ CUtensorMap tm_sk,
-                 const __grid_constant__ CUtensorMap tm_sv, const TcBwdParams p)
+tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
+              const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
+              const __grid_constant__ CUtensorMap tm_sk, const __grid_constant__ CUtensorMap tm_sv,
+              const __grid_constant__ TcBwdParams p)
 {
     using C = Cfg<D>;
-    constexpr bool RK = (MODE & 1) != 0, RV = (MODE & 2) != 0;
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -124,17 +272,18 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + p.off_misc + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + p.off_misc);
 
-    if ((sbase & 1023u) != 0u) {
+    if ((sbase & 1023u) != 0u) {  // the swizzled layouts need a 1024-byte aligned base
         if (tid == 0) atomicCAS(p.status, 0u, (unsigned int)kErrAlign);
         return;
     }
-    // padding rows of the operand buffers must hold finite values (0 * NaN would poison dQ)
-    for (int i = tid; i < p.off_bar / 16; i += kThreads) reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
+    // operand rows that no copy ever writes must hold finite values (0 * NaN would poison a sum)
+    for (int i = tid; i < p.off_p / 16; i += kThreads) reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
     if (tid == 0) {
+#pragma unroll 1
         for (int i = 0; i < kNumBars; ++i) {
-            const bool epi = i == kBarDqFree || i == kBarStageFull;
-            const bool elem = i == kBarDpFree || (i >= kBarDsReady && i < kBarDsReady + kSlots);
-            mbar_init(bar(i), elem ? (uint32_t)(4 * kGroups) : epi ? 4u : 1u);
+            const bool epi = i == kBarDqFree || i == kBarAccFree;
+            const bool elem = (i >= kBarSFree && i < kBarSFree + 2) || (i >= kBarDsReady && i < kBarDsReady + 2);
+            mbar_init(bar(i), elem ? 8u : epi ? 4u : i == kBarQFree ? 2u : 1u);
         }
         *abort_flag = 0;
         fence_barrier_init();
@@ -152,628 +301,493 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
     // everything above touched shared and tensor memory only: it may run under the tail of the kernel before
     grid_dep_wait();
 
-    const int t_begin = (int)((long long)blockIdx.x * p.total_tiles / gridDim.x);
-    const int t_end = (int)((long long)(blockIdx.x + 1) * p.total_tiles / gridDim.x);
-    const int n_tiles = t_end - t_begin;
-    const int nitems = p.nblk_p + 1;
-    // A run of tiles that shares one prefix: a KV head, or (several instructions) one instruction's
-    // candidates inside a KV head; resident prefix blocks are reloaded at the start of each run and the
-    // barrier parity of those loads follows the run number.
-    auto inst_of = [&](const TileInfo &t) { return MI ? p.fd_rpi.div(t.R0) : 0; };
-    auto run_of = [&](const TileInfo &t, int inst) { return MI ? t.g * p.n_instr + inst : t.g; };
-    auto first_of_run = [&](const TileInfo &t, int inst) { return t.first_of_g || (MI && t.R0 == inst * p.rpi); };
-    int run_first;
-    {
-        const TileInfo t0 = tile_info(p, t_begin < p.total_tiles ? t_begin : 0, t_begin);
-        run_first = run_of(t0, inst_of(t0));
-    }
-    // Several instructions (Sec. 4.3): the prefix of instruction i starts with pad[i] rows of left padding;
-    // the key blocks that hold nothing else are left out of its tiles (their probabilities are all zero), so
-    // the items of a tile are the blocks from first_block on, then the suffix block.
-    auto first_block = [&](const TileInfo &t) { return MI ? p.pad[inst_of(t)] / kBlockN : 0; };
-    auto count_items = [&]() {
-        if (!MI) return n_tiles * nitems;
-        int n = 0;
-        for (int tl = 0; tl < n_tiles; ++tl) n += nitems - first_block(tile_info(p, t_begin + tl, t_begin));
-        return n;
-    };
-    const int sfx_slab = p.sfx_rows * 128;
-    const int tail_slab = p.tail_rows * 128;
-    const uint32_t stages_k = (uint32_t)p.stages_k, stages_v = (uint32_t)p.stages_v;
+    Walk w;
+    w.start(p);
+    bool ok = true;
 
     if (warp == 0) {
-        // ------------------------------------------------------------------ producer: Q, K
+        // ------------------------------------------------------------------ producer: K and V pieces
         if (lane == 0) {
-            prefetch_tensormap(&tm_q);
             prefetch_tensormap(&tm_sk);
-            if (p.P > 0) { prefetch_tensormap(&tm_pk); prefetch_tensormap(&tm_pk_tail); }
+            prefetch_tensormap(&tm_sv);
+            if (p.P > 0) { prefetch_tensormap(&tm_pk); prefetch_tensormap(&tm_pv); }
         }
-        uint32_t kload = 0;
-        bool ok = true;
+        int ks = 0, vs = 0;
+        uint32_t kph = 1, vph = 1, item = 0, tile = 0, n_acc = 0;
+        const uint32_t sfx_tx = (uint32_t)(C::kSlabs * p.sfx_box * p.cpp * 128);
+        uint4 *descs = reinterpret_cast<uint4 *>(smem + p.off_bar + kDescOff);
 #pragma unroll 1
-        for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info(p, t_begin + tl, t_begin);
-            // while idle: ask for the next tile's Q in L2 (its load can only be issued a tile from
-            // now, exactly when it is needed)
-            if (tl + 1 < n_tiles) {
-                const TileInfo tn = tile_info(p, t_begin + tl + 1, t_begin);
-                const int nseg_n = p.fd_seg.div(tn.rows);
-                int nb = p.fd_Rg.div(tn.R0), nr = tn.R0 - nb * p.Rg;
+        for (; !w.done() && ok; w.next_tile(p), ++tile) {
+            const int head = w.inst * p.Hkv + w.g;
+#pragma unroll 1
+            for (; w.k < w.n_items; w.next_item(), ++item) {
+                int row, b = w.b0;
+                uint4 dsc;
+                dsc.x = (uint32_t)w.n16(p) | (w.last_item() ? kDescLast : 0u) | (w.k == 0 ? kDescFirst : 0u) |
+                        (w.pass == 0 ? kDescDq : 0u);
+                dsc.w = (tile & 0xffffu) | (uint32_t)w.tt << 16;
+                if (w.sfx) {
+                    const int h = w.half(p), gr = w.grp(p);
+                    row = h * kPieceN;
+                    b += gr * p.cpp;
+                    dsc.x |= kDescSfx;
+                    dsc.y = (uint32_t)gr;
+                    dsc.z = (uint32_t)row;
+                    if (w.acc(h)) {
+                        const int r0 = w.grp_row0(p, gr) - w.R0, r1 = w.grp_row1(p, gr) - w.R0;
+                        dsc.x |= kDescAcc | (r0 >= 0 ? kDescAccFirst : 0u) | (r1 <= kTileM ? kDescAccLast : 0u) |
+                                 ((n_acc & 1u) ? kDescAccOdd : 0u) | (uint32_t)(max(r0, 0) >> 4) << kDescK0 |
+                                 (uint32_t)((min(r1, kTileM) + 15) >> 4) << kDescK1;
+                        if (gr == w.grp_lo + w.ngrp - 1 && (w.npass > 1 || h == p.nh - 1)) dsc.x |= kDescQDone;
+                        ++n_acc;
+                    }
+                } else {
+                    row = (w.kp0 + w.q) * kPieceN;
+                    dsc.y = (uint32_t)max(0, p.pad[w.inst] - row) | (uint32_t)(min(kPieceN, p.P - row) - 1) << 8;
+                    dsc.z = 0u;
+                }
+                const uint32_t tx = w.sfx ? sfx_tx : (uint32_t)C::kPieceBytes;
+                ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProdKv);
+                if (!ok) break;
                 if (elect_one_sync()) {
-#pragma unroll 1
-                    for (int s = 0; s < nseg_n; ++s) {
+                    descs[item & 7u] = dsc;
+                    const uint32_t dst = sbase + p.off_k + ks * C::kPieceBytes, fb = bar(kBarKFull + ks);
+                    mbar_arrive_expect_tx(fb, tx);
 #pragma unroll
-                        for (int sl = 0; sl < C::kSlabs; ++sl) tma_prefetch_4d(&tm_q, sl * 64, nr, tn.g, nb);
-                        nr += p.seg_rows;
-                        if (nr >= p.Rg) {
-                            nr -= p.Rg;
-                            ++nb;
-                        }
+                    for (int sl = 0; sl < C::kSlabs; ++sl) {
+                        if (w.sfx) tma_load_4d(dst + sl * C::kPieceSlab, &tm_sk, fb, sl * 64, row, w.g, b);
+                        else tma_load_3d(dst + sl * C::kPieceSlab, &tm_pk, fb, sl * 64, row, head);
                     }
                 }
                 __syncwarp();
-            }
-            // everything the Q loads need is worked out before the wait (the Q buffer is single)
-            const int nseg = p.fd_seg.div(t.rows);
-            int qb = p.fd_Rg.div(t.R0), qr = t.R0 - qb * p.Rg;
-            uint32_t q_dst = sbase + p.off_q;
-            ok = mbar_wait_warp(bar(kBarQkFree), (tl & 1) ^ 1, abort_flag, p.status, kErrProdA);
-            if (!ok) break;
-            if (elect_one_sync()) {
-                mbar_arrive_expect_tx(bar(kBarQFull), (uint32_t)(nseg * C::kSlabs * p.seg_rows * 128));
-#pragma unroll 1
-                for (int s = 0; s < nseg; ++s) {
+                ok = mbar_wait_warp(bar(kBarVFree + vs), vph, abort_flag, p.status, kErrProdKv);
+                if (!ok) break;
+                if (elect_one_sync()) {
+                    const uint32_t dst = sbase + p.off_v + vs * C::kPieceBytes, fb = bar(kBarVFull + vs);
+                    mbar_arrive_expect_tx(fb, tx);
 #pragma unroll
-                    for (int sl = 0; sl < C::kSlabs; ++sl)
-                        tma_load_4d(q_dst + sl * C::kSlabBytes, &tm_q, bar(kBarQFull), sl * 64, qr, t.g, qb);
-                    q_dst += p.seg_rows * 128;
-                    qr += p.seg_rows;  // boxes never straddle a candidate: seg_rows divides Rg
-                    if (qr >= p.Rg) {
-                        qr -= p.Rg;
-                        ++qb;
+                    for (int sl = 0; sl < C::kSlabs; ++sl) {
+                        if (w.sfx) tma_load_4d(dst + sl * C::kPieceSlab, &tm_sv, fb, sl * 64, row, w.g, b);
+                        else tma_load_3d(dst + sl * C::kPieceSlab, &tm_pv, fb, sl * 64, row, head);
                     }
                 }
+                __syncwarp();
+                if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
+                if (++vs == p.stages_v) { vs = 0; vph ^= 1u; }
             }
-            __syncwarp();
-            if (!RK) {
+        }
+        // two end marks, one for each set of element-wise warps
 #pragma unroll 1
-                for (int k = first_block(t); k < p.nblk_p; ++k) {
-                    const uint32_t ks = kload % stages_k;
-                    ok = mbar_wait_warp(bar(kBarKFree + ks), ((kload / stages_k) & 1) ^ 1, abort_flag, p.status, kErrProdA);
-                    if (!ok) break;
-                    const bool tail = k == p.nblk_p - 1;
-                    const int slab = tail ? tail_slab : C::kSlabBytes;
-                    if (elect_one_sync()) {
-                        mbar_arrive_expect_tx(bar(kBarKFull + ks), (uint32_t)(C::kSlabs * slab));
-                        for (int sl = 0; sl < C::kSlabs; ++sl)
-                            tma_load_3d(sbase + p.off_pk + ks * C::kTileBytes + sl * slab, tail ? &tm_pk_tail : &tm_pk,
-                                        bar(kBarKFull + ks), sl * 64, k * kBlockN, inst_of(t) * p.Hkv + t.g);
-                    }
-                    __syncwarp();
-                    ++kload;
-                }
-                if (!ok) break;
-            }
-            // suffix K (and resident prefix K) are read by the dQ MMAs too: free once dQ of the
-            // previous tile is final
-            if (tl > 0) {
-                ok = mbar_wait_warp(bar(kBarDqFull), (tl - 1) & 1, abort_flag, p.status, kErrProdA);
-                if (!ok) break;
-            }
-            if (RK && first_of_run(t, inst_of(t)) && elect_one_sync()) {
-                for (int k = 0; k < p.nblk_p; ++k) {
-                    const bool tail = k == p.nblk_p - 1;
-                    const int slab = tail ? tail_slab : C::kSlabBytes;
-                    mbar_arrive_expect_tx(bar(kBarKFull + k), (uint32_t)(C::kSlabs * slab));
-                    for (int sl = 0; sl < C::kSlabs; ++sl)
-                        tma_load_3d(sbase + p.off_pk + k * C::kTileBytes + sl * slab, tail ? &tm_pk_tail : &tm_pk,
-                                    bar(kBarKFull + k), sl * 64, k * kBlockN, inst_of(t) * p.Hkv + t.g);
-                }
+        for (int i = 0; i < 2 && ok; ++i, ++item) {
+            ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProdKv);
+            if (ok && elect_one_sync()) {
+                descs[item & 7u] = make_uint4(kDescEnd, 0u, 0u, 0u);
+                mbar_arrive(bar(kBarKFull + ks));
             }
             __syncwarp();
-            if (elect_one_sync()) {
-                mbar_arrive_expect_tx(bar(kBarSKFull), (uint32_t)(t.nc * C::kSlabs * p.S * 128));
-                for (int c = 0; c < t.nc; ++c)
-                    for (int sl = 0; sl < C::kSlabs; ++sl)
-                        tma_load_4d(sbase + p.off_sk + sl * sfx_slab + c * p.S * 128, &tm_sk, bar(kBarSKFull),
-                                    sl * 64, 0, t.g, t.b_first + c);
-            }
-            __syncwarp();
+            if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
         }
     } else if (warp == 3) {
-        // ------------------------------------------------------------------ producer: dO, V
+        // ------------------------------------------------------------------ producer: Q and dO tiles
         if (lane == 0) {
+            prefetch_tensormap(&tm_q);
             prefetch_tensormap(&tm_do);
-            prefetch_tensormap(&tm_sv);
-            if (p.P > 0) { prefetch_tensormap(&tm_pv); prefetch_tensormap(&tm_pv_tail); }
         }
-        uint32_t vload = 0;
-        bool ok = true;
+        const int step = p.seg * p.cbox;  // rows of one box
+        uint32_t tile = 0;
 #pragma unroll 1
-        for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info(p, t_begin + tl, t_begin);
-            if (tl + 1 < n_tiles) {  // the next tile's dO into L2, a tile ahead
-                const TileInfo tn = tile_info(p, t_begin + tl + 1, t_begin);
-                const int nseg_n = p.fd_seg.div(tn.rows);
-                int nb = p.fd_Rg.div(tn.R0), nr = tn.R0 - nb * p.Rg;
-                if (elect_one_sync()) {
-#pragma unroll 1
-                    for (int s = 0; s < nseg_n; ++s) {
+        while (!w.done() && ok) {
+            // The tile's row table: -lse log2(e) and D; rows that do not exist get probability zero.
+            float st[4], dr[4];
 #pragma unroll
-                        for (int sl = 0; sl < C::kSlabs; ++sl) tma_prefetch_4d(&tm_do, sl * 64, nr, tn.g, nb);
-                        nr += p.seg_rows;
-                        if (nr >= p.Rg) {
-                            nr -= p.Rg;
-                            ++nb;
-                        }
-                    }
-                }
-                __syncwarp();
+            for (int i = 0; i < 4; ++i) {
+                const int row = 32 * i + lane, R = w.R0 + row;
+                const int c = p.fd_Rp.div(R), r = R - c * p.Rp;
+                const bool v = row < w.rows && r < p.Rg;
+                const size_t at = ((size_t)(w.b0 + c) * p.Hq + (size_t)w.g * p.n_rep) * p.S + r;
+                st[i] = v ? -p.lse[at] * kLog2e : -INFINITY;
+                dr[i] = v ? p.row_dot[at] : 0.f;
             }
-            const int nseg = p.fd_seg.div(t.rows);
-            int qb = p.fd_Rg.div(t.R0), qr = t.R0 - qb * p.Rg;
-            uint32_t do_dst = sbase + p.off_do;
-            ok = mbar_wait_warp(bar(kBarDvFree), (tl & 1) ^ 1, abort_flag, p.status, kErrProdB);
-            if (!ok) break;
-            if (elect_one_sync()) {
-                mbar_arrive_expect_tx(bar(kBarDoFull), (uint32_t)(nseg * C::kSlabs * p.seg_rows * 128));
-#pragma unroll 1
-                for (int s = 0; s < nseg; ++s) {
+            const int nb = (w.rows + step - 1) / step;
+            const int R = w.R0 + lane * step;
+            const int c = p.fd_Rp.div(R), r = R - c * p.Rp, g = w.g, b = w.b0 + c;
+            // While idle, ask for the next tile's rows in L2: the buffers are single, so their copies can only
+            // be issued right when they are needed.
+            w.next_tile(p);
+            if (!w.done() && lane < (w.rows + step - 1) / step) {
+                const int Rn = w.R0 + lane * step;
+                const int cn = p.fd_Rp.div(Rn), rn = Rn - cn * p.Rp;
 #pragma unroll
-                    for (int sl = 0; sl < C::kSlabs; ++sl)
-                        tma_load_4d(do_dst + sl * C::kSlabBytes, &tm_do, bar(kBarDoFull), sl * 64, qr, t.g, qb);
-                    do_dst += p.seg_rows * 128;
-                    qr += p.seg_rows;
-                    if (qr >= p.Rg) {
-                        qr -= p.Rg;
-                        ++qb;
-                    }
+                for (int sl = 0; sl < C::kSlabs; ++sl) {
+                    tma_prefetch_4d(&tm_q, sl * 64, rn, w.g, w.b0 + cn);
+                    tma_prefetch_4d(&tm_do, sl * 64, rn, w.g, w.b0 + cn);
                 }
-                if (RV && first_of_run(t, inst_of(t))) {
-                    for (int k = 0; k < p.nblk_p; ++k) {
-                        const bool tail = k == p.nblk_p - 1;
-                        const int slab = tail ? tail_slab : C::kSlabBytes;
-                        mbar_arrive_expect_tx(bar(kBarVFull + k), (uint32_t)(C::kSlabs * slab));
-                        for (int sl = 0; sl < C::kSlabs; ++sl)
-                            tma_load_3d(sbase + p.off_pv + k * C::kTileBytes + sl * slab, tail ? &tm_pv_tail : &tm_pv,
-                                        bar(kBarVFull + k), sl * 64, k * kBlockN, inst_of(t) * p.Hkv + t.g);
-                    }
-                }
-                mbar_arrive_expect_tx(bar(kBarSVFull), (uint32_t)(t.nc * C::kSlabs * p.S * 128));
-                for (int c = 0; c < t.nc; ++c)
-                    for (int sl = 0; sl < C::kSlabs; ++sl)
-                        tma_load_4d(sbase + p.off_sv + sl * sfx_slab + c * p.S * 128, &tm_sv, bar(kBarSVFull),
-                                    sl * 64, 0, t.g, t.b_first + c);
             }
             __syncwarp();
-            if (!RV) {
-#pragma unroll 1
-                for (int k = first_block(t); k < p.nblk_p; ++k) {
-                    const uint32_t vs = vload % stages_v;
-                    ok = mbar_wait_warp(bar(kBarVFree + vs), ((vload / stages_v) & 1) ^ 1, abort_flag, p.status, kErrProdB);
-                    if (!ok) break;
-                    const bool tail = k == p.nblk_p - 1;
-                    const int slab = tail ? tail_slab : C::kSlabBytes;
-                    if (elect_one_sync()) {
-                        mbar_arrive_expect_tx(bar(kBarVFull + vs), (uint32_t)(C::kSlabs * slab));
-                        for (int sl = 0; sl < C::kSlabs; ++sl)
-                            tma_load_3d(sbase + p.off_pv + vs * C::kTileBytes + sl * slab, tail ? &tm_pv_tail : &tm_pv,
-                                        bar(kBarVFull + vs), sl * 64, k * kBlockN, inst_of(t) * p.Hkv + t.g);
-                    }
-                    __syncwarp();
-                    ++vload;
+            ok = mbar_wait_warp(bar(kBarQFree), (tile & 1u) ^ 1u, abort_flag, p.status, kErrProdQ);
+            if (!ok) break;
+            PSKV_TRACE_EVENT(2, tile);
+            if (lane == 0) mbar_arrive_expect_tx(bar(kBarQFull), (uint32_t)(nb * 2 * C::kSlabs * step * 128));
+            __syncwarp();
+            if (lane < nb) {
+#pragma unroll
+                for (int sl = 0; sl < C::kSlabs; ++sl) {
+                    const uint32_t off = (uint32_t)(sl * C::kSlabBytes + lane * step * 128);
+                    tma_load_4d(sbase + p.off_q + off, &tm_q, bar(kBarQFull), sl * 64, r, g, b);
+                    tma_load_4d(sbase + p.off_do + off, &tm_do, bar(kBarQFull), sl * 64, r, g, b);
                 }
             }
+            // Table tile & 1 was last read for tile - 2; the MMAs behind kBarQFree of tile - 1 came after that.
+            float2 *rows = reinterpret_cast<float2 *>(smem + p.off_rows) + (tile & 1u) * kTileM;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) rows[32 * i + lane] = make_float2(st[i], dr[i]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarRowsFull + (tile & 1u)));
+            ++tile;
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------------ S = Q K^T
-        const int total_items = count_items();
-        int tl = 0;
-        uint32_t kuse = 0;
-        TileInfo t = tile_info(p, t_begin, t_begin);
-        int kf = first_block(t), k = kf;
+        // ------------------------------------------------------------------ S = Q K^T, dP = dO V^T
         const uint64_t q_desc = make_smem_desc(sbase + p.off_q, 0, 1024);
-        bool ok = true;
-#pragma unroll 1
-        for (int i = 0; i < total_items && ok; ++i) {
-            const int slot = i % kSlots;
-            const bool prefix = k < p.nblk_p;
-            const int n = prefix ? prefix_block_rows(p, k) : t.n_sfx;
-            const int slab = prefix ? n * 128 : sfx_slab;
-            const bool last_of_tile = k == nitems - 1;
-            const bool ring_k = prefix && !RK;
-            const uint32_t idesc = make_idesc_bf16(kTileM, n, 0);
-            const uint64_t slab16 = (uint64_t)(slab >> 4);
-            // ---- S: the slot is free once the dQ MMAs of item i-2 have completed
-            ok = mbar_wait_warp(bar(kBarDqDone + slot), ((i / kSlots) & 1) ^ 1, abort_flag, p.status, kErrMmaS);
-            if (!ok) break;
-            if (k == kf) ok = mbar_wait_warp(bar(kBarQFull), tl & 1, abort_flag, p.status, kErrMmaS);
-            if (!ok) break;
-            if (MI && RK && k == kf && first_of_run(t, inst_of(t))) {
-                // the resident blocks this run leaves out were fetched with the others: pass their barriers
-                // too, so that every block's barrier has completed once per run
-                for (int kk = 0; kk < kf && kk < p.nblk_p && ok; ++kk)
-                    ok = mbar_wait_warp(bar(kBarKFull + kk), (run_of(t, inst_of(t)) - run_first) & 1, abort_flag, p.status,
-                                        kErrMmaS);
-                if (!ok) break;
-            }
-            uint32_t kaddr;
-            if (prefix) {
-                if (RK) {
-                    if (first_of_run(t, inst_of(t)))
-                        ok = mbar_wait_warp(bar(kBarKFull + k), (run_of(t, inst_of(t)) - run_first) & 1, abort_flag,
-                                            p.status, kErrMmaS);
-                    kaddr = sbase + p.off_pk + k * C::kTileBytes;
-                } else {
-                    const uint32_t ks = kuse % stages_k;
-                    ok = mbar_wait_warp(bar(kBarKFull + ks), (kuse / stages_k) & 1, abort_flag, p.status, kErrMmaS);
-                    kaddr = sbase + p.off_pk + ks * C::kTileBytes;
-                }
-            } else {
-                ok = mbar_wait_warp(bar(kBarSKFull), tl & 1, abort_flag, p.status, kErrMmaS);
-                kaddr = sbase + p.off_sk;
-            }
-            if (!ok) break;
-            PSKV_TRACE_EVENT(10, i);
-            tc_fence_after();
-            {
-                const uint64_t k_desc = make_smem_desc(kaddr, 0, 1024);
-                const uint32_t d_tmem = tmem + slot * kBlockN;
-                if (elect_one_sync()) {
-#pragma unroll
-                    for (int ks16 = 0; ks16 < D / 16; ++ks16) {
-                        const uint64_t qoff = (uint64_t)(((ks16 >> 2) * C::kSlabBytes + (ks16 & 3) * 32) >> 4);
-                        const uint64_t koff = (uint64_t)(ks16 >> 2) * slab16 + (uint64_t)(((ks16 & 3) * 32) >> 4);
-                        mma_ss(d_tmem, q_desc + qoff, k_desc + koff, idesc, ks16 > 0 ? 1u : 0u);
-                    }
-                    tc_commit(bar(kBarSFull + slot));
-                    if (last_of_tile) tc_commit(bar(kBarQkFree));
-                }
-                __syncwarp();
-            }
-            if (ring_k) ++kuse;
-            if (++k == nitems) {
-                if (++tl < n_tiles) {
-                    t = tile_info(p, t_begin + tl, t_begin);
-                    kf = first_block(t);
-                }
-                k = kf;
-            }
-        }
-    } else if (warp == 2) {
-        // ------------------------------------------------------------------ dP = dO V^T, dQ += dS K
-        // This warp alternates: dP of item i+1 (its buffer comes free early in the element-wise
-        // stage of item i), then dQ of item i (whose dS comes at the end of that stage).  The score
-        // MMAs of warp 1 run beside both, so two threads keep the tensor pipe fed.
-        const int total_items = count_items();
-        int tl = 0;
-        uint32_t kuse = 0;
-        TileInfo t = tile_info(p, t_begin, t_begin);
-        int kf = first_block(t), k = kf;
-        const uint32_t idesc_dq = make_idesc_bf16(kTileM, D, 1);
         const uint64_t do_desc = make_smem_desc(sbase + p.off_do, 0, 1024);
-        bool ok = true;
-        // cursor of the dP stream
-        int ptl = 0, pkf = kf, pk = kf;
-        uint32_t vuse = 0;
-        TileInfo pt = t;
-        auto issue_dp = [&](int i) -> bool {
-            const int tl = ptl, k = pk;
-            const TileInfo &t = pt;
-            const bool prefix = k < p.nblk_p;
-            const int n = prefix ? prefix_block_rows(p, k) : t.n_sfx;
-            const int slab = prefix ? n * 128 : sfx_slab;
-            const bool last_of_tile = k == nitems - 1;
-            const bool ring_v = prefix && !RV;
-            const uint32_t idesc = make_idesc_bf16(kTileM, n, 0);
-            const uint64_t slab16 = (uint64_t)(slab >> 4);
-            bool ok = true;
-                // ---- dP: its single slot is free once the element-wise warps have read item i-1
-                ok = mbar_wait_warp(bar(kBarDpFree), (i & 1) ^ 1, abort_flag, p.status, kErrMmaDq);
-                if (!ok) return false;
-                if (k == pkf) ok = mbar_wait_warp(bar(kBarDoFull), tl & 1, abort_flag, p.status, kErrMmaDq);
-                if (!ok) return false;
-                if (MI && RV && k == pkf && first_of_run(t, inst_of(t))) {  // (as for the K blocks in warp 1)
-                    for (int kk = 0; kk < pkf && kk < p.nblk_p && ok; ++kk)
-                        ok = mbar_wait_warp(bar(kBarVFull + kk), (run_of(t, inst_of(t)) - run_first) & 1, abort_flag,
-                                            p.status, kErrMmaDq);
-                    if (!ok) return false;
-                }
-                uint32_t vaddr;
-                if (prefix) {
-                    if (RV) {
-                        if (first_of_run(t, inst_of(t)))
-                            ok = mbar_wait_warp(bar(kBarVFull + k), (run_of(t, inst_of(t)) - run_first) & 1, abort_flag,
-                                                p.status, kErrMmaDq);
-                        vaddr = sbase + p.off_pv + k * C::kTileBytes;
-                    } else {
-                        const uint32_t vs = vuse % stages_v;
-                        ok = mbar_wait_warp(bar(kBarVFull + vs), (vuse / stages_v) & 1, abort_flag, p.status, kErrMmaDq);
-                        vaddr = sbase + p.off_pv + vs * C::kTileBytes;
-                    }
-                } else {
-                    ok = mbar_wait_warp(bar(kBarSVFull), tl & 1, abort_flag, p.status, kErrMmaDq);
-                    vaddr = sbase + p.off_sv;
-                }
-                if (!ok) return false;
-                PSKV_TRACE_EVENT(12, i);
-                tc_fence_after();
-                {
-                    const uint64_t v_desc = make_smem_desc(vaddr, 0, 1024);
-                    if (elect_one_sync()) {
-#pragma unroll
-                        for (int ks16 = 0; ks16 < D / 16; ++ks16) {
-                            const uint64_t aoff = (uint64_t)(((ks16 >> 2) * C::kSlabBytes + (ks16 & 3) * 32) >> 4);
-                            const uint64_t voff = (uint64_t)(ks16 >> 2) * slab16 + (uint64_t)(((ks16 & 3) * 32) >> 4);
-                            mma_ss(tmem + kDpCol, do_desc + aoff, v_desc + voff, idesc, ks16 > 0 ? 1u : 0u);
-                        }
-                        tc_commit(bar(kBarDpFull));
-                        if (ring_v) tc_commit(bar(kBarVFree + (vuse % stages_v)));
-                        if (last_of_tile) tc_commit(bar(kBarDvFree));
-                    }
-                    __syncwarp();
-                }
-            if (!ok) return false;
-            if (ring_v) ++vuse;
-            if (++pk == nitems) {
-                if (++ptl < n_tiles) {
-                    pt = tile_info(p, t_begin + ptl, t_begin);
-                    pkf = first_block(pt);
-                }
-                pk = pkf;
-            }
-            return true;
-        };
-        if (total_items > 0) ok = issue_dp(0);
+        const uint4 *descs = reinterpret_cast<const uint4 *>(smem + p.off_bar + kDescOff);
+        int ks = 0, vs = 0;
+        uint32_t kph = 0, vph = 0;
 #pragma unroll 1
-        for (int i = 0; i < total_items && ok; ++i) {
-            if (i + 1 < total_items) {
-                ok = issue_dp(i + 1);
-                if (!ok) break;
-            }
-            const int slot = i % kSlots;
-            const bool prefix = k < p.nblk_p;
-            const int n = prefix ? prefix_block_rows(p, k) : t.n_sfx;
-            const int slab = prefix ? n * 128 : sfx_slab;
-            const bool last_of_tile = k == nitems - 1;
-            const bool ring = prefix && !RK;
-            ok = mbar_wait_warp(bar(kBarDsReady + slot), (i / kSlots) & 1, abort_flag, p.status, kErrMmaDq);
+        for (uint32_t item = 0;; ++item) {
+            const uint32_t slot = item & 1u;
+            const uint32_t d_tmem = tmem + slot * kSlotCols;
+            const uint64_t k_desc = make_smem_desc(sbase + p.off_k + ks * C::kPieceBytes, 0, 1024);
+            const uint64_t v_desc = make_smem_desc(sbase + p.off_v + vs * C::kPieceBytes, 0, 1024);
+            PSKV_TRACE_EVENT(12, item);
+            ok = mbar_wait_warp(bar(kBarKFull + ks), kph, abort_flag, p.status, kErrMmaS);
             if (!ok) break;
-            if (k == kf && tl > 0) {
-                ok = mbar_wait_warp(bar(kBarDqFree), (tl - 1) & 1, abort_flag, p.status, kErrMmaDq);
-                if (!ok) break;
-            }
-            uint32_t kaddr;
-            if (prefix) kaddr = sbase + p.off_pk + (RK ? (uint32_t)k : kuse % stages_k) * C::kTileBytes;
-            else kaddr = sbase + p.off_sk;
-            PSKV_TRACE_EVENT(11, i);
+            const uint32_t x = __shfl_sync(0xffffffffu, descs[item & 7u].x, 0);
+            if (x & kDescEnd) break;
+            const uint32_t idesc = make_idesc_bf16(kTileM, (int)(x & kDescN), 0);
+            if (x & kDescFirst) ok = mbar_wait_warp(bar(kBarQFull), descs[item & 7u].w & 1u, abort_flag, p.status, kErrMmaS);
+            if (ok) ok = mbar_wait_warp(bar(kBarSFree + slot), ((item >> 1) & 1u) ^ 1u, abort_flag, p.status, kErrMmaS);
+            if (ok) ok = mbar_wait_warp(bar(kBarVFull + vs), vph, abort_flag, p.status, kErrMmaS);
+            if (!ok) break;
+            PSKV_TRACE_EVENT(15, item);
             tc_fence_after();
-            const uint32_t ds_tmem = tmem + slot * kBlockN;  // bf16 pairs: 8 columns per 16 keys
-            const uint64_t k_desc = make_smem_desc(kaddr, (uint32_t)slab, 1024);  // K as [keys][d]: d contiguous
-            const int nk = n >> 4;
-            const uint32_t acc0 = k > kf ? 1u : 0u;
             if (elect_one_sync()) {
 #pragma unroll
-                for (int ks16 = 0; ks16 < kBlockN / 16; ++ks16) {
-                    if (ks16 < nk)
-                        mma_ts(tmem + kDqCol, ds_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8, k_desc + (uint64_t)(ks16 * (2048 >> 4)), idesc_dq,
-                               ks16 > 0 ? 1u : acc0);
+                for (int i = 0; i < D / 16; ++i) {
+                    const uint64_t aoff = (uint64_t)(((i >> 2) * C::kSlabBytes + (i & 3) * 32) >> 4);
+                    const uint64_t boff = (uint64_t)(((i >> 2) * C::kPieceSlab + (i & 3) * 32) >> 4);
+                    mma_ss(d_tmem, q_desc + aoff, k_desc + boff, idesc, i > 0 ? 1u : 0u);
                 }
-                tc_commit(bar(kBarDqDone + slot));
-                if (ring) tc_commit(bar(kBarKFree + (kuse % stages_k)));
-                if (last_of_tile) tc_commit(bar(kBarDqFull));
+#pragma unroll
+                for (int i = 0; i < D / 16; ++i) {
+                    const uint64_t aoff = (uint64_t)(((i >> 2) * C::kSlabBytes + (i & 3) * 32) >> 4);
+                    const uint64_t boff = (uint64_t)(((i >> 2) * C::kPieceSlab + (i & 3) * 32) >> 4);
+                    mma_ss(d_tmem + kColDp, do_desc + aoff, v_desc + boff, idesc, i > 0 ? 1u : 0u);
+                }
+                tc_commit(bar(kBarSFull + slot));
+                tc_commit(bar(kBarVFree + vs));
+                if (x & kDescLast) tc_commit(bar(kBarQFree));
             }
             __syncwarp();
-            if (ring) ++kuse;
-            if (++k == nitems) {
-                if (++tl < n_tiles) {
-                    t = tile_info(p, t_begin + tl, t_begin);
-                    kf = first_block(t);
-                }
-                k = kf;
-            }
+            PSKV_TRACE_EVENT(10, item);
+            if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
+            if (++vs == p.stages_v) { vs = 0; vph ^= 1u; }
         }
-    } else if (warp < 4 + 4 * kGroups) {
-        // ------------------------------------------------------------------ element-wise warps (4..19)
-        // Four warpgroups share every item: the 128 score columns are four pieces of 32 and group j
-        // takes piece j.  Thread <-> query row (tensor-memory lane).  Each thread pulls its piece
-        // of S and of dP into registers, hands dP back at once (the next item's dP MMAs are
-        // waiting for that buffer), then forms dS = 2^(S sl2 - lse2) (dP - D) and writes it as
-        // bf16 pairs over the first half of the S piece it came from.
-        const int wg = (warp - 4) >> 2;
-        const int row = 32 * (warp & 3) + lane;
-        const int c0 = wg * kPiece;  // first column of my piece
-        const uint32_t my_tmem = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + c0;
-        int item = 0;
-        bool ok = true;
+    } else if (warp == 2) {
+        // ------------------------------------------------------------------ dQ += dS K, dV^T += dO^T P, dK^T += Q^T dS
+        const uint32_t idesc_dq = make_idesc_bf16(kTileM, D, 1);
+        // A operands with d contiguous.  Head dim 128: two 64-column slabs of dO / of Q.  Head dim 64: M is still
+        // 128, rows 0-63 from the slab of dO and rows 64-127 from the slab of Q, which lies behind it.
+        const uint64_t dot_desc = make_smem_desc(sbase + p.off_do, D == 128 ? C::kSlabBytes : p.off_q - p.off_do, 1024);
+        const uint64_t qt_desc = D == 128 ? make_smem_desc(sbase + p.off_q, C::kSlabBytes, 1024) : dot_desc;
+        const uint64_t p_desc = make_smem_desc(sbase + p.off_p, kDsBytes, 1024);
+        const uint4 *descs = reinterpret_cast<const uint4 *>(smem + p.off_bar + kDescOff);
+        int ks = 0;
+        uint32_t kph = 0, dqph = 1, accph = 1;
 #pragma unroll 1
-        for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info(p, t_begin + tl, t_begin);
-            const bool valid = row < t.rows;
-            const int R = t.R0 + (valid ? row : 0);
-            const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-            const int sfx_lo = (b - t.b_first) * p.S;
-            const int sfx_hi = sfx_lo + (r - p.fd_S.div(r) * p.S);
-            const size_t grow = ((size_t)b * p.Hq + (size_t)t.g * p.n_rep) * p.S + r;
-            // padding rows: lse = +inf makes every probability (and so every dS) zero
-            const float neg_lse2 = valid ? -p.lse[grow] * kLog2e : -INFINITY;
-            const float drow = valid ? p.row_dot[grow] : 0.f;
-            const int pad = MI ? p.pad[inst_of(t)] : 0;
-#pragma unroll 1
-            for (int k = pad / kBlockN; k < nitems && ok; ++k, ++item) {
-                const int slot = item % kSlots;
-                int n, lo, hi;
-                if (k < p.nblk_p) {
-                    n = prefix_block_rows(p, k);
-                    lo = max(0, pad - k * kBlockN);  // left padding of this tile's instruction
-                    hi = min(kBlockN, p.P - k * kBlockN) - 1;
-                } else {
-                    n = t.n_sfx;
-                    lo = valid ? sfx_lo : 1;
-                    hi = valid ? sfx_hi : 0;
-                }
-                // my piece: 0 = not read by the dQ MMAs, 1 = no valid column for any row of this
-                // warp (zeros), 2 = some columns masked, 3 = every column valid for every row
-                int kind = 0;
-                if (c0 < n) {
-                    const bool all_valid = lo <= c0 && hi >= c0 + kPiece - 1;
-                    const bool none_valid = hi < lo || hi < c0 || lo > c0 + kPiece - 1;
-                    kind = __all_sync(0xffffffffu, all_valid) ? 3 : __all_sync(0xffffffffu, none_valid) ? 1 : 2;
-                }
-                const uint32_t s_tmem = my_tmem + slot * kBlockN;
-                const uint32_t dp_tmem = my_tmem + kDpCol;
-
-                ok = mbar_wait_warp(bar(kBarSFull + slot), (item / kSlots) & 1, abort_flag, p.status, kErrElem);
-                if (!ok) break;
-                ok = mbar_wait_warp(bar(kBarDpFull), item & 1, abort_flag, p.status, kErrElem);
-                if (!ok) break;
-                PSKV_TRACE_EVENT(20, item);
-                tc_fence_after();
-                // two halves of 16 columns; dP goes back as soon as the second half is in registers
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    constexpr int kHalf = kPiece / 2;
-                    uint32_t rs[kHalf], rd[kHalf], pk[kHalf / 2];
-                    if (kind >= 2) {
-                        tmem_ld16(s_tmem + hf * kHalf, rs);
-                        tmem_ld16(dp_tmem + hf * kHalf, rd);
-                        tmem_wait_ld();
-                    }
-                    if (hf == 1) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(bar(kBarDpFree));
-                    }
-                    if (kind >= 2) {
-                        float e[kHalf];
-#pragma unroll
-                        for (int c = 0; c < kHalf; c += 2) {
-                            float x0 = __uint_as_float(rs[c]), x1 = __uint_as_float(rs[c + 1]);
-                            fma_f32x2(x0, x1, p.sl2, neg_lse2);
-                            e[c] = ex2_approx(x0);
-                            e[c + 1] = ex2_approx(x1);
-                        }
-                        if (kind == 2) {
-                            const unsigned span = (unsigned)(hi - lo);
-                            const int base = c0 + hf * kHalf - lo;
-                            const bool any_col = hi >= lo;
-#pragma unroll
-                            for (int c = 0; c < kHalf; ++c) e[c] = (any_col && (unsigned)(base + c) <= span) ? e[c] : 0.f;
-                        }
-#pragma unroll
-                        for (int c = 0; c < kHalf / 2; ++c) {
-                            float d0 = __uint_as_float(rd[2 * c]), d1 = __uint_as_float(rd[2 * c + 1]);
-                            add_f32x2(d0, d1, -drow, -drow);
-                            mul_f32x2(d0, d1, e[2 * c], e[2 * c + 1]);
-                            pk[c] = pack_bf16x2(d0, d1);
-                        }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < kHalf / 2; ++c) pk[c] = 0u;
-                    }
-                    if (kind != 0) tmem_st8(s_tmem + hf * (kHalf / 2), pk);
-                }
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kBarDsReady + slot));
-                PSKV_TRACE_EVENT(24, item);
+        for (uint32_t item = 0;; ++item) {
+            const uint32_t slot = item & 1u;
+            const uint64_t ds_a = make_smem_desc(sbase + p.off_ds + slot * kDsBytes, kDsBytes, 1024);
+            const uint64_t k_desc = make_smem_desc(sbase + p.off_k + ks * C::kPieceBytes, C::kPieceSlab, 1024);
+            ok = mbar_wait_warp(bar(kBarKFull + ks), kph, abort_flag, p.status, kErrMmaGrad);
+            if (!ok) break;
+            const uint32_t x = __shfl_sync(0xffffffffu, descs[item & 7u].x, 0);
+            if (x & kDescEnd) break;
+            const int n = (int)(x & kDescN);
+            const uint32_t acc0 = (x & kDescFirst) ? 0u : 1u;
+            PSKV_TRACE_EVENT(13, item);
+            ok = mbar_wait_warp(bar(kBarDsReady + slot), (item >> 1) & 1u, abort_flag, p.status, kErrMmaGrad);
+            if (ok && (x & (kDescDq | kDescFirst)) == (kDescDq | kDescFirst)) {  // the previous dQ must have been read out
+                ok = mbar_wait_warp(bar(kBarDqFree), dqph, abort_flag, p.status, kErrMmaGrad);
+                dqph ^= 1u;
             }
+            if (!ok) break;
+            tc_fence_after();
+            if ((x & kDescDq) && elect_one_sync()) {
+#pragma unroll
+                for (int i = 0; i < kPieceN / 16; ++i)
+                    if (i * 16 < n)
+                        mma_ss(tmem + kColDq, ds_a + (uint64_t)(i * 32 >> 4), k_desc + (uint64_t)(i * 2048 >> 4), idesc_dq,
+                               i > 0 ? 1u : acc0);
+            }
+            __syncwarp();
+            if (x & kDescAcc) {
+                if (x & kDescAccFirst) {
+                    PSKV_TRACE_EVENT(16, item);
+                    ok = mbar_wait_warp(bar(kBarAccFree), accph, abort_flag, p.status, kErrMmaGrad);
+                    accph ^= 1u;
+                    if (!ok) break;
+                    tc_fence_after();
+                }
+                PSKV_TRACE_EVENT(11, item);
+                const uint32_t idesc_acc = make_idesc_bf16_ab(128, n, 1, 1);
+                // rows of the tile that belong to the group (the others are zero in P and dS)
+                const int k0 = (int)((x >> kDescK0) & 15u), k1 = (int)((x >> kDescK1) & 15u);
+                if (elect_one_sync()) {
+                    uint32_t a = (x & kDescAccFirst) ? 0u : 1u;
+#pragma unroll 1
+                    for (int i = k0; i < k1; ++i) {
+                        const uint64_t off = (uint64_t)(i * (2048 >> 4));
+                        mma_ss(tmem + kColDv, dot_desc + off, p_desc + off, idesc_acc, a);
+                        mma_ss(tmem + kColDk, qt_desc + off, ds_a + off, idesc_acc, a);
+                        a = 1u;
+                    }
+                    tc_commit(bar(kBarPFree));
+                    if (x & kDescAccLast) tc_commit(bar(kBarAccFull));
+                    if (x & kDescQDone) tc_commit(bar(kBarQFree));
+                }
+                __syncwarp();
+            }
+            if (elect_one_sync()) {
+                tc_commit(bar(kBarDsFree + slot));
+                tc_commit(bar(kBarKFree + ks));
+                if ((x & (kDescLast | kDescDq)) == (kDescLast | kDescDq)) tc_commit(bar(kBarDqFull));
+            }
+            __syncwarp();
+            PSKV_TRACE_EVENT(14, item);
+            if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
+        }
+    } else if (warp < 20) {
+        // ------------------------------------------------------------------ element-wise warps (4..19)
+        const int set = (warp - 4) >> 3;        // items of parity `set`
+        const int c0 = ((warp >> 2) & 1) ? 0 : 32;   // my 32 of the piece's 64 keys
+        const int row = 32 * (warp & 3) + lane;
+        const uint32_t my_tmem = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + set * kSlotCols + c0;
+        uint8_t *p_row = smem + p.off_p + row * 128;
+        uint8_t *ds_row = smem + p.off_ds + set * kDsBytes + row * 128;
+        const uint4 *descs = reinterpret_cast<const uint4 *>(smem + p.off_bar + kDescOff);
+        int ks = set;
+        uint32_t kph = 0, tile = 0xffffffffu;  // (no tile has this number and index)
+        if (ks >= p.stages_k) { ks -= p.stages_k; kph ^= 1u; }
+        float neg_lse2 = 0.f, drow = 0.f;
+        int my_grp = -1, my_lo = 0, my_hi = 0;
+#pragma unroll 1
+        for (uint32_t item = (uint32_t)set;; item += 2) {
+            const uint32_t sph = (item >> 1) & 1u;
+            PSKV_TRACE_EVENT(26, item);
+            ok = mbar_wait_warp(bar(kBarKFull + ks), kph, abort_flag, p.status, kErrElem);
+            if (!ok) break;
+            const uint4 dsc = descs[item & 7u];
+            if (dsc.x & kDescEnd) break;
+            ks += 2;
+            if (ks >= p.stages_k) {
+                ks -= p.stages_k;
+                kph ^= 1u;
+            }
+            if (dsc.w != tile) {
+                tile = dsc.w;
+                ok = mbar_wait_warp(bar(kBarRowsFull + (tile & 1u)), (tile >> 1) & 1u, abort_flag, p.status, kErrElem);
+                if (!ok) break;
+                const float2 rt = reinterpret_cast<const float2 *>(smem + p.off_rows)[(tile & 1u) * kTileM + row];
+                neg_lse2 = rt.x;
+                drow = rt.y;
+                // candidate group of my row, first key column of its candidate in the piece, last visible one
+                const int R = (int)(tile >> 16) * kTileM + row, c = p.fd_Rp.div(R), r = R - c * p.Rp;
+                my_grp = p.fd_cpp.div(c);
+                my_lo = (c - my_grp * p.cpp) * p.Sp;
+                my_hi = my_lo + r - p.fd_S.div(r) * p.S;
+            }
+            const bool acc = (dsc.x & kDescAcc) != 0u;
+            int lo, hi;  // visible columns of my row
+            if (dsc.x & kDescSfx) {
+                const bool mine = (int)dsc.y == my_grp;
+                lo = mine ? my_lo : 1;
+                hi = mine ? my_hi - (int)dsc.z : 0;
+            } else {
+                lo = (int)(dsc.y & 0xffu);
+                hi = (int)(dsc.y >> 8);
+            }
+            // my 32 columns: 0 = not read by the MMAs, 1 = nothing visible to any row of this warp (zeros),
+            // 2 = some masked, 3 = all visible to all rows
+            int kind = 0;
+            if (c0 < (int)(dsc.x & kDescN)) {
+                const bool all_valid = lo <= c0 && hi >= c0 + 31;
+                const bool none_valid = hi < lo || hi < c0 || lo > c0 + 31;
+                kind = __all_sync(0xffffffffu, all_valid) ? 3 : __all_sync(0xffffffffu, none_valid) ? 1 : 2;
+            }
+            PSKV_TRACE_EVENT(25, item);
+            ok = mbar_wait_warp(bar(kBarSFull + set), sph, abort_flag, p.status, kErrElem);
+            if (!ok) break;
+            PSKV_TRACE_EVENT(20, item);
+            tc_fence_after();
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t rs[16], rd[16], pk[8], pp[8];
+                if (kind >= 2) {
+                    tmem_ld16(my_tmem + hf * 16, rs);
+                    tmem_ld16(my_tmem + kColDp + hf * 16, rd);
+                    tmem_wait_ld();
+                }
+                if (hf == 1) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kBarSFree + set));
+                }
+                if (kind >= 2) {
+                    float e[16];
+#pragma unroll
+                    for (int i = 0; i < 16; i += 2) {
+                        float x0 = __uint_as_float(rs[i]), x1 = __uint_as_float(rs[i + 1]);
+                        fma_f32x2(x0, x1, p.sl2, neg_lse2);
+                        e[i] = ex2_approx(x0);
+                        e[i + 1] = ex2_approx(x1);
+                    }
+                    if (kind == 2) {
+                        const unsigned span = (unsigned)(hi - lo);
+                        const int base = c0 + hf * 16 - lo;
+                        const bool any_col = hi >= lo;
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) e[i] = (any_col && (unsigned)(base + i) <= span) ? e[i] : 0.f;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        float d0 = __uint_as_float(rd[2 * i]), d1 = __uint_as_float(rd[2 * i + 1]);
+                        add_f32x2(d0, d1, -drow, -drow);
+                        mul_f32x2(d0, d1, e[2 * i], e[2 * i + 1]);
+                        pk[i] = pack_bf16x2(d0, d1);
+                        pp[i] = pack_bf16x2(e[2 * i], e[2 * i + 1]);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) pk[i] = pp[i] = 0u;
+                }
+                if (hf == 0) {
+                    PSKV_TRACE_EVENT(21, item);
+                    ok = mbar_wait_warp(bar(kBarDsFree + set), sph ^ 1u, abort_flag, p.status, kErrElem);
+                    if (ok && acc)
+                        ok = mbar_wait_warp(bar(kBarPFree), (dsc.x & kDescAccOdd) ? 0u : 1u, abort_flag, p.status, kErrElem);
+                    if (!ok) break;
+                    PSKV_TRACE_EVENT(22, item);
+                }
+                if (kind != 0) {
+                    // 128-byte rows, 16-byte chunks swizzled by the row
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int off = (((c0 >> 3) + 2 * hf + i) ^ (row & 7)) << 4;
+                        *reinterpret_cast<uint4 *>(ds_row + off) = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                        if (acc)
+                            *reinterpret_cast<uint4 *>(p_row + off) = make_uint4(pp[4 * i], pp[4 * i + 1], pp[4 * i + 2], pp[4 * i + 3]);
+                    }
+                }
+            }
+            if (!ok) break;
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarDsReady + set));
+            PSKV_TRACE_EVENT(24, item);
         }
     } else {
         // ------------------------------------------------------------------ epilogue warps (20..23)
         const int ew = warp & 3;
         const int row = 32 * ew + lane;
         const uint32_t lane_addr = (uint32_t)(32 * ew) << 16;
-        const uint32_t stage = sbase + p.off_stage;
-        const bool issuer = warp == 4 + 4 * kGroups;
-        if (issuer && lane == 0) prefetch_tensormap(&tm_dq);
-        bool ok = true;
+        uint32_t dqph = 0, accph = 0;
 #pragma unroll 1
-        for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info(p, t_begin + tl, t_begin);
-            ok = mbar_wait_warp(bar(kBarDqFull), tl & 1, abort_flag, p.status, kErrEpi);
-            if (!ok) break;
-            tc_fence_after();
-            const int nseg = p.fd_seg.div(t.rows);
-            // dQ leaves tensor memory in two load round trips back to back (the first slab is scaled and packed
-            // to bf16 in registers while the second one is on its way) and goes back to the MMA issuer right
-            // after them: the first dQ MMAs of the next tile wait for exactly that, and with the first slab's
-            // staging and stores between the two loads they waited 2 500-4 100 cycles a tile.
-            uint32_t pk0[C::kSlabs > 1 ? 32 : 1];
-            uint32_t o0[32], o1[32];
-            tmem_ld32(tmem + lane_addr + kDqCol, o0);
-            tmem_ld32(tmem + lane_addr + kDqCol + 32, o1);
-            tmem_wait_ld();
-            if (C::kSlabs > 1) {
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    pk0[c] = pack_bf16x2(__uint_as_float(o0[2 * c]) * p.scale, __uint_as_float(o0[2 * c + 1]) * p.scale);
-                    pk0[16 + c] = pack_bf16x2(__uint_as_float(o1[2 * c]) * p.scale, __uint_as_float(o1[2 * c + 1]) * p.scale);
-                }
-                tmem_ld32(tmem + lane_addr + kDqCol + 64, o0);
-                tmem_ld32(tmem + lane_addr + kDqCol + 96, o1);
-                tmem_wait_ld();
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarDqFree));
+        for (; !w.done() && ok; w.next_tile(p)) {
 #pragma unroll 1
-            for (int sl = 0; sl < C::kSlabs; ++sl) {
-                const uint32_t round = (uint32_t)(tl * C::kSlabs + sl);
-                ok = mbar_wait_warp(bar(kBarStageFree), (round & 1) ^ 1, abort_flag, p.status, kErrEpi);
+            for (; w.j < w.n_sfx; ++w.j) {
+                const int h = w.half(p), gr = w.grp(p);
+                if (!w.acc(h) || w.grp_row1(p, gr) > w.R0 + kTileM) continue;
+                // ---- accumulators of a candidate group: lane <-> column d, tensor-memory column <-> key
+                ok = mbar_wait_warp(bar(kBarAccFull), accph, abort_flag, p.status, kErrEpi);
                 if (!ok) break;
-                uint8_t *srow = smem + p.off_stage + row * 128;
-                if (C::kSlabs > 1 && sl == 0) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        *reinterpret_cast<uint4 *>(srow + ((c ^ (row & 7)) << 4)) =
-                            make_uint4(pk0[4 * c], pk0[4 * c + 1], pk0[4 * c + 2], pk0[4 * c + 3]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint4 v;
-                        v.x = pack_bf16x2(__uint_as_float(o0[8 * c]) * p.scale, __uint_as_float(o0[8 * c + 1]) * p.scale);
-                        v.y = pack_bf16x2(__uint_as_float(o0[8 * c + 2]) * p.scale, __uint_as_float(o0[8 * c + 3]) * p.scale);
-                        v.z = pack_bf16x2(__uint_as_float(o0[8 * c + 4]) * p.scale, __uint_as_float(o0[8 * c + 5]) * p.scale);
-                        v.w = pack_bf16x2(__uint_as_float(o0[8 * c + 6]) * p.scale, __uint_as_float(o0[8 * c + 7]) * p.scale);
-                        *reinterpret_cast<uint4 *>(srow + ((c ^ (row & 7)) << 4)) = v;
+                accph ^= 1u;
+                PSKV_TRACE_EVENT(30, w.u);
+                tc_fence_after();
+                const int n = w.n16(p);
+                int b = w.b0 + gr * p.cpp, t = h * kPieceN;   // candidate and key of the coming eight columns
+                const int b_end = w.b0 + w.ncand;
+#pragma unroll 1
+                for (int col = 0; col < n; col += 16) {
+                    uint32_t av[16], ak[16];
+                    if (D == 128 || ew < 2) tmem_ld16(tmem + lane_addr + kColDv + col, av);
+                    if (D == 128 || ew >= 2) tmem_ld16(tmem + lane_addr + kColDk + col, ak);
+                    tmem_wait_ld();
+                    if (col + 16 >= n) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kBarAccFree));
                     }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint4 v;
-                        v.x = pack_bf16x2(__uint_as_float(o1[8 * c]) * p.scale, __uint_as_float(o1[8 * c + 1]) * p.scale);
-                        v.y = pack_bf16x2(__uint_as_float(o1[8 * c + 2]) * p.scale, __uint_as_float(o1[8 * c + 3]) * p.scale);
-                        v.z = pack_bf16x2(__uint_as_float(o1[8 * c + 4]) * p.scale, __uint_as_float(o1[8 * c + 5]) * p.scale);
-                        v.w = pack_bf16x2(__uint_as_float(o1[8 * c + 6]) * p.scale, __uint_as_float(o1[8 * c + 7]) * p.scale);
-                        *reinterpret_cast<uint4 *>(srow + (((4 + c) ^ (row & 7)) << 4)) = v;
+                    for (int i8 = 0; i8 < 16; i8 += 8) {
+                        // eight columns lie inside one candidate (Sp is a multiple of 8)
+                        const size_t o = (((size_t)b * p.Hkv + w.g) * p.S + t) * D + (D == 128 ? row : row & 63);
+                        const int nk = b < b_end ? p.S - t : 0;
+                        if (D == 128 || ew < 2) {
+                            __nv_bfloat16 *dst = p.dv + o;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                if (i < nk) dst[i * D] = __float2bfloat16_rn(__uint_as_float(av[i8 + i]));
+                        }
+                        if (D == 128 || ew >= 2) {
+                            __nv_bfloat16 *dst = p.dk + o;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                if (i < nk) dst[i * D] = __float2bfloat16_rn(__uint_as_float(ak[i8 + i]) * p.scale);
+                        }
+                        t += 8;
+                        if (t == p.Sp && p.cpp > 1) {
+                            t = 0;
+                            ++b;
+                        }
                     }
                 }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kBarStageFull));
-                if (issuer) {
-                    ok = mbar_wait_warp(bar(kBarStageFull), round & 1, abort_flag, p.status, kErrEpi);
-                    if (!ok) break;
-                    if (elect_one_sync()) {
-                        for (int s = 0; s < nseg; ++s) {
-                            const int R = t.R0 + s * p.seg_rows;
-                            const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-                            tma_store_4d(&tm_dq, stage + s * p.seg_rows * 128, sl * 64, r, t.g, b);
-                        }
-                        tma_store_commit();
-                        tma_store_wait_read();
-                        mbar_arrive(bar(kBarStageFree));
-                    }
+                PSKV_TRACE_EVENT(31, w.u);
+            }
+            if (!ok) break;
+            if (w.pass != 0) continue;
+            // ---- dQ of the tile
+            ok = mbar_wait_warp(bar(kBarDqFull), dqph, abort_flag, p.status, kErrEpi);
+            if (!ok) break;
+            dqph ^= 1u;
+            PSKV_TRACE_EVENT(33, w.u);
+            tc_fence_after();
+            const int R = w.R0 + row, c = p.fd_Rp.div(R), r = R - c * p.Rp;
+            const bool stored = row < w.rows && r < p.Rg;
+            __nv_bfloat16 *dst = p.dq + (((size_t)(w.b0 + c) * p.Hq + (size_t)w.g * p.n_rep) * p.S + r) * D;
+#pragma unroll 1
+            for (int q4 = 0; q4 < D / 32; ++q4) {
+                uint32_t o[32], v[16];
+                tmem_ld32(tmem + lane_addr + kColDq + q4 * 32, o);
+                tmem_wait_ld();
+                if (q4 == D / 32 - 1) {
+                    tc_fence_before();
                     __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kBarDqFree));
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    v[i] = pack_bf16x2(__uint_as_float(o[2 * i]) * p.scale, __uint_as_float(o[2 * i + 1]) * p.scale);
+                if (stored) {
+                    store_sector(dst + q4 * 32, v, p.dq_sectors != 0);
+                    store_sector(dst + q4 * 32 + 16, v + 8, p.dq_sectors != 0);
                 }
             }
+            PSKV_TRACE_EVENT(34, w.u);
         }
-        if (issuer && elect_one_sync()) tma_store_wait_all();
     }
 
     PSKV_TRACE_FLUSH;
-    if (*abort_flag != 0) __nanosleep(20000);
+    if (*abort_flag != 0) __nanosleep(20000);  // let copies and MMAs still in flight drain
     tc_fence_before();
     __syncthreads();
     if (warp == 2) tmem_dealloc(tmem, 512);
@@ -783,167 +797,160 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 
 struct BwdPlan {
     bool ok;
-    int tile_rows, seg_rows, tiles_per_group, sfx_rows;
-    int nblk_p, tail_rows, resident, stages_k, stages_v;
-    int off_pk, off_pv, off_q, off_do, off_sk, off_sv, off_stage, off_bar, off_misc, smem_bytes;
+    int cu, cpp, nh, Rp, Sp, seg, cbox, sfx_box, nblk, upi;
+    int stages_k, stages_v;
+    int off_do, off_q, off_k, off_v, off_p, off_ds, off_rows, off_bar, off_misc, smem_bytes;
 };
 
-BwdPlan plan_bwd(const Dims &dm)
+// Chooses the candidates per unit and lays out shared memory.  The cost of a choice is what the busiest SM
+// does: its units times their items (64-key pieces summed over tiles and passes) plus a fixed share per tile,
+// worth about one item.
+BwdPlan plan_bwd(const Dims &dm, int n_instr)
 {
     BwdPlan pl;
     memset(&pl, 0, sizeof(pl));
-    int nc_best = 0;
-    if (!pick_tile_rows(dm, &pl.tile_rows, &pl.seg_rows, &pl.tiles_per_group, &nc_best)) return pl;
-    pl.sfx_rows = round_up(nc_best * dm.S, 16);
-    pl.nblk_p = (dm.P + kBlockN - 1) / kBlockN;
-    pl.tail_rows = pl.nblk_p ? round_up(dm.P - (pl.nblk_p - 1) * kBlockN, 16) : 0;
-    const int slabs = dm.d / 64;
-    const int tile_bytes = slabs * kTileM * 128;
-    const int sfx_bytes = round_up(slabs * pl.sfx_rows * 128, 1024);
-    const int tail_bytes = round_up(slabs * pl.tail_rows * 128, 1024);
-    const int fixed = 2 * tile_bytes /*Q, dO*/ + 2 * sfx_bytes + kStagingBytes + kBarBytes + 64;
-    const int resident_bytes = pl.nblk_p ? (pl.nblk_p - 1) * tile_bytes + tail_bytes : 0;
-    int k_bytes = 0, v_bytes = 0;
-    if (pl.nblk_p <= kMaxStages && fixed + 2 * resident_bytes <= kMaxSmem) {
-        pl.resident = 3;  // K and V resident
-        pl.stages_k = pl.stages_v = pl.nblk_p > 0 ? pl.nblk_p : 1;
-        k_bytes = v_bytes = resident_bytes;
-    } else if (pl.nblk_p <= kMaxStages && fixed + resident_bytes + tile_bytes <= kMaxSmem) {
-        // K resident, V through a ring: a K block is needed through a whole item (its dQ MMA comes
-        // after the element-wise stage), a V block only for its dP MMA
-        pl.resident = 1;
-        pl.stages_k = pl.nblk_p;
-        int nv = (kMaxSmem - fixed - resident_bytes) / tile_bytes;
-        pl.stages_v = nv > kMaxStages ? kMaxStages : nv;
-        k_bytes = resident_bytes;
-        v_bytes = pl.stages_v * tile_bytes;
-    } else {
-        // ring mode: K gets the larger share of the stages that fit, for the same reason
-        int n = (kMaxSmem - fixed) / tile_bytes;
-        if (n > 2 * kMaxStages) n = 2 * kMaxStages;
-        if (n < 2) return pl;
-        pl.stages_v = n >= 6 ? 2 : 1;
-        pl.stages_k = n - pl.stages_v;
-        if (pl.stages_k > kMaxStages) pl.stages_k = kMaxStages;
-        k_bytes = pl.stages_k * tile_bytes;
-        v_bytes = pl.stages_v * tile_bytes;
+    const int Rg = dm.n_rep * dm.S, Kq = dm.B / n_instr;
+    pl.Rp = round_up(Rg, 8);
+    pl.Sp = round_up(dm.S, 8);
+    pl.nh = (dm.S + kPieceN - 1) / kPieceN;
+    pl.nblk = (dm.P + kPieceN - 1) / kPieceN;
+    const int sms = sm_count();
+    double best = -1.0;
+    for (int cu = 1; cu <= 16 && cu <= Kq; ++cu) {
+        const int tiles = (cu * pl.Rp + kTileM - 1) / kTileM;
+        const int seg = gcd_int(pl.Rp, kTileM);
+        if (cu > 1 && tiles > 1 && seg < 32) break;  // tiles that straddle candidates take 128 / seg boxes
+        if (tiles > 8 && cu > 1) break;
+        int cpp = 1, sfx = 0;
+        if (tiles == 1) {
+            cpp = pl.nh > 1 ? 1 : kPieceN / pl.Sp < cu ? kPieceN / pl.Sp : cu;
+            sfx = (cu + cpp - 1) / cpp * pl.nh;
+        } else {
+            for (int t = 0; t < tiles; ++t) {
+                const int r1 = (t + 1) * kTileM < cu * pl.Rp ? (t + 1) * kTileM : cu * pl.Rp;
+                sfx += (r1 - 1) / pl.Rp - t * kTileM / pl.Rp + 1;
+            }
+            sfx *= 2 * pl.nh - 1;  // pass 0: every piece; each later pass: one
+        }
+        const long long units = (long long)((Kq + cu - 1) / cu) * n_instr * dm.Hkv;
+        const double cost = (double)((units + sms - 1) / sms) * (tiles * (pl.nblk + 1) + sfx * 1.3);
+        if (best < 0.0 || cost < best * 0.97) {
+            best = cost;
+            pl.cu = cu;
+            pl.cpp = cpp;
+            pl.seg = tiles == 1 ? pl.Rp : cu == 1 ? kTileM : seg;
+            pl.cbox = tiles == 1 && n_instr == 1 ? cu : 1;  // (a box must not reach into the next instruction)
+        }
     }
-    pl.off_pk = 0;
-    pl.off_pv = k_bytes;
-    pl.off_q = k_bytes + v_bytes;
-    pl.off_do = pl.off_q + tile_bytes;
-    pl.off_sk = pl.off_do + tile_bytes;
-    pl.off_sv = pl.off_sk + sfx_bytes;
-    pl.off_stage = pl.off_sv + sfx_bytes;
-    pl.off_bar = pl.off_stage + kStagingBytes;
+    pl.sfx_box = pl.nh > 1 ? kPieceN : pl.Sp;
+    pl.upi = (Kq + pl.cu - 1) / pl.cu;
+    const int slabs = dm.d / 64;
+    const int tile_bytes = slabs * kTileM * 128, piece_bytes = slabs * kPieceN * 128;
+    const int fixed = 2 * tile_bytes + 3 * kDsBytes + kRowsBytes + kBarBytes + 64;
+    int n = (kMaxSmem - fixed) / piece_bytes;
+    if (n > 2 * kMaxRing) n = 2 * kMaxRing;
+    if (n < 2) return pl;
+    pl.stages_v = n / 2;  // a K piece is needed until its dQ product, a V piece only for dP
+    pl.stages_k = n - pl.stages_v;
+    pl.off_do = 0;
+    pl.off_q = tile_bytes;
+    pl.off_k = 2 * tile_bytes;
+    pl.off_v = pl.off_k + pl.stages_k * piece_bytes;
+    pl.off_p = pl.off_v + pl.stages_v * piece_bytes;
+    pl.off_ds = pl.off_p + kDsBytes;
+    pl.off_rows = pl.off_ds + 2 * kDsBytes;
+    pl.off_bar = pl.off_rows + kRowsBytes;
     pl.off_misc = pl.off_bar + kBarBytes;
     pl.smem_bytes = pl.off_misc + 64;
-    pl.ok = pl.smem_bytes <= kMaxSmem;
+    pl.ok = pl.smem_bytes <= kMaxSmem && (long long)pl.upi * n_instr * dm.Hkv < 2000000000ll;
     return pl;
 }
 
 template <int D>
-cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_word, cudaStream_t stream, int parts, int n_instr, const int *prefix_len)
+cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_word, cudaStream_t stream, int n_instr,
+                   const int *prefix_len, int split)
 {
     const Dims &dm = a.dims;
     const int Rg = dm.n_rep * dm.S;
-    CUtensorMap tm_q, tm_do, tm_dq, tm_pk, tm_pv, tm_pk_tail, tm_pv_tail, tm_sk, tm_sv;
+    CUtensorMap tm_q, tm_do, tm_pk, tm_pv, tm_sk, tm_sv;
     memset(&tm_pk, 0, sizeof(tm_pk));
     memset(&tm_pv, 0, sizeof(tm_pv));
-    memset(&tm_pk_tail, 0, sizeof(tm_pk_tail));
-    memset(&tm_pv_tail, 0, sizeof(tm_pv_tail));
     {
+        // q / dout viewed as [B][Hkv][Rg][D]: the n_rep heads of a KV head are contiguous rows.  A box that
+        // reaches past a candidate's last row reads zeros there.
         cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)Rg, (cuuint64_t)dm.Hkv, (cuuint64_t)dm.B};
         cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)Rg * D * 2, (cuuint64_t)dm.Hkv * Rg * D * 2};
-        cuuint32_t box[4] = {64, (cuuint32_t)plan.seg_rows, 1, 1};
+        cuuint32_t box[4] = {64, (cuuint32_t)plan.seg, 1, (cuuint32_t)plan.cbox};
         if (!encode_map(&tm_q, a.q, 4, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_do, a.dout, 4, dims, str, box)) return cudaErrorInvalidValue;
-        if (!encode_map(&tm_dq, a.dq, 4, dims, str, box)) return cudaErrorInvalidValue;
     }
     {
         cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)dm.S, (cuuint64_t)dm.Hkv, (cuuint64_t)dm.B};
         cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)dm.S * D * 2, (cuuint64_t)dm.Hkv * dm.S * D * 2};
-        cuuint32_t box[4] = {64, (cuuint32_t)dm.S, 1, 1};
+        cuuint32_t box[4] = {64, (cuuint32_t)plan.sfx_box, 1, (cuuint32_t)plan.cpp};
         if (!encode_map(&tm_sk, a.suffix_k, 4, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_sv, a.suffix_v, 4, dims, str, box)) return cudaErrorInvalidValue;
     }
     if (dm.P > 0) {
         cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)dm.P, (cuuint64_t)dm.Hkv * (cuuint64_t)n_instr};
         cuuint64_t str[2] = {(cuuint64_t)D * 2, (cuuint64_t)dm.Pstride * D * 2};
-        cuuint32_t box[3] = {64, (cuuint32_t)kBlockN, 1};
-        cuuint32_t box_tail[3] = {64, (cuuint32_t)plan.tail_rows, 1};
+        cuuint32_t box[3] = {64, (cuuint32_t)kPieceN, 1};
         if (!encode_map(&tm_pk, a.prefix_k, 3, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_pv, a.prefix_v, 3, dims, str, box)) return cudaErrorInvalidValue;
-        if (!encode_map(&tm_pk_tail, a.prefix_k, 3, dims, str, box_tail)) return cudaErrorInvalidValue;
-        if (!encode_map(&tm_pv_tail, a.prefix_v, 3, dims, str, box_tail)) return cudaErrorInvalidValue;
     }
     TcBwdParams p;
+    memset(&p, 0, sizeof(p));
     p.lse = a.lse;
     p.row_dot = a.row_dot;
+    p.dq = a.dq;
+    p.dq_sectors = (reinterpret_cast<uintptr_t>(a.dq) & 31u) == 0;
+    p.dk = a.dk_suffix;
+    p.dv = a.dv_suffix;
     p.status = status_word;
     p.sl2 = a.scale * kLog2e;
     p.scale = a.scale;
-    p.B = dm.B; p.Hq = dm.Hq; p.Hkv = dm.Hkv; p.S = dm.S; p.P = dm.P; p.n_rep = dm.n_rep;
-    p.Rg = Rg;
-    p.tile_rows = plan.tile_rows;
-    p.seg_rows = plan.seg_rows;
-    p.tiles_per_group = plan.tiles_per_group;
-    p.fd_tpg.init(plan.tiles_per_group);
-    p.fd_Rg.init(Rg);
+    p.Hq = dm.Hq; p.Hkv = dm.Hkv; p.S = dm.S; p.P = dm.P; p.n_rep = dm.n_rep;
+    p.Rg = Rg; p.Rp = plan.Rp; p.Sp = plan.Sp;
+    p.cu = plan.cu; p.cpp = plan.cpp; p.nh = plan.nh; p.seg = plan.seg; p.cbox = plan.cbox; p.sfx_box = plan.sfx_box;
+    p.nblk = plan.nblk;
+    p.Kq = dm.B / n_instr;
+    p.upi = plan.upi;
+    p.upg = plan.upi * n_instr;
+    p.fd_upg.init(p.upg);
+    p.fd_upi.init(p.upi);
+    p.fd_Rp.init(p.Rp);
     p.fd_S.init(dm.S);
-    p.fd_seg.init(plan.seg_rows);
-    p.total_tiles = plan.tiles_per_group * dm.Hkv;
-    p.nblk_p = plan.nblk_p;
-    p.tail_rows = plan.tail_rows;
-    p.stages_k = plan.stages_k > 0 ? plan.stages_k : 1;
-    p.stages_v = plan.stages_v > 0 ? plan.stages_v : 1;
-    p.sfx_rows = plan.sfx_rows;
-    p.off_pk = plan.off_pk; p.off_pv = plan.off_pv; p.off_q = plan.off_q; p.off_do = plan.off_do;
-    p.off_sk = plan.off_sk; p.off_sv = plan.off_sv; p.off_stage = plan.off_stage; p.off_bar = plan.off_bar;
-    p.off_misc = plan.off_misc;
-    p.n_instr = n_instr;
-    p.rpi = dm.B / n_instr * Rg;
-    p.fd_rpi.init(p.rpi > 0 ? p.rpi : 1);
-    for (int i = 0; i < kMaxInstr; ++i) p.pad[i] = (n_instr > 1 && i < n_instr) ? dm.P - prefix_len[i] : 0;
+    p.fd_cpp.init(p.cpp);
+    p.stages_k = plan.stages_k; p.stages_v = plan.stages_v;
+    p.off_do = plan.off_do; p.off_q = plan.off_q; p.off_k = plan.off_k; p.off_v = plan.off_v; p.off_p = plan.off_p;
+    p.off_ds = plan.off_ds; p.off_rows = plan.off_rows; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
+    for (int i = 0; i < n_instr && n_instr > 1; ++i) p.pad[i] = dm.P - prefix_len[i];
 
-    const bool mi = n_instr > 1;
-    auto kernel = plan.resident == 3 ? (mi ? tc_bwd_dq_kernel<D, 3, true> : tc_bwd_dq_kernel<D, 3, false>)
-                  : plan.resident == 1 ? (mi ? tc_bwd_dq_kernel<D, 1, true> : tc_bwd_dq_kernel<D, 1, false>)
-                                       : (mi ? tc_bwd_dq_kernel<D, 0, true> : tc_bwd_dq_kernel<D, 0, false>);
-    static PerDeviceOnce attr_set[8];
-    if (cudaError_t e0 = ensure_max_smem(kernel, attr_set[plan.resident + (mi ? 4 : 0)]); e0 != cudaSuccess) return e0;
-    // The suffix-gradient kernel streams every dO row anyway, so where the shape allows it forms the row
-    // statistic D = <dout, out> itself and runs FIRST (it then stands for both the "row statistic" and the
-    // "suffix gradients" part); the query-side kernel behind it reads D.  Otherwise: a streaming pre-pass
-    // for D, then dQ, then dK_suffix / dV_suffix.
-    const bool d_in_dkv = tc_bwd_dkv_row_dot_supported(dm);
-    cudaError_t e = cudaSuccess;
-    if (parts & kBwdPartRowDot) {
-        e = d_in_dkv ? launch_tc_bwd_dkv(a, status_word, stream, true) : launch_simt_row_dot(a, stream);
-        if (e != cudaSuccess) return e;
-    }
-    if (parts & kBwdPartDq) {
-        const int grid = even_grid(p.total_tiles, sm_count());
+    static PerDeviceOnce attr_set;
+    if (cudaError_t e = ensure_max_smem(tc_bwd_kernel<D>, attr_set); e != cudaSuccess) return e;
+    const int units = p.upg * dm.Hkv;
+    if (split > units) split = units;
+    for (int s = 0; s < split; ++s) {
+        p.unit0 = (int)((long long)units * s / split);
+        p.n_units = (int)((long long)units * (s + 1) / split) - p.unit0;
+        cudaError_t e;
         {
-            KernelTiming timing(kKernelBwdDqTc, stream);
-            e = launch_dependent(kernel, grid, kThreads, plan.smem_bytes, stream, tm_q, tm_do, tm_dq, tm_pk, tm_pv,
-                                 tm_pk_tail, tm_pv_tail, tm_sk, tm_sv, p);
+            KernelTiming timing(kKernelBwdTc, stream);
+            e = launch_dependent(tc_bwd_kernel<D>, even_grid(p.n_units, sm_count()), kThreads, plan.smem_bytes, stream, tm_q,
+                                 tm_do, tm_pk, tm_pv, tm_sk, tm_sv, p);
         }
         count_launches(1);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    if (!(parts & kBwdPartDkv)) return cudaSuccess;
-    if (d_in_dkv) return cudaSuccess;  // done together with the row statistic (also for callers that ask part by part)
-    if (tc_bwd_dkv_supported(dm)) return launch_tc_bwd_dkv(a, status_word, stream);
-    return mma_bwd_dkv_supported(dm) ? launch_mma_bwd_dkv(a, stream) : launch_simt_bwd_dkv(a, stream);
+    return cudaSuccess;
 }
 
 }  // namespace
 
 #ifdef PSKV_TRACE
-// Debug builds only: copies this kernel's event trace of CTA 0 to the host.
-extern "C" int pskv_debug_read_trace_dq(long long *host, int max_events)
+// Debug builds only: copies this kernel's event trace of one CTA to the host.
+extern "C" int pskv_debug_read_trace_bwd(long long *host, int max_events)
 {
     static long long buf[kTraceWarps * kTraceCap * 2];
     unsigned int cnt[kTraceWarps];
@@ -964,33 +971,32 @@ bool tc_bwd_supported(const Dims &dm)
 {
     if (dm.Skv != dm.S || dm.ragged) return false;  // full-suffix operator only
     if (dm.d != 64 && dm.d != 128) return false;
-    if ((long long)dm.B * dm.n_rep * dm.S > 2000000000ll) return false;
-    const BwdPlan pl = plan_bwd(dm);
-    return pl.ok && (long long)pl.tiles_per_group * dm.Hkv <= 2000000000ll;
+    if ((long long)dm.B * dm.n_rep * dm.S > 2000000000ll || dm.n_rep * (long long)dm.S > 1000000ll) return false;
+    return plan_bwd(dm, 1).ok && get_encode_fn() != nullptr;
 }
 
 size_t tc_bwd_workspace_bytes(const Dims &dm) { return (size_t)dm.B * dm.Hq * dm.S * sizeof(float); }
 
-// One launch can serve several instructions when an instruction's rows in a KV head's row list are a whole
-// number of tiles (every tile then lies inside one instruction).
 bool tc_bwd_fused_supported(const Dims &dm, int n_instr)
 {
-    if (n_instr < 2 || n_instr > kMaxFusedInstructions || dm.B % n_instr != 0 || dm.P < 1 || dm.Pstride != dm.P ||
-        !tc_bwd_supported(dm))
-        return false;
-    const BwdPlan pl = plan_bwd(dm);
-    return pl.ok && ((long long)(dm.B / n_instr) * dm.n_rep * dm.S) % pl.tile_rows == 0;
+    return n_instr >= 2 && n_instr <= kMaxFusedInstructions && dm.B % n_instr == 0 && dm.P >= 1 && dm.Pstride == dm.P &&
+           tc_bwd_supported(dm) && plan_bwd(dm, n_instr).ok;
 }
 
-cudaError_t launch_tc_bwd(const BwdArgs &a, void *, unsigned int *status_word, cudaStream_t stream, int parts,
-                          int n_instr, const int *prefix_len)
+cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStream_t stream, int parts, int n_instr,
+                          const int *prefix_len, int split)
 {
-    const BwdPlan plan = plan_bwd(a.dims);
-    if (!plan.ok) return cudaErrorInvalidValue;
-    if (n_instr > 1 && (!prefix_len || !tc_bwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
     if (n_instr < 1) n_instr = 1;
-    return a.dims.d == 128 ? launch<128>(a, plan, status_word, stream, parts, n_instr, prefix_len)
-                           : launch<64>(a, plan, status_word, stream, parts, n_instr, prefix_len);
+    if (n_instr > 1 && (!prefix_len || !tc_bwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
+    const BwdPlan plan = plan_bwd(a.dims, n_instr);
+    if (!plan.ok) return cudaErrorInvalidValue;
+    if (parts & kBwdPartRowDot) {
+        const cudaError_t e = launch_simt_row_dot(a, stream);
+        if (e != cudaSuccess) return e;
+    }
+    if (!(parts & kBwdPartGrad)) return cudaSuccess;
+    return a.dims.d == 128 ? launch<128>(a, plan, status_word, stream, n_instr, prefix_len, split)
+                           : launch<64>(a, plan, status_word, stream, n_instr, prefix_len, split);
 }
 
 }  // namespace pskv
