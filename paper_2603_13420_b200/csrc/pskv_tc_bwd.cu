@@ -805,7 +805,7 @@ struct BwdPlan {
 // Chooses the candidates per unit and lays out shared memory.  The cost of a choice is what the busiest SM
 // does: its units times their items (64-key pieces summed over tiles and passes) plus a fixed share per tile,
 // worth about one item.
-BwdPlan plan_bwd(const Dims &dm, int n_instr)
+BwdPlan make_plan(const Dims &dm, int n_instr)
 {
     BwdPlan pl;
     memset(&pl, 0, sizeof(pl));
@@ -864,6 +864,12 @@ BwdPlan plan_bwd(const Dims &dm, int n_instr)
     pl.smem_bytes = pl.off_misc + 64;
     pl.ok = pl.smem_bytes <= kMaxSmem && (long long)pl.upi * n_instr * dm.Hkv < 2000000000ll;
     return pl;
+}
+
+const BwdPlan &plan_bwd(const Dims &dm, int n_instr)
+{
+    static thread_local PlanTable<BwdPlan> table;
+    return table.get(dm, n_instr, [&] { return make_plan(dm, n_instr); });
 }
 
 template <int D>
@@ -988,7 +994,7 @@ cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStrea
 {
     if (n_instr < 1) n_instr = 1;
     if (n_instr > 1 && (!prefix_len || !tc_bwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
-    const BwdPlan plan = plan_bwd(a.dims, n_instr);
+    const BwdPlan &plan = plan_bwd(a.dims, n_instr);
     if (!plan.ok) return cudaErrorInvalidValue;
     if (parts & kBwdPartRowDot) {
         const cudaError_t e = launch_simt_row_dot(a, stream);

@@ -72,7 +72,7 @@ struct TileInfo {
     bool first_of_g;
 };
 
-// `Params` is any kernel parameter block with fields B, Rg, S, tile_rows, tiles_per_group, fd_tpg, fd_Rg.
+// `Params` is any kernel parameter block with fields B, Rg, Sp, tile_rows, tiles_per_group, fd_tpg, fd_Rg.
 template <class Params>
 __device__ __forceinline__ TileInfo tile_info(const Params &p, int tile, int t_begin)
 {
@@ -86,7 +86,7 @@ __device__ __forceinline__ TileInfo tile_info(const Params &p, int tile, int t_b
     t.b_first = p.fd_Rg.div(t.R0);
     const int b_last = p.fd_Rg.div(t.R0 + t.rows - 1);
     t.nc = b_last - t.b_first + 1;
-    t.n_sfx = (t.nc * p.S + 15) & ~15;
+    t.n_sfx = (t.nc * p.Sp + 15) & ~15;
     return t;
 }
 
@@ -105,39 +105,6 @@ inline int even_grid(int units, int sms)
 inline int gcd_int(int a, int b) { return b == 0 ? a : gcd_int(b, a % b); }
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-
-// Picks the rows per tile: the largest multiple of 8 up to 128 such that the suffix keys of all
-// candidates a tile can touch fit one 128-key block (candidates x S <= 128).  `nc_max` receives
-// that largest number of candidates.
-inline bool pick_tile_rows(const Dims &dm, int *tile_rows, int *seg_rows, int *tiles_per_group, int *nc_max_out)
-{
-    if (dm.S % 8 != 0 || dm.S > kBlockN) return false;
-    const int Rg = dm.n_rep * dm.S;
-    const long long total = (long long)dm.B * Rg;
-    for (int m = kTileM; m >= 8; m -= 8) {
-        const int seg = gcd_int(Rg, m);
-        if (seg % 8 != 0) continue;
-        // worst number of candidates a window [t*m, t*m + m) overlaps; the pattern repeats every Rg/seg tiles
-        const long long ntiles = (total + m - 1) / m;
-        const long long period = (long long)Rg / seg;
-        const long long check = ntiles < period ? ntiles : period;
-        int nc_max = 0;
-        for (long long t = 0; t < check; ++t) {
-            const long long r0 = t * m;
-            long long r1 = r0 + m;
-            if (r1 > total) r1 = total;
-            const int nc = (int)((r1 - 1) / Rg - r0 / Rg + 1);
-            if (nc > nc_max) nc_max = nc;
-        }
-        if (nc_max * dm.S > kBlockN) continue;
-        *tile_rows = m;
-        *seg_rows = seg;
-        *tiles_per_group = (int)ntiles;
-        *nc_max_out = nc_max;
-        return true;
-    }
-    return false;
-}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
@@ -279,6 +246,38 @@ inline int sm_count()
     }
     return n;
 }
+
+// A tiling is a pure function of the call's sizes and the device's SM count, and a call asks for it three or four
+// times (workspace size, kernel family, launch); the choice looks at up to a few hundred candidates (4 us).  Each
+// thread keeps the last ones it worked out, by value of everything that goes in.
+template <class Plan, int kEntries = 16>
+struct PlanTable {
+    struct Entry {
+        bool used;
+        Dims dims;
+        int sms, n_instr;
+        Plan plan;
+    };
+    Entry entries[kEntries];
+
+    template <class Make>
+    const Plan &get(const Dims &dm, int n_instr, Make make)
+    {
+        const int sms = sm_count();
+        unsigned int h = (unsigned int)n_instr;
+        const int key[9] = {dm.B, dm.Hq, dm.Hkv, dm.S, dm.P, dm.d, dm.Pstride, dm.Skv, dm.ragged};
+        for (int v : key) h = (h ^ (unsigned int)v) * 0x01000193u;
+        Entry &e = entries[(h >> 16) % kEntries];
+        if (!e.used || memcmp(&e.dims, &dm, sizeof(dm)) != 0 || e.sms != sms || e.n_instr != n_instr) {
+            e.plan = make();
+            e.dims = dm;
+            e.sms = sms;
+            e.n_instr = n_instr;
+            e.used = true;
+        }
+        return e.plan;
+    }
+};
 
 }  // namespace
 }  // namespace pskv

@@ -61,9 +61,11 @@ struct TcFwdParams {
     FwdArgs args;         // the call's raw arguments, for the rows that are redone row by row
     float sl2;            // scale * log2(e)
     int B, Hq, Hkv, S, P, n_rep;
-    int Rg;               // rows per candidate in one KV-head group: n_rep * S
+    int Rg;               // rows a candidate takes in the row list of a KV-head group (its n_rep * S real rows, padded)
+    int Rr;               // its real rows: n_rep * S
+    int Sp;               // key columns a candidate takes in a tile's suffix block: S rounded up to 8
     int tile_rows;        // rows of the flat row list per tile (<= 128, multiple of seg_rows)
-    int seg_rows;         // rows per Q / out TMA box: gcd(Rg, tile_rows)
+    int seg_rows;         // rows per Q / out TMA box: gcd(Rg, tile_rows) (rows past Rr are zero-filled, never stored)
     int tiles_per_group;
     FastDiv fd_tpg, fd_Rg, fd_S, fd_seg;  // divisions by tiles_per_group, Rg, S, seg_rows
     int total_tiles;
@@ -411,12 +413,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             } else {
                 // suffix K of the candidates this tile touches: one box per candidate
                 if (elect_one_sync()) {
-                    mbar_arrive_expect_tx(bar(kBarSKFull), (uint32_t)(t.nc * C::kSlabs * p.S * 128));
+                    mbar_arrive_expect_tx(bar(kBarSKFull), (uint32_t)(t.nc * C::kSlabs * p.Sp * 128));
 #pragma unroll 1
                     for (int c = 0; c < t.nc; ++c)
 #pragma unroll 1
                         for (int sl = 0; sl < C::kSlabs; ++sl)
-                            tma_load_4d(sbase + p.off_sk + sl * sfx_slab + c * p.S * 128, &tm_sk, bar(kBarSKFull),
+                            tma_load_4d(sbase + p.off_sk + sl * sfx_slab + c * p.Sp * 128, &tm_sk, bar(kBarSKFull),
                                         sl * 64, 0, t.g, t.b_first + c);
                 }
                 __syncwarp();
@@ -555,6 +557,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                                 for (int s = 0; s < nseg; ++s) {
                                     const int R = u.R0 + s * p.seg_rows;
                                     const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
+                                    if (r >= p.Rr) continue;  // padding only
                                     tma_store_4d(&tm_out, stage + (p.slab_stage ? 0 : sl) * kStagingBytes + s * p.seg_rows * 128,
                                                  sl * 64, r, u.g, b);
                                 }
@@ -575,12 +578,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 if (pend_sv && p.alias_stage && !pend_store) sv_ready = true;
                 if (sv_ready) {
                     if (elect_one_sync()) {
-                        mbar_arrive_expect_tx(bar(kBarSVFull), (uint32_t)(t.nc * C::kSlabs * p.S * 128));
+                        mbar_arrive_expect_tx(bar(kBarSVFull), (uint32_t)(t.nc * C::kSlabs * p.Sp * 128));
 #pragma unroll 1
                         for (int c = 0; c < t.nc; ++c)
 #pragma unroll 1
                             for (int sl = 0; sl < C::kSlabs; ++sl)
-                                tma_load_4d(sbase + p.off_sv + sl * sfx_slab + c * p.S * 128, &tm_sv, bar(kBarSVFull),
+                                tma_load_4d(sbase + p.off_sv + sl * sfx_slab + c * p.Sp * 128, &tm_sv, bar(kBarSVFull),
                                             sl * 64, 0, t.g, t.b_first + c);
                     }
                     __syncwarp();
@@ -806,7 +809,9 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 const int R = t.R0 + row;
                 const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
                 const int i = r - p.fd_S.div(r) * p.S;  // query index inside the candidate
-                if (SR) {
+                if (r >= p.Rr) {
+                    // a padding row between two candidates: sees no suffix key, is never stored
+                } else if (SR) {
                     // query i is suffix token L - S + i of its candidate: suffix keys 0 .. L - S + i
                     const int pos = suffix_tokens(p.suffix_len, b, p.S, p.Skv) - p.S + i;
                     if (p.long_sfx) {
@@ -819,8 +824,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         hi_sfx = lo_sfx + pos;
                     }
                 } else {
-                    lo_sfx = (b - t.b_first) * p.S;  // first suffix column of this row's candidate
-                    hi_sfx = lo_sfx + i;             // causal: suffix keys 0..i
+                    lo_sfx = (b - t.b_first) * p.Sp;  // first suffix column of this row's candidate
+                    hi_sfx = lo_sfx + i;              // causal: suffix keys 0..i
                 }
             }
             lsum = 0.f;
@@ -1046,10 +1051,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBarStageFull));
             }
-            const bool stored = row < u.rows;
+            const int R = u.R0 + row;
+            const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
+            const bool stored = row < u.rows && r < p.Rr;
             if (stored) {
-                const int R = u.R0 + row;
-                const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
                 const size_t grow = ((size_t)b * p.Hq + (size_t)u.g * p.n_rep) * p.S + r;
                 p.lse[grow] = row_ok ? log2f(l) * kLn2 : __int_as_float(0x7fc00000);
             }
@@ -1078,6 +1083,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             for (int r = warp; r < t.rows; r += kThreads / 32) {
                 const int R = t.R0 + r;
                 const int b = p.fd_Rg.div(R), rr = R - b * p.Rg;
+                if (rr >= p.Rr) continue;
                 const long long grow = ((long long)b * p.Hq + (long long)t.g * p.n_rep) * p.S + rr;
                 const float v = p.lse[grow];
                 if (v != v) {
@@ -1106,14 +1112,59 @@ struct TilePlan {
     int cbox, Spad, cpb;  // suffix-ring mode: candidates per tile, rows per candidate in a block, candidates per block
     int long_sfx;         // suffix-ring mode: tiles inside one candidate, its suffix keys in 128-key blocks
     int tile_rows, seg_rows, tiles_per_group, sfx_rows;
+    int Rp, Sp;           // rows / suffix key columns a candidate takes (base tiling)
+    double cost;          // estimated SM cycles of a KV head's tiles
     int nblk_p, tail_rows, resident, stages, alias_stage, slab_stage, ml_tiles;
     int off_pk, off_pv, off_q, off_sk, off_sv, off_stage, off_bar, off_misc, off_ml, smem_bytes;
 };
 
-// Picks the rows per tile -- the largest multiple of 8 up to 128 such that the suffix keys of all
-// candidates a tile can touch fit one 128-key block (candidates x S <= 128) -- and lays out shared
-// memory: all prefix blocks of a KV head if they fit beside the other buffers (resident mode), else
-// rings of 2..4 block stages.
+// Cycles of a tile, for the choice of a tiling: about 2 000 per key block, 1 700 for the tile itself, and 60 per
+// box of Q and of `out` (one thread issues them; with sixteen boxes of 8 rows that is 1 000 cycles in which the
+// single Q buffer is waited for).
+double tile_cost(int blocks, int boxes) { return 2000.0 * blocks + 1700.0 + 60.0 * boxes; }
+
+// Rows a candidate takes in the row list (Rp >= n_rep * S) and rows per tile, both multiples of 8, such that the
+// suffix keys of all candidates a tile can touch (Sp columns each) fit one 128-key block.  Suffix lengths are
+// rarely multiples of anything, so a candidate's rows are padded: by as much as makes the launch cheapest,
+// which is more than to the next multiple of 8 where that lets a tile be fetched in few boxes
+// (4 heads x 53 rows: 224 rows, 32-row boxes) or end where a candidate ends (4 x 113: 480 rows, tiles of 120).
+// Measured against the suffix-ring tiling that took every length that is no multiple of 8 (whole calls):
+// B = 333, 32/8 heads, P = 217, S = 53 173 -> 120 us; B = 64, 32/32, P = 230, S = 85 74 -> 57; B = 42, 32/8, P = 112,
+// S = 117 44 -> 36; and against tiles of the largest divisor: B = 128, 32/8, P = 256, S = 80 (336 rows, three tiles
+// of 112, instead of four of 80) 101 -> 82.
+bool pick_tile_rows(const Dims &dm, TilePlan *pl, int *nc_max)
+{
+    const int Sp = round_up(dm.S, 8);
+    if (Sp > kBlockN) return false;
+    const int Rg = dm.n_rep * dm.S, nblk = (dm.P + kBlockN - 1) / kBlockN;
+    double best = -1.0;
+    for (int Rp = round_up(Rg, 8); Rp < Rg + kTileM; Rp += 8) {
+        if ((long long)dm.B * Rp > 2000000000ll) break;
+        if (best >= 0.0 && (double)(((long long)dm.B * Rp + kTileM - 1) / kTileM) * tile_cost(nblk + 1, 1) >= best) break;
+        for (int m = kTileM; m >= 8; m -= 8) {
+            const int seg = gcd_int(Rp, m);
+            // candidates that a window of m rows can touch, its offset in a candidate being a multiple of seg
+            int nc = m % Rp == 0 ? m / Rp : Rp % m == 0 ? 1 : (m - seg + Rp - 1) / Rp + 1;
+            if (nc > dm.B) nc = dm.B;
+            if (nc * Sp > kBlockN) continue;
+            const long long tiles = ((long long)dm.B * Rp + m - 1) / m;
+            const double cost = (double)tiles * tile_cost(nblk + 1, m / seg);
+            if (best < 0.0 || cost < best) {
+                best = cost;
+                pl->Rp = Rp;
+                pl->tile_rows = m;
+                pl->seg_rows = seg;
+                pl->tiles_per_group = (int)tiles;
+                *nc_max = nc;
+            }
+        }
+    }
+    if (best < 0.0) return false;
+    pl->Sp = Sp;
+    pl->cost = best;
+    return true;
+}
+
 // Suffix-ring mode: a tile is the largest run of whole candidates with at most 128 rows; the
 // suffix keys follow the prefix blocks through K/V rings, 128 / Spad candidates per block.
 TilePlan plan_suffix_ring(const Dims &dm)
@@ -1159,6 +1210,7 @@ TilePlan plan_suffix_ring(const Dims &dm)
         }
         pl.tile_rows = pl.seg_rows = Rg * pl.cbox;
         pl.tiles_per_group = (dm.B + pl.cbox - 1) / pl.cbox;
+        pl.cost = (double)pl.tiles_per_group * tile_cost(nblk + (pl.cbox + pl.cpb - 1) / pl.cpb, 1);
     }
     pl.nblk_p = (dm.P + kBlockN - 1) / kBlockN;
     pl.tail_rows = pl.nblk_p ? round_up(dm.P - (pl.nblk_p - 1) * kBlockN, 16) : 0;
@@ -1183,13 +1235,15 @@ TilePlan plan_suffix_ring(const Dims &dm)
     return pl;
 }
 
+// Lays out shared memory: all prefix blocks of a KV head if they fit beside the other buffers (resident mode), else
+// rings of 2..4 block stages.
 TilePlan plan_base(const Dims &dm)
 {
     TilePlan pl;
     memset(&pl, 0, sizeof(pl));
     int nc_best = 0;
-    if (!pick_tile_rows(dm, &pl.tile_rows, &pl.seg_rows, &pl.tiles_per_group, &nc_best)) return pl;
-    pl.sfx_rows = round_up(nc_best * dm.S, 16);
+    if (!pick_tile_rows(dm, &pl, &nc_best)) return pl;
+    pl.sfx_rows = round_up(nc_best * pl.Sp, 16);
     pl.nblk_p = (dm.P + kBlockN - 1) / kBlockN;
     pl.tail_rows = pl.nblk_p ? round_up(dm.P - (pl.nblk_p - 1) * kBlockN, 16) : 0;
 
@@ -1249,15 +1303,26 @@ TilePlan plan_base(const Dims &dm)
     return pl;
 }
 
-// The full-suffix operator takes the tiling with the suffix in one block when it has one; the
-// decode-shaped operator, and full-suffix shapes that tiling cannot take, go to suffix-ring mode.
-TilePlan plan_tiles(const Dims &dm)
+// The full-suffix operator takes the tiling with the suffix in one block when it has one; the decode-shaped operator
+// and suffixes beyond one block go to suffix-ring mode, and so do groups of a few rows, whose padding to 8 rows
+// would cost more than the ring's extra suffix blocks (one row per candidate and head: an eighth of the tile).
+TilePlan make_plan(const Dims &dm)
 {
     if (dm.Skv == dm.S && !dm.ragged) {
         const TilePlan pl = plan_base(dm);
+        if (pl.ok && dm.n_rep * dm.S % 8 != 0 && dm.n_rep * dm.S <= kTileM / 2) {
+            const TilePlan ring = plan_suffix_ring(dm);
+            if (ring.ok && !ring.long_sfx && ring.cost < pl.cost) return ring;
+        }
         if (pl.ok) return pl;
     }
     return plan_suffix_ring(dm);
+}
+
+const TilePlan &plan_tiles(const Dims &dm)
+{
+    static thread_local PlanTable<TilePlan> table;
+    return table.get(dm, 1, [&] { return make_plan(dm); });
 }
 
 template <int D>
@@ -1286,7 +1351,7 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     {
         cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)dm.Skv, (cuuint64_t)dm.Hkv, (cuuint64_t)dm.B};
         cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)dm.Skv * D * 2, (cuuint64_t)dm.Hkv * dm.Skv * D * 2};
-        cuuint32_t box[4] = {64, (cuuint32_t)(plan.long_sfx ? kBlockN : dm.Skv), 1, 1};
+        cuuint32_t box[4] = {64, (cuuint32_t)(plan.long_sfx ? kBlockN : plan.mode == 2 ? dm.Skv : plan.Sp), 1, 1};
         if (!encode_map(&tm_sk, a.suffix_k, 4, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_sv, a.suffix_v, 4, dims, str, box)) return cudaErrorInvalidValue;
     }
@@ -1306,12 +1371,14 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     p.args = a;
     p.sl2 = a.scale * kLog2e;
     p.B = dm.B; p.Hq = dm.Hq; p.Hkv = dm.Hkv; p.S = dm.S; p.P = dm.P; p.n_rep = dm.n_rep;
-    p.Rg = Rg;
+    p.Rg = plan.mode == 2 ? Rg : plan.Rp;
+    p.Rr = Rg;
+    p.Sp = plan.mode == 2 ? dm.S : plan.Sp;
     p.tile_rows = plan.tile_rows;
     p.seg_rows = plan.seg_rows;
     p.tiles_per_group = plan.tiles_per_group;
     p.fd_tpg.init(plan.tiles_per_group);
-    p.fd_Rg.init(Rg);
+    p.fd_Rg.init(p.Rg);
     p.fd_S.init(dm.S);
     p.fd_seg.init(plan.seg_rows);
     p.total_tiles = plan.tiles_per_group * dm.Hkv;
@@ -1330,7 +1397,7 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     p.fd_cpb.init(p.cpb);
     p.long_sfx = plan.long_sfx;
     p.n_instr = n_instr;
-    p.rpi = dm.B / n_instr * Rg;
+    p.rpi = dm.B / n_instr * p.Rg;
     p.fd_rpi.init(p.rpi > 0 ? p.rpi : 1);
     for (int i = 0; i < kMaxInstr; ++i) p.pad[i] = (n_instr > 1 && i < n_instr) ? dm.P - prefix_len[i] : 0;
     // Dealing by cost balances the causal skew but lets every CTA touch every candidate's suffix K/V
@@ -1383,7 +1450,7 @@ bool tc_fwd_supported(const Dims &dm)
 {
     if (dm.d != 64 && dm.d != 128) return false;
     if ((long long)dm.B * dm.n_rep * dm.S > 2000000000ll) return false;  // flat row index fits an int
-    const TilePlan pl = plan_tiles(dm);
+    const TilePlan &pl = plan_tiles(dm);
     return pl.ok && (long long)pl.tiles_per_group * dm.Hkv <= 2000000000ll;  // ... and so does the tile index
 }
 
@@ -1397,14 +1464,14 @@ bool tc_fwd_fused_supported(const Dims &dm, int n_instr)
     if (n_instr < 2 || n_instr > kMaxFusedInstructions || dm.B % n_instr != 0 || dm.P < 1 || dm.Pstride != dm.P ||
         dm.ragged || !tc_fwd_supported(dm))
         return false;
-    const TilePlan pl = plan_tiles(dm);
-    return pl.ok && pl.mode != 2 && ((long long)(dm.B / n_instr) * dm.n_rep * dm.S) % pl.tile_rows == 0;
+    const TilePlan &pl = plan_tiles(dm);
+    return pl.ok && pl.mode != 2 && ((long long)(dm.B / n_instr) * pl.Rp) % pl.tile_rows == 0;
 }
 
 cudaError_t launch_tc_fwd(const FwdArgs &a, void *workspace, unsigned int *status_word, cudaStream_t stream,
                           int n_instr, const int *prefix_len)
 {
-    const TilePlan plan = plan_tiles(a.dims);
+    const TilePlan &plan = plan_tiles(a.dims);
     if (!plan.ok) return cudaErrorInvalidValue;
     if (n_instr > 1 && (!prefix_len || !tc_fwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
     if (n_instr < 1) n_instr = 1;

@@ -1,0 +1,48 @@
+"""The tensor-core forward at the edges of its tiling: candidates whose rows or keys are no multiple of 8, padded to the next
+multiple or as far as a tile's end, boxes that hold padding only, a short last tile, suffixes of one whole key block."""
+import pytest
+
+import paper_2603_13420_b200 as pskv
+import parity
+from paper_2603_13420_b200.inputs import Workload, make_inputs
+
+SHAPES = [
+    # B, Hq, Hkv, d, P, S
+    (19, 2, 2, 128, 40, 1),      # one row per candidate: whole candidates, suffix keys in several blocks
+    (21, 4, 4, 128, 200, 13),    # 16 rows per candidate, eight to a tile
+    (9, 8, 2, 128, 217, 53),     # 212 rows padded to 224: tiles straddle candidates, boxes of 32 rows
+    (5, 8, 2, 64, 129, 45),
+    (3, 8, 2, 128, 78, 113),     # 452 rows padded to 480: four tiles of 120 rows inside a candidate
+    (4, 2, 2, 128, 600, 121),    # prefix streamed
+    (3, 7, 1, 128, 100, 35),     # seven heads per KV head
+    (2, 8, 2, 128, 0, 127),      # no prefix
+    (33, 3, 3, 64, 31, 9),
+    (300, 8, 2, 128, 257, 21),   # several tiles per CTA
+]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_forward_matches_the_oracle(shape):
+    B, Hq, Hkv, d, P, S = shape
+    w = Workload("tiles", 900 + sum(shape), B=B, Hq=Hq, Hkv=Hkv, d=d, P=P, S=S)
+    assert pskv.pskv_kernel_family(0, B, Hq, Hkv, S, P, d) == 1
+    cand = None if B <= 64 else [0, 1, 2, 149, 150, 297, 298, 299]
+    parity.fwd_parity(w, cand=cand, strict_abs=(P + S >= 128))
+
+
+@pytest.mark.gpu
+def test_rows_outside_the_safe_exponent_range_next_to_padding_rows():
+    """Scores of several hundred nats in the last real rows before a candidate's padding, and in the first after it."""
+    w = Workload("tiles", 977, B=6, Hq=8, Hkv=2, d=128, P=90, S=53)
+    t = make_inputs(w)
+    q = t["q"].float()
+    q[1, 3, 52] *= 60.0
+    q[2, 0, 0] *= -60.0
+    q[5, 7, 52] *= 60.0
+    t["q"] = q.to(t["q"].dtype)
+    out, lse, _ = parity.run_fwd_gpu(t, w.scale)
+    ref_out, ref_lse = parity.oracle_fwd(t, w.scale)
+    assert abs(ref_lse).max() > 100.0
+    parity.check_tensor("out", parity.to_f64(out), ref_out)
+    parity.check_lse(parity.to_f64(lse), ref_lse)
