@@ -1,10 +1,12 @@
-"""ctypes binding of libpskv.so: argument marshalling only.
+"""Python binding of libpskv.so: argument marshalling only.
 
 Each function has the name and argument order of its C entry point in
 ``include/pskv.h``; tensors are torch CUDA tensors whose ``data_ptr()`` is
 handed through, sizes are read from the tensors' shapes, and the work is
-enqueued on torch's current stream.  Nothing is computed here and there is no
-fallback: if the shared library has not been built, loading fails.
+enqueued on torch's current stream.  The calls a search makes all the time go
+through the extension module ``_native`` (``csrc/pskv_python.cpp``), the others
+through ctypes.  Nothing is computed here and there is no fallback: if the
+libraries have not been built, loading fails.
 """
 from __future__ import annotations
 
@@ -26,6 +28,7 @@ PSKV_ERR_CUDA = 5
 PSKV_ERR_DEVICE_TIMEOUT = 6
 
 _lib = None
+_native = None
 
 
 class PskvError(RuntimeError):
@@ -118,6 +121,34 @@ def lib() -> ctypes.CDLL:
         L.pskv_enable_cta_pairs.restype = None
         _lib = L
     return _lib
+
+
+# the C entry points _native calls, in the order it expects them
+_NATIVE_ENTRIES = (
+    "pskv_attn_fwd", "pskv_attn_fwd_workspace_bytes", "pskv_attn_bwd", "pskv_attn_bwd_lse", "pskv_attn_bwd_workspace_bytes",
+    "pskv_attn_fwd_decode", "pskv_attn_fwd_decode_workspace_bytes", "pskv_attn_fwd_multi", "pskv_attn_fwd_multi_workspace_bytes",
+    "pskv_attn_bwd_multi", "pskv_attn_bwd_multi_workspace_bytes", "pskv_target_ce_fwd", "pskv_target_ce_fwd_workspace_bytes")
+
+
+def native():
+    """The extension module, bound to the loaded library."""
+    global _native
+    if _native is None:
+        L = lib()
+        try:
+            from . import _native as module
+        except ImportError as e:
+            raise RuntimeError("the extension module _native.so is missing or does not load: build it with `python -m "
+                               "paper_2603_13420_b200.build` (there is no fallback)") from e
+        module.init(*[ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _NATIVE_ENTRIES])
+        _native = module
+    return _native
+
+
+def _checked(r, where):
+    if type(r) is int:
+        raise PskvError(r, where)
+    return r
 
 
 def _ptr(t):
@@ -221,61 +252,23 @@ def _workspace(nbytes, device, workspace):
 def pskv_attn_fwd(q, prefix_k, prefix_v, suffix_k, suffix_v, scale, out=None, lse=None,
                   workspace=None):
     """out [B,Hq,S,d] bf16 and lse [B,Hq,S] fp32; q/suffix_* are per candidate, prefix_* [Hkv,P,d] shared."""
-    dims = _dims(q, prefix_k, suffix_k)
-    B, Hq, Hkv, S, P, d = dims
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((B, Hq, S), dtype=torch.float32, device=q.device)
-    ws = _workspace(pskv_attn_fwd_workspace_bytes(*dims), q.device, workspace)
-    st = lib().pskv_attn_fwd(_ptr(q), _ptr(prefix_k), _ptr(prefix_v), _ptr(suffix_k), _ptr(suffix_v),
-                             float(scale), _ptr(out), _ptr(lse), *dims,
-                             _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_attn_fwd")
-    return out, lse
+    return _checked((_native or native()).fwd(q, prefix_k, prefix_v, suffix_k, suffix_v, scale, out, lse, workspace), "pskv_attn_fwd")
 
 
 def pskv_attn_bwd(dout, q, prefix_k, prefix_v, suffix_k, suffix_v, out, lse, scale,
                   dq=None, dk_suffix=None, dv_suffix=None, workspace=None):
     """dq, dk_suffix, dv_suffix (bf16) of L = sum(out * dout); the prefix cache gets no gradient."""
-    dims = _dims(q, prefix_k, suffix_k)
-    if dq is None:
-        dq = torch.empty_like(q)
-    if dk_suffix is None:
-        dk_suffix = torch.empty_like(suffix_k)
-    if dv_suffix is None:
-        dv_suffix = torch.empty_like(suffix_v)
-    ws = _workspace(pskv_attn_bwd_workspace_bytes(*dims), q.device, workspace)
-    st = lib().pskv_attn_bwd(_ptr(dout), _ptr(q), _ptr(prefix_k), _ptr(prefix_v), _ptr(suffix_k),
-                             _ptr(suffix_v), _ptr(out), _ptr(lse), float(scale),
-                             _ptr(dq), _ptr(dk_suffix), _ptr(dv_suffix), *dims,
-                             _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_attn_bwd")
-    return dq, dk_suffix, dv_suffix
+    return _checked((_native or native()).bwd(dout, None, q, prefix_k, prefix_v, suffix_k, suffix_v, out, lse, scale,
+                                              dq, dk_suffix, dv_suffix, workspace), "pskv_attn_bwd")
 
 
 def pskv_attn_bwd_lse(dout, dlse, q, prefix_k, prefix_v, suffix_k, suffix_v, out, lse, scale,
                       dq=None, dk_suffix=None, dv_suffix=None, workspace=None):
     """Backward of L = sum(out * dout) + sum(lse * dlse): pskv_attn_bwd with a gradient on lse (fp32 [B,Hq,S])."""
-    dims = _dims(q, prefix_k, suffix_k)
-    if dq is None:
-        dq = torch.empty_like(q)
-    if dk_suffix is None:
-        dk_suffix = torch.empty_like(suffix_k)
-    if dv_suffix is None:
-        dv_suffix = torch.empty_like(suffix_v)
     if dlse is None or dlse.dtype != torch.float32 or tuple(dlse.shape) != tuple(q.shape[:3]):
         raise ValueError("dlse must be a float32 CUDA tensor of shape [B,Hq,S]")
-    ws = _workspace(pskv_attn_bwd_workspace_bytes(*dims), q.device, workspace)
-    st = lib().pskv_attn_bwd_lse(_ptr(dout), _ptr(dlse), _ptr(q), _ptr(prefix_k), _ptr(prefix_v), _ptr(suffix_k),
-                                 _ptr(suffix_v), _ptr(out), _ptr(lse), float(scale),
-                                 _ptr(dq), _ptr(dk_suffix), _ptr(dv_suffix), *dims,
-                                 _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_attn_bwd_lse")
-    return dq, dk_suffix, dv_suffix
+    return _checked((_native or native()).bwd(dout, dlse, q, prefix_k, prefix_v, suffix_k, suffix_v, out, lse, scale,
+                                              dq, dk_suffix, dv_suffix, workspace), "pskv_attn_bwd_lse")
 
 
 def pskv_attn_bwd_prefix_workspace_bytes(B, Hq, Hkv, S, P, d) -> int:
@@ -301,19 +294,6 @@ def pskv_attn_bwd_prefix(dout, dlse, q, prefix_k, prefix_v, out, lse, scale, dk_
     return dk_prefix, dv_prefix
 
 
-def _multi_dims(q, prefix_k, suffix_k, prefix_len):
-    B, Hq, S, d = q.shape
-    Hkv = suffix_k.shape[1]
-    Bp = len(prefix_len)
-    Pmax = 0 if prefix_k is None else prefix_k.shape[2]
-    return [int(B), int(Bp), int(Hq), int(Hkv), int(S), int(Pmax), int(d)]
-
-
-def _host_lens(prefix_len):
-    arr = (ctypes.c_int * len(prefix_len))(*[int(x) for x in prefix_len])
-    return arr
-
-
 def pskv_attn_fwd_multi_workspace_bytes(B, Bp, Hq, Hkv, S, Pmax, d) -> int:
     return int(lib().pskv_attn_fwd_multi_workspace_bytes(B, Bp, Hq, Hkv, S, Pmax, d))
 
@@ -327,40 +307,15 @@ def pskv_attn_fwd_multi(q, prefix_k, prefix_v, prefix_len, suffix_k, suffix_v, s
     """Forward with one left-padded prefix cache per instruction: prefix_k / prefix_v are
     [Bp, Hkv, Pmax, d], prefix_len (host ints) the true lengths, candidate b uses instruction
     b // (B // Bp).  Padding rows may hold any finite values."""
-    dims = _multi_dims(q, prefix_k, suffix_k, prefix_len)
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
-    ws = _workspace(max(256, pskv_attn_fwd_multi_workspace_bytes(*dims)), q.device, workspace)
-    lens = _host_lens(prefix_len)
-    st = lib().pskv_attn_fwd_multi(_ptr(q), _ptr(prefix_k), _ptr(prefix_v), ctypes.cast(lens, ctypes.c_void_p),
-                                   _ptr(suffix_k), _ptr(suffix_v), float(scale), _ptr(out), _ptr(lse), *dims,
-                                   _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_attn_fwd_multi")
-    return out, lse
+    return _checked((_native or native()).fwd_multi(q, prefix_k, prefix_v, prefix_len, suffix_k, suffix_v, scale, out, lse, workspace),
+                    "pskv_attn_fwd_multi")
 
 
 def pskv_attn_bwd_multi(dout, q, prefix_k, prefix_v, prefix_len, suffix_k, suffix_v, out, lse, scale,
                         dq=None, dk_suffix=None, dv_suffix=None, workspace=None):
     """Backward of pskv_attn_fwd_multi: dq, dk_suffix, dv_suffix; the prefix caches get no gradient."""
-    dims = _multi_dims(q, prefix_k, suffix_k, prefix_len)
-    if dq is None:
-        dq = torch.empty_like(q)
-    if dk_suffix is None:
-        dk_suffix = torch.empty_like(suffix_k)
-    if dv_suffix is None:
-        dv_suffix = torch.empty_like(suffix_v)
-    ws = _workspace(pskv_attn_bwd_multi_workspace_bytes(*dims), q.device, workspace)
-    lens = _host_lens(prefix_len)
-    st = lib().pskv_attn_bwd_multi(_ptr(dout), _ptr(q), _ptr(prefix_k), _ptr(prefix_v),
-                                   ctypes.cast(lens, ctypes.c_void_p), _ptr(suffix_k), _ptr(suffix_v), _ptr(out),
-                                   _ptr(lse), float(scale), _ptr(dq), _ptr(dk_suffix), _ptr(dv_suffix), *dims,
-                                   _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_attn_bwd_multi")
-    return dq, dk_suffix, dv_suffix
+    return _checked((_native or native()).bwd_multi(dout, q, prefix_k, prefix_v, prefix_len, suffix_k, suffix_v, out, lse, scale,
+                                                    dq, dk_suffix, dv_suffix, workspace), "pskv_attn_bwd_multi")
 
 
 def _decode_dims(q, prefix_k, suffix_k):
@@ -390,18 +345,8 @@ def pskv_attn_fwd_decode(q, prefix_k, prefix_v, suffix_k, suffix_v, suffix_len, 
                          workspace=None):
     """Decode-shaped forward: q [B,Hq,Sq,d] are the last Sq of each candidate's suffix_len[b] cached
     suffix tokens (suffix_k / suffix_v [B,Hkv,Skv,d]; suffix_len an int32 CUDA tensor [B] or None)."""
-    dims = _decode_dims(q, prefix_k, suffix_k)
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
-    ws = _workspace(pskv_attn_fwd_decode_workspace_bytes(*dims), q.device, workspace)
-    st = lib().pskv_attn_fwd_decode(_ptr(q), _ptr(prefix_k), _ptr(prefix_v), _ptr(suffix_k), _ptr(suffix_v),
-                                    _len_ptr(suffix_len, dims[0]), float(scale), _ptr(out), _ptr(lse), *dims,
-                                    _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_attn_fwd_decode")
-    return out, lse
+    return _checked((_native or native()).fwd_decode(q, prefix_k, prefix_v, suffix_k, suffix_v, suffix_len, scale, out, lse, workspace),
+                    "pskv_attn_fwd_decode")
 
 
 def pskv_attn_bwd_decode(dout, q, prefix_k, prefix_v, suffix_k, suffix_v, suffix_len, out, lse, scale,
@@ -431,22 +376,7 @@ def pskv_target_ce_fwd_workspace_bytes(N, Lr, Dm, V) -> int:
 def pskv_target_ce_fwd(hidden, weight, target, mask, nll=None, lse=None, loss=None, workspace=None):
     """Masked target cross-entropy fused with the vocabulary projection: hidden bf16 [N,Lr,Dm], weight
     bf16 [V,Dm], target int32 [N,Lr], mask fp32 [N,Lr].  Returns nll [N,Lr], lse [N,Lr], loss [N] (fp32)."""
-    N, Lr, Dm = (int(x) for x in hidden.shape)
-    V = int(weight.shape[0])
-    if target.dtype != torch.int32 or mask.dtype != torch.float32:
-        raise ValueError("target must be int32 and mask float32")
-    if tuple(target.shape) != (N, Lr) or tuple(mask.shape) != (N, Lr) or int(weight.shape[1]) != Dm:
-        raise ValueError("shape mismatch")
-    f32 = dict(dtype=torch.float32, device=hidden.device)
-    nll = torch.empty((N, Lr), **f32) if nll is None else nll
-    lse = torch.empty((N, Lr), **f32) if lse is None else lse
-    loss = torch.empty((N,), **f32) if loss is None else loss
-    ws = _workspace(pskv_target_ce_fwd_workspace_bytes(N, Lr, Dm, V), hidden.device, workspace)
-    st = lib().pskv_target_ce_fwd(_ptr(hidden), _ptr(weight), _ptr(target), _ptr(mask), _ptr(nll), _ptr(lse),
-                                  _ptr(loss), N, Lr, Dm, V, _ptr(ws), ws.numel() * ws.element_size(), _stream())
-    if st != PSKV_OK:
-        raise PskvError(st, "pskv_target_ce_fwd")
-    return nll, lse, loss
+    return _checked((_native or native()).target_ce(hidden, weight, target, mask, nll, lse, loss, workspace), "pskv_target_ce_fwd")
 
 
 def pskv_attn_bwd_static_max_rows() -> int:

@@ -1,4 +1,4 @@
-"""Build libpskv.so in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Build libpskv.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the Python face _native.so with g++.
 
     python -m paper_2603_13420_b200.build [--force] [--verbose]
 """
@@ -13,6 +13,8 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_PATH = os.path.join(PKG_DIR, "libpskv.so")
+NATIVE_SRC = os.path.join(CSRC, "pskv_python.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
 
 SOURCES = ["pskv_api.cu", "pskv_simt.cu", "pskv_tc_fwd.cu", "pskv_tc_fwd_pair.cu", "pskv_tc_bwd.cu", "pskv_tc_bwd_prefix.cu", "pskv_noalloc.cu", "pskv_selftest.cu", "pskv_ce.cu"]
 
@@ -30,16 +32,36 @@ def _deps():
     return deps
 
 
+def _older(target, sources) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in sources)
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
-        return True
-    built = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(p) > built for p in _deps())
+    return _older(LIB_PATH, _deps()) or _older(NATIVE_PATH, [NATIVE_SRC, _deps()[0]])
+
+
+def _build_native() -> None:
+    """The Python extension module; it needs torch's headers and libraries, not CUDA kernels."""
+    import importlib.util
+    import sysconfig
+
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    inc = os.path.join(torch_dir, "include")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = NATIVE_PATH + ".tmp.%d" % os.getpid()
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I", INCLUDE, "-I", inc,
+                    "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(cuda, "include"), NATIVE_SRC, "-o", tmp, "-L", os.path.join(torch_dir, "lib"),
+                    "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"], check=True)
+    os.replace(tmp, NATIVE_PATH)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source into paper_2603_13420_b200/libpskv.so and return its path."""
-    if not force and not is_stale():
+    """Compile every CUDA source into paper_2603_13420_b200/libpskv.so, and the extension module beside it; returns the
+    library's path."""
+    if force or _older(NATIVE_PATH, [NATIVE_SRC, _deps()[0]]):
+        _build_native()
+    if not force and not _older(LIB_PATH, _deps()):
         return LIB_PATH
     objs = []
     procs = []
