@@ -5,6 +5,8 @@
 // followed by the causally visible suffix keys (Eq. 2).
 #include "pskv_common.cuh"
 #include "pskv_rows.cuh"
+#include "pskv_sm100.cuh"
+#include "pskv_tc_common.cuh"
 
 namespace pskv {
 namespace {
@@ -99,6 +101,8 @@ simt_row_dot_kernel(BwdArgs a)
     constexpr int kLanesPerRow = D / 8;             // 16 (d = 128) or 8 (d = 64)
     constexpr int kRowsPerLoad = 32 / kLanesPerRow;  // rows one warp-wide load covers
     constexpr int kRowsPerWarp = kRowsPerLoad * kRowDotUnroll;
+    sm100::grid_dep_launch();  // the gradient kernel behind this one sets itself up under its tail
+    sm100::grid_dep_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long rows = (long long)a.dims.B * a.dims.Hq * a.dims.S;
     const long long first = ((long long)blockIdx.x * kWarpsPerBlock + warp) * kRowsPerWarp;
@@ -282,13 +286,20 @@ cudaError_t launch_simt_fwd(const FwdArgs &a, cudaStream_t stream)
 cudaError_t launch_simt_row_dot(const BwdArgs &a, cudaStream_t stream)
 {
     const long long rows = (long long)a.dims.B * a.dims.Hq * a.dims.S;
-    KernelTiming timing(kKernelRowDot, stream);
-    if (a.dims.d == 128)
-        simt_row_dot_kernel<128><<<blocks_for((rows + 2 * kRowDotUnroll - 1) / (2 * kRowDotUnroll)), kWarpsPerBlock * 32, 0,
-                                   stream>>>(a);
-    else
-        simt_row_dot_kernel<64><<<blocks_for((rows + 4 * kRowDotUnroll - 1) / (4 * kRowDotUnroll)), kWarpsPerBlock * 32, 0,
-                                  stream>>>(a);
+    const int per_warp = (a.dims.d == 128 ? 2 : 4) * kRowDotUnroll;
+    const int grid = (int)blocks_for((rows + per_warp - 1) / per_warp);
+    // A launch of at most one wave of blocks sets out under the tail of the kernel before it, and lets the gradient
+    // kernel set itself up under its own: 16.4 -> 15.2 us for a step of 8 candidates of 8 tokens.  Larger ones
+    // follow in plain stream order: overlapped, a step of 512 candidates of 48 tokens took 545 instead of 525 us.
+    const bool overlap = grid <= 8 * sm_count();
+    cudaError_t e = cudaSuccess;
+    {
+        KernelTiming timing(kKernelRowDot, stream);
+        auto kernel = a.dims.d == 128 ? simt_row_dot_kernel<128> : simt_row_dot_kernel<64>;
+        if (overlap) e = launch_dependent(kernel, grid, kWarpsPerBlock * 32, 0, stream, a);
+        else kernel<<<grid, kWarpsPerBlock * 32, 0, stream>>>(a);
+    }
+    if (e != cudaSuccess) return e;
     count_launches(1);
     return cudaGetLastError();
 }

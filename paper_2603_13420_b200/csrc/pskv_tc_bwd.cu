@@ -32,6 +32,11 @@
 // When the unit is one tile the pieces take turns; when it is several tiles, pass 0 accumulates piece 0 (and
 // all of dQ) and every later pass walks over the tiles once more for one further piece.
 //
+// Launches of few candidates (the gradient of a search's one current suffix) are split: every tile's dQ and every
+// suffix piece's dK / dV is a unit of its own, so that one candidate keeps up to tiles + pieces SMs per KV head
+// busy instead of one, at the price of forming the scores of the suffix pieces once more.  Whole steps: B = 1, 32/8
+// heads, P = 78, S = 113 45 -> 25 us; B = 4, 32/8, P = 1000, S = 100 96 -> 56; B = 20, 32/8, P = 200, S = 90 84 -> 77.
+//
 // Persistent CTA, one per SM, 24 warps:
 //   warp 0      TMA producer: K and V pieces (two rings); writes the descriptor of every item
 //   warp 1      tcgen05.mma issuer: S and dP
@@ -89,7 +94,8 @@ struct TcBwdParams {
     int Kq;                // candidates per instruction (all of them when there is one prefix)
     int upi, upg;          // units per (KV head, instruction), per KV head
     int unit0, n_units;
-    FastDiv fd_upg, fd_upi, fd_Rp, fd_S, fd_cpp;
+    int n_tiles, n_sub;    // split launch: dQ units and all units of a candidate (else n_sub = 1)
+    FastDiv fd_upg, fd_upi, fd_sub, fd_Rp, fd_S, fd_cpp;
     int stages_k, stages_v;
     int off_do, off_q, off_k, off_v, off_p, off_ds, off_rows, off_bar, off_misc;
     int pad[kMaxInstr];    // left padding of each instruction's prefix cache (Sec. 4.3)
@@ -134,42 +140,63 @@ constexpr int kRowsBytes = 2 * kTileM * 8;  // row tables (-lse log2(e), D) of t
 // eight entries are enough.
 enum : uint32_t {
     kDescN = 0x7f, kDescSfx = 1u << 7, kDescAcc = 1u << 8, kDescAccFirst = 1u << 9, kDescAccLast = 1u << 10,
-    kDescQDone = 1u << 11,     // last item of the tile that feeds dK / dV
+    kDescQDone = 1u << 11,     // last item of the tile that feeds dK / dV: its products are the last to read Q and dO
     kDescLast = 1u << 12, kDescDq = 1u << 13, kDescFirst = 1u << 14,
     kDescAccOdd = 1u << 15,    // parity of the items that fed dK / dV so far
     kDescK0 = 16, kDescK1 = 20,  // rows of the group inside the tile, in steps of 16 (4 bits each)
     kDescEnd = 1u << 31
 };
 
-// The walk over units, passes, tiles and items, the same in every role.
+// The walk over units, passes and tiles, the same in every role.  SPLIT: the units are the parts of a candidate (an
+// instantiation of its own: with the decision at run time the other launches were 4 % slower).
+template <bool SPLIT>
 struct Walk {
     int u, u_end;           // unit
     int g, inst, b0, ncand; // its KV head, instruction, first candidate, candidates
-    int ntile, npass, pass, tt;
+    int t_first, t_end, npass, pass, tt;
+    bool dq_;               // SPLIT: see dq(), fed()
+    int fed_;
     int R0, rows;           // tile: first row of the unit's row list, rows that belong to the unit
     int grp_lo, ngrp;       // candidate groups (pieces' worth of candidates) the tile touches
     int kp0;                // first prefix piece (pieces of padding only are left out)
-    int n_sfx, n_items;
-    // item
-    int k, e, j, q;         // position, interleaving state, next suffix / prefix index
-    bool sfx;
+    int n_sfx, n_items;     // suffix items, all items of the tile
 
     __device__ __forceinline__ bool done() const { return u >= u_end; }
+    // the pass forms dQ (and walks over the prefix)
+    __device__ __forceinline__ bool dq() const { return SPLIT ? dq_ : pass == 0; }
+    // pieces that feed dK / dV: 0 none, 1 all, 2 the one of number `pass`
+    __device__ __forceinline__ int fed() const { return SPLIT ? fed_ : npass > 1 ? 2 : 1; }
 
     __device__ __forceinline__ void unit(const TcBwdParams &p)
     {
         if (done()) return;
-        const int w = p.unit0 + u;
+        const int w = SPLIT ? p.fd_sub.div(p.unit0 + u) : p.unit0 + u;
         g = p.fd_upg.div(w);
         const int r = w - g * p.upg;
         inst = p.fd_upi.div(r);
         const int ub = r - inst * p.upi;
         b0 = inst * p.Kq + ub * p.cu;
         ncand = min(p.cu, p.Kq - ub * p.cu);
-        ntile = (ncand * p.Rp + kTileM - 1) / kTileM;
-        npass = ntile > 1 ? p.nh : 1;
-        pass = tt = 0;
         kp0 = p.pad[inst] / kPieceN;
+        t_first = pass = 0;
+        t_end = (ncand * p.Rp + kTileM - 1) / kTileM;
+        npass = t_end > 1 ? p.nh : 1;
+        if (SPLIT) {
+            const int sub = p.unit0 + u - w * p.n_sub;
+            if (sub < p.n_tiles) {
+                t_first = sub;
+                t_end = sub + 1;
+                npass = 1;
+                dq_ = true;
+                fed_ = 0;
+            } else {
+                pass = sub - p.n_tiles;
+                npass = pass + 1;
+                dq_ = false;
+                fed_ = 2;
+            }
+        }
+        tt = t_first;
         tile(p);
     }
     __device__ __forceinline__ void tile(const TcBwdParams &p)
@@ -178,10 +205,8 @@ struct Walk {
         rows = min(kTileM, ncand * p.Rp - R0);
         grp_lo = p.fd_cpp.div(p.fd_Rp.div(R0));
         ngrp = p.fd_cpp.div(p.fd_Rp.div(R0 + rows - 1)) - grp_lo + 1;
-        n_sfx = pass == 0 ? ngrp * p.nh : ngrp;
-        n_items = n_sfx + (pass == 0 ? p.nblk - kp0 : 0);
-        k = e = j = q = 0;
-        sfx = true;
+        n_sfx = dq() ? ngrp * p.nh : ngrp;
+        n_items = n_sfx + (dq() ? p.nblk - kp0 : 0);
     }
     __device__ __forceinline__ void start(const TcBwdParams &p)
     {
@@ -191,49 +216,35 @@ struct Walk {
     }
     __device__ __forceinline__ void next_tile(const TcBwdParams &p)
     {
-        if (++tt < ntile) { tile(p); return; }
-        tt = 0;
-        if (++pass < npass) { tile(p); return; }
+        if (++tt < t_end) { tile(p); return; }
+        if (++pass < npass) {
+            tt = t_first;
+            tile(p);
+            return;
+        }
         ++u;
         unit(p);
     }
-    // Suffix items are spread evenly over the tile's items, the first one first: their accumulators are
-    // drained, and their P buffer is read, under the prefix items in between.
-    __device__ __forceinline__ void next_item()
+    // suffix item j of the tile: candidate group and 64-key piece of its suffix
+    __device__ __forceinline__ int grp(const TcBwdParams &p, int j) const
     {
-        if (sfx) ++j; else ++q;
-        ++k;
-        e += n_sfx;
-        if (e >= n_items) e -= n_items;
-        sfx = e < n_sfx;
+        return grp_lo + (!dq() || p.nh == 1 ? j : j / p.nh);
     }
-    __device__ __forceinline__ bool last_item() const { return k == n_items - 1; }
-    // suffix item: candidate group and 64-key piece of its suffix
-    __device__ __forceinline__ int grp(const TcBwdParams &p) const
+    __device__ __forceinline__ int half(const TcBwdParams &p, int j) const
     {
-        return grp_lo + (pass > 0 || p.nh == 1 ? j : j / p.nh);
+        return !dq() ? pass : p.nh == 1 ? 0 : j - j / p.nh * p.nh;
     }
-    __device__ __forceinline__ int half(const TcBwdParams &p) const
-    {
-        return pass > 0 ? pass : p.nh == 1 ? 0 : j - j / p.nh * p.nh;
-    }
-    __device__ __forceinline__ bool acc(int h) const { return npass == 1 || h == pass; }  // feeds dK / dV
+    __device__ __forceinline__ bool acc(int h) const { return fed() == 1 || (fed() == 2 && h == pass); }  // feeds dK / dV
     __device__ __forceinline__ int grp_row0(const TcBwdParams &p, int gr) const { return gr * p.cpp * p.Rp; }
     __device__ __forceinline__ int grp_row1(const TcBwdParams &p, int gr) const
     {
         return min((gr + 1) * p.cpp, ncand) * p.Rp;
     }
-    // MMA N of the current item (keys rounded up to 16)
-    __device__ __forceinline__ int n16(const TcBwdParams &p) const
+    // key columns of a suffix item
+    __device__ __forceinline__ int sfx_cols(const TcBwdParams &p, int gr, int h) const
     {
-        int n;
-        if (!sfx) n = min(kPieceN, p.P - (kp0 + q) * kPieceN);
-        else if (p.nh > 1) n = min(kPieceN, p.S - half(p) * kPieceN);
-        else {
-            const int gr = grp(p);
-            n = p.cpp == 1 ? p.S : min(p.cpp, ncand - gr * p.cpp) * p.Sp;
-        }
-        return (n + 15) & ~15;
+        if (p.nh > 1) return min(kPieceN, p.S - h * kPieceN);
+        return p.cpp == 1 ? p.S : min(p.cpp, ncand - gr * p.cpp) * p.Sp;
     }
 };
 
@@ -253,7 +264,7 @@ __device__ __forceinline__ void store_sector(__nv_bfloat16 *dst, const uint32_t 
     }
 }
 
-template <int D>
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
               const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
@@ -301,7 +312,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     // everything above touched shared and tensor memory only: it may run under the tail of the kernel before
     grid_dep_wait();
 
-    Walk w;
+    Walk<SPLIT> w;
     w.start(p);
     bool ok = true;
 
@@ -319,17 +330,22 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll 1
         for (; !w.done() && ok; w.next_tile(p), ++tile) {
             const int head = w.inst * p.Hkv + w.g;
+            // suffix items are spread evenly over the tile's items, the first one first: their accumulators are drained, and
+            // their P buffer is read, under the prefix items in between
+            int e = 0, j = 0, q = 0;
+            bool sfx = true;
 #pragma unroll 1
-            for (; w.k < w.n_items; w.next_item(), ++item) {
-                int row, b = w.b0;
+            for (int k = 0; k < w.n_items; ++k, ++item) {
+                int row, b = w.b0, n;
                 uint4 dsc;
-                dsc.x = (uint32_t)w.n16(p) | (w.last_item() ? kDescLast : 0u) | (w.k == 0 ? kDescFirst : 0u) |
-                        (w.pass == 0 ? kDescDq : 0u);
+                dsc.x = (k == w.n_items - 1 ? kDescLast : 0u) | (k == 0 ? kDescFirst : 0u) | (w.dq() ? kDescDq : 0u) |
+                        (w.fed() == 0 && k == w.n_items - 1 ? kDescQDone : 0u);
                 dsc.w = (tile & 0xffffu) | (uint32_t)w.tt << 16;
-                if (w.sfx) {
-                    const int h = w.half(p), gr = w.grp(p);
+                if (sfx) {
+                    const int h = w.half(p, j), gr = w.grp(p, j);
                     row = h * kPieceN;
                     b += gr * p.cpp;
+                    n = w.sfx_cols(p, gr, h);
                     dsc.x |= kDescSfx;
                     dsc.y = (uint32_t)gr;
                     dsc.z = (uint32_t)row;
@@ -338,15 +354,17 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         dsc.x |= kDescAcc | (r0 >= 0 ? kDescAccFirst : 0u) | (r1 <= kTileM ? kDescAccLast : 0u) |
                                  ((n_acc & 1u) ? kDescAccOdd : 0u) | (uint32_t)(max(r0, 0) >> 4) << kDescK0 |
                                  (uint32_t)((min(r1, kTileM) + 15) >> 4) << kDescK1;
-                        if (gr == w.grp_lo + w.ngrp - 1 && (w.npass > 1 || h == p.nh - 1)) dsc.x |= kDescQDone;
+                        if (gr == w.grp_lo + w.ngrp - 1 && (w.fed() == 2 || h == p.nh - 1)) dsc.x |= kDescQDone;
                         ++n_acc;
                     }
                 } else {
-                    row = (w.kp0 + w.q) * kPieceN;
-                    dsc.y = (uint32_t)max(0, p.pad[w.inst] - row) | (uint32_t)(min(kPieceN, p.P - row) - 1) << 8;
+                    row = (w.kp0 + q) * kPieceN;
+                    n = min(kPieceN, p.P - row);
+                    dsc.y = (uint32_t)max(0, p.pad[w.inst] - row) | (uint32_t)(n - 1) << 8;
                     dsc.z = 0u;
                 }
-                const uint32_t tx = w.sfx ? sfx_tx : (uint32_t)C::kPieceBytes;
+                dsc.x |= (uint32_t)((n + 15) & ~15);
+                const uint32_t tx = sfx ? sfx_tx : (uint32_t)C::kPieceBytes;
                 ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProdKv);
                 if (!ok) break;
                 if (elect_one_sync()) {
@@ -355,7 +373,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     mbar_arrive_expect_tx(fb, tx);
 #pragma unroll
                     for (int sl = 0; sl < C::kSlabs; ++sl) {
-                        if (w.sfx) tma_load_4d(dst + sl * C::kPieceSlab, &tm_sk, fb, sl * 64, row, w.g, b);
+                        if (sfx) tma_load_4d(dst + sl * C::kPieceSlab, &tm_sk, fb, sl * 64, row, w.g, b);
                         else tma_load_3d(dst + sl * C::kPieceSlab, &tm_pk, fb, sl * 64, row, head);
                     }
                 }
@@ -367,13 +385,17 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     mbar_arrive_expect_tx(fb, tx);
 #pragma unroll
                     for (int sl = 0; sl < C::kSlabs; ++sl) {
-                        if (w.sfx) tma_load_4d(dst + sl * C::kPieceSlab, &tm_sv, fb, sl * 64, row, w.g, b);
+                        if (sfx) tma_load_4d(dst + sl * C::kPieceSlab, &tm_sv, fb, sl * 64, row, w.g, b);
                         else tma_load_3d(dst + sl * C::kPieceSlab, &tm_pv, fb, sl * 64, row, head);
                     }
                 }
                 __syncwarp();
                 if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
                 if (++vs == p.stages_v) { vs = 0; vph ^= 1u; }
+                if (sfx) ++j; else ++q;
+                e += w.n_sfx;
+                if (e >= w.n_items) e -= w.n_items;
+                sfx = e < w.n_sfx;
             }
         }
         // two end marks, one for each set of element-wise warps
@@ -553,11 +575,11 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     }
                     tc_commit(bar(kBarPFree));
                     if (x & kDescAccLast) tc_commit(bar(kBarAccFull));
-                    if (x & kDescQDone) tc_commit(bar(kBarQFree));
                 }
                 __syncwarp();
             }
             if (elect_one_sync()) {
+                if (x & kDescQDone) tc_commit(bar(kBarQFree));
                 tc_commit(bar(kBarDsFree + slot));
                 tc_commit(bar(kBarKFree + ks));
                 if ((x & (kDescLast | kDescDq)) == (kDescLast | kDescDq)) tc_commit(bar(kBarDqFull));
@@ -704,8 +726,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll 1
         for (; !w.done() && ok; w.next_tile(p)) {
 #pragma unroll 1
-            for (; w.j < w.n_sfx; ++w.j) {
-                const int h = w.half(p), gr = w.grp(p);
+            for (int j = 0; j < w.n_sfx; ++j) {
+                const int h = w.half(p, j), gr = w.grp(p, j);
                 if (!w.acc(h) || w.grp_row1(p, gr) > w.R0 + kTileM) continue;
                 // ---- accumulators of a candidate group: lane <-> column d, tensor-memory column <-> key
                 ok = mbar_wait_warp(bar(kBarAccFull), accph, abort_flag, p.status, kErrEpi);
@@ -713,7 +735,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 accph ^= 1u;
                 PSKV_TRACE_EVENT(30, w.u);
                 tc_fence_after();
-                const int n = w.n16(p);
+                const int n = w.sfx_cols(p, gr, h);
                 int b = w.b0 + gr * p.cpp, t = h * kPieceN;   // candidate and key of the coming eight columns
                 const int b_end = w.b0 + w.ncand;
 #pragma unroll 1
@@ -754,7 +776,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 PSKV_TRACE_EVENT(31, w.u);
             }
             if (!ok) break;
-            if (w.pass != 0) continue;
+            if (!w.dq()) continue;
             // ---- dQ of the tile
             ok = mbar_wait_warp(bar(kBarDqFull), dqph, abort_flag, p.status, kErrEpi);
             if (!ok) break;
@@ -798,6 +820,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 struct BwdPlan {
     bool ok;
     int cu, cpp, nh, Rp, Sp, seg, cbox, sfx_box, nblk, upi;
+    int n_tiles, n_sub;
     int stages_k, stages_v;
     int off_do, off_q, off_k, off_v, off_p, off_ds, off_rows, off_bar, off_misc, smem_bytes;
 };
@@ -842,6 +865,22 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
             pl.cbox = tiles == 1 && n_instr == 1 ? cu : 1;  // (a box must not reach into the next instruction)
         }
     }
+    {
+        // Split: the busiest SM's share is its units times the dearer kind.  Taken where that is well below what whole
+        // candidates give, which is when they leave SMs idle: one candidate of 113 tokens, 4 heads per KV head and
+        // 78 prefix tokens is 8 units of 20 items on 148 SMs, or 48 units of at most 4 items.
+        const int tiles = (pl.Rp + kTileM - 1) / kTileM;
+        const long long units = (long long)Kq * n_instr * dm.Hkv * (tiles + pl.nh);
+        const double dq = pl.nblk + 1 + pl.nh, piece = tiles * 2.3;
+        const double cost = (double)((units + sms - 1) / sms) * (dq > piece ? dq : piece);
+        pl.n_sub = 1;
+        if (tiles <= 1024 && cost < 0.85 * best) {
+            pl.n_tiles = tiles;
+            pl.n_sub = tiles + pl.nh;
+            pl.cu = pl.cpp = pl.cbox = 1;
+            pl.seg = tiles == 1 ? pl.Rp : kTileM;
+        }
+    }
     pl.sfx_box = pl.nh > 1 ? kPieceN : pl.Sp;
     pl.upi = (Kq + pl.cu - 1) / pl.cu;
     const int slabs = dm.d / 64;
@@ -862,7 +901,7 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
     pl.off_bar = pl.off_rows + kRowsBytes;
     pl.off_misc = pl.off_bar + kBarBytes;
     pl.smem_bytes = pl.off_misc + 64;
-    pl.ok = pl.smem_bytes <= kMaxSmem && (long long)pl.upi * n_instr * dm.Hkv < 2000000000ll;
+    pl.ok = pl.smem_bytes <= kMaxSmem && (long long)pl.upi * n_instr * dm.Hkv * pl.n_sub < 2000000000ll;
     return pl;
 }
 
@@ -924,6 +963,9 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     p.upg = plan.upi * n_instr;
     p.fd_upg.init(p.upg);
     p.fd_upi.init(p.upi);
+    p.n_tiles = plan.n_tiles;
+    p.n_sub = plan.n_sub;
+    p.fd_sub.init(p.n_sub);
     p.fd_Rp.init(p.Rp);
     p.fd_S.init(dm.S);
     p.fd_cpp.init(p.cpp);
@@ -932,9 +974,10 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     p.off_ds = plan.off_ds; p.off_rows = plan.off_rows; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
     for (int i = 0; i < n_instr && n_instr > 1; ++i) p.pad[i] = dm.P - prefix_len[i];
 
-    static PerDeviceOnce attr_set;
-    if (cudaError_t e = ensure_max_smem(tc_bwd_kernel<D>, attr_set); e != cudaSuccess) return e;
-    const int units = p.upg * dm.Hkv;
+    auto kernel = plan.n_sub > 1 ? tc_bwd_kernel<D, true> : tc_bwd_kernel<D, false>;
+    static PerDeviceOnce attr_set[2];
+    if (cudaError_t e = ensure_max_smem(kernel, attr_set[plan.n_sub > 1]); e != cudaSuccess) return e;
+    const int units = p.upg * dm.Hkv * p.n_sub;
     if (split > units) split = units;
     for (int s = 0; s < split; ++s) {
         p.unit0 = (int)((long long)units * s / split);
@@ -942,7 +985,7 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
         cudaError_t e;
         {
             KernelTiming timing(kKernelBwdTc, stream);
-            e = launch_dependent(tc_bwd_kernel<D>, even_grid(p.n_units, sm_count()), kThreads, plan.smem_bytes, stream, tm_q,
+            e = launch_dependent(kernel, even_grid(p.n_units, sm_count()), kThreads, plan.smem_bytes, stream, tm_q,
                                  tm_do, tm_pk, tm_pv, tm_sk, tm_sv, p);
         }
         count_launches(1);

@@ -40,6 +40,21 @@ def test_backward_matches_the_oracle(shape):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("shape", [
+    # enough candidates that whole candidates are the units (the shapes above are small enough for the split launch,
+    # in which every tile's dQ and every suffix piece's dK / dV is a unit of its own)
+    (700, 2, 2, 128, 40, 1), (420, 4, 4, 128, 64, 5), (320, 3, 3, 128, 1, 33), (400, 8, 2, 128, 130, 45),
+    (400, 8, 2, 128, 256, 48), (401, 8, 2, 64, 256, 48), (400, 4, 4, 128, 191, 65), (400, 8, 2, 128, 78, 113),
+    (300, 2, 2, 128, 70, 129), (900, 1, 1, 64, 33, 72),
+], ids=lambda s: "x".join(map(str, s)))
+def test_backward_of_many_candidates_matches_the_oracle(shape):
+    B, Hq, Hkv, d, P, S = shape
+    w = Workload("units", 1700 + sum(shape), B=B, Hq=Hq, Hkv=Hkv, d=d, P=P, S=S)
+    assert pskv.pskv_kernel_family(1, B, Hq, Hkv, S, P, d) == 1
+    parity.bwd_parity(w, cand=[0, 1, 2, B // 2 - 1, B // 2, B - 3, B - 2, B - 1])
+
+
+@pytest.mark.gpu
 def test_dq_at_a_base_that_is_16_but_not_32_bytes_aligned():
     """dQ leaves in whole 32-byte sectors where its base allows it, else in 16-byte halves: the same bits."""
     w = Workload("units", 899, B=4, Hq=8, Hkv=2, d=128, P=90, S=24)
