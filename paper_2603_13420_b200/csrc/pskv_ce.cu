@@ -8,13 +8,14 @@
 // (max, sum) per row and pick out the target's logit while the tensor cores already work on the next
 // block in the other half of tensor memory.
 //
-// Work units are (vocabulary panel of 8 blocks, 128-row tile).  Row tiles are taken in groups of a
+// Work units are (vocabulary panel of up to 16 blocks, 128-row tile); the panel is as wide as lets the units
+// fill whole rounds of the SMs (ce_panel).  Row tiles are taken in groups of a
 // quarter of the CTA count; inside a group the units are numbered panel-major, row tile fastest, and
 // CTA c takes units c, c + G, c + 2G, ...: the CTAs running at any moment work on about four weight
 // panels (16 MB each) against one group of row tiles (1 MB each), a working set that stays in L2, so
 // the weight matrix comes from HBM once per row group and the hidden states once.  Each unit
-// leaves one partial (max, sum) per row; two small kernels merge the partials of a row into lse
-// and nll = mask * (lse - target logit) and form the masked average per candidate.
+// leaves one partial (max, sum) per row; a small kernel, one block per candidate, merges the partials of its rows
+// into lse and nll = mask * (lse - target logit) and forms the masked average.
 //
 // Roles (256 threads): warp 0 TMA producer (hidden tile and weight block, 64 columns of the hidden
 // dimension per stage, 4 stages), warp 1 tcgen05.mma issuer, warp 2 owns the tensor-memory
@@ -34,7 +35,7 @@ constexpr int kCeM = 128;        // rows per tile (tensor-memory lanes)
 constexpr int kCeN = 256;        // vocabulary entries per block (one MMA N, half of tensor memory)
 constexpr int kCeK = 64;         // hidden columns per stage: one 128-byte swizzle slab
 constexpr int kCeStages = 4;
-constexpr int kCePanel = 8;      // blocks per panel
+constexpr int kCeMaxPanel = 16;  // blocks per panel at most
 constexpr int kCeThreads = 256;
 constexpr int kCeABytes = kCeM * 128, kCeBBytes = kCeN * 128, kCeStageBytes = kCeABytes + kCeBBytes;
 
@@ -45,11 +46,11 @@ enum { kCeBarFull = 0, kCeBarEmpty = kCeStages, kCeBarAccFull = 2 * kCeStages, k
 
 struct CeParams {
     const int *target;     // [R]
-    float *part_m, *part_l;  // [npanel][Rpad], log2 domain
+    float2 *part;          // [R][npanel] (max, sum), log2 domain
     float *tlogit;         // [R] logit of the target token (natural units)
     unsigned int *status;
-    int R, Rpad, Dm, V;
-    int nrt, nvb, npanel, units, ksteps;
+    int R, Dm, V;
+    int nrt, nvb, panel, npanel, units, ksteps;
     int rg;                // row tiles per group
 };
 
@@ -115,9 +116,9 @@ ce_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ 
             const int u = (int)blockIdx.x + tl * (int)gridDim.x;
             int pn, rt;
             ce_unit(p, u, pn, rt);
-            const int vb_end = min(p.nvb, (pn + 1) * kCePanel);
+            const int vb_end = min(p.nvb, (pn + 1) * p.panel);
 #pragma unroll 1
-            for (int vb = pn * kCePanel; vb < vb_end && ok; ++vb) {
+            for (int vb = pn * p.panel; vb < vb_end && ok; ++vb) {
 #pragma unroll 1
                 for (int ks = 0; ks < p.ksteps; ++ks, ++it) {
                     const uint32_t s = it % kCeStages;
@@ -146,9 +147,9 @@ ce_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ 
             const int u = (int)blockIdx.x + tl * (int)gridDim.x;
             int pn, rt;
             ce_unit(p, u, pn, rt);
-            const int vb_end = min(p.nvb, (pn + 1) * kCePanel);
+            const int vb_end = min(p.nvb, (pn + 1) * p.panel);
 #pragma unroll 1
-            for (int vb = pn * kCePanel; vb < vb_end && ok; ++vb, ++blk) {
+            for (int vb = pn * p.panel; vb < vb_end && ok; ++vb, ++blk) {
                 const uint32_t a = blk & 1u;
                 // the accumulator half is free once the fold warps have read block blk - 2 out of it
                 ok = mbar_wait_warp(bar(kCeBarAccFree + a), ((blk >> 1) & 1) ^ 1, abort_flag, p.status, kErrCeMma);
@@ -186,14 +187,14 @@ ce_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ 
             const int u = (int)blockIdx.x + tl * (int)gridDim.x;
             int pn, rt;
             ce_unit(p, u, pn, rt);
-            const int vb_end = min(p.nvb, (pn + 1) * kCePanel);
+            const int vb_end = min(p.nvb, (pn + 1) * p.panel);
             const int grow = rt * kCeM + row;
             const bool valid = grow < p.R;
             const int z = valid ? p.target[grow] : -1;
             float m = -INFINITY, l = 0.f, zt = 0.f;  // running max and sum in the log2 domain
             bool have_zt = false;
 #pragma unroll 1
-            for (int vb = pn * kCePanel; vb < vb_end && ok; ++vb, ++blk) {
+            for (int vb = pn * p.panel; vb < vb_end && ok; ++vb, ++blk) {
                 const uint32_t a = blk & 1u;
                 ok = mbar_wait_warp(bar(kCeBarAccFull + a), (blk >> 1) & 1, abort_flag, p.status, kErrCeFold);
                 if (!ok) break;
@@ -237,8 +238,7 @@ ce_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ 
                 if (lane == 0) mbar_arrive(bar(kCeBarAccFree + a));
             }
             if (ok && valid) {
-                p.part_m[(size_t)pn * p.Rpad + grow] = m;
-                p.part_l[(size_t)pn * p.Rpad + grow] = l;
+                p.part[(size_t)grow * p.npanel + pn] = make_float2(m, l);
                 if (have_zt) p.tlogit[grow] = zt;
             }
         }
@@ -250,47 +250,62 @@ ce_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ 
     if (warp == 2) tmem_dealloc(tmem, 512);
 }
 
-// Merges the partials of every row: one thread per row (consecutive threads read consecutive
-// addresses of every panel's partial arrays), lse and nll per row.
-__global__ void __launch_bounds__(256)
-ce_rows_kernel(const float *part_m, const float *part_l, const float *tlogit, const int *target, const float *mask,
-               float *nll, float *lse, long long R, int Rpad, int npanel, int V)
+// One block per candidate, a warp per row at a time: merges the partials of the candidate's rows (contiguous, one lane
+// each) into lse and nll, then the masked average.  (One thread per row, walking over the panels, took 13 to 30 us,
+// and a third launch, in calls whose projection takes 40 to 400.)
+constexpr int kCeFinalWarps = 8;
+__global__ void __launch_bounds__(32 * kCeFinalWarps)
+ce_finalize_kernel(const float2 *part, const float *tlogit, const int *target, const float *mask, float *nll, float *lse,
+                   float *loss, int Lr, int npanel, int V)
 {
-    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    float M = -INFINITY;
-    for (int pn = 0; pn < npanel; ++pn) M = fmaxf(M, part_m[(size_t)pn * Rpad + r]);
-    float L = 0.f;
-    for (int pn = 0; pn < npanel; ++pn) L += part_l[(size_t)pn * Rpad + r] * exp2f(part_m[(size_t)pn * Rpad + r] - M);
-    const float ls = (M + log2f(L)) * kLn2;
-    lse[r] = ls;
-    const float w = mask[r];
-    float v = 0.f;
-    if (w != 0.f) {
-        const int z = target[r];
-        v = (z >= 0 && z < V) ? w * (ls - tlogit[r]) : __int_as_float(0x7fc00000);  // a bad token id shows as NaN
-    }
-    nll[r] = v;
-}
-
-// Masked average per candidate: one warp per candidate.
-__global__ void __launch_bounds__(256)
-ce_finalize_kernel(const float *nll, const float *mask, float *loss, int N, int Lr)
-{
-    const int warp = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (warp >= N) return;
+    __shared__ float num_s[kCeFinalWarps], den_s[kCeFinalWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float num = 0.f, den = 0.f;
-    for (int i = lane; i < Lr; i += 32) {
-        const size_t r = (size_t)warp * Lr + i;
-        num += nll[r];
-        den += mask[r];
-    }
+    for (int i = warp; i < Lr; i += kCeFinalWarps) {
+        const size_t r = (size_t)blockIdx.x * Lr + i;
+        const float2 *pr = part + r * npanel;
+        float M = -INFINITY, L = 0.f;
+        for (int pn = lane; pn < npanel; pn += 32) {
+            const float2 x = pr[pn];
+            const float m = fmaxf(M, x.x);
+            // (a panel may hold nothing but -inf logits: m - M would be inf - inf)
+            L = (M == m ? L : L * exp2f(M - m)) + (x.x == m ? x.y : x.y * exp2f(x.x - m));
+            M = m;
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, M, o), l2 = __shfl_xor_sync(0xffffffffu, L, o);
+            const float m = fmaxf(M, m2);
+            L = (M == m ? L : L * exp2f(M - m)) + (m2 == m ? l2 : l2 * exp2f(m2 - m));
+            M = m;
+        }
+        const float ls = (M + log2f(L)) * kLn2;
+        const float w = mask[r];
+        float v = 0.f;
+        if (w != 0.f) {
+            const int z = target[r];
+            v = (z >= 0 && z < V) ? w * (ls - tlogit[r]) : __int_as_float(0x7fc00000);  // a bad token id shows as NaN
+        }
+        if (lane == 0) {
+            lse[r] = ls;
+            nll[r] = v;
+        }
+        num += v;
+        den += w;
     }
-    if (lane == 0) loss[warp] = den != 0.f ? num / den : 0.f;
+    if (lane == 0) {
+        num_s[warp] = num;
+        den_s[warp] = den;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        num = den = 0.f;
+        for (int k = 0; k < kCeFinalWarps; ++k) {
+            num += num_s[k];
+            den += den_s[k];
+        }
+        loss[blockIdx.x] = den != 0.f ? num / den : 0.f;
+    }
 }
 
 inline bool encode_2d(CUtensorMap *map, const void *base, int cols, long long rows, int box_rows)
@@ -302,20 +317,43 @@ inline bool encode_2d(CUtensorMap *map, const void *base, int cols, long long ro
 }
 
 struct CePlan {
-    int nrt, nvb, npanel, Rpad, ksteps;
+    int nrt, nvb, panel, npanel, Rpad, ksteps;
     size_t part_bytes, ws_bytes;
 };
+
+// Blocks per panel: a CTA's time is its units times their blocks, so the width is the one whose units fill the last
+// round of the SMs best, 8 where nothing is clearly better.  204 rows of a 32 000-word vocabulary are 32 units of
+// 8 blocks on 148 SMs, or 250 of one; 10 240 rows of 128 256 words 34.05 rounds of 8, or 38.9 of 7.  Whole calls at
+// Dm = 4096 against 8 blocks throughout: 204 rows x 32 000 words 191 -> 77 us, 270 x 128 256 449 -> 366, 512 x 32 000
+// 193 -> 130, 3 540 x 32 000 815 -> 711, 10 240 x 128 256 8.10 -> 7.98 ms.
+int ce_panel(int nrt, int nvb)
+{
+    const int sms = sm_count();
+    auto cost = [&](int panel) {
+        const long long units = (long long)((nvb + panel - 1) / panel) * nrt;
+        return (double)((units + sms - 1) / sms) * (panel + 0.1);
+    };
+    int best = 8;
+    double best_cost = 0.99 * cost(8);
+    for (int panel = kCeMaxPanel; panel >= 1; --panel)
+        if (cost(panel) < best_cost) {
+            best = panel;
+            best_cost = cost(panel);
+        }
+    return best;
+}
 
 CePlan ce_plan(long long R, int Dm, int V)
 {
     CePlan pl;
     pl.nrt = (int)((R + kCeM - 1) / kCeM);
     pl.nvb = (V + kCeN - 1) / kCeN;
-    pl.npanel = (pl.nvb + kCePanel - 1) / kCePanel;
+    pl.panel = ce_panel(pl.nrt, pl.nvb);
+    pl.npanel = (pl.nvb + pl.panel - 1) / pl.panel;
     pl.Rpad = pl.nrt * kCeM;
     pl.ksteps = (Dm + kCeK - 1) / kCeK;
-    pl.part_bytes = (size_t)pl.npanel * pl.Rpad * sizeof(float);
-    pl.ws_bytes = 2 * pl.part_bytes + (size_t)pl.Rpad * sizeof(float);
+    pl.part_bytes = (size_t)pl.npanel * pl.Rpad * sizeof(float2);
+    pl.ws_bytes = pl.part_bytes + (size_t)pl.Rpad * sizeof(float);
     return pl;
 }
 
@@ -344,12 +382,11 @@ cudaError_t launch_ce_fwd(const CeArgs &a, void *workspace, unsigned int *status
     if (!encode_2d(&tm_w, a.weight, a.Dm, a.V, kCeN)) return cudaErrorInvalidValue;
     CeParams p;
     p.target = a.target;
-    p.part_m = static_cast<float *>(workspace);
-    p.part_l = p.part_m + (size_t)pl.npanel * pl.Rpad;
-    p.tlogit = p.part_l + (size_t)pl.npanel * pl.Rpad;
+    p.part = static_cast<float2 *>(workspace);
+    p.tlogit = reinterpret_cast<float *>(p.part + (size_t)pl.npanel * pl.Rpad);
     p.status = status_word;
-    p.R = (int)R; p.Rpad = pl.Rpad; p.Dm = a.Dm; p.V = a.V;
-    p.nrt = pl.nrt; p.nvb = pl.nvb; p.npanel = pl.npanel; p.units = pl.npanel * pl.nrt; p.ksteps = pl.ksteps;
+    p.R = (int)R; p.Dm = a.Dm; p.V = a.V;
+    p.nrt = pl.nrt; p.nvb = pl.nvb; p.panel = pl.panel; p.npanel = pl.npanel; p.units = pl.npanel * pl.nrt; p.ksteps = pl.ksteps;
     p.rg = sm_count() / 4 < 1 ? 1 : sm_count() / 4;
     if (p.rg > pl.nrt) p.rg = pl.nrt;
     const int smem_bytes = kCeStages * kCeStageBytes + 8 * kCeNumBars + 64;
@@ -364,13 +401,10 @@ cudaError_t launch_ce_fwd(const CeArgs &a, void *workspace, unsigned int *status
     if (e != cudaSuccess) return e;
     {
         KernelTiming timing(kKernelCeFinalize, stream);
-        ce_rows_kernel<<<(unsigned)((R + 255) / 256), 256, 0, stream>>>(p.part_m, p.part_l, p.tlogit, a.target, a.mask, a.nll,
-                                                                       a.lse, R, pl.Rpad, pl.npanel, a.V);
-        const int warps_per_block = 8;
-        ce_finalize_kernel<<<(a.N + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, stream>>>(
-            a.nll, a.mask, a.loss, a.N, a.Lr);
+        ce_finalize_kernel<<<(unsigned)a.N, 32 * kCeFinalWarps, 0, stream>>>(p.part, p.tlogit, a.target, a.mask, a.nll, a.lse,
+                                                                            a.loss, a.Lr, pl.npanel, a.V);
     }
-    count_launches(3);
+    count_launches(2);
     return cudaGetLastError();
 }
 
