@@ -1192,17 +1192,19 @@ TilePlan plan_suffix_ring(const Dims &dm)
         pl.Spad = round_up(dm.Skv, 8);
         pl.cpb = kBlockN / pl.Spad;
         const int cmax = kTileM / Rg < dm.B ? kTileM / Rg : dm.B;
-        // Candidates per tile: as many as fit, unless a few less give every SM a tile (or one round of tiles
-        // less): a CTA's time is its tiles times the key blocks of a tile.  With 512 candidates of one query row
-        // x 4 heads, 32 per tile are 128 tiles of 18 blocks on 148 SMs, 30 per tile are 144 tiles of 17.
+        // Candidates per tile: as many as fit, unless fewer give more SMs a tile or make a round less: a CTA's time is
+        // its tiles times the key blocks of a tile, and the suffix blocks of a tile grow with its candidates.  With 512
+        // candidates of one query row x 4 heads, 32 per tile are 128 tiles of 18 blocks on 148 SMs, 30 per tile
+        // are 144 tiles of 17; 24 candidates with 126 cached tokens are 8 tiles of 28 blocks, or 96 of 6 (25 -> 13 us; 40
+        // candidates of 64 tokens on 32/32 heads 27 -> 16; 131 with a prefix of 1872 28 -> 24).
         const int sms = sm_count();
         const int nblk = (dm.P + kBlockN - 1) / kBlockN;
         long long best_cost = -1;
         pl.cbox = cmax;
-        for (int c = cmax; c >= 1 && c >= cmax - 8; --c) {
+        for (int c = cmax; c >= 1; --c) {
             const long long tiles = (long long)dm.Hkv * ((dm.B + c - 1) / c);
             const long long rounds = (tiles + sms - 1) / sms;
-            const long long cost = rounds * (nblk + (c + pl.cpb - 1) / pl.cpb);
+            const long long cost = rounds * (nblk + (c + pl.cpb - 1) / pl.cpb + 1);
             if (best_cost < 0 || cost < best_cost) {
                 best_cost = cost;
                 pl.cbox = c;
