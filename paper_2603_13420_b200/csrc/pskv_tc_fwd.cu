@@ -64,10 +64,13 @@ struct TcFwdParams {
     int Rg;               // rows a candidate takes in the row list of a KV-head group (its n_rep * S real rows, padded)
     int Rr;               // its real rows: n_rep * S
     int Sp;               // key columns a candidate takes in a tile's suffix block: S rounded up to 8
+    int Sh;               // rows a query head takes in the row list: S, or S padded to whole tiles (head_box)
+    int one_box;          // 1: a tile's Q is one box per slab (whole candidates, or rows of one head), else runs of seg_rows
+    int head_box;         // 1: Q / out maps are [B][Hq][S][D] and a tile lies inside one head
     int tile_rows;        // rows of the flat row list per tile (<= 128, multiple of seg_rows)
     int seg_rows;         // rows per Q / out TMA box: gcd(Rg, tile_rows) (rows past Rr are zero-filled, never stored)
     int tiles_per_group;
-    FastDiv fd_tpg, fd_Rg, fd_S, fd_seg;  // divisions by tiles_per_group, Rg, S, seg_rows
+    FastDiv fd_tpg, fd_Rg, fd_S, fd_seg;  // divisions by tiles_per_group, Rg, Sh, seg_rows
     int total_tiles;
     int nblk_p;           // prefix key blocks: ceil(P / 128)
     int tail_rows;        // rows held by the last prefix block (multiple of 16, <= 128)
@@ -127,6 +130,19 @@ enum {
 constexpr int kBarBytes = 512;
 static_assert(kNumBars * 8 <= kBarBytes, "barrier area");
 
+// Q / out box coordinates of row r of a group: (row, head) -- the group's row list seen as one head, or the head itself
+template <bool SR>
+__device__ __forceinline__ void q_coords(const TcFwdParams &p, int r, int g, int &c1, int &c2)
+{
+    c1 = r;
+    c2 = g;
+    if (SR && p.head_box) {
+        const int h = p.fd_S.div(r);
+        c1 = r - h * p.Sh;
+        c2 = g * p.n_rep + h;
+    }
+}
+
 // rows held (and MMA N used) by prefix block k
 __device__ __forceinline__ int prefix_block_rows(const TcFwdParams &p, int k)
 {
@@ -152,7 +168,7 @@ __device__ __forceinline__ int sfx_block_rows(const TcFwdParams &p, int nc, int 
 __device__ __forceinline__ int sfx_blocks_long(const TcFwdParams &p, const TileInfo &t)
 {
     const int r0 = t.R0 - t.b_first * p.Rg;
-    const int s0 = r0 - p.fd_S.div(r0) * p.S;  // query index of the tile's first row
+    const int s0 = r0 - p.fd_S.div(r0) * p.Sh;  // query index of the tile's first row
     const int s_max = (s0 + t.rows > p.S) ? p.S - 1 : s0 + t.rows - 1;  // rows wrap into the next head
     const int pos = suffix_tokens(p.suffix_len, t.b_first, p.S, p.Skv) - p.S + s_max;
     return (pos >> 7) + 1;
@@ -233,7 +249,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int t_begin = (int)((long long)blockIdx.x * p.total_tiles / gridDim.x);
     const int t_end = (int)((long long)(blockIdx.x + 1) * p.total_tiles / gridDim.x);
     const int G = (int)gridDim.x;
-    const int n_sp = (SR && p.deal_by_cost) ? p.S / p.tile_rows : 1;  // tiles per head
+    const int n_sp = (SR && p.deal_by_cost) ? p.Sh / p.tile_rows : 1;  // tiles per head
     const bool dealt = n_sp > 1;
     auto rank_at = [&](int tl) { return tl * G + ((tl & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
     auto tile_at = [&](int tl) {
@@ -291,7 +307,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // score MMA of the previous tile done" to "Q of this tile requested" is exposed.
             // (Suffix-ring mode: one box per slab holds the tile's whole candidates; a box reaching
             // past the last candidate is filled with zeros and still counts its full size.)
-            const int nseg = SR ? 1 : p.fd_seg.div(t.rows);  // one box per run of seg_rows rows
+            const int nseg = (SR && p.one_box) ? 1 : p.fd_seg.div(t.rows);  // one box per run of seg_rows rows
             int qb = p.fd_Rg.div(t.R0), qr = t.R0 - qb * p.Rg;
             const uint32_t q_bytes = (uint32_t)(nseg * C::kSlabs * p.seg_rows * 128);
             const uint32_t seg_bytes = (uint32_t)(p.seg_rows * 128);
@@ -300,13 +316,15 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // be issued a tile from now, right when it is needed, and then finds the data close by.
             if (tl + 1 < n_tiles) {
                 const TileInfo tn = tile_info(p, tile_at(tl + 1), t_begin);
-                const int nseg_n = SR ? 1 : p.fd_seg.div(tn.rows);
+                const int nseg_n = (SR && p.one_box) ? 1 : p.fd_seg.div(tn.rows);
                 int nb = p.fd_Rg.div(tn.R0), nr = tn.R0 - nb * p.Rg;
                 if (elect_one_sync()) {
 #pragma unroll 1
                     for (int s = 0; s < nseg_n; ++s) {
+                        int c1, c2;
+                        q_coords<SR>(p, nr, tn.g, c1, c2);
 #pragma unroll
-                        for (int sl = 0; sl < C::kSlabs; ++sl) tma_prefetch_4d(&tm_q, sl * 64, nr, tn.g, nb);
+                        for (int sl = 0; sl < C::kSlabs; ++sl) tma_prefetch_4d(&tm_q, sl * 64, c1, c2, nb);
                         nr += p.seg_rows;
                         if (nr >= p.Rg) {
                             nr -= p.Rg;
@@ -325,9 +343,11 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 mbar_arrive_expect_tx(bar(kBarQFull), q_bytes);
 #pragma unroll 1
                 for (int s = 0; s < nseg; ++s) {
+                    int c1, c2;
+                    q_coords<SR>(p, qr, t.g, c1, c2);
 #pragma unroll
                     for (int sl = 0; sl < C::kSlabs; ++sl)
-                        tma_load_4d(q_dst + sl * C::kSlabBytes, &tm_q, bar(kBarQFull), sl * 64, qr, t.g, qb);
+                        tma_load_4d(q_dst + sl * C::kSlabBytes, &tm_q, bar(kBarQFull), sl * 64, c1, c2, qb);
                     q_dst += seg_bytes;
                     qr += p.seg_rows;  // boxes never straddle a candidate: seg_rows divides Rg
                     if (qr >= p.Rg) {
@@ -547,7 +567,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     if (!ok) break;
                     if (ready) {
                         const TileInfo u = tile_info(p, tile_at(tl - 1), t_begin);
-                        const int nseg = SR ? 1 : p.fd_seg.div(u.rows);  // (one box of whole candidates)
+                        const int nseg = (SR && p.one_box) ? 1 : p.fd_seg.div(u.rows);
                         const int sl_first = p.slab_stage ? store_slab : 0;
                         const int sl_end = p.slab_stage ? store_slab + 1 : C::kSlabs;
                         if (elect_one_sync()) {
@@ -558,8 +578,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                                     const int R = u.R0 + s * p.seg_rows;
                                     const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
                                     if (r >= p.Rr) continue;  // padding only
+                                    int c1, c2;
+                                    q_coords<SR>(p, r, u.g, c1, c2);
                                     tma_store_4d(&tm_out, stage + (p.slab_stage ? 0 : sl) * kStagingBytes + s * p.seg_rows * 128,
-                                                 sl * 64, r, u.g, b);
+                                                 sl * 64, c1, c2, b);
                                 }
                             tma_store_commit();
                             tma_store_wait_read();  // the staging buffer may be overwritten after this
@@ -808,8 +830,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (row < t.rows) {
                 const int R = t.R0 + row;
                 const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-                const int i = r - p.fd_S.div(r) * p.S;  // query index inside the candidate
-                if (r >= p.Rr) {
+                const int i = r - p.fd_S.div(r) * p.Sh;  // query index inside the candidate
+                if (r >= p.Rr || (SR && i >= p.S)) {
                     // a padding row between two candidates: sees no suffix key, is never stored
                 } else if (SR) {
                     // query i is suffix token L - S + i of its candidate: suffix keys 0 .. L - S + i
@@ -1053,9 +1075,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             }
             const int R = u.R0 + row;
             const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-            const bool stored = row < u.rows && r < p.Rr;
+            const int hd = SR ? p.fd_S.div(r) : 0, skip = hd * (p.Sh - p.S);  // (head_box: padding rows before this head)
+            const bool stored = row < u.rows && r < p.Rr && (!SR || r - hd * p.Sh < p.S);
             if (stored) {
-                const size_t grow = ((size_t)b * p.Hq + (size_t)u.g * p.n_rep) * p.S + r;
+                const size_t grow = ((size_t)b * p.Hq + (size_t)u.g * p.n_rep) * p.S + r - skip;
                 p.lse[grow] = row_ok ? log2f(l) * kLn2 : __int_as_float(0x7fc00000);
             }
             const unsigned bad = __ballot_sync(0xffffffffu, stored && !row_ok);
@@ -1083,8 +1106,9 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             for (int r = warp; r < t.rows; r += kThreads / 32) {
                 const int R = t.R0 + r;
                 const int b = p.fd_Rg.div(R), rr = R - b * p.Rg;
-                if (rr >= p.Rr) continue;
-                const long long grow = ((long long)b * p.Hq + (long long)t.g * p.n_rep) * p.S + rr;
+                const int hd = SR ? p.fd_S.div(rr) : 0;
+                if (rr >= p.Rr || (SR && rr - hd * p.Sh >= p.S)) continue;
+                const long long grow = ((long long)b * p.Hq + (long long)t.g * p.n_rep) * p.S + rr - hd * (p.Sh - p.S);
                 const float v = p.lse[grow];
                 if (v != v) {
                     if (MI) {  // the row's own prefix cache, without its left padding
@@ -1112,7 +1136,8 @@ struct TilePlan {
     int cbox, Spad, cpb;  // suffix-ring mode: candidates per tile, rows per candidate in a block, candidates per block
     int long_sfx;         // suffix-ring mode: tiles inside one candidate, its suffix keys in 128-key blocks
     int tile_rows, seg_rows, tiles_per_group, sfx_rows;
-    int Rp, Sp;           // rows / suffix key columns a candidate takes (base tiling)
+    int Rp, Sp;           // rows / suffix key columns a candidate takes
+    int Sh, one_box, head_box;  // see TcFwdParams
     double cost;          // estimated SM cycles of a KV head's tiles
     int nblk_p, tail_rows, resident, stages, alias_stage, slab_stage, ml_tiles;
     int off_pk, off_pv, off_q, off_sk, off_sv, off_stage, off_bar, off_misc, off_ml, smem_bytes;
@@ -1121,7 +1146,7 @@ struct TilePlan {
 // Cycles of a tile, for the choice of a tiling: about 2 000 per key block, 1 700 for the tile itself, and 60 per
 // box of Q and of `out` (one thread issues them; with sixteen boxes of 8 rows that is 1 000 cycles in which the
 // single Q buffer is waited for).
-double tile_cost(int blocks, int boxes) { return 2000.0 * blocks + 1700.0 + 60.0 * boxes; }
+double tile_cost(double blocks, int boxes) { return 2000.0 * blocks + 1700.0 + 60.0 * boxes; }
 
 // Rows a candidate takes in the row list (Rp >= n_rep * S) and rows per tile, both multiples of 8, such that the
 // suffix keys of all candidates a tile can touch (Sp columns each) fit one 128-key block.  Suffix lengths are
@@ -1132,11 +1157,13 @@ double tile_cost(int blocks, int boxes) { return 2000.0 * blocks + 1700.0 + 60.0
 // B = 333, 32/8 heads, P = 217, S = 53 173 -> 120 us; B = 64, 32/32, P = 230, S = 85 74 -> 57; B = 42, 32/8, P = 112,
 // S = 117 44 -> 36; and against tiles of the largest divisor: B = 128, 32/8, P = 256, S = 80 (336 rows, three tiles
 // of 112, instead of four of 80) 101 -> 82.
-bool pick_tile_rows(const Dims &dm, TilePlan *pl, int *nc_max)
+//
+// ring: the suffix keys come in several blocks through the K / V rings, so a tile may touch any number of candidates.
+bool pick_tile_rows(const Dims &dm, bool ring, TilePlan *pl, int *nc_max)
 {
     const int Sp = round_up(dm.S, 8);
     if (Sp > kBlockN) return false;
-    const int Rg = dm.n_rep * dm.S, nblk = (dm.P + kBlockN - 1) / kBlockN;
+    const int Rg = dm.n_rep * dm.S, nblk = (dm.P + kBlockN - 1) / kBlockN, cpb = kBlockN / Sp;
     double best = -1.0;
     for (int Rp = round_up(Rg, 8); Rp < Rg + kTileM; Rp += 8) {
         if ((long long)dm.B * Rp > 2000000000ll) break;
@@ -1146,9 +1173,11 @@ bool pick_tile_rows(const Dims &dm, TilePlan *pl, int *nc_max)
             // candidates that a window of m rows can touch, its offset in a candidate being a multiple of seg
             int nc = m % Rp == 0 ? m / Rp : Rp % m == 0 ? 1 : (m - seg + Rp - 1) / Rp + 1;
             if (nc > dm.B) nc = dm.B;
-            if (nc * Sp > kBlockN) continue;
+            if (!ring && nc * Sp > kBlockN) continue;
             const long long tiles = ((long long)dm.B * Rp + m - 1) / m;
-            const double cost = (double)tiles * tile_cost(nblk + 1, m / seg);
+            // suffix blocks of a tile: one, or (ring) one and a share for each candidate it touches beyond the first
+            const double sfx = ring ? 1.0 + (double)(m - seg) / Rp / cpb : 1.0;
+            const double cost = (double)tiles * tile_cost(nblk + sfx, m / seg);
             if (best < 0.0 || cost < best) {
                 best = cost;
                 pl->Rp = Rp;
@@ -1165,6 +1194,31 @@ bool pick_tile_rows(const Dims &dm, TilePlan *pl, int *nc_max)
     return true;
 }
 
+// Shared memory of the suffix-ring mode: K and V rings, Q, the staging buffer.
+void layout_ring(const Dims &dm, TilePlan *pl)
+{
+    pl->nblk_p = (dm.P + kBlockN - 1) / kBlockN;
+    pl->tail_rows = pl->nblk_p ? round_up(dm.P - (pl->nblk_p - 1) * kBlockN, 16) : 0;
+    const int slabs = dm.d / 64;
+    const int tile_bytes = slabs * kTileM * 128;
+    const int ml_bytes = 4 * kGroups * kTileM * 4;
+    const int stage_bytes = slabs * kStagingBytes;
+    const int fixed = tile_bytes /*Q*/ + stage_bytes + ml_bytes + 64 + kBarBytes;
+    int st = (kMaxSmem - fixed) / (2 * tile_bytes);
+    if (st > kMaxStages) st = kMaxStages;
+    if (st < 1) return;
+    pl->stages = st;
+    pl->off_pk = 0;
+    pl->off_pv = st * tile_bytes;
+    pl->off_q = 2 * st * tile_bytes;
+    pl->off_sk = pl->off_sv = pl->off_stage = pl->off_q + tile_bytes;  // no suffix buffers of their own
+    pl->off_bar = pl->off_stage + stage_bytes;
+    pl->off_misc = pl->off_bar + kBarBytes;
+    pl->off_ml = pl->off_misc + 64;
+    pl->smem_bytes = pl->off_ml + ml_bytes;
+    pl->ok = pl->smem_bytes <= kMaxSmem;
+}
+
 // Suffix-ring mode: a tile is the largest run of whole candidates with at most 128 rows; the
 // suffix keys follow the prefix blocks through K/V rings, 128 / Spad candidates per block.
 TilePlan plan_suffix_ring(const Dims &dm)
@@ -1174,20 +1228,31 @@ TilePlan plan_suffix_ring(const Dims &dm)
     const int Rg = dm.n_rep * dm.S;
     pl.mode = 2;
     if (Rg > kTileM || dm.Skv > kBlockN) {
-        // long suffixes: a tile is a run of rows inside one candidate (the largest divisor of its
-        // row count that fits a tile), the candidate's suffix keys come in blocks of 128
+        // Long suffixes: a tile lies inside one candidate, whose suffix keys come in blocks of 128.  Beyond 128 queries
+        // it lies inside one head too: a head's rows are padded to whole tiles, so any length does, and a tile's
+        // cost follows from its position, so that tiles can be dealt out by cost.  Else, and where heads would be
+        // padded to more tiles, a tile is the largest divisor of the candidate's rows that fits.  (Lengths without such a
+        // divisor went to the CUDA-core kernel: 1.57 ms for a prompt of 1039 tokens, 12.2 for 3001, now 22 and 131 us.)
         int rows = 0;
         for (int m = kTileM; m >= 16 && !rows; --m)
             if (Rg % m == 0) rows = m;
         if (!rows && Rg <= kTileM) rows = Rg;
+        const int per_head = (dm.S + kTileM - 1) / kTileM;
+        if (dm.S > kTileM && (!rows || (long long)dm.n_rep * per_head <= Rg / rows)) {
+            rows = round_up((dm.S + per_head - 1) / per_head, 8);
+            pl.head_box = 1;
+            pl.Sh = rows * per_head;
+        }
         if (!rows) return pl;  // no usable divisor: the general kernels take the shape
-        if ((long long)dm.B * (Rg / rows) > 2000000000ll) return pl;
+        pl.Rp = pl.head_box ? dm.n_rep * pl.Sh : Rg;
+        pl.one_box = 1;
+        if ((long long)dm.B * pl.Rp > 2000000000ll) return pl;
         pl.long_sfx = 1;
         pl.Spad = 8;
         pl.cpb = 1;
         pl.cbox = 1;
         pl.tile_rows = pl.seg_rows = rows;
-        pl.tiles_per_group = dm.B * (Rg / rows);
+        pl.tiles_per_group = dm.B * (pl.Rp / rows);
     } else {
         pl.Spad = round_up(dm.Skv, 8);
         pl.cpb = kBlockN / pl.Spad;
@@ -1210,30 +1275,13 @@ TilePlan plan_suffix_ring(const Dims &dm)
                 pl.cbox = c;
             }
         }
+        pl.Rp = Rg;
+        pl.one_box = 1;
         pl.tile_rows = pl.seg_rows = Rg * pl.cbox;
         pl.tiles_per_group = (dm.B + pl.cbox - 1) / pl.cbox;
         pl.cost = (double)pl.tiles_per_group * tile_cost(nblk + (pl.cbox + pl.cpb - 1) / pl.cpb, 1);
     }
-    pl.nblk_p = (dm.P + kBlockN - 1) / kBlockN;
-    pl.tail_rows = pl.nblk_p ? round_up(dm.P - (pl.nblk_p - 1) * kBlockN, 16) : 0;
-    const int slabs = dm.d / 64;
-    const int tile_bytes = slabs * kTileM * 128;
-    const int ml_bytes = 4 * kGroups * kTileM * 4;
-    const int stage_bytes = slabs * kStagingBytes;
-    const int fixed = tile_bytes /*Q*/ + stage_bytes + ml_bytes + 64 + kBarBytes;
-    int st = (kMaxSmem - fixed) / (2 * tile_bytes);
-    if (st > kMaxStages) st = kMaxStages;
-    if (st < 1) return pl;
-    pl.stages = st;
-    pl.off_pk = 0;
-    pl.off_pv = st * tile_bytes;
-    pl.off_q = 2 * st * tile_bytes;
-    pl.off_sk = pl.off_sv = pl.off_stage = pl.off_q + tile_bytes;  // no suffix buffers of their own
-    pl.off_bar = pl.off_stage + stage_bytes;
-    pl.off_misc = pl.off_bar + kBarBytes;
-    pl.off_ml = pl.off_misc + 64;
-    pl.smem_bytes = pl.off_ml + ml_bytes;
-    pl.ok = pl.smem_bytes <= kMaxSmem;
+    layout_ring(dm, &pl);
     return pl;
 }
 
@@ -1244,7 +1292,7 @@ TilePlan plan_base(const Dims &dm)
     TilePlan pl;
     memset(&pl, 0, sizeof(pl));
     int nc_best = 0;
-    if (!pick_tile_rows(dm, &pl, &nc_best)) return pl;
+    if (!pick_tile_rows(dm, false, &pl, &nc_best)) return pl;
     pl.sfx_rows = round_up(nc_best * pl.Sp, 16);
     pl.nblk_p = (dm.P + kBlockN - 1) / kBlockN;
     pl.tail_rows = pl.nblk_p ? round_up(dm.P - (pl.nblk_p - 1) * kBlockN, 16) : 0;
@@ -1305,26 +1353,50 @@ TilePlan plan_base(const Dims &dm)
     return pl;
 }
 
-// The full-suffix operator takes the tiling with the suffix in one block when it has one; the decode-shaped operator
-// and suffixes beyond one block go to suffix-ring mode, and so do groups of a few rows, whose padding to 8 rows
-// would cost more than the ring's extra suffix blocks (one row per candidate and head: an eighth of the tile).
-TilePlan make_plan(const Dims &dm)
+// Suffix-ring mode with tiles that end anywhere in the row list: one query head per KV head and 66 suffix keys are 66
+// rows of a 128-row tile where a tile's suffix keys have to fit one block, or 120 rows and two or three suffix blocks.
+TilePlan plan_straddle(const Dims &dm)
+{
+    TilePlan pl;
+    memset(&pl, 0, sizeof(pl));
+    int nc = 0;
+    if (!pick_tile_rows(dm, true, &pl, &nc)) return pl;
+    pl.mode = 2;
+    pl.Spad = pl.Sp;
+    pl.cpb = kBlockN / pl.Sp;
+    pl.cbox = 1;
+    layout_ring(dm, &pl);
+    return pl;
+}
+
+// The full-suffix operator takes the tiling with the suffix in one block unless another one is clearly cheaper: tiles
+// that straddle candidates, or, for groups of a few rows, whole candidates without padding (one row per candidate and
+// head padded to 8 would be an eighth of the tile).  The decode-shaped operator and suffixes beyond one block are the
+// suffix-ring mode's.  Straddling tiles fetch the prefix for every tile, so they have to be cheaper by 40 % by count of
+// blocks where it would stay resident (B = 74, 32/8 heads, P = 256, S = 75: 57 us instead of 49 at a count 12 %
+// lower), by 8 % where it is streamed either way (B = 58, 32/32, P = 1735, S = 66 221 -> 168 us; B = 66, 32/8, P = 803,
+// S = 109 152 -> 145).
+TilePlan make_plan(const Dims &dm, int n_instr)
 {
     if (dm.Skv == dm.S && !dm.ragged) {
         const TilePlan pl = plan_base(dm);
+        if (n_instr > 1) return pl;  // (several instructions in one launch: only this tiling)
         if (pl.ok && dm.n_rep * dm.S % 8 != 0 && dm.n_rep * dm.S <= kTileM / 2) {
             const TilePlan ring = plan_suffix_ring(dm);
             if (ring.ok && !ring.long_sfx && ring.cost < pl.cost) return ring;
         }
-        if (pl.ok) return pl;
+        if (pl.ok) {
+            const TilePlan ring = plan_straddle(dm);
+            return ring.ok && (pl.resident ? 1.4 : 1.08) * ring.cost < pl.cost ? ring : pl;
+        }
     }
     return plan_suffix_ring(dm);
 }
 
-const TilePlan &plan_tiles(const Dims &dm)
+const TilePlan &plan_tiles(const Dims &dm, int n_instr = 1)
 {
     static thread_local PlanTable<TilePlan> table;
-    return table.get(dm, 1, [&] { return make_plan(dm); });
+    return table.get(dm, n_instr, [&] { return make_plan(dm, n_instr); });
 }
 
 template <int D>
@@ -1343,7 +1415,11 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
         cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)Rg, (cuuint64_t)dm.Hkv, (cuuint64_t)dm.B};
         cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)Rg * D * 2, (cuuint64_t)dm.Hkv * Rg * D * 2};
         cuuint32_t box[4] = {64, (cuuint32_t)plan.seg_rows, 1, 1};
-        if (plan.mode == 2) {  // one box = the whole candidates of a tile, or the tile's rows of one candidate
+        if (plan.head_box) {  // heads of their own
+            dims[1] = (cuuint64_t)dm.S;
+            dims[2] = (cuuint64_t)dm.Hq;
+            str[1] = (cuuint64_t)dm.S * D * 2;
+        } else if (plan.mode == 2 && plan.one_box) {  // one box = the whole candidates of a tile, or the tile's rows of one candidate
             box[1] = (cuuint32_t)(plan.long_sfx ? plan.tile_rows : Rg);
             box[3] = (cuuint32_t)plan.cbox;
         }
@@ -1373,15 +1449,18 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     p.args = a;
     p.sl2 = a.scale * kLog2e;
     p.B = dm.B; p.Hq = dm.Hq; p.Hkv = dm.Hkv; p.S = dm.S; p.P = dm.P; p.n_rep = dm.n_rep;
-    p.Rg = plan.mode == 2 ? Rg : plan.Rp;
-    p.Rr = Rg;
+    p.Rg = plan.Rp;
+    p.Sh = plan.head_box ? plan.Sh : dm.S;
+    p.Rr = dm.n_rep * p.Sh;
+    p.one_box = plan.one_box;
+    p.head_box = plan.head_box;
     p.Sp = plan.mode == 2 ? dm.S : plan.Sp;
     p.tile_rows = plan.tile_rows;
     p.seg_rows = plan.seg_rows;
     p.tiles_per_group = plan.tiles_per_group;
     p.fd_tpg.init(plan.tiles_per_group);
     p.fd_Rg.init(p.Rg);
-    p.fd_S.init(dm.S);
+    p.fd_S.init(p.Sh);
     p.fd_seg.init(plan.seg_rows);
     p.total_tiles = plan.tiles_per_group * dm.Hkv;
     p.nblk_p = plan.nblk_p;
@@ -1404,7 +1483,7 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     for (int i = 0; i < kMaxInstr; ++i) p.pad[i] = (n_instr > 1 && i < n_instr) ? dm.P - prefix_len[i] : 0;
     // Dealing by cost balances the causal skew but lets every CTA touch every candidate's suffix K/V
     // at several times; it pays when those tensors stay in L2 between the touches.
-    p.deal_by_cost = plan.long_sfx && dm.S % plan.tile_rows == 0 && dm.S / plan.tile_rows > 1 &&
+    p.deal_by_cost = plan.long_sfx && p.Sh % plan.tile_rows == 0 && p.Sh / plan.tile_rows > 1 &&
                      4.0 * dm.B * dm.Hkv * dm.Skv * D <= 48.0e6;
     p.off_pk = plan.off_pk; p.off_pv = plan.off_pv; p.off_q = plan.off_q; p.off_sk = plan.off_sk;
     p.off_sv = plan.off_sv; p.off_stage = plan.off_stage; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
@@ -1466,17 +1545,17 @@ bool tc_fwd_fused_supported(const Dims &dm, int n_instr)
     if (n_instr < 2 || n_instr > kMaxFusedInstructions || dm.B % n_instr != 0 || dm.P < 1 || dm.Pstride != dm.P ||
         dm.ragged || !tc_fwd_supported(dm))
         return false;
-    const TilePlan &pl = plan_tiles(dm);
+    const TilePlan &pl = plan_tiles(dm, n_instr);
     return pl.ok && pl.mode != 2 && ((long long)(dm.B / n_instr) * pl.Rp) % pl.tile_rows == 0;
 }
 
 cudaError_t launch_tc_fwd(const FwdArgs &a, void *workspace, unsigned int *status_word, cudaStream_t stream,
                           int n_instr, const int *prefix_len)
 {
-    const TilePlan &plan = plan_tiles(a.dims);
+    if (n_instr < 1) n_instr = 1;
+    const TilePlan plan = plan_tiles(a.dims, n_instr);  // (a copy: the next look-up may replace the table's entry)
     if (!plan.ok) return cudaErrorInvalidValue;
     if (n_instr > 1 && (!prefix_len || !tc_fwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
-    if (n_instr < 1) n_instr = 1;
     if (n_instr == 1 && cta_pairs_enabled() && tc_fwd_pair_supported(a.dims))
         return launch_tc_fwd_pair(a, status_word, stream);
     return a.dims.d == 128 ? launch<128>(a, plan, workspace, status_word, stream, n_instr, prefix_len)

@@ -1,5 +1,7 @@
 """The tensor-core forward at the edges of its tiling: candidates whose rows or keys are no multiple of 8, padded to the next
-multiple or as far as a tile's end, boxes that hold padding only, a short last tile, suffixes of one whole key block."""
+multiple or as far as a tile's end, boxes that hold padding only, a short last tile, suffixes of one
+whole key block, tiles that straddle candidates with suffix keys in several blocks, lengths beyond 128 that have no
+divisor."""
 import pytest
 
 import paper_2603_13420_b200 as pskv
@@ -18,6 +20,14 @@ SHAPES = [
     (2, 8, 2, 128, 0, 127),      # no prefix
     (33, 3, 3, 64, 31, 9),
     (300, 8, 2, 128, 257, 21),   # several tiles per CTA
+    (5, 4, 4, 128, 300, 66),     # tiles that straddle candidates, a suffix block per candidate
+    (9, 2, 2, 64, 40, 85),
+    (300, 2, 2, 128, 200, 70),
+    (11, 3, 3, 128, 700, 45),    # ... two candidates to a suffix block
+    (1, 4, 2, 128, 0, 131),      # beyond 128 queries: tiles inside one head, heads padded to whole tiles
+    (2, 4, 4, 64, 60, 139),
+    (1, 2, 1, 128, 0, 1039),
+    (1, 8, 2, 128, 33, 513),
 ]
 
 
