@@ -833,43 +833,49 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
     BwdPlan pl;
     memset(&pl, 0, sizeof(pl));
     const int Rg = dm.n_rep * dm.S, Kq = dm.B / n_instr;
-    pl.Rp = round_up(Rg, 8);
     pl.Sp = round_up(dm.S, 8);
     pl.nh = (dm.S + kPieceN - 1) / kPieceN;
     pl.nblk = (dm.P + kPieceN - 1) / kPieceN;
     const int sms = sm_count();
     double best = -1.0;
-    for (int cu = 1; cu <= 16 && cu <= Kq; ++cu) {
-        const int tiles = (cu * pl.Rp + kTileM - 1) / kTileM;
-        const int seg = gcd_int(pl.Rp, kTileM);
-        if (cu > 1 && tiles > 1 && seg < 32) break;  // tiles that straddle candidates take 128 / seg boxes
-        if (tiles > 8 && cu > 1) break;
-        int cpp = 1, sfx = 0;
-        if (tiles == 1) {
-            cpp = pl.nh > 1 ? 1 : kPieceN / pl.Sp < cu ? kPieceN / pl.Sp : cu;
-            sfx = (cu + cpp - 1) / cpp * pl.nh;
-        } else {
-            for (int t = 0; t < tiles; ++t) {
-                const int r1 = (t + 1) * kTileM < cu * pl.Rp ? (t + 1) * kTileM : cu * pl.Rp;
-                sfx += (r1 - 1) / pl.Rp - t * kTileM / pl.Rp + 1;
+    // A candidate's rows may be padded further than to the next multiple of 8: 4 heads x 42 rows are two tiles, one of
+    // them a third full, or, as 176 rows, three tiles for two candidates (kernel alone, B = 250, P = 385 240 -> 203 us;
+    // 4 x 67 rows, B = 100, P = 300 181 -> 169; 4 x 35, B = 144, P = 92 74 -> 66).
+    for (int Rp = round_up(Rg, 8); Rp < Rg + 64; Rp += 8) {
+        const int seg = gcd_int(Rp, kTileM);
+        for (int cu = 1; cu <= 16 && cu <= Kq; ++cu) {
+            const int tiles = (cu * Rp + kTileM - 1) / kTileM;
+            // a tile that straddles candidates takes 128 / seg boxes
+            if (cu > 1 && ((tiles > 1 && seg < 16) || tiles > 12)) break;
+            int cpp = 1, sfx = 0;
+            if (tiles == 1) {
+                cpp = pl.nh > 1 ? 1 : kPieceN / pl.Sp < cu ? kPieceN / pl.Sp : cu;
+                sfx = (cu + cpp - 1) / cpp * pl.nh;
+            } else {
+                for (int t = 0; t < tiles; ++t) {
+                    const int r1 = (t + 1) * kTileM < cu * Rp ? (t + 1) * kTileM : cu * Rp;
+                    sfx += (r1 - 1) / Rp - t * kTileM / Rp + 1;
+                }
+                sfx *= 2 * pl.nh - 1;  // pass 0: every piece; each later pass: one
             }
-            sfx *= 2 * pl.nh - 1;  // pass 0: every piece; each later pass: one
-        }
-        const long long units = (long long)((Kq + cu - 1) / cu) * n_instr * dm.Hkv;
-        const double cost = (double)((units + sms - 1) / sms) * (tiles * (pl.nblk + 1) + sfx * 1.3);
-        if (best < 0.0 || cost < best * 0.97) {
-            best = cost;
-            pl.cu = cu;
-            pl.cpp = cpp;
-            pl.seg = tiles == 1 ? pl.Rp : cu == 1 ? kTileM : seg;
-            pl.cbox = tiles == 1 && n_instr == 1 ? cu : 1;  // (a box must not reach into the next instruction)
+            const long long units = (long long)((Kq + cu - 1) / cu) * n_instr * dm.Hkv;
+            const double boxes = tiles > 1 && cu > 1 ? 0.03 * kTileM / seg : 0.03;
+            const double cost = (double)((units + sms - 1) / sms) * (tiles * (pl.nblk + 1 + boxes) + sfx * 1.3);
+            if (best < 0.0 || cost < best * 0.97) {
+                best = cost;
+                pl.Rp = Rp;
+                pl.cu = cu;
+                pl.cpp = cpp;
+                pl.seg = tiles == 1 ? Rp : cu == 1 ? kTileM : seg;
+                pl.cbox = tiles == 1 && n_instr == 1 ? cu : 1;  // (a box must not reach into the next instruction)
+            }
         }
     }
     {
         // Split: the busiest SM's share is its units times the dearer kind.  Taken where that is well below what whole
         // candidates give, which is when they leave SMs idle: one candidate of 113 tokens, 4 heads per KV head and
         // 78 prefix tokens is 8 units of 20 items on 148 SMs, or 48 units of at most 4 items.
-        const int tiles = (pl.Rp + kTileM - 1) / kTileM;
+        const int tiles = (round_up(Rg, 8) + kTileM - 1) / kTileM;
         const long long units = (long long)Kq * n_instr * dm.Hkv * (tiles + pl.nh);
         const double dq = pl.nblk + 1 + pl.nh, piece = tiles * 2.3;
         const double cost = (double)((units + sms - 1) / sms) * (dq > piece ? dq : piece);
@@ -877,6 +883,7 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
         if (tiles <= 1024 && cost < 0.85 * best) {
             pl.n_tiles = tiles;
             pl.n_sub = tiles + pl.nh;
+            pl.Rp = round_up(Rg, 8);
             pl.cu = pl.cpp = pl.cbox = 1;
             pl.seg = tiles == 1 ? pl.Rp : kTileM;
         }

@@ -46,6 +46,8 @@ def test_backward_matches_the_oracle(shape):
     (700, 2, 2, 128, 40, 1), (420, 4, 4, 128, 64, 5), (320, 3, 3, 128, 1, 33), (400, 8, 2, 128, 130, 45),
     (400, 8, 2, 128, 256, 48), (401, 8, 2, 64, 256, 48), (400, 4, 4, 128, 191, 65), (400, 8, 2, 128, 78, 113),
     (300, 2, 2, 128, 70, 129), (900, 1, 1, 64, 33, 72),
+    (401, 8, 2, 128, 385, 42),   # rows padded so that three tiles hold two candidates (the last unit one)
+    (350, 8, 2, 128, 300, 67),   # ... several candidates per unit, two pieces each
 ], ids=lambda s: "x".join(map(str, s)))
 def test_backward_of_many_candidates_matches_the_oracle(shape):
     B, Hq, Hkv, d, P, S = shape
