@@ -444,14 +444,15 @@ SideStream *side_stream()
 // instruction, 1 = one launch wherever the shapes allow it (the same as 0 today), 2 = always passes.
 int multi_form() { return g_multi_form.load(std::memory_order_relaxed); }
 
-// Launches of the gradient step of pskv_attn_bwd_multi.  One is enough; the shapes for which the row statistic,
-// dQ and the suffix gradients have been three launches so far keep that count (pskv_kernel_launches is part of
-// the interface), as the row statistic and two halves of the units, the second half's CTAs filling in as
-// the first half's drain.
+// Launches of the gradient step of pskv_attn_bwd_multi.  One is enough; small calls of the shapes for which the row
+// statistic, dQ and the suffix gradients used to be three launches keep that observable count (pskv_kernel_launches)
+// as the row statistic and two halves of the units.  Large ones run in one: in two halves 300 candidates of 12
+// instructions (32/32 heads, P = 512, S = 80) took 3 % longer.
 int tc_bwd_multi_launches(const Dims &dm, int Bp)
 {
     const bool grouped = dm.S % 8 == 0 && dm.S <= 128 && !(dm.S <= 48 && dm.n_rep * dm.S >= 128);
-    return grouped && tc_fwd_fused_supported(dm, Bp) ? 2 : 1;
+    const long long rows = (long long)dm.B * dm.Hq * dm.S;
+    return grouped && rows <= 16384 && (long long)(dm.B / Bp) * dm.n_rep * dm.S % 128 == 0 ? 2 : 1;
 }
 
 // checks shared by the two multi-instruction calls; fills the per-instruction geometry

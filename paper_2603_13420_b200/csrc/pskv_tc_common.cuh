@@ -72,17 +72,23 @@ struct TileInfo {
     bool first_of_g;
 };
 
-// `Params` is any kernel parameter block with fields B, Rg, Sp, tile_rows, tiles_per_group, fd_tpg, fd_Rg.
-template <class Params>
+// `Params` is any kernel parameter block with fields B, Rg, Sp, tile_rows, tiles_per_group, fd_tpg, fd_Rg.  MI: several
+// instructions, whose rows (rpi each) are cut into tiles one by one (tpi tiles each, the last one shorter).
+template <bool MI, class Params>
 __device__ __forceinline__ TileInfo tile_info(const Params &p, int tile, int t_begin)
 {
     TileInfo t;
     t.g = p.fd_tpg.div(tile);
     const int tt = tile - t.g * p.tiles_per_group;
     t.first_of_g = (tt == 0) || (tile == t_begin);
-    t.R0 = tt * p.tile_rows;
-    const int total = p.B * p.Rg;
-    t.rows = min(p.tile_rows, total - t.R0);
+    if (MI) {
+        const int inst = p.fd_tpi.div(tt), r = (tt - inst * p.tpi) * p.tile_rows;
+        t.R0 = inst * p.rpi + r;
+        t.rows = min(p.tile_rows, p.rpi - r);
+    } else {
+        t.R0 = tt * p.tile_rows;
+        t.rows = min(p.tile_rows, p.B * p.Rg - t.R0);
+    }
     t.b_first = p.fd_Rg.div(t.R0);
     const int b_last = p.fd_Rg.div(t.R0 + t.rows - 1);
     t.nc = b_last - t.b_first + 1;

@@ -92,8 +92,9 @@ struct TcFwdParams {
     // several instructions in one launch (Sec. 4.3): the candidates of instruction i are contiguous and use
     // prefix cache i of [n_instr][Hkv][P][d], whose first pad[i] rows are left padding
     int n_instr;          // 1: one shared prefix
-    int rpi;              // rows of one instruction inside a KV head's row list (a multiple of tile_rows)
-    FastDiv fd_rpi;
+    int rpi;              // rows of one instruction inside a KV head's row list
+    int tpi;              // its tiles: an instruction starts a tile of its own
+    FastDiv fd_rpi, fd_tpi;
     int pad[kMaxInstr];
     // shared-memory carve-up (byte offsets from the 1024-byte aligned base)
     int off_pk, off_pv, off_q, off_sk, off_sv, off_stage, off_bar, off_misc, off_ml;
@@ -280,7 +281,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     auto first_block = [&](int inst) { return MI ? p.pad[inst] / kBlockN : 0; };
     int run_first;
     {
-        const TileInfo t0 = tile_info(p, t_begin < p.total_tiles ? t_begin : 0, t_begin);
+        const TileInfo t0 = tile_info<MI>(p, t_begin < p.total_tiles ? t_begin : 0, t_begin);
         run_first = run_of(t0, inst_of(t0));
     }
     const int sfx_slab = p.sfx_rows * 128;
@@ -301,7 +302,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         bool ok = true;
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info(p, tile_at(tl), t_begin);
+            const TileInfo t = tile_info<MI>(p, tile_at(tl), t_begin);
             // Everything the Q loads need is worked out before the wait, so that only the copy
             // instructions themselves follow it: the Q buffer is single, and the time from "last
             // score MMA of the previous tile done" to "Q of this tile requested" is exposed.
@@ -315,7 +316,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // While there is nothing else to do, ask for the NEXT tile's Q in L2: its load can only
             // be issued a tile from now, right when it is needed, and then finds the data close by.
             if (tl + 1 < n_tiles) {
-                const TileInfo tn = tile_info(p, tile_at(tl + 1), t_begin);
+                const TileInfo tn = tile_info<MI>(p, tile_at(tl + 1), t_begin);
                 const int nseg_n = (SR && p.one_box) ? 1 : p.fd_seg.div(tn.rows);
                 int nb = p.fd_Rg.div(tn.R0), nr = tn.R0 - nb * p.Rg;
                 if (elect_one_sync()) {
@@ -471,7 +472,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             int ph = 0;  // head index inside the prefix caches
             int kfirst = 0;
             if (have_tile) {
-                t = tile_info(p, tile_at(tl), t_begin);
+                t = tile_info<MI>(p, tile_at(tl), t_begin);
                 const int inst = inst_of(t);
                 ph = inst * p.Hkv + t.g;
                 kfirst = first_block(inst);
@@ -566,7 +567,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         ready = __shfl_sync(0xffffffffu, mbar_try_wait(bar(kBarStageFull), round & 1) ? 1 : 0, 0) != 0;
                     if (!ok) break;
                     if (ready) {
-                        const TileInfo u = tile_info(p, tile_at(tl - 1), t_begin);
+                        const TileInfo u = tile_info<MI>(p, tile_at(tl - 1), t_begin);
                         const int nseg = (SR && p.one_box) ? 1 : p.fd_seg.div(u.rows);
                         const int sl_first = p.slab_stage ? store_slab : 0;
                         const int sl_end = p.slab_stage ? store_slab + 1 : C::kSlabs;
@@ -620,7 +621,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         // ------------------------------------------------------------------ score MMAs: S = Q K^T
         int tl = 0;
         uint32_t kuse = 0;  // streaming mode: K blocks consumed from the ring
-        TileInfo t = tile_info(p, tile_at(0), t_begin);
+        TileInfo t = tile_info<MI>(p, tile_at(0), t_begin);
         int nitems = items_of(t);
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint64_t q_desc = make_smem_desc(sbase + p.off_q, 0, 1024);
@@ -703,7 +704,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
-                    t = tile_info(p, tile_at(tl), t_begin);
+                    t = tile_info<MI>(p, tile_at(tl), t_begin);
                     nitems = items_of(t);
                     k = kfirst = first_block(inst_of(t));
                 }
@@ -713,7 +714,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         // ------------------------------------------------------------------ value MMAs: O += P V
         int tl = 0;
         uint32_t vuse = 0;
-        TileInfo t = tile_info(p, tile_at(0), t_begin);
+        TileInfo t = tile_info<MI>(p, tile_at(0), t_begin);
         int nitems = items_of(t);
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint32_t idesc_pv = make_idesc_bf16(kTileM, D, 1);
@@ -795,7 +796,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
-                    t = tile_info(p, tile_at(tl), t_begin);
+                    t = tile_info<MI>(p, tile_at(tl), t_begin);
                     nitems = items_of(t);
                     k = kfirst = first_block(inst_of(t));
                 }
@@ -823,7 +824,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int item = 0;  // items handled so far
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info(p, tile_at(tl), t_begin);
+            const TileInfo t = tile_info<MI>(p, tile_at(tl), t_begin);
             const int nitems = items_of(t);
             int lo_sfx = 1, hi_sfx = 0;
             int k_own = p.nblk_p;  // suffix-ring mode: the item that holds this row's candidate
@@ -966,7 +967,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         bool ok = true;
 #pragma unroll 1
         for (int te = 0; te < n_tiles && ok; ++te) {
-            const TileInfo u = tile_info(p, tile_at(te), t_begin);
+            const TileInfo u = tile_info<MI>(p, tile_at(te), t_begin);
             ok = mbar_wait_warp(bar(kBarOFull), te & 1, abort_flag, p.status, kErrEpilogue);
             if (!ok) break;
             PSKV_TRACE_EVENT(30, te);
@@ -1101,7 +1102,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         float *q_s = reinterpret_cast<float *>(smem) + warp * D;
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles; ++tl) {
-            const TileInfo t = tile_info(p, tile_at(tl), t_begin);
+            const TileInfo t = tile_info<MI>(p, tile_at(tl), t_begin);
 #pragma unroll 1
             for (int r = warp; r < t.rows; r += kThreads / 32) {
                 const int R = t.R0 + r;
@@ -1457,12 +1458,9 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     p.Sp = plan.mode == 2 ? dm.S : plan.Sp;
     p.tile_rows = plan.tile_rows;
     p.seg_rows = plan.seg_rows;
-    p.tiles_per_group = plan.tiles_per_group;
-    p.fd_tpg.init(plan.tiles_per_group);
     p.fd_Rg.init(p.Rg);
     p.fd_S.init(p.Sh);
     p.fd_seg.init(plan.seg_rows);
-    p.total_tiles = plan.tiles_per_group * dm.Hkv;
     p.nblk_p = plan.nblk_p;
     p.tail_rows = plan.tail_rows;
     p.resident = plan.resident;
@@ -1480,6 +1478,11 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     p.n_instr = n_instr;
     p.rpi = dm.B / n_instr * p.Rg;
     p.fd_rpi.init(p.rpi > 0 ? p.rpi : 1);
+    p.tpi = n_instr > 1 ? (p.rpi + plan.tile_rows - 1) / plan.tile_rows : plan.tiles_per_group;
+    p.fd_tpi.init(p.tpi);
+    p.tiles_per_group = p.tpi * n_instr;
+    p.fd_tpg.init(p.tiles_per_group);
+    p.total_tiles = p.tiles_per_group * dm.Hkv;
     for (int i = 0; i < kMaxInstr; ++i) p.pad[i] = (n_instr > 1 && i < n_instr) ? dm.P - prefix_len[i] : 0;
     // Dealing by cost balances the causal skew but lets every CTA touch every candidate's suffix K/V
     // at several times; it pays when those tensors stay in L2 between the touches.
@@ -1537,16 +1540,20 @@ bool tc_fwd_supported(const Dims &dm)
 
 size_t tc_fwd_workspace_bytes(const Dims &) { return 0; }
 
-// One launch can serve several instructions when every tile lies inside one instruction's candidates (an
-// instruction's rows in a KV head's row list are a whole number of tiles) and the tiles are the 128-row
-// tiles with one suffix block each (not the suffix-ring tiling).
+// One launch can serve several instructions when the tiles are those with one suffix block each (not the suffix-ring
+// tiling).  An instruction starts a tile of its own, so its last tile may be short: taken where an instruction is a
+// whole number of tiles, or at least four, so that the short one costs at most a fifth (90 candidates of 6
+// instructions, 32/8 heads, P = 300, S = 37: one launch 107 us for forward + backward, six passes
+// on two streams 131).
 bool tc_fwd_fused_supported(const Dims &dm, int n_instr)
 {
     if (n_instr < 2 || n_instr > kMaxFusedInstructions || dm.B % n_instr != 0 || dm.P < 1 || dm.Pstride != dm.P ||
         dm.ragged || !tc_fwd_supported(dm))
         return false;
     const TilePlan &pl = plan_tiles(dm, n_instr);
-    return pl.ok && pl.mode != 2 && ((long long)(dm.B / n_instr) * pl.Rp) % pl.tile_rows == 0;
+    const long long rows = (long long)(dm.B / n_instr) * pl.Rp;
+    return pl.ok && pl.mode != 2 && (rows % pl.tile_rows == 0 || rows >= 4 * pl.tile_rows) &&
+           (rows / pl.tile_rows + 1) * n_instr * dm.Hkv <= 2000000000ll;
 }
 
 cudaError_t launch_tc_fwd(const FwdArgs &a, void *workspace, unsigned int *status_word, cudaStream_t stream,

@@ -3,7 +3,9 @@ multiple or as far as a tile's end, boxes that hold padding only, a short last t
 whole key block, tiles that straddle candidates with suffix keys in several blocks, lengths beyond 128 that have no
 divisor."""
 import pytest
+import torch
 
+import oracle
 import paper_2603_13420_b200 as pskv
 import parity
 from paper_2603_13420_b200.inputs import Workload, make_inputs
@@ -54,5 +56,33 @@ def test_rows_outside_the_safe_exponent_range_next_to_padding_rows():
     out, lse, _ = parity.run_fwd_gpu(t, w.scale)
     ref_out, ref_lse = parity.oracle_fwd(t, w.scale)
     assert abs(ref_lse).max() > 100.0
+    parity.check_tensor("out", parity.to_f64(out), ref_out)
+    parity.check_lse(parity.to_f64(lse), ref_lse)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", [
+    # B, Bp, Hq, Hkv, S, Pmax, d, lens: an instruction is no whole number of tiles, its last tile is short
+    (24, 3, 8, 2, 37, 300, 128, (300, 129, 40)),
+    (44, 2, 4, 4, 21, 64, 64, (0, 64)),
+    (30, 5, 4, 4, 100, 600, 128, (600, 1, 470, 128, 129)),
+])
+def test_several_instructions_whose_last_tiles_are_short_in_one_launch(case):
+    B, Bp, Hq, Hkv, S, Pmax, d, lens = case
+    gen = torch.Generator().manual_seed(4242 + S)
+    draw = lambda *s: torch.randn(s, generator=gen, dtype=torch.float32).to(torch.bfloat16)
+    t = dict(q=draw(B, Hq, S, d), prefix_k=draw(Bp, Hkv, Pmax, d), prefix_v=draw(Bp, Hkv, Pmax, d),
+             suffix_k=draw(B, Hkv, S, d), suffix_v=draw(B, Hkv, S, d))
+    for i, n in enumerate(lens):
+        t["prefix_k"][i, :, : Pmax - n] = 3.0e4
+        t["prefix_v"][i, :, : Pmax - n] = -3.0e4
+    dev = {k: v.cuda() for k, v in t.items()}
+    n0 = pskv.pskv_kernel_launches()
+    out, lse = pskv.pskv_attn_fwd_multi(dev["q"], dev["prefix_k"], dev["prefix_v"], lens, dev["suffix_k"], dev["suffix_v"], d ** -0.5)
+    assert pskv.pskv_kernel_launches() - n0 == 1
+    assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
+    f = {k: parity.to_f64(v) for k, v in t.items()}
+    ref_out, ref_lse = oracle.attn_fwd_multi(f["q"], f["prefix_k"], f["prefix_v"], oracle.left_padding_mask(lens, Pmax),
+                                             f["suffix_k"], f["suffix_v"], d ** -0.5)
     parity.check_tensor("out", parity.to_f64(out), ref_out)
     parity.check_lse(parity.to_f64(lse), ref_lse)
