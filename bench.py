@@ -711,7 +711,7 @@ def ce_run(pskv, device, peaks, iters, warmup, with_library=True):
            "roofline": {"kernel": "ce_fwd_kernel", "bound": "tensor", "achieved": fl / ms / 1e9, "peak": peaks["bf16_tflops"],
                         "unit": "TFLOP/s", "frac": fl / ms / 1e9 / peaks["bf16_tflops"],
                         "traffic": 3.65e9,  # profiles/ce_fwd_kernel_512x20_V128256.md (algorithmic 1.13 GB)
-                        "note": "call = GEMM kernel + a 40 us finalize kernel; peak = measured bf16 burst (a library GEMM)"}}
+                        "note": "call = GEMM kernel + a finalize kernel of about 15 us; peak = measured bf16 burst (a library GEMM)"}}
     if with_library:
         tl = t.view(-1).long()
 
