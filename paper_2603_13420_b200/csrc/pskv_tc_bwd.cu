@@ -98,6 +98,7 @@ struct TcBwdParams {
     FastDiv fd_upg, fd_upi, fd_sub, fd_Rp, fd_S, fd_cpp;
     int stages_k, stages_v;
     int off_do, off_q, off_k, off_v, off_p, off_ds, off_rows, off_bar, off_misc;
+    int zero_lo, zero_hi;  // operand buffers with rows that no copy may reach before the MMAs read them
     int pad[kMaxInstr];    // left padding of each instruction's prefix cache (Sec. 4.3)
 };
 
@@ -287,20 +288,22 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         if (tid == 0) atomicCAS(p.status, 0u, (unsigned int)kErrAlign);
         return;
     }
-    // operand rows that no copy ever writes must hold finite values (0 * NaN would poison a sum)
-    for (int i = tid; i < p.off_p / 16; i += kThreads) reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
-    if (tid == 0) {
+    // Operand rows that no copy ever writes must hold finite values (0 * NaN would poison a sum).  Zeroing all
+    // buffers in every launch, with the barriers set up by one thread, cost 2 us: one candidate, 32/8 heads, P = 78, S =
+    // 113 22.9 instead of 20.9 us, 12 candidates, 32/32 heads, P = 90, S = 77 27.0 instead of 24.9.
+    for (int i = p.zero_lo / 16 + tid; i < p.zero_hi / 16; i += kThreads)
+        reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0, 0, 0, 0);
+    if (warp == 3) {
 #pragma unroll 1
-        for (int i = 0; i < kNumBars; ++i) {
+        for (int i = lane; i < kNumBars; i += 32) {
             const bool epi = i == kBarDqFree || i == kBarAccFree;
             const bool elem = (i >= kBarSFree && i < kBarSFree + 2) || (i >= kBarDsReady && i < kBarDsReady + 2);
             mbar_init(bar(i), elem ? 8u : epi ? 4u : i == kBarQFree ? 2u : 1u);
         }
-        *abort_flag = 0;
+        if (lane == 0) *abort_flag = 0;
         fence_barrier_init();
     }
     fence_proxy_async();
-    __syncthreads();
     if (warp == 2) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
@@ -978,6 +981,9 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     p.fd_cpp.init(p.cpp);
     p.stages_k = plan.stages_k; p.stages_v = plan.stages_v;
     p.off_do = plan.off_do; p.off_q = plan.off_q; p.off_k = plan.off_k; p.off_v = plan.off_v; p.off_p = plan.off_p;
+    // The MMAs contract over rows and keys in steps of 16: boxes of a multiple of 16 rows (keys) leave none unwritten.
+    p.zero_lo = plan.seg * plan.cbox % 16 != 0 ? plan.off_do : plan.off_k;
+    p.zero_hi = plan.sfx_box * plan.cpp % 16 != 0 ? plan.off_p : plan.off_k;
     p.off_ds = plan.off_ds; p.off_rows = plan.off_rows; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
     for (int i = 0; i < n_instr && n_instr > 1; ++i) p.pad[i] = dm.P - prefix_len[i];
 
