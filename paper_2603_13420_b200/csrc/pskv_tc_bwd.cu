@@ -2,7 +2,7 @@
 //   dQ        = scale * sum_j dS_j K_j              over the shared prefix keys and the visible suffix keys
 //   dK_suffix = scale * sum over rows of dS^T Q     (suffix keys only: the prefix cache is frozen, Sec. 4.2)
 //   dV_suffix =         sum over rows of  P^T dO
-//   with P = exp(S - lse), S = scale Q K^T, dP = dO V^T, dS = P o (dP - D), D = <dO, O> (a pre-pass).
+//   with P = exp(S - lse), S = scale Q K^T, dP = dO V^T, dS = P o (dP - D), D = <dO, O> (a pre-pass, or in here: DROW).
 // Q and dO are fetched once; nothing is read or recomputed twice except in the passes named below.
 //
 // A CTA works on units.  A unit is `cu` neighbouring candidates of one KV head, so that the sums over rows
@@ -74,7 +74,9 @@ enum : unsigned int {
 
 struct TcBwdParams {
     const float *lse;      // [B*Hq*S] from the forward pass
-    const float *row_dot;  // [B*Hq*S] D
+    const float *row_dot;  // [B*Hq*S] D, or (DROW) what it is formed from:
+    const __nv_bfloat16 *out, *dout;
+    const float *dlse;     // gradient on lse, or nullptr
     __nv_bfloat16 *dq;       // [B,Hq,S,d]
     __nv_bfloat16 *dk, *dv;  // [B,Hkv,S,d]
     unsigned int *status;
@@ -265,7 +267,48 @@ __device__ __forceinline__ void store_sector(__nv_bfloat16 *dst, const uint32_t 
     }
 }
 
-template <int D, bool SPLIT>
+// The rows [first, first + 8) of a CTA's one tile: (-lse log2(e), D) into the row table, D = <dout, out> less the
+// gradient on lse, formed as the pre-pass does.
+template <int D>
+__device__ __forceinline__ void row_dots(const TcBwdParams &p, int b0, int g, int R0, int rows, float2 *table, int first, int lane)
+{
+    constexpr int kLanes = D / 8, kRows = 32 / kLanes, kLoads = 8 / kRows;  // lanes of a row, rows of a load
+    const int sub = lane / kLanes, col = lane % kLanes * 8;
+    uint4 o[kLoads], d[kLoads];
+    float2 st[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+        const int row = first + u * kRows + sub, R = R0 + row, c = p.fd_Rp.div(R), r = R - c * p.Rp;
+        const bool v = row < rows && r < p.Rg;  // rows that do not exist get probability zero
+        o[u] = d[u] = make_uint4(0, 0, 0, 0);
+        st[u] = make_float2(-INFINITY, 0.f);
+        if (v) {
+            const size_t at = ((size_t)(b0 + c) * p.Hq + (size_t)g * p.n_rep) * p.S + r;
+            o[u] = *reinterpret_cast<const uint4 *>(p.out + at * D + col);
+            d[u] = *reinterpret_cast<const uint4 *>(p.dout + at * D + col);
+            st[u] = make_float2(-p.lse[at] * kLog2e, p.dlse ? p.dlse[at] : 0.f);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+        const __nv_bfloat162 *ob = reinterpret_cast<const __nv_bfloat162 *>(&o[u]);
+        const __nv_bfloat162 *gb = reinterpret_cast<const __nv_bfloat162 *>(&d[u]);
+        float acc = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float2 x = __bfloat1622float2(ob[e]), y = __bfloat1622float2(gb[e]);
+            acc = fmaf(x.x, y.x, acc);
+            acc = fmaf(x.y, y.y, acc);
+        }
+#pragma unroll
+        for (int off = kLanes / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane % kLanes == 0)
+            table[first + u * kRows + sub] = make_float2(st[u].x, acc - st[u].y);
+    }
+}
+
+// DROW: every CTA has one tile, and forms its D itself instead of reading it from a pre-pass.
+template <int D, bool SPLIT, bool DROW>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
               const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
@@ -298,7 +341,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         for (int i = lane; i < kNumBars; i += 32) {
             const bool epi = i == kBarDqFree || i == kBarAccFree;
             const bool elem = (i >= kBarSFree && i < kBarSFree + 2) || (i >= kBarDsReady && i < kBarDsReady + 2);
-            mbar_init(bar(i), elem ? 8u : epi ? 4u : i == kBarQFree ? 2u : 1u);
+            mbar_init(bar(i), elem ? 8u : epi ? 4u : i == kBarQFree ? 2u : DROW && i == kBarRowsFull ? 16u : 1u);
         }
         if (lane == 0) *abort_flag = 0;
         fence_barrier_init();
@@ -425,7 +468,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // The tile's row table: -lse log2(e) and D; rows that do not exist get probability zero.
             float st[4], dr[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 4 && !DROW; ++i) {
                 const int row = 32 * i + lane, R = w.R0 + row;
                 const int c = p.fd_Rp.div(R), r = R - c * p.Rp;
                 const bool v = row < w.rows && r < p.Rg;
@@ -462,12 +505,14 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     tma_load_4d(sbase + p.off_do + off, &tm_do, bar(kBarQFull), sl * 64, r, g, b);
                 }
             }
-            // Table tile & 1 was last read for tile - 2; the MMAs behind kBarQFree of tile - 1 came after that.
-            float2 *rows = reinterpret_cast<float2 *>(smem + p.off_rows) + (tile & 1u) * kTileM;
+            if (!DROW) {
+                // Table tile & 1 was last read for tile - 2; the MMAs behind kBarQFree of tile - 1 came after that.
+                float2 *rows = reinterpret_cast<float2 *>(smem + p.off_rows) + (tile & 1u) * kTileM;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) rows[32 * i + lane] = make_float2(st[i], dr[i]);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarRowsFull + (tile & 1u)));
+                for (int i = 0; i < 4; ++i) rows[32 * i + lane] = make_float2(st[i], dr[i]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kBarRowsFull + (tile & 1u)));
+            }
             ++tile;
         }
     } else if (warp == 1) {
@@ -603,6 +648,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int ks = set;
         uint32_t kph = 0, tile = 0xffffffffu;  // (no tile has this number and index)
         if (ks >= p.stages_k) { ks -= p.stages_k; kph ^= 1u; }
+        if (DROW) {  // under the first copies
+            row_dots<D>(p, w.b0, w.g, w.R0, w.rows, reinterpret_cast<float2 *>(smem + p.off_rows),
+                        32 * (warp & 3) + 8 * ((warp - 4) >> 2), lane);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarRowsFull));
+        }
         float neg_lse2 = 0.f, drow = 0.f;
         int my_grp = -1, my_lo = 0, my_hi = 0;
 #pragma unroll 1
@@ -921,9 +972,20 @@ const BwdPlan &plan_bwd(const Dims &dm, int n_instr)
     return table.get(dm, n_instr, [&] { return make_plan(dm, n_instr); });
 }
 
+// D in the kernel: the smallest launches, whose CTAs have one tile each.  Its loads then run under those of the tile's
+// operands, and a launch in the chain of three goes away.  Whole steps, with the pre-pass and with D in here: 8 candidates, 4/4
+// heads, d = 64, P = 32, S = 8 14.1 and 12.0 us; 9, 32/8 heads, P = 256, S = 30 21.8 and 18.2; 2, 32/32 heads, P = 200, S =
+// 128 24.3 and 21.6, P = 300, S = 50 21.7 and 21.2.  With several tiles per CTA every tile waits for its own D: 1
+// candidate, 32/8 heads, P = 78, S = 113 (four tiles in a unit) 25.3 and 28.8, 12 candidates, 32/32 heads, P = 90, S = 77
+// (three units per CTA) 38.7 and 43.9.
+bool row_dot_in_kernel(const Dims &dm, const BwdPlan &plan)
+{
+    return plan.cu * plan.Rp <= kTileM && (long long)plan.upi * dm.Hkv * plan.n_sub <= sm_count();
+}
+
 template <int D>
 cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_word, cudaStream_t stream, int n_instr,
-                   const int *prefix_len, int split)
+                   const int *prefix_len, int split, bool drow)
 {
     const Dims &dm = a.dims;
     const int Rg = dm.n_rep * dm.S;
@@ -957,6 +1019,9 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     memset(&p, 0, sizeof(p));
     p.lse = a.lse;
     p.row_dot = a.row_dot;
+    p.out = a.out;
+    p.dout = a.dout;
+    p.dlse = a.dlse;
     p.dq = a.dq;
     p.dq_sectors = (reinterpret_cast<uintptr_t>(a.dq) & 31u) == 0;
     p.dk = a.dk_suffix;
@@ -987,9 +1052,11 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     p.off_ds = plan.off_ds; p.off_rows = plan.off_rows; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
     for (int i = 0; i < n_instr && n_instr > 1; ++i) p.pad[i] = dm.P - prefix_len[i];
 
-    auto kernel = plan.n_sub > 1 ? tc_bwd_kernel<D, true> : tc_bwd_kernel<D, false>;
-    static PerDeviceOnce attr_set[2];
-    if (cudaError_t e = ensure_max_smem(kernel, attr_set[plan.n_sub > 1]); e != cudaSuccess) return e;
+    const bool sp = plan.n_sub > 1;
+    auto kernel = drow ? (sp ? tc_bwd_kernel<D, true, true> : tc_bwd_kernel<D, false, true>)
+                       : (sp ? tc_bwd_kernel<D, true, false> : tc_bwd_kernel<D, false, false>);
+    static PerDeviceOnce attr_set[4];
+    if (cudaError_t e = ensure_max_smem(kernel, attr_set[2 * drow + sp]); e != cudaSuccess) return e;
     const int units = p.upg * dm.Hkv * p.n_sub;
     if (split > units) split = units;
     for (int s = 0; s < split; ++s) {
@@ -1052,13 +1119,14 @@ cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStrea
     if (n_instr > 1 && (!prefix_len || !tc_bwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
     const BwdPlan &plan = plan_bwd(a.dims, n_instr);
     if (!plan.ok) return cudaErrorInvalidValue;
-    if (parts & kBwdPartRowDot) {
+    const bool drow = parts == kBwdPartAll && n_instr == 1 && split == 1 && row_dot_in_kernel(a.dims, plan);
+    if ((parts & kBwdPartRowDot) && !drow) {
         const cudaError_t e = launch_simt_row_dot(a, stream);
         if (e != cudaSuccess) return e;
     }
     if (!(parts & kBwdPartGrad)) return cudaSuccess;
-    return a.dims.d == 128 ? launch<128>(a, plan, status_word, stream, n_instr, prefix_len, split)
-                           : launch<64>(a, plan, status_word, stream, n_instr, prefix_len, split);
+    return a.dims.d == 128 ? launch<128>(a, plan, status_word, stream, n_instr, prefix_len, split, drow)
+                           : launch<64>(a, plan, status_word, stream, n_instr, prefix_len, split, drow);
 }
 
 }  // namespace pskv
