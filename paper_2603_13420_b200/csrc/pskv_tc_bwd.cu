@@ -37,6 +37,16 @@
 // busy instead of one, at the price of forming the scores of the suffix pieces once more.  Whole steps: B = 1, 32/8
 // heads, P = 78, S = 113 45 -> 25 us; B = 4, 32/8, P = 1000, S = 100 96 -> 56; B = 20, 32/8, P = 200, S = 90 84 -> 77.
 //
+// Two terms (TWO): P and dS go to shared memory as sums of two bf16 values (16 bits of mantissa), and the contractions run over
+// both.  Taken where the suffix length is no multiple of 8 or exceeds 64 (multiples of 8 up to 128: for dK / dV alone):
+// the CUDA-core kernels, which these lengths came from, hold P and dS in fp32, and one bf16 term is not that.  Distance
+// (2-norm) of dQ / dK / dV from 64-bit gradients, B = 333, 32/8 heads, P = 217, S = 53: CUDA cores 2.40e-3 / 1.80e-3 / 1.67e-3,
+// one term 3.25e-3 / 2.51e-3 / 2.35e-3, two terms 2.40e-3 / 1.80e-3 / 1.67e-3 (the rounding of the results, and of `out` inside
+// D).  Price of the second term, kernel and pre-pass: that shape 290 -> 312 us, B = 100, 32/32 heads, P = 78, S = 113 192 ->
+// 223, B = 250, 32/8, P = 385, S = 42 210 -> 256, one candidate, 32/8, P = 78, S = 113 17.2 -> 19.9 (CUDA cores: 21.4 ms, 10.3 ms,
+// 20 ms, 233 us).  The second terms take the memory of three stages; with three K stages and one V stage left the
+// second and third of these took 243 and 271 us, with two and two 266 and 310 (both with the spills the loop had then).
+//
 // Persistent CTA, one per SM, 24 warps:
 //   warp 0      TMA producer: K and V pieces (two rings); writes the descriptor of every item
 //   warp 1      tcgen05.mma issuer: S and dP
@@ -83,6 +93,7 @@ struct TcBwdParams {
     float sl2;             // scale * log2(e)
     float scale;
     int dq_sectors;        // dq is 32-byte aligned
+    int dq_two;            // TWO: dQ over both terms too
     int Hq, Hkv, S, P, n_rep;
     int Rg;                // rows of a candidate in one KV-head group: n_rep * S
     int Rp;                // rows it takes in the unit's row list: Rg rounded up to 8
@@ -267,6 +278,20 @@ __device__ __forceinline__ void store_sector(__nv_bfloat16 *dst, const uint32_t 
     }
 }
 
+// Eight values as bf16; `two`: with what the rounding leaves (exact in fp32) as bf16 in the buffer behind.
+__device__ __forceinline__ void store_terms(uint8_t *dst, const float *x, bool two)
+{
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) hi[i] = pack_bf16x2(x[2 * i], x[2 * i + 1]);
+    *reinterpret_cast<uint4 *>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    if (!two) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        lo[i] = pack_bf16x2(x[2 * i] - __uint_as_float(hi[i] << 16), x[2 * i + 1] - __uint_as_float(hi[i] & 0xffff0000u));
+    *reinterpret_cast<uint4 *>(dst + kDsBytes) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+}
+
 // The rows [first, first + 8) of a CTA's one tile: (-lse log2(e), D) into the row table, D = <dout, out> less the
 // gradient on lse, formed as the pre-pass does.
 template <int D>
@@ -307,8 +332,8 @@ __device__ __forceinline__ void row_dots(const TcBwdParams &p, int b0, int g, in
     }
 }
 
-// DROW: every CTA has one tile, and forms its D itself instead of reading it from a pre-pass.
-template <int D, bool SPLIT, bool DROW>
+// DROW: every CTA has one tile, and forms its D itself instead of reading it from a pre-pass.  TWO: P and dS as two terms.
+template <int D, bool SPLIT, bool DROW, bool TWO>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
               const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
@@ -316,6 +341,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
               const __grid_constant__ TcBwdParams p)
 {
     using C = Cfg<D>;
+    constexpr int kTerms = TWO ? 2 : 1;
+    constexpr uint64_t kLoTerm = (uint64_t)(kDsBytes >> 4);  // descriptor distance from a P / dS buffer to its second term
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -576,7 +603,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll 1
         for (uint32_t item = 0;; ++item) {
             const uint32_t slot = item & 1u;
-            const uint64_t ds_a = make_smem_desc(sbase + p.off_ds + slot * kDsBytes, kDsBytes, 1024);
+            const uint64_t ds_a = make_smem_desc(sbase + p.off_ds + slot * kTerms * kDsBytes, kDsBytes, 1024);
             const uint64_t k_desc = make_smem_desc(sbase + p.off_k + ks * C::kPieceBytes, C::kPieceSlab, 1024);
             ok = mbar_wait_warp(bar(kBarKFull + ks), kph, abort_flag, p.status, kErrMmaGrad);
             if (!ok) break;
@@ -598,6 +625,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     if (i * 16 < n)
                         mma_ss(tmem + kColDq, ds_a + (uint64_t)(i * 32 >> 4), k_desc + (uint64_t)(i * 2048 >> 4), idesc_dq,
                                i > 0 ? 1u : acc0);
+                if (TWO && p.dq_two) {
+#pragma unroll
+                    for (int i = 0; i < kPieceN / 16; ++i)
+                        if (i * 16 < n)
+                            mma_ss(tmem + kColDq, ds_a + kLoTerm + (uint64_t)(i * 32 >> 4), k_desc + (uint64_t)(i * 2048 >> 4), idesc_dq, 1u);
+                }
             }
             __syncwarp();
             if (x & kDescAcc) {
@@ -620,6 +653,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         mma_ss(tmem + kColDv, dot_desc + off, p_desc + off, idesc_acc, a);
                         mma_ss(tmem + kColDk, qt_desc + off, ds_a + off, idesc_acc, a);
                         a = 1u;
+                        if (TWO) {
+                            mma_ss(tmem + kColDv, dot_desc + off, p_desc + kLoTerm + off, idesc_acc, 1u);
+                            mma_ss(tmem + kColDk, qt_desc + off, ds_a + kLoTerm + off, idesc_acc, 1u);
+                        }
                     }
                     tc_commit(bar(kBarPFree));
                     if (x & kDescAccLast) tc_commit(bar(kBarAccFull));
@@ -643,7 +680,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         const int row = 32 * (warp & 3) + lane;
         const uint32_t my_tmem = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + set * kSlotCols + c0;
         uint8_t *p_row = smem + p.off_p + row * 128;
-        uint8_t *ds_row = smem + p.off_ds + set * kDsBytes + row * 128;
+        uint8_t *ds_row = smem + p.off_ds + set * kTerms * kDsBytes + row * 128;
         const uint4 *descs = reinterpret_cast<const uint4 *>(smem + p.off_bar + kDescOff);
         int ks = set;
         uint32_t kph = 0, tile = 0xffffffffu;  // (no tile has this number and index)
@@ -717,6 +754,54 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kBarSFree + set));
+                }
+                if (TWO) {
+                    // eight columns at a time, stored as they are made (the waits first): with sixteen of P and dS held in
+                    // fp32 across the waits the loop spilled
+                    if (hf == 0) {
+                        PSKV_TRACE_EVENT(21, item);
+                        ok = mbar_wait_warp(bar(kBarDsFree + set), sph ^ 1u, abort_flag, p.status, kErrElem);
+                        if (ok && acc)
+                            ok = mbar_wait_warp(bar(kBarPFree), (dsc.x & kDescAccOdd) ? 0u : 1u, abort_flag, p.status, kErrElem);
+                        if (!ok) break;
+                        PSKV_TRACE_EVENT(22, item);
+                    }
+                    if (kind == 0) continue;
+                    const bool lo_term = acc || p.dq_two;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        float e[8], ds[8];
+                        if (kind >= 2) {
+#pragma unroll
+                            for (int c = 0; c < 8; c += 2) {
+                                float x0 = __uint_as_float(rs[8 * i + c]), x1 = __uint_as_float(rs[8 * i + c + 1]);
+                                fma_f32x2(x0, x1, p.sl2, neg_lse2);
+                                e[c] = ex2_approx(x0);
+                                e[c + 1] = ex2_approx(x1);
+                            }
+                            if (kind == 2) {
+                                const unsigned span = (unsigned)(hi - lo);
+                                const int base = c0 + hf * 16 + 8 * i - lo;
+                                const bool any_col = hi >= lo;
+#pragma unroll
+                                for (int c = 0; c < 8; ++c) e[c] = (any_col && (unsigned)(base + c) <= span) ? e[c] : 0.f;
+                            }
+#pragma unroll
+                            for (int c = 0; c < 8; c += 2) {
+                                ds[c] = __uint_as_float(rd[8 * i + c]);
+                                ds[c + 1] = __uint_as_float(rd[8 * i + c + 1]);
+                                add_f32x2(ds[c], ds[c + 1], -drow, -drow);
+                                mul_f32x2(ds[c], ds[c + 1], e[c], e[c + 1]);
+                            }
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) e[c] = ds[c] = 0.f;
+                        }
+                        const int off = (((c0 >> 3) + 2 * hf + i) ^ (row & 7)) << 4;
+                        store_terms(ds_row + off, ds, lo_term);
+                        if (acc) store_terms(p_row + off, e, true);
+                    }
+                    continue;
                 }
                 if (kind >= 2) {
                     float e[16];
@@ -875,6 +960,7 @@ struct BwdPlan {
     bool ok;
     int cu, cpp, nh, Rp, Sp, seg, cbox, sfx_box, nblk, upi;
     int n_tiles, n_sub;
+    int terms;             // bf16 terms of P and dS
     int stages_k, stages_v;
     int off_do, off_q, off_k, off_v, off_p, off_ds, off_rows, off_bar, off_misc, smem_bytes;
 };
@@ -946,19 +1032,21 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
     pl.upi = (Kq + pl.cu - 1) / pl.cu;
     const int slabs = dm.d / 64;
     const int tile_bytes = slabs * kTileM * 128, piece_bytes = slabs * kPieceN * 128;
-    const int fixed = 2 * tile_bytes + 3 * kDsBytes + kRowsBytes + kBarBytes + 64;
+    pl.terms = dm.S % 8 != 0 || dm.S > kPieceN ? 2 : 1;  // (see the head of this file)
+    const int fixed = 2 * tile_bytes + 3 * pl.terms * kDsBytes + kRowsBytes + kBarBytes + 64;
     int n = (kMaxSmem - fixed) / piece_bytes;
     if (n > 2 * kMaxRing) n = 2 * kMaxRing;
     if (n < 2) return pl;
-    pl.stages_v = n / 2;  // a K piece is needed until its dQ product, a V piece only for dP
+    // a K piece is needed until its dQ product, a V piece only for dP (three and one rather than two and two: see above)
+    pl.stages_v = n > 4 ? n / 2 : 1;
     pl.stages_k = n - pl.stages_v;
     pl.off_do = 0;
     pl.off_q = tile_bytes;
     pl.off_k = 2 * tile_bytes;
     pl.off_v = pl.off_k + pl.stages_k * piece_bytes;
     pl.off_p = pl.off_v + pl.stages_v * piece_bytes;
-    pl.off_ds = pl.off_p + kDsBytes;
-    pl.off_rows = pl.off_ds + 2 * kDsBytes;
+    pl.off_ds = pl.off_p + pl.terms * kDsBytes;
+    pl.off_rows = pl.off_ds + 2 * pl.terms * kDsBytes;
     pl.off_bar = pl.off_rows + kRowsBytes;
     pl.off_misc = pl.off_bar + kBarBytes;
     pl.smem_bytes = pl.off_misc + 64;
@@ -983,7 +1071,7 @@ bool row_dot_in_kernel(const Dims &dm, const BwdPlan &plan)
     return plan.cu * plan.Rp <= kTileM && (long long)plan.upi * dm.Hkv * plan.n_sub <= sm_count();
 }
 
-template <int D>
+template <int D, bool TWO>
 cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_word, cudaStream_t stream, int n_instr,
                    const int *prefix_len, int split, bool drow)
 {
@@ -1023,6 +1111,7 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     p.dout = a.dout;
     p.dlse = a.dlse;
     p.dq = a.dq;
+    p.dq_two = dm.S % 8 != 0 || dm.S > kTileM;
     p.dq_sectors = (reinterpret_cast<uintptr_t>(a.dq) & 31u) == 0;
     p.dk = a.dk_suffix;
     p.dv = a.dv_suffix;
@@ -1053,8 +1142,8 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     for (int i = 0; i < n_instr && n_instr > 1; ++i) p.pad[i] = dm.P - prefix_len[i];
 
     const bool sp = plan.n_sub > 1;
-    auto kernel = drow ? (sp ? tc_bwd_kernel<D, true, true> : tc_bwd_kernel<D, false, true>)
-                       : (sp ? tc_bwd_kernel<D, true, false> : tc_bwd_kernel<D, false, false>);
+    auto kernel = drow ? (sp ? tc_bwd_kernel<D, true, true, TWO> : tc_bwd_kernel<D, false, true, TWO>)
+                       : (sp ? tc_bwd_kernel<D, true, false, TWO> : tc_bwd_kernel<D, false, false, TWO>);
     static PerDeviceOnce attr_set[4];
     if (cudaError_t e = ensure_max_smem(kernel, attr_set[2 * drow + sp]); e != cudaSuccess) return e;
     const int units = p.upg * dm.Hkv * p.n_sub;
@@ -1125,8 +1214,9 @@ cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStrea
         if (e != cudaSuccess) return e;
     }
     if (!(parts & kBwdPartGrad)) return cudaSuccess;
-    return a.dims.d == 128 ? launch<128>(a, plan, status_word, stream, n_instr, prefix_len, split, drow)
-                           : launch<64>(a, plan, status_word, stream, n_instr, prefix_len, split, drow);
+    auto run = plan.terms == 2 ? (a.dims.d == 128 ? launch<128, true> : launch<64, true>)
+                               : (a.dims.d == 128 ? launch<128, false> : launch<64, false>);
+    return run(a, plan, status_word, stream, n_instr, prefix_len, split, drow);
 }
 
 }  // namespace pskv
