@@ -187,7 +187,15 @@ __device__ __forceinline__ int sfx_long_rows(const TcFwdParams &p, int j)
 // in as many blocks as it takes -- the mode of the decode-shaped operator, where a 128-row tile
 // spans many candidates, and of full-suffix shapes the other two modes cannot tile.  A compile-time
 // switch so that each launch carries only the code of its own mode.
-template <int D, int MODE, bool MI>
+//
+// TWO (suffix-ring): probabilities as the sum of two bf16 values, the second in the half of a piece that the first leaves free, and
+// a value contraction over each.  For the lengths that came from the CUDA-core kernel (two_terms in plan_suffix_ring), whose
+// probabilities are fp32.  Distance (2-norm) of `out` from 64 bits, a prompt of 1039 tokens, 32/8 heads: CUDA cores 1.625e-3,
+// one term 2.310e-3, two terms 1.625e-3 (the rounding of the result); of lse 4.9e-8, 7.6e-8 and, with the logarithm in 64
+// bits, 4.1e-8 (131 tokens: 4.8e-8, 8.0e-8 and 5.4e-8: what is left is the tensor cores' fp32 sum of a score; one rounding of
+// the result is 2.7e-8).  Price: 131 tokens 8.7 -> 9.0 us, 1039 21.0 -> 24.0, 4093 131 -> 170 (CUDA cores 52 us, 1.58 and
+// 22.2 ms).
+template <int D, int MODE, bool MI, bool TWO = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_out,
               const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
@@ -785,9 +793,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (elect_one_sync()) {
 #pragma unroll
                 for (int ks16 = 0; ks16 < kBlockN / 16; ++ks16) {
-                    if (ks16 < nk)
-                        mma_ts(tmem + kOCol, p_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8, v_desc + (uint64_t)(ks16 * (2048 >> 4)), idesc_pv,
-                               ks16 > 0 ? 1u : acc0);
+                    if (ks16 < nk) {
+                        const uint32_t p_cols = p_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8;
+                        const uint64_t v_rows = v_desc + (uint64_t)(ks16 * (2048 >> 4));
+                        mma_ts(tmem + kOCol, p_cols, v_rows, idesc_pv, ks16 > 0 ? 1u : acc0);
+                        if (TWO) mma_ts(tmem + kOCol, p_cols + kPiece / 2, v_rows, idesc_pv, 1u);
+                    }
                 }
                 tc_commit(bar(kBarPvDone + slot));
                 if (free_stage) tc_commit(bar(kBarVFree + (vuse % (uint32_t)p.stages)));
@@ -935,11 +946,19 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                                 pk[2 * c] = pack_bf16x2(e[4 * c], e[4 * c + 1]);
                                 pk[2 * c + 1] = pack_bf16x2(e[4 * c + 2], e[4 * c + 3]);
                             }
+                            if (TWO) {  // what the rounding leaves is exact in fp32
+                                uint32_t lo[kPiece / 2];
+#pragma unroll
+                                for (int c = 0; c < kPiece / 2; ++c)
+                                    lo[c] = pack_bf16x2(e[2 * c] - __uint_as_float(pk[c] << 16), e[2 * c + 1] - __uint_as_float(pk[c] & 0xffff0000u));
+                                tmem_st16(s_tmem + kPiece / 2, lo);
+                            }
                             ls0 += ls2;
                             ls1 += ls3;
                         } else {
 #pragma unroll
                             for (int c = 0; c < kPiece / 2; ++c) pk[c] = 0u;
+                            if (TWO) tmem_st16(s_tmem + kPiece / 2, pk);
                         }
                         lsum += ls0 + ls1;
                         tmem_st16(s_tmem, pk);
@@ -1086,7 +1105,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             const bool stored = row < u.rows && r < p.Rr && (!SR || r - hd * p.Sh < p.S);
             if (stored) {
                 const size_t grow = ((size_t)b * p.Hq + (size_t)u.g * p.n_rep) * p.S + r - skip;
-                p.lse[grow] = row_ok ? log2f(l) * kLn2 : __int_as_float(0x7fc00000);
+                // (log2f is good to 2^-22 absolute, more than the CUDA-core kernel loses, whose sum is relative to the maximum)
+                p.lse[grow] = row_ok ? (TWO ? (float)log((double)l) : log2f(l) * kLn2) : __int_as_float(0x7fc00000);
             }
             const unsigned bad = __ballot_sync(0xffffffffu, stored && !row_ok);
             if (bad != 0u && lane == 0) atomicAdd(cta_redo, __popc(bad));
@@ -1142,6 +1162,7 @@ struct TilePlan {
     int mode;   // kernel template MODE: 0 rings, 1 resident prefix, 2 suffix-ring
     int cbox, Spad, cpb;  // suffix-ring mode: candidates per tile, rows per candidate in a block, candidates per block
     int long_sfx;         // suffix-ring mode: tiles inside one candidate, its suffix keys in 128-key blocks
+    int two_terms;        // suffix-ring mode: probabilities as two bf16 terms
     int tile_rows, seg_rows, tiles_per_group, sfx_rows;
     int Rp, Sp;           // rows / suffix key columns a candidate takes
     int Sh, one_box, head_box;  // see TcFwdParams
@@ -1239,11 +1260,13 @@ TilePlan plan_suffix_ring(const Dims &dm)
         // it lies inside one head too: a head's rows are padded to whole tiles, so any length does, and a tile's
         // cost follows from its position, so that tiles can be dealt out by cost.  Else, and where heads would be
         // padded to more tiles, a tile is the largest divisor of the candidate's rows that fits.  (Lengths without such a
-        // divisor went to the CUDA-core kernel: 1.57 ms for a prompt of 1039 tokens, 12.2 for 3001, now 22 and 131 us.)
+        // divisor went to the CUDA-core kernel: 1.58 ms for a prompt of 1039 tokens, 12.2 for 3001, now 24 and 108 us;
+        // they keep its precision, see TWO at the kernel.)
         int rows = 0;
         for (int m = kTileM; m >= 16 && !rows; --m)
             if (Rg % m == 0) rows = m;
         if (!rows && Rg <= kTileM) rows = Rg;
+        pl.two_terms = !rows;
         const int per_head = (dm.S + kTileM - 1) / kTileM;
         if (dm.S > kTileM && (!rows || (long long)dm.n_rep * per_head <= Rg / rows)) {
             rows = round_up((dm.S + per_head - 1) / per_head, 8);
@@ -1507,11 +1530,11 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     }
 
     const bool mi = n_instr > 1;  // (never with the suffix-ring tiling)
-    auto kernel = plan.mode == 2 ? tc_fwd_kernel<D, 2, false>
+    auto kernel = plan.mode == 2 ? (plan.two_terms ? tc_fwd_kernel<D, 2, false, true> : tc_fwd_kernel<D, 2, false>)
                   : plan.mode == 1 ? (mi ? tc_fwd_kernel<D, 1, true> : tc_fwd_kernel<D, 1, false>)
                                    : (mi ? tc_fwd_kernel<D, 0, true> : tc_fwd_kernel<D, 0, false>);
-    static PerDeviceOnce attr_set[6];
-    if (cudaError_t e = ensure_max_smem(kernel, attr_set[plan.mode + (mi ? 3 : 0)]); e != cudaSuccess) return e;
+    static PerDeviceOnce attr_set[7];
+    if (cudaError_t e = ensure_max_smem(kernel, attr_set[plan.two_terms ? 6 : plan.mode + (mi ? 3 : 0)]); e != cudaSuccess) return e;
     const int grid = even_grid(p.total_tiles, sm_count());
     cudaError_t launch_err;
     {

@@ -1,5 +1,6 @@
 """Gradients of suffix lengths that are no multiple of 8, or beyond 64, are as exact as fp32 probabilities and dS make them: what is
-left is the rounding of the result to bf16.  (dQ of a multiple of 8 up to 128 takes dS rounded to bf16, as up to 64.)"""
+left is the rounding of the result to bf16.  (dQ of a multiple of 8 up to 128 takes dS rounded to bf16, as up to 64.)
+The same of the forward of more than 128 queries whose rows have no divisor between 16 and 128."""
 import numpy as np
 import pytest
 import torch
@@ -48,3 +49,19 @@ def test_gradients_are_off_by_the_rounding_of_the_result_alone(shape):
         # Two bf16 terms hold 16 bits: 2^-17 relative, a few hundredths of the result's own rounding (2^-9) even where the terms
         # of a sum cancel tenfold.  One term (2^-9 again) would give a factor of 1.4.
         assert err <= 1.05 * _rounding(r), (name, err / _rounding(r))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [
+    # B, Hq, Hkv, d, P, S: rows without a divisor between 16 and 128
+    (1, 4, 1, 128, 0, 131), (2, 2, 2, 64, 75, 139), (1, 2, 1, 128, 0, 1039), (1, 3, 3, 128, 40, 257),
+], ids=lambda s: "x".join(map(str, s)))
+def test_forward_of_lengths_without_a_divisor_is_off_by_the_rounding_of_the_result_alone(shape):
+    B, Hq, Hkv, d, P, S = shape
+    w = Workload("precision", 400 + sum(shape), B=B, Hq=Hq, Hkv=Hkv, d=d, P=P, S=S)
+    t = make_inputs(w)
+    out, lse, _ = parity.run_fwd_gpu(t, w.scale)
+    ref_out, ref_lse = parity.oracle_fwd(t, w.scale)
+    assert np.linalg.norm(parity.to_f64(out) - ref_out) <= 1.05 * _rounding(ref_out)
+    # fp32 scores of about 10 log2 units, a sum over the keys and the rounding of the result, 2^-24 each
+    assert np.linalg.norm(parity.to_f64(lse) - ref_lse) <= 2.0 ** -24 * np.linalg.norm(ref_lse)
