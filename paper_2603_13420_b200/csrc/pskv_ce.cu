@@ -318,8 +318,18 @@ inline bool encode_2d(CUtensorMap *map, const void *base, int cols, long long ro
 
 struct CePlan {
     int nrt, nvb, panel, npanel, Rpad, ksteps;
-    size_t part_bytes, ws_bytes;
+    size_t ws_bytes;
 };
+
+// Units a call may have: the workspace holds the partials of that many.  It never falls as rows are added, so that scratch
+// sized for a program's largest batch serves its smaller ones, and depends on the sizes alone, so that the query gives the same
+// bytes wherever it is made.  32 units for each of 148 SMs, or panels of five blocks, leave out no width that
+// would be more than half a percent cheaper.
+long long ce_max_units(int nrt, int nvb)
+{
+    const long long narrow = (long long)nvb * nrt, cap = 32 * 148, wide = (long long)((nvb + 4) / 5) * nrt;
+    return wide > cap ? wide : narrow < cap ? narrow : cap;
+}
 
 // Blocks per panel: a CTA's time is its units times their blocks, so the width is the one whose units fill the last
 // round of the SMs best, 8 where nothing is clearly better.  204 rows of a 32 000-word vocabulary are 32 units of
@@ -329,6 +339,7 @@ struct CePlan {
 int ce_panel(int nrt, int nvb)
 {
     const int sms = sm_count();
+    const long long most = ce_max_units(nrt, nvb);
     auto cost = [&](int panel) {
         const long long units = (long long)((nvb + panel - 1) / panel) * nrt;
         return (double)((units + sms - 1) / sms) * (panel + 0.1);
@@ -336,7 +347,7 @@ int ce_panel(int nrt, int nvb)
     int best = 8;
     double best_cost = 0.99 * cost(8);
     for (int panel = kCeMaxPanel; panel >= 1; --panel)
-        if (cost(panel) < best_cost) {
+        if (cost(panel) < best_cost && (long long)((nvb + panel - 1) / panel) * nrt <= most) {
             best = panel;
             best_cost = cost(panel);
         }
@@ -352,8 +363,7 @@ CePlan ce_plan(long long R, int Dm, int V)
     pl.npanel = (pl.nvb + pl.panel - 1) / pl.panel;
     pl.Rpad = pl.nrt * kCeM;
     pl.ksteps = (Dm + kCeK - 1) / kCeK;
-    pl.part_bytes = (size_t)pl.npanel * pl.Rpad * sizeof(float2);
-    pl.ws_bytes = pl.part_bytes + (size_t)pl.Rpad * sizeof(float);
+    pl.ws_bytes = (size_t)ce_max_units(pl.nrt, pl.nvb) * kCeM * sizeof(float2) + (size_t)pl.Rpad * sizeof(float);
     return pl;
 }
 

@@ -113,3 +113,29 @@ def test_target_ce_arguments_are_checked_on_the_host():
     need = pskv.pskv_target_ce_fwd_workspace_bytes(512, 20, 4096, 128256)
     assert need % 256 == 0 and need >= 2 * 63 * 10240 * 4
     assert pskv.pskv_target_ce_fwd_workspace_bytes(4, 4, 60, 100) == 0
+
+
+@pytest.mark.parametrize("V", [300, 4096, 32000, 50257, 128256, 256000])
+def test_workspace_never_falls_as_rows_are_added(V):
+    """Scratch sized for the largest batch of a program serves its smaller ones (a last, partial batch)."""
+    for Lr in (1, 20, 93):
+        sizes = [pskv.pskv_target_ce_fwd_workspace_bytes(N, Lr, 4096, V) for N in range(1, 40000 // Lr, max(1, 64 // Lr))]
+        assert sizes[0] > 0 and sizes == sorted(sizes)
+    sizes = [pskv.pskv_target_ce_fwd_workspace_bytes(3, Lr, 4096, V) for Lr in range(1, 3000)]
+    assert sizes == sorted(sizes)
+
+
+@pytest.mark.gpu
+def test_one_workspace_serves_every_smaller_batch():
+    Dm, V, Lr = 64, 32000, 128
+    gen = torch.Generator(device="cpu").manual_seed(77)
+    w = (torch.randn((V, Dm), generator=gen) / math.sqrt(Dm)).to(torch.bfloat16).cuda()
+    ws = torch.empty(pskv.pskv_target_ce_fwd_workspace_bytes(20, Lr, Dm, V), dtype=torch.uint8, device="cuda")
+    for N in range(20, 0, -1):
+        h = torch.randn((N, Lr, Dm), generator=gen).to(torch.bfloat16).cuda()
+        t = torch.randint(0, V, (N, Lr), generator=gen, dtype=torch.int32).cuda()
+        m = torch.ones((N, Lr), device="cuda")
+        a = pskv.pskv_target_ce_fwd(h, w, t, m, workspace=ws)
+        b = pskv.pskv_target_ce_fwd(h, w, t, m)
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
+    assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
