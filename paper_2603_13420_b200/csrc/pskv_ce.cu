@@ -14,8 +14,8 @@
 // CTA c takes units c, c + G, c + 2G, ...: the CTAs running at any moment work on about four weight
 // panels (16 MB each) against one group of row tiles (1 MB each), a working set that stays in L2, so
 // the weight matrix comes from HBM once per row group and the hidden states once.  Each unit
-// leaves one partial (max, sum) per row; a small kernel, one block per candidate, merges the partials of its rows
-// into lse and nll = mask * (lse - target logit) and forms the masked average.
+// leaves one partial (max, sum) per row; a small kernel merges the partials of a row into lse and nll = mask * (lse -
+// target logit) and forms the masked average of each candidate (with many rows per candidate a second one does).
 //
 // Roles (256 threads): warp 0 TMA producer (hidden tile and weight block, 64 columns of the hidden
 // dimension per stage, 4 stages), warp 1 tcgen05.mma issuer, warp 2 owns the tensor-memory
@@ -250,25 +250,31 @@ ce_fwd_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ 
     if (warp == 2) tmem_dealloc(tmem, 512);
 }
 
-// One block per candidate, a warp per row at a time: merges the partials of the candidate's rows (contiguous, one lane
-// each) into lse and nll, then the masked average.  (One thread per row, walking over the panels, took 13 to 30 us,
-// and a third launch, in calls whose projection takes 40 to 400.)
+// Merges the partials of a row (contiguous, one lane each) into lse and nll by one warp, and forms the masked average of a
+// candidate.  WHOLE: a block per candidate does both, its warps taking the rows in turn.  Else a block takes kCeFinalWarps rows
+// of the list of all rows, and ce_average_kernel follows.  (One thread per row, walking over the panels, took 13 to 30 us in
+// calls whose projection takes 40 to 400.)
 constexpr int kCeFinalWarps = 8;
+// Up to three rows per warp a second launch costs more than it gives.  Whole calls, one kernel and two: 1 candidate x 8 rows
+// (Dm = 1024, 32 000 words) 18.2 and 19.6 us, x 20 21.0 and 20.5, x 32 20.4 and 18.6, x 64 21.7 and 15.5, x 256 52 and 21; 512 x
+// 20 (Dm = 256, 4 096 words) 37.9 and 38.2, x 96 144 and 139; 1 x 30 000 (Dm = 256, 4 096 words) 3 660 and 98.
+constexpr int kCeWholeRows = 24;
+template <bool WHOLE>
 __global__ void __launch_bounds__(32 * kCeFinalWarps)
 ce_finalize_kernel(const float2 *part, const float *tlogit, const int *target, const float *mask, float *nll, float *lse,
-                   float *loss, int Lr, int npanel, int V)
+                   float *loss, long long R, int Lr, int npanel, int V)
 {
     __shared__ float num_s[kCeFinalWarps], den_s[kCeFinalWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float num = 0.f, den = 0.f;
-    for (int i = warp; i < Lr; i += kCeFinalWarps) {
-        const size_t r = (size_t)blockIdx.x * Lr + i;
-        const float2 *pr = part + r * npanel;
+    const long long first = (long long)blockIdx.x * (WHOLE ? Lr : kCeFinalWarps), end = WHOLE ? first + Lr : min(R, first + kCeFinalWarps);
+    for (long long r = first + warp; r < end; r += kCeFinalWarps) {
+        const float2 *pr = part + (size_t)r * npanel;
         float M = -INFINITY, L = 0.f;
         for (int pn = lane; pn < npanel; pn += 32) {
             const float2 x = pr[pn];
             const float m = fmaxf(M, x.x);
-            // (a panel may hold nothing but -inf logits: m - M would be inf - inf)
+            // (equal maxima need no factor; a lane that has seen no panel holds -inf, and -inf - -inf is not 0)
             L = (M == m ? L : L * exp2f(M - m)) + (x.x == m ? x.y : x.y * exp2f(x.x - m));
             M = m;
         }
@@ -292,6 +298,39 @@ ce_finalize_kernel(const float2 *part, const float *tlogit, const int *target, c
         }
         num += v;
         den += w;
+    }
+    if (!WHOLE) return;
+    if (lane == 0) {
+        num_s[warp] = num;
+        den_s[warp] = den;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        num = den = 0.f;
+        for (int k = 0; k < kCeFinalWarps; ++k) {
+            num += num_s[k];
+            den += den_s[k];
+        }
+        loss[blockIdx.x] = den != 0.f ? num / den : 0.f;
+    }
+}
+
+// Masked average of a candidate of many rows: one block per candidate.
+__global__ void __launch_bounds__(32 * kCeFinalWarps)
+ce_average_kernel(const float *nll, const float *mask, float *loss, int Lr)
+{
+    __shared__ float num_s[kCeFinalWarps], den_s[kCeFinalWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float num = 0.f, den = 0.f;
+    for (int i = threadIdx.x; i < Lr; i += 32 * kCeFinalWarps) {
+        const size_t r = (size_t)blockIdx.x * Lr + i;
+        num += nll[r];
+        den += mask[r];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
     }
     if (lane == 0) {
         num_s[warp] = num;
@@ -411,10 +450,14 @@ cudaError_t launch_ce_fwd(const CeArgs &a, void *workspace, unsigned int *status
     if (e != cudaSuccess) return e;
     {
         KernelTiming timing(kKernelCeFinalize, stream);
-        ce_finalize_kernel<<<(unsigned)a.N, 32 * kCeFinalWarps, 0, stream>>>(p.part, p.tlogit, a.target, a.mask, a.nll, a.lse,
-                                                                            a.loss, a.Lr, pl.npanel, a.V);
+        const bool whole = a.Lr <= kCeWholeRows;
+        const unsigned blocks = whole ? (unsigned)a.N : (unsigned)((R + kCeFinalWarps - 1) / kCeFinalWarps);
+        auto kernel = whole ? ce_finalize_kernel<true> : ce_finalize_kernel<false>;
+        kernel<<<blocks, 32 * kCeFinalWarps, 0, stream>>>(p.part, p.tlogit, a.target, a.mask, a.nll, a.lse, a.loss, R, a.Lr,
+                                                          pl.npanel, a.V);
+        if (!whole) ce_average_kernel<<<(unsigned)a.N, 32 * kCeFinalWarps, 0, stream>>>(a.nll, a.mask, a.loss, a.Lr);
+        count_launches(whole ? 2 : 3);
     }
-    count_launches(2);
     return cudaGetLastError();
 }
 

@@ -139,3 +139,26 @@ def test_one_workspace_serves_every_smaller_batch():
         b = pskv.pskv_target_ce_fwd(h, w, t, m)
         assert all(torch.equal(x, y) for x, y in zip(a, b))
     assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", [
+    # N, Lr, Dm, V: a candidate's rows merged by one block up to 24, by blocks of eight rows beyond
+    (7, 24, 64, 3000), (7, 25, 64, 3000), (3, 251, 64, 9000), (1, 2048, 32, 700)])
+def test_candidates_of_many_rows(case):
+    N, Lr, Dm, V = case
+    h, w, t, m = make(N, Lr, Dm, V, seed=5000 + sum(case))
+    nll = parity.Guarded((N, Lr), torch.float32, "cuda")
+    lse = parity.Guarded((N, Lr), torch.float32, "cuda")
+    loss = parity.Guarded((N,), torch.float32, "cuda")
+    if N == 1:
+        m[0] = (torch.arange(Lr) % 3 != 0).float()
+        t[0, 0] = 5
+    n0 = pskv.pskv_kernel_launches()
+    pskv.pskv_target_ce_fwd(h.cuda(), w.cuda(), t.cuda(), m.cuda(), nll=nll.view, lse=lse.view, loss=loss.view)
+    assert pskv.pskv_kernel_launches() - n0 == (2 if Lr <= 24 else 3)
+    assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
+    nll.check("nll"); lse.check("lse"); loss.check("loss")
+    rn, rl, rs = oracle.target_ce_fwd(parity.to_f64(h), parity.to_f64(w), t.numpy(), m.numpy().astype(np.float64))
+    for got, ref in ((nll, rn), (lse, rl), (loss, rs)):   # (bound: as above)
+        assert np.max(np.abs(parity.to_f64(got.view) - ref) / np.maximum(np.abs(ref), 1.0)) <= 1e-3
