@@ -72,16 +72,16 @@ struct TileInfo {
     bool first_of_g;
 };
 
-// `Params` is any kernel parameter block with fields B, Rg, Sp, tile_rows, tiles_per_group, fd_tpg, fd_Rg.  MI: several
+// `Params` is any kernel parameter block with fields B, Rg, Sp, tile_rows, tiles_per_group, fd_tpg, fd_Rg.  SHORT: several
 // instructions, whose rows (rpi each) are cut into tiles one by one (tpi tiles each, the last one shorter).
-template <bool MI, class Params>
+template <bool SHORT, class Params>
 __device__ __forceinline__ TileInfo tile_info(const Params &p, int tile, int t_begin)
 {
     TileInfo t;
     t.g = p.fd_tpg.div(tile);
     const int tt = tile - t.g * p.tiles_per_group;
     t.first_of_g = (tt == 0) || (tile == t_begin);
-    if (MI) {
+    if (SHORT) {
         const int inst = p.fd_tpi.div(tt), r = (tt - inst * p.tpi) * p.tile_rows;
         t.R0 = inst * p.rpi + r;
         t.rows = min(p.tile_rows, p.rpi - r);

@@ -55,6 +55,22 @@ enum : unsigned int {
     kErrSoftmax = 0x105, kErrEpilogue = 0x106, kErrAlign = 0x107
 };
 
+// MODE 3.  The compiler reads runs of the kernel's parameters in one instruction where they are aligned, and what that makes of the
+// walk over tiles differs: with the fields behind these moved by 12 bytes the kernel for several instructions took 140 us for 8
+// x 64 candidates, 32/8 heads, P = 256, S = 48, moved by 0 or 16 132; the others want the 12 (149 candidates, 4/4 heads, P =
+// 315, S = 8: 10.3 us, else 11.4).
+template <bool SEVERAL>
+struct BoxFields {
+    int Sh;               // rows a query head takes in the row list: S, or S padded to whole tiles (head_box)
+    int one_box;          // 1: a tile's Q is one box per slab (whole candidates, or rows of one head), else runs of seg_rows
+    int head_box;         // 1: Q / out maps are [B][Hq][S][D] and a tile lies inside one head
+};
+template <>
+struct BoxFields<true> {
+    int Sh, one_box, head_box, unused;
+};
+
+template <int MI>
 struct TcFwdParams {
     float *lse;
     unsigned int *status;
@@ -64,9 +80,7 @@ struct TcFwdParams {
     int Rg;               // rows a candidate takes in the row list of a KV-head group (its n_rep * S real rows, padded)
     int Rr;               // its real rows: n_rep * S
     int Sp;               // key columns a candidate takes in a tile's suffix block: S rounded up to 8
-    int Sh;               // rows a query head takes in the row list: S, or S padded to whole tiles (head_box)
-    int one_box;          // 1: a tile's Q is one box per slab (whole candidates, or rows of one head), else runs of seg_rows
-    int head_box;         // 1: Q / out maps are [B][Hq][S][D] and a tile lies inside one head
+    BoxFields<(MI != 0)> box;
     int tile_rows;        // rows of the flat row list per tile (<= 128, multiple of seg_rows)
     int seg_rows;         // rows per Q / out TMA box: gcd(Rg, tile_rows) (rows past Rr are zero-filled, never stored)
     int tiles_per_group;
@@ -93,8 +107,8 @@ struct TcFwdParams {
     // prefix cache i of [n_instr][Hkv][P][d], whose first pad[i] rows are left padding
     int n_instr;          // 1: one shared prefix
     int rpi;              // rows of one instruction inside a KV head's row list
-    int tpi;              // its tiles: an instruction starts a tile of its own
     FastDiv fd_rpi, fd_tpi;
+    int tpi;              // tiles of an instruction, where each starts a tile of its own and its last tile is short
     int pad[kMaxInstr];
     // shared-memory carve-up (byte offsets from the 1024-byte aligned base)
     int off_pk, off_pv, off_q, off_sk, off_sv, off_stage, off_bar, off_misc, off_ml;
@@ -133,20 +147,21 @@ constexpr int kBarBytes = 512;
 static_assert(kNumBars * 8 <= kBarBytes, "barrier area");
 
 // Q / out box coordinates of row r of a group: (row, head) -- the group's row list seen as one head, or the head itself
-template <bool SR>
-__device__ __forceinline__ void q_coords(const TcFwdParams &p, int r, int g, int &c1, int &c2)
+template <bool ANY, class Params>
+__device__ __forceinline__ void q_coords(const Params &p, int r, int g, int &c1, int &c2)
 {
     c1 = r;
     c2 = g;
-    if (SR && p.head_box) {
+    if (ANY && p.box.head_box) {
         const int h = p.fd_S.div(r);
-        c1 = r - h * p.Sh;
+        c1 = r - h * p.box.Sh;
         c2 = g * p.n_rep + h;
     }
 }
 
 // rows held (and MMA N used) by prefix block k
-__device__ __forceinline__ int prefix_block_rows(const TcFwdParams &p, int k)
+template <class Params>
+__device__ __forceinline__ int prefix_block_rows(const Params &p, int k)
 {
     return k == p.nblk_p - 1 ? p.tail_rows : kBlockN;
 }
@@ -156,27 +171,31 @@ static_assert(kBlockN == 4 * kPiece, "two softmax groups x two pieces cover a sc
 
 // Suffix-ring mode: candidates [first, first + count) of a tile that suffix block j holds, and the
 // MMA N (rows rounded up to 16) of that block.
-__device__ __forceinline__ int sfx_block_cands(const TcFwdParams &p, int nc, int j)
+template <class Params>
+__device__ __forceinline__ int sfx_block_cands(const Params &p, int nc, int j)
 {
     return min(p.cpb, nc - j * p.cpb);
 }
-__device__ __forceinline__ int sfx_block_rows(const TcFwdParams &p, int nc, int j)
+template <class Params>
+__device__ __forceinline__ int sfx_block_rows(const Params &p, int nc, int j)
 {
     return (sfx_block_cands(p, nc, j) * p.Spad + 15) & ~15;
 }
 
 // Suffix-ring mode with long suffixes: the tile's rows belong to one candidate; it needs that
 // candidate's suffix keys up to the last one any of its rows may see, in blocks of 128.
-__device__ __forceinline__ int sfx_blocks_long(const TcFwdParams &p, const TileInfo &t)
+template <bool ANY, class Params>
+__device__ __forceinline__ int sfx_blocks_long(const Params &p, const TileInfo &t)
 {
     const int r0 = t.R0 - t.b_first * p.Rg;
-    const int s0 = r0 - p.fd_S.div(r0) * p.Sh;  // query index of the tile's first row
+    const int s0 = r0 - p.fd_S.div(r0) * (ANY ? p.box.Sh : p.S);  // query index of the tile's first row
     const int s_max = (s0 + t.rows > p.S) ? p.S - 1 : s0 + t.rows - 1;  // rows wrap into the next head
     const int pos = suffix_tokens(p.suffix_len, t.b_first, p.S, p.Skv) - p.S + s_max;
     return (pos >> 7) + 1;
 }
 // MMA N of long-suffix block j (its 128-row box is zero-filled past the end of the cache)
-__device__ __forceinline__ int sfx_long_rows(const TcFwdParams &p, int j)
+template <class Params>
+__device__ __forceinline__ int sfx_long_rows(const Params &p, int j)
 {
     return min(kBlockN, (p.Skv - j * kBlockN + 15) & ~15);
 }
@@ -185,27 +204,32 @@ __device__ __forceinline__ int sfx_long_rows(const TcFwdParams &p, int j)
 // and the suffix keys of a tile sit in one block with buffers of its own; MODE 2 (suffix-ring): a
 // tile is a run of whole candidates and their suffix keys follow the prefix through the same rings
 // in as many blocks as it takes -- the mode of the decode-shaped operator, where a 128-row tile
-// spans many candidates, and of full-suffix shapes the other two modes cannot tile.  A compile-time
-// switch so that each launch carries only the code of its own mode.
+// spans many candidates, and of full-suffix shapes the other two modes cannot tile; MODE 3: the same with tiles that
+// straddle candidates or lie inside a head whose rows are padded to whole tiles.  A compile-time
+// switch so that each launch carries only the code of its own mode (with MODE 3's decisions taken at run time in MODE 2, 729
+// beams, 32/32 heads, 4 tokens over 147 cached ones took 644 us instead of 572).
+// MI 1: several instructions, each a whole number of tiles; 2: the last tile of each is short.  Apart because a tile's
+// place is worked out by every role (8 x 64 candidates, 32/8 heads, P = 256, S = 48: 139 us with the second's division, 132).
 //
-// TWO (suffix-ring): probabilities as the sum of two bf16 values, the second in the half of a piece that the first leaves free, and
+// TWO (MODE 3): probabilities as the sum of two bf16 values, the second in the half of a piece that the first leaves free, and
 // a value contraction over each.  For the lengths that came from the CUDA-core kernel (two_terms in plan_suffix_ring), whose
 // probabilities are fp32.  Distance (2-norm) of `out` from 64 bits, a prompt of 1039 tokens, 32/8 heads: CUDA cores 1.625e-3,
 // one term 2.310e-3, two terms 1.625e-3 (the rounding of the result); of lse 4.9e-8, 7.6e-8 and, with the logarithm in 64
 // bits, 4.1e-8 (131 tokens: 4.8e-8, 8.0e-8 and 5.4e-8: what is left is the tensor cores' fp32 sum of a score; one rounding of
 // the result is 2.7e-8).  Price: 131 tokens 8.7 -> 9.0 us, 1039 21.0 -> 24.0, 4093 131 -> 170 (CUDA cores 52 us, 1.58 and
 // 22.2 ms).
-template <int D, int MODE, bool MI, bool TWO = false>
+template <int D, int MODE, int MI, bool TWO = false>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_out,
               const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
               const __grid_constant__ CUtensorMap tm_pk_tail, const __grid_constant__ CUtensorMap tm_pv_tail,
               const __grid_constant__ CUtensorMap tm_sk, const __grid_constant__ CUtensorMap tm_sv,
-              const TcFwdParams p)
+              const TcFwdParams<MI> p)
 {
     using C = Cfg<D>;
     constexpr bool RES = MODE == 1;
-    constexpr bool SR = MODE == 2;
+    constexpr bool SR = MODE >= 2, ANY = MODE == 3;
+    constexpr bool PAD = MODE != 2;  // a candidate's rows may be followed by rows that do not exist
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
@@ -264,7 +288,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int t_begin = (int)((long long)blockIdx.x * p.total_tiles / gridDim.x);
     const int t_end = (int)((long long)(blockIdx.x + 1) * p.total_tiles / gridDim.x);
     const int G = (int)gridDim.x;
-    const int n_sp = (SR && p.deal_by_cost) ? p.Sh / p.tile_rows : 1;  // tiles per head
+    const int Sh = ANY ? p.box.Sh : p.S;
+    const int n_sp = (SR && p.deal_by_cost) ? Sh / p.tile_rows : 1;  // tiles per head
     const bool dealt = n_sp > 1;
     auto rank_at = [&](int tl) { return tl * G + ((tl & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
     auto tile_at = [&](int tl) {
@@ -280,7 +305,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int n_tiles = !dealt ? t_end - t_begin : (n_rounds - 1) + (rank_at(n_rounds - 1) < p.total_tiles ? 1 : 0);
     // items of a tile: prefix blocks + the suffix block(s)
     auto items_of = [&](const TileInfo &t) {
-        return p.nblk_p + (!SR ? 1 : p.long_sfx ? sfx_blocks_long(p, t) : p.fd_cpb.div(t.nc + p.cpb - 1));
+        return p.nblk_p + (!SR ? 1 : p.long_sfx ? sfx_blocks_long<ANY>(p, t) : p.fd_cpb.div(t.nc + p.cpb - 1));
     };
     // A run of tiles that shares one prefix: a KV head, or (several instructions) one instruction's
     // candidates inside a KV head.  Runs are numbered in tile order; the resident prefix is reloaded at the
@@ -295,7 +320,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     auto first_block = [&](int inst) { return MI ? p.pad[inst] / kBlockN : 0; };
     int run_first;
     {
-        const TileInfo t0 = tile_info<MI>(p, t_begin < p.total_tiles ? t_begin : 0, t_begin);
+        const TileInfo t0 = tile_info<MI == 2>(p, t_begin < p.total_tiles ? t_begin : 0, t_begin);
         run_first = run_of(t0, inst_of(t0));
     }
     const int sfx_slab = p.sfx_rows * 128;
@@ -316,13 +341,13 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         bool ok = true;
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info<MI>(p, tile_at(tl), t_begin);
+            const TileInfo t = tile_info<MI == 2>(p, tile_at(tl), t_begin);
             // Everything the Q loads need is worked out before the wait, so that only the copy
             // instructions themselves follow it: the Q buffer is single, and the time from "last
             // score MMA of the previous tile done" to "Q of this tile requested" is exposed.
             // (Suffix-ring mode: one box per slab holds the tile's whole candidates; a box reaching
             // past the last candidate is filled with zeros and still counts its full size.)
-            const int nseg = (SR && p.one_box) ? 1 : p.fd_seg.div(t.rows);  // one box per run of seg_rows rows
+            const int nseg = (SR && (!ANY || p.box.one_box)) ? 1 : p.fd_seg.div(t.rows);  // one box per run of seg_rows rows
             int qb = p.fd_Rg.div(t.R0), qr = t.R0 - qb * p.Rg;
             const uint32_t q_bytes = (uint32_t)(nseg * C::kSlabs * p.seg_rows * 128);
             const uint32_t seg_bytes = (uint32_t)(p.seg_rows * 128);
@@ -337,7 +362,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll 1
                 for (int s = 0; s < nseg; ++s) {
                     int c1, c2;
-                    q_coords<SR>(p, qr, t.g, c1, c2);
+                    q_coords<ANY>(p, qr, t.g, c1, c2);
 #pragma unroll
                     for (int sl = 0; sl < C::kSlabs; ++sl)
                         tma_load_4d(q_dst + sl * C::kSlabBytes, &tm_q, bar(kBarQFull), sl * 64, c1, c2, qb);
@@ -439,14 +464,14 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // Ask for the NEXT tile's Q in L2: its load can only be issued a tile from now, right when it is needed,
             // and then finds the data close by.  (Behind this tile's copies: the first ones of a launch are waited for.)
             if (tl + 1 < n_tiles) {
-                const TileInfo tn = tile_info<MI>(p, tile_at(tl + 1), t_begin);
-                const int nseg_n = (SR && p.one_box) ? 1 : p.fd_seg.div(tn.rows);
+                const TileInfo tn = tile_info<MI == 2>(p, tile_at(tl + 1), t_begin);
+                const int nseg_n = (SR && (!ANY || p.box.one_box)) ? 1 : p.fd_seg.div(tn.rows);
                 int nb = p.fd_Rg.div(tn.R0), nr = tn.R0 - nb * p.Rg;
                 if (elect_one_sync()) {
 #pragma unroll 1
                     for (int s = 0; s < nseg_n; ++s) {
                         int c1, c2;
-                        q_coords<SR>(p, nr, tn.g, c1, c2);
+                        q_coords<ANY>(p, nr, tn.g, c1, c2);
 #pragma unroll
                         for (int sl = 0; sl < C::kSlabs; ++sl) tma_prefetch_4d(&tm_q, sl * 64, c1, c2, nb);
                         nr += p.seg_rows;
@@ -486,7 +511,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             int ph = 0;  // head index inside the prefix caches
             int kfirst = 0;
             if (have_tile) {
-                t = tile_info<MI>(p, tile_at(tl), t_begin);
+                t = tile_info<MI == 2>(p, tile_at(tl), t_begin);
                 const int inst = inst_of(t);
                 ph = inst * p.Hkv + t.g;
                 kfirst = first_block(inst);
@@ -581,8 +606,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         ready = __shfl_sync(0xffffffffu, mbar_try_wait(bar(kBarStageFull), round & 1) ? 1 : 0, 0) != 0;
                     if (!ok) break;
                     if (ready) {
-                        const TileInfo u = tile_info<MI>(p, tile_at(tl - 1), t_begin);
-                        const int nseg = (SR && p.one_box) ? 1 : p.fd_seg.div(u.rows);
+                        const TileInfo u = tile_info<MI == 2>(p, tile_at(tl - 1), t_begin);
+                        const int nseg = (SR && (!ANY || p.box.one_box)) ? 1 : p.fd_seg.div(u.rows);
                         const int sl_first = p.slab_stage ? store_slab : 0;
                         const int sl_end = p.slab_stage ? store_slab + 1 : C::kSlabs;
                         if (elect_one_sync()) {
@@ -592,9 +617,9 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                                 for (int s = 0; s < nseg; ++s) {
                                     const int R = u.R0 + s * p.seg_rows;
                                     const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-                                    if (r >= p.Rr) continue;  // padding only
+                                    if (PAD && r >= p.Rr) continue;  // padding only
                                     int c1, c2;
-                                    q_coords<SR>(p, r, u.g, c1, c2);
+                                    q_coords<ANY>(p, r, u.g, c1, c2);
                                     tma_store_4d(&tm_out, stage + (p.slab_stage ? 0 : sl) * kStagingBytes + s * p.seg_rows * 128,
                                                  sl * 64, c1, c2, b);
                                 }
@@ -635,7 +660,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         // ------------------------------------------------------------------ score MMAs: S = Q K^T
         int tl = 0;
         uint32_t kuse = 0;  // streaming mode: K blocks consumed from the ring
-        TileInfo t = tile_info<MI>(p, tile_at(0), t_begin);
+        TileInfo t = tile_info<MI == 2>(p, tile_at(0), t_begin);
         int nitems = items_of(t);
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint64_t q_desc = make_smem_desc(sbase + p.off_q, 0, 1024);
@@ -718,7 +743,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
-                    t = tile_info<MI>(p, tile_at(tl), t_begin);
+                    t = tile_info<MI == 2>(p, tile_at(tl), t_begin);
                     nitems = items_of(t);
                     k = kfirst = first_block(inst_of(t));
                 }
@@ -728,7 +753,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         // ------------------------------------------------------------------ value MMAs: O += P V
         int tl = 0;
         uint32_t vuse = 0;
-        TileInfo t = tile_info<MI>(p, tile_at(0), t_begin);
+        TileInfo t = tile_info<MI == 2>(p, tile_at(0), t_begin);
         int nitems = items_of(t);
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint32_t idesc_pv = make_idesc_bf16(kTileM, D, 1);
@@ -813,7 +838,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
-                    t = tile_info<MI>(p, tile_at(tl), t_begin);
+                    t = tile_info<MI == 2>(p, tile_at(tl), t_begin);
                     nitems = items_of(t);
                     k = kfirst = first_block(inst_of(t));
                 }
@@ -841,15 +866,15 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int item = 0;  // items handled so far
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles && ok; ++tl) {
-            const TileInfo t = tile_info<MI>(p, tile_at(tl), t_begin);
+            const TileInfo t = tile_info<MI == 2>(p, tile_at(tl), t_begin);
             const int nitems = items_of(t);
             int lo_sfx = 1, hi_sfx = 0;
             int k_own = p.nblk_p;  // suffix-ring mode: the item that holds this row's candidate
             if (row < t.rows) {
                 const int R = t.R0 + row;
                 const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-                const int i = r - p.fd_S.div(r) * p.Sh;  // query index inside the candidate
-                if (r >= p.Rr || (SR && i >= p.S)) {
+                const int i = r - p.fd_S.div(r) * Sh;  // query index inside the candidate
+                if ((PAD && r >= p.Rr) || (ANY && i >= p.S)) {
                     // a padding row between two candidates: sees no suffix key, is never stored
                 } else if (SR) {
                     // query i is suffix token L - S + i of its candidate: suffix keys 0 .. L - S + i
@@ -992,7 +1017,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         bool ok = true;
 #pragma unroll 1
         for (int te = 0; te < n_tiles && ok; ++te) {
-            const TileInfo u = tile_info<MI>(p, tile_at(te), t_begin);
+            const TileInfo u = tile_info<MI == 2>(p, tile_at(te), t_begin);
             ok = mbar_wait_warp(bar(kBarOFull), te & 1, abort_flag, p.status, kErrEpilogue);
             if (!ok) break;
             PSKV_TRACE_EVENT(30, te);
@@ -1101,8 +1126,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             }
             const int R = u.R0 + row;
             const int b = p.fd_Rg.div(R), r = R - b * p.Rg;
-            const int hd = SR ? p.fd_S.div(r) : 0, skip = hd * (p.Sh - p.S);  // (head_box: padding rows before this head)
-            const bool stored = row < u.rows && r < p.Rr && (!SR || r - hd * p.Sh < p.S);
+            const int hd = ANY ? p.fd_S.div(r) : 0, skip = ANY ? hd * (p.box.Sh - p.S) : 0;  // (head_box: padding rows before this head)
+            const bool stored = row < u.rows && (!PAD || r < p.Rr) && (!ANY || r - hd * p.box.Sh < p.S);
             if (stored) {
                 const size_t grow = ((size_t)b * p.Hq + (size_t)u.g * p.n_rep) * p.S + r - skip;
                 // (log2f is good to 2^-22 absolute, more than the CUDA-core kernel loses, whose sum is relative to the maximum)
@@ -1128,14 +1153,14 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         float *q_s = reinterpret_cast<float *>(smem) + warp * D;
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles; ++tl) {
-            const TileInfo t = tile_info<MI>(p, tile_at(tl), t_begin);
+            const TileInfo t = tile_info<MI == 2>(p, tile_at(tl), t_begin);
 #pragma unroll 1
             for (int r = warp; r < t.rows; r += kThreads / 32) {
                 const int R = t.R0 + r;
                 const int b = p.fd_Rg.div(R), rr = R - b * p.Rg;
-                const int hd = SR ? p.fd_S.div(rr) : 0;
-                if (rr >= p.Rr || (SR && rr - hd * p.Sh >= p.S)) continue;
-                const long long grow = ((long long)b * p.Hq + (long long)t.g * p.n_rep) * p.S + rr - hd * (p.Sh - p.S);
+                const int hd = ANY ? p.fd_S.div(rr) : 0;
+                if ((PAD && rr >= p.Rr) || (ANY && rr - hd * p.box.Sh >= p.S)) continue;
+                const long long grow = ((long long)b * p.Hq + (long long)t.g * p.n_rep) * p.S + rr - (ANY ? hd * (p.box.Sh - p.S) : 0);
                 const float v = p.lse[grow];
                 if (v != v) {
                     if (MI) {  // the row's own prefix cache, without its left padding
@@ -1159,7 +1184,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 
 struct TilePlan {
     bool ok;
-    int mode;   // kernel template MODE: 0 rings, 1 resident prefix, 2 suffix-ring
+    int mode;   // kernel template MODE: 0 rings, 1 resident prefix, 2 suffix-ring, 3 suffix-ring with any row list
     int cbox, Spad, cpb;  // suffix-ring mode: candidates per tile, rows per candidate in a block, candidates per block
     int long_sfx;         // suffix-ring mode: tiles inside one candidate, its suffix keys in 128-key blocks
     int two_terms;        // suffix-ring mode: probabilities as two bf16 terms
@@ -1268,10 +1293,14 @@ TilePlan plan_suffix_ring(const Dims &dm)
         if (!rows && Rg <= kTileM) rows = Rg;
         pl.two_terms = !rows;
         const int per_head = (dm.S + kTileM - 1) / kTileM;
-        if (dm.S > kTileM && (!rows || (long long)dm.n_rep * per_head <= Rg / rows)) {
+        const long long head_tiles = (long long)dm.n_rep * per_head;
+        if (dm.S > kTileM && (!rows || head_tiles < Rg / rows || (head_tiles == Rg / rows && dm.S % rows != 0))) {
             rows = round_up((dm.S + per_head - 1) / per_head, 8);
-            pl.head_box = 1;
-            pl.Sh = rows * per_head;
+            if (dm.S % rows != 0) {
+                pl.mode = 3;
+                pl.head_box = 1;
+                pl.Sh = rows * per_head;
+            }
         }
         if (!rows) return pl;  // no usable divisor: the general kernels take the shape
         pl.Rp = pl.head_box ? dm.n_rep * pl.Sh : Rg;
@@ -1391,7 +1420,7 @@ TilePlan plan_straddle(const Dims &dm)
     memset(&pl, 0, sizeof(pl));
     int nc = 0;
     if (!pick_tile_rows(dm, true, &pl, &nc)) return pl;
-    pl.mode = 2;
+    pl.mode = 3;
     pl.Spad = pl.Sp;
     pl.cpb = kBlockN / pl.Sp;
     pl.cbox = 1;
@@ -1449,7 +1478,7 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
             dims[1] = (cuuint64_t)dm.S;
             dims[2] = (cuuint64_t)dm.Hq;
             str[1] = (cuuint64_t)dm.S * D * 2;
-        } else if (plan.mode == 2 && plan.one_box) {  // one box = the whole candidates of a tile, or the tile's rows of one candidate
+        } else if (plan.mode >= 2 && plan.one_box) {  // one box = the whole candidates of a tile, or the tile's rows of one candidate
             box[1] = (cuuint32_t)(plan.long_sfx ? plan.tile_rows : Rg);
             box[3] = (cuuint32_t)plan.cbox;
         }
@@ -1459,7 +1488,7 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
     {
         cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)dm.Skv, (cuuint64_t)dm.Hkv, (cuuint64_t)dm.B};
         cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)dm.Skv * D * 2, (cuuint64_t)dm.Hkv * dm.Skv * D * 2};
-        cuuint32_t box[4] = {64, (cuuint32_t)(plan.long_sfx ? kBlockN : plan.mode == 2 ? dm.Skv : plan.Sp), 1, 1};
+        cuuint32_t box[4] = {64, (cuuint32_t)(plan.long_sfx ? kBlockN : plan.mode >= 2 ? dm.Skv : plan.Sp), 1, 1};
         if (!encode_map(&tm_sk, a.suffix_k, 4, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_sv, a.suffix_v, 4, dims, str, box)) return cudaErrorInvalidValue;
     }
@@ -1473,77 +1502,84 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
         if (!encode_map(&tm_pk_tail, a.prefix_k, 3, dims, str, box_tail)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_pv_tail, a.prefix_v, 3, dims, str, box_tail)) return cudaErrorInvalidValue;
     }
-    TcFwdParams p;
-    p.lse = a.lse;
-    p.status = status_word;
-    p.args = a;
-    p.sl2 = a.scale * kLog2e;
-    p.B = dm.B; p.Hq = dm.Hq; p.Hkv = dm.Hkv; p.S = dm.S; p.P = dm.P; p.n_rep = dm.n_rep;
-    p.Rg = plan.Rp;
-    p.Sh = plan.head_box ? plan.Sh : dm.S;
-    p.Rr = dm.n_rep * p.Sh;
-    p.one_box = plan.one_box;
-    p.head_box = plan.head_box;
-    p.Sp = plan.mode == 2 ? dm.S : plan.Sp;
-    p.tile_rows = plan.tile_rows;
-    p.seg_rows = plan.seg_rows;
-    p.fd_Rg.init(p.Rg);
-    p.fd_S.init(p.Sh);
-    p.fd_seg.init(plan.seg_rows);
-    p.nblk_p = plan.nblk_p;
-    p.tail_rows = plan.tail_rows;
-    p.resident = plan.resident;
-    p.stages = plan.stages > 0 ? plan.stages : 1;
-    p.sfx_rows = plan.sfx_rows;
-    p.alias_stage = plan.alias_stage;
-    p.slab_stage = plan.slab_stage;
-    p.ml_mask = plan.ml_tiles == 1 ? 0 : 3;
-    p.suffix_len = a.suffix_len;
-    p.Skv = dm.Skv;
-    p.Spad = plan.Spad > 0 ? plan.Spad : 8;
-    p.cpb = plan.cpb > 0 ? plan.cpb : 1;
-    p.fd_cpb.init(p.cpb);
-    p.long_sfx = plan.long_sfx;
-    p.n_instr = n_instr;
-    p.rpi = dm.B / n_instr * p.Rg;
-    p.fd_rpi.init(p.rpi > 0 ? p.rpi : 1);
-    p.tpi = n_instr > 1 ? (p.rpi + plan.tile_rows - 1) / plan.tile_rows : plan.tiles_per_group;
-    p.fd_tpi.init(p.tpi);
-    p.tiles_per_group = p.tpi * n_instr;
-    p.fd_tpg.init(p.tiles_per_group);
-    p.total_tiles = p.tiles_per_group * dm.Hkv;
-    for (int i = 0; i < kMaxInstr; ++i) p.pad[i] = (n_instr > 1 && i < n_instr) ? dm.P - prefix_len[i] : 0;
-    // Dealing by cost balances the causal skew but lets every CTA touch every candidate's suffix K/V
-    // at several times; it pays when those tensors stay in L2 between the touches.
-    p.deal_by_cost = plan.long_sfx && p.Sh % plan.tile_rows == 0 && p.Sh / plan.tile_rows > 1 &&
-                     4.0 * dm.B * dm.Hkv * dm.Skv * D <= 48.0e6;
-    p.off_pk = plan.off_pk; p.off_pv = plan.off_pv; p.off_q = plan.off_q; p.off_sk = plan.off_sk;
-    p.off_sv = plan.off_sv; p.off_stage = plan.off_stage; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
-    p.off_ml = plan.off_ml;
-    // The MMAs read keys in steps of 16: candidates that take a multiple of 16 leave no row of a block unwritten, and
-    // the boxes of prefix and long-suffix blocks are whole blocks, filled with zeros past the end.
-    p.zero_lo = p.zero_hi = 0;
-    if (plan.mode == 2) {
-        if (!plan.long_sfx && dm.Skv % 16 != 0) p.zero_lo = plan.off_pv, p.zero_hi = plan.off_q;
-    } else if (plan.Sp % 16 != 0) {
-        p.zero_lo = plan.off_sv, p.zero_hi = plan.off_sv + D / 64 * plan.sfx_rows * 128;
-    }
+    // one instantiation: its parameters and its launch
+    auto run = [&](auto kernel, auto &&p, int slot) {
+        p.lse = a.lse;
+        p.status = status_word;
+        p.args = a;
+        p.sl2 = a.scale * kLog2e;
+        p.B = dm.B; p.Hq = dm.Hq; p.Hkv = dm.Hkv; p.S = dm.S; p.P = dm.P; p.n_rep = dm.n_rep;
+        p.Rg = plan.Rp;
+        p.box.Sh = plan.head_box ? plan.Sh : dm.S;
+        p.Rr = dm.n_rep * p.box.Sh;
+        p.box.one_box = plan.one_box;
+        p.box.head_box = plan.head_box;
+        p.Sp = plan.mode >= 2 ? dm.S : plan.Sp;
+        p.tile_rows = plan.tile_rows;
+        p.seg_rows = plan.seg_rows;
+        p.fd_Rg.init(p.Rg);
+        p.fd_S.init(p.box.Sh);
+        p.fd_seg.init(plan.seg_rows);
+        p.nblk_p = plan.nblk_p;
+        p.tail_rows = plan.tail_rows;
+        p.resident = plan.resident;
+        p.stages = plan.stages > 0 ? plan.stages : 1;
+        p.sfx_rows = plan.sfx_rows;
+        p.alias_stage = plan.alias_stage;
+        p.slab_stage = plan.slab_stage;
+        p.ml_mask = plan.ml_tiles == 1 ? 0 : 3;
+        p.suffix_len = a.suffix_len;
+        p.Skv = dm.Skv;
+        p.Spad = plan.Spad > 0 ? plan.Spad : 8;
+        p.cpb = plan.cpb > 0 ? plan.cpb : 1;
+        p.fd_cpb.init(p.cpb);
+        p.long_sfx = plan.long_sfx;
+        p.n_instr = n_instr;
+        p.rpi = dm.B / n_instr * p.Rg;
+        p.fd_rpi.init(p.rpi > 0 ? p.rpi : 1);
+        p.tpi = n_instr > 1 ? (p.rpi + plan.tile_rows - 1) / plan.tile_rows : plan.tiles_per_group;
+        p.fd_tpi.init(p.tpi);
+        p.tiles_per_group = p.tpi * n_instr;
+        p.fd_tpg.init(p.tiles_per_group);
+        p.total_tiles = p.tiles_per_group * dm.Hkv;
+        for (int i = 0; i < kMaxInstr; ++i) p.pad[i] = (n_instr > 1 && i < n_instr) ? dm.P - prefix_len[i] : 0;
+        // Dealing by cost balances the causal skew but lets every CTA touch every candidate's suffix K/V
+        // at several times; it pays when those tensors stay in L2 between the touches.
+        p.deal_by_cost = plan.long_sfx && p.box.Sh % plan.tile_rows == 0 && p.box.Sh / plan.tile_rows > 1 &&
+                         4.0 * dm.B * dm.Hkv * dm.Skv * D <= 48.0e6;
+        p.off_pk = plan.off_pk; p.off_pv = plan.off_pv; p.off_q = plan.off_q; p.off_sk = plan.off_sk;
+        p.off_sv = plan.off_sv; p.off_stage = plan.off_stage; p.off_bar = plan.off_bar; p.off_misc = plan.off_misc;
+        p.off_ml = plan.off_ml;
+        // The MMAs read keys in steps of 16: candidates that take a multiple of 16 leave no row of a block unwritten, and
+        // the boxes of prefix and long-suffix blocks are whole blocks, filled with zeros past the end.
+        p.zero_lo = p.zero_hi = 0;
+        if (plan.mode >= 2) {
+            if (!plan.long_sfx && dm.Skv % 16 != 0) p.zero_lo = plan.off_pv, p.zero_hi = plan.off_q;
+        } else if (plan.Sp % 16 != 0) {
+            p.zero_lo = plan.off_sv, p.zero_hi = plan.off_sv + D / 64 * plan.sfx_rows * 128;
+        }
 
-    const bool mi = n_instr > 1;  // (never with the suffix-ring tiling)
-    auto kernel = plan.mode == 2 ? (plan.two_terms ? tc_fwd_kernel<D, 2, false, true> : tc_fwd_kernel<D, 2, false>)
-                  : plan.mode == 1 ? (mi ? tc_fwd_kernel<D, 1, true> : tc_fwd_kernel<D, 1, false>)
-                                   : (mi ? tc_fwd_kernel<D, 0, true> : tc_fwd_kernel<D, 0, false>);
-    static PerDeviceOnce attr_set[7];
-    if (cudaError_t e = ensure_max_smem(kernel, attr_set[plan.two_terms ? 6 : plan.mode + (mi ? 3 : 0)]); e != cudaSuccess) return e;
-    const int grid = even_grid(p.total_tiles, sm_count());
-    cudaError_t launch_err;
-    {
-        KernelTiming timing(kKernelFwdTc, stream);
-        launch_err = launch_dependent(kernel, grid, kThreads, plan.smem_bytes, stream, tm_q, tm_out, tm_pk, tm_pv, tm_pk_tail,
-                                      tm_pv_tail, tm_sk, tm_sv, p);
+        static PerDeviceOnce attr_set[9];
+        if (cudaError_t e = ensure_max_smem(kernel, attr_set[slot]); e != cudaSuccess) return e;
+        const int grid = even_grid(p.total_tiles, sm_count());
+        cudaError_t launch_err;
+        {
+            KernelTiming timing(kKernelFwdTc, stream);
+            launch_err = launch_dependent(kernel, grid, kThreads, plan.smem_bytes, stream, tm_q, tm_out, tm_pk, tm_pv, tm_pk_tail,
+                                          tm_pv_tail, tm_sk, tm_sv, p);
+        }
+        count_launches(1);
+        return launch_err != cudaSuccess ? launch_err : cudaGetLastError();
+    };
+    if (n_instr > 1) {  // (never with the suffix-ring tiling) whole tiles of every instruction, or the last one of each short
+        const bool whole = (long long)(dm.B / n_instr) * plan.Rp % plan.tile_rows == 0;
+        if (whole) return plan.mode == 1 ? run(tc_fwd_kernel<D, 1, 1>, TcFwdParams<1>(), 4) : run(tc_fwd_kernel<D, 0, 1>, TcFwdParams<1>(), 5);
+        return plan.mode == 1 ? run(tc_fwd_kernel<D, 1, 2>, TcFwdParams<2>(), 6) : run(tc_fwd_kernel<D, 0, 2>, TcFwdParams<2>(), 7);
     }
-    count_launches(1);
-    return launch_err != cudaSuccess ? launch_err : cudaGetLastError();
+    if (plan.mode == 3 && plan.two_terms) return run(tc_fwd_kernel<D, 3, 0, true>, TcFwdParams<0>(), 8);
+    return run(plan.mode == 3 ? tc_fwd_kernel<D, 3, 0> : plan.mode == 2 ? tc_fwd_kernel<D, 2, 0> : plan.mode == 1 ? tc_fwd_kernel<D, 1, 0>
+                                                                                                             : tc_fwd_kernel<D, 0, 0>,
+               TcFwdParams<0>(), plan.mode);
 }
 
 }  // namespace
@@ -1589,7 +1625,7 @@ bool tc_fwd_fused_supported(const Dims &dm, int n_instr)
         return false;
     const TilePlan &pl = plan_tiles(dm, n_instr);
     const long long rows = (long long)(dm.B / n_instr) * pl.Rp;
-    return pl.ok && pl.mode != 2 && (rows % pl.tile_rows == 0 || rows >= 4 * pl.tile_rows) &&
+    return pl.ok && pl.mode < 2 && (rows % pl.tile_rows == 0 || rows >= 4 * pl.tile_rows) &&
            (rows / pl.tile_rows + 1) * n_instr * dm.Hkv <= 2000000000ll;
 }
 
