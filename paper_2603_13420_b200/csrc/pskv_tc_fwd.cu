@@ -1428,13 +1428,22 @@ TilePlan plan_straddle(const Dims &dm)
     return pl;
 }
 
+// Estimated cycles of the SM with the most tiles.
+double busiest(const Dims &dm, const TilePlan &pl)
+{
+    const long long sms = sm_count(), tiles = (long long)pl.tiles_per_group * dm.Hkv;
+    return (double)((tiles + sms - 1) / sms) * pl.cost / pl.tiles_per_group;
+}
+
 // The full-suffix operator takes the tiling with the suffix in one block unless another one is clearly cheaper: tiles
 // that straddle candidates, or, for groups of a few rows, whole candidates without padding (one row per candidate and
 // head padded to 8 would be an eighth of the tile).  The decode-shaped operator and suffixes beyond one block are the
 // suffix-ring mode's.  Straddling tiles fetch the prefix for every tile, so they have to be cheaper by 40 % by count of
 // blocks where it would stay resident (B = 74, 32/8 heads, P = 256, S = 75: 57 us instead of 49 at a count 12 %
 // lower), by 8 % where it is streamed either way (B = 58, 32/32, P = 1735, S = 66 221 -> 168 us; B = 66, 32/8, P = 803,
-// S = 109 152 -> 145).
+// S = 109 152 -> 145), on the whole and on the SM with the most tiles: fewer tiles gain nothing where they take as many rounds
+// (B = 65, 4/4, P = 1183, S = 81 33.3 us straddling, 25.6 not; B = 35, 8/2, P = 315, S = 67 16.7 and 12.8), and a round less
+// is not enough by itself (B = 23, 8/8, P = 365, S = 84 13.8 and 13.2).
 TilePlan make_plan(const Dims &dm, int n_instr)
 {
     if (dm.Skv == dm.S && !dm.ragged) {
@@ -1446,7 +1455,8 @@ TilePlan make_plan(const Dims &dm, int n_instr)
         }
         if (pl.ok) {
             const TilePlan ring = plan_straddle(dm);
-            return ring.ok && (pl.resident ? 1.4 : 1.08) * ring.cost < pl.cost ? ring : pl;
+            const double margin = pl.resident ? 1.4 : 1.08;
+            return ring.ok && margin * ring.cost < pl.cost && margin * busiest(dm, ring) < busiest(dm, pl) ? ring : pl;
         }
     }
     return plan_suffix_ring(dm);
