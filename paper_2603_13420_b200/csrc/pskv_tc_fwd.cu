@@ -1196,10 +1196,11 @@ struct TilePlan {
     int off_pk, off_pv, off_q, off_sk, off_sv, off_stage, off_bar, off_misc, off_ml, smem_bytes;
 };
 
-// Cycles of a tile, for the choice of a tiling: about 2 000 per key block, 1 700 for the tile itself, and 60 per
-// box of Q and of `out` (one thread issues them; with sixteen boxes of 8 rows that is 1 000 cycles in which the
-// single Q buffer is waited for).
-double tile_cost(double blocks, int boxes) { return 2000.0 * blocks + 1700.0 + 60.0 * boxes; }
+// Cycles of a tile, for the choice of a tiling: about 2 000 per key block, 1 700 for the tile itself, and 100 per
+// 64-column slab of a box of Q and of `out`: one thread asks for the next tile's boxes, fetches and stores them, and the single Q
+// buffer is waited for (448 tiles of one box, 28 candidates, 32/8 heads, P = 190, S = 61, 15.8 us; 440 of sixteen 17.2; 262
+// candidates, 4/4 heads, P = 20, S = 8 8.3 us in 68 tiles of sixteen boxes, 6.7 in 132 of eight).
+double tile_cost(double blocks, double slabs) { return 2000.0 * blocks + 1700.0 + 100.0 * slabs; }
 
 // Rows a candidate takes in the row list (Rp >= n_rep * S) and rows per tile, both multiples of 8, such that the
 // suffix keys of all candidates a tile can touch (Sp columns each) fit one 128-key block.  Suffix lengths are
@@ -1212,15 +1213,26 @@ double tile_cost(double blocks, int boxes) { return 2000.0 * blocks + 1700.0 + 6
 // of 112, instead of four of 80) 101 -> 82.
 //
 // ring: the suffix keys come in several blocks through the K / V rings, so a tile may touch any number of candidates.
-bool pick_tile_rows(const Dims &dm, bool ring, TilePlan *pl, int *nc_max)
+// several: tiles for several instructions in one launch, where an instruction had better be whole tiles: the sum over all
+// tiles decides, and boxes count less.
+bool pick_tile_rows(const Dims &dm, bool ring, bool several, TilePlan *pl, int *nc_max)
 {
     const int Sp = round_up(dm.S, 8);
     if (Sp > kBlockN) return false;
     const int Rg = dm.n_rep * dm.S, nblk = (dm.P + kBlockN - 1) / kBlockN, cpb = kBlockN / Sp;
+    // The busiest SM's tiles decide, and among equals the sum over all: 133 candidates of 7 heads x 40 rows are 291 tiles of 128
+    // rows in sixteen boxes or 333 of 112 in seven, which is cheaper in sum, but three rounds of the SMs instead of two.
+    const long long sms = sm_count();
+    const double slabs = several ? 0.6 : dm.d / 64;  // of a box
+    auto score = [&](long long tiles, double cycles) {
+        const long long all = tiles * dm.Hkv;
+        if (several) return (double)tiles * cycles;
+        return ((double)((all + sms - 1) / sms) + 0.25 * (double)all / (double)sms) * cycles;
+    };
     double best = -1.0;
     for (int Rp = round_up(Rg, 8); Rp < Rg + kTileM; Rp += 8) {
         if ((long long)dm.B * Rp > 2000000000ll) break;
-        if (best >= 0.0 && (double)(((long long)dm.B * Rp + kTileM - 1) / kTileM) * tile_cost(nblk + 1, 1) >= best) break;
+        if (best >= 0.0 && score(((long long)dm.B * Rp + kTileM - 1) / kTileM, tile_cost(nblk + 1, slabs)) >= best) break;
         for (int m = kTileM; m >= 8; m -= 8) {
             const int seg = gcd_int(Rp, m);
             // candidates that a window of m rows can touch, its offset in a candidate being a multiple of seg
@@ -1230,9 +1242,10 @@ bool pick_tile_rows(const Dims &dm, bool ring, TilePlan *pl, int *nc_max)
             const long long tiles = ((long long)dm.B * Rp + m - 1) / m;
             // suffix blocks of a tile: one, or (ring) one and a share for each candidate it touches beyond the first
             const double sfx = ring ? 1.0 + (double)(m - seg) / Rp / cpb : 1.0;
-            const double cost = (double)tiles * tile_cost(nblk + sfx, m / seg);
-            if (best < 0.0 || cost < best) {
-                best = cost;
+            const double cycles = tile_cost(nblk + sfx, slabs * (m / seg)), sc = score(tiles, cycles);
+            if (best < 0.0 || sc < best) {
+                best = sc;
+                pl->cost = (double)tiles * cycles;
                 pl->Rp = Rp;
                 pl->tile_rows = m;
                 pl->seg_rows = seg;
@@ -1243,7 +1256,6 @@ bool pick_tile_rows(const Dims &dm, bool ring, TilePlan *pl, int *nc_max)
     }
     if (best < 0.0) return false;
     pl->Sp = Sp;
-    pl->cost = best;
     return true;
 }
 
@@ -1338,7 +1350,7 @@ TilePlan plan_suffix_ring(const Dims &dm)
         pl.one_box = 1;
         pl.tile_rows = pl.seg_rows = Rg * pl.cbox;
         pl.tiles_per_group = (dm.B + pl.cbox - 1) / pl.cbox;
-        pl.cost = (double)pl.tiles_per_group * tile_cost(nblk + (pl.cbox + pl.cpb - 1) / pl.cpb, 1);
+        pl.cost = (double)pl.tiles_per_group * tile_cost(nblk + (pl.cbox + pl.cpb - 1) / pl.cpb, dm.d / 64);
     }
     layout_ring(dm, &pl);
     return pl;
@@ -1346,12 +1358,12 @@ TilePlan plan_suffix_ring(const Dims &dm)
 
 // Lays out shared memory: all prefix blocks of a KV head if they fit beside the other buffers (resident mode), else
 // rings of 2..4 block stages.
-TilePlan plan_base(const Dims &dm)
+TilePlan plan_base(const Dims &dm, bool several)
 {
     TilePlan pl;
     memset(&pl, 0, sizeof(pl));
     int nc_best = 0;
-    if (!pick_tile_rows(dm, false, &pl, &nc_best)) return pl;
+    if (!pick_tile_rows(dm, false, several, &pl, &nc_best)) return pl;
     pl.sfx_rows = round_up(nc_best * pl.Sp, 16);
     pl.nblk_p = (dm.P + kBlockN - 1) / kBlockN;
     pl.tail_rows = pl.nblk_p ? round_up(dm.P - (pl.nblk_p - 1) * kBlockN, 16) : 0;
@@ -1419,7 +1431,7 @@ TilePlan plan_straddle(const Dims &dm)
     TilePlan pl;
     memset(&pl, 0, sizeof(pl));
     int nc = 0;
-    if (!pick_tile_rows(dm, true, &pl, &nc)) return pl;
+    if (!pick_tile_rows(dm, true, false, &pl, &nc)) return pl;
     pl.mode = 3;
     pl.Spad = pl.Sp;
     pl.cpb = kBlockN / pl.Sp;
@@ -1447,7 +1459,7 @@ double busiest(const Dims &dm, const TilePlan &pl)
 TilePlan make_plan(const Dims &dm, int n_instr)
 {
     if (dm.Skv == dm.S && !dm.ragged) {
-        const TilePlan pl = plan_base(dm);
+        const TilePlan pl = plan_base(dm, n_instr > 1);
         if (n_instr > 1) return pl;  // (several instructions in one launch: only this tiling)
         if (pl.ok && dm.n_rep * dm.S % 8 != 0 && dm.n_rep * dm.S <= kTileM / 2) {
             const TilePlan ring = plan_suffix_ring(dm);

@@ -30,6 +30,9 @@ SHAPES = [
     (2, 4, 4, 64, 60, 139),
     (1, 2, 1, 128, 0, 1039),
     (1, 8, 2, 128, 33, 513),
+    (262, 4, 4, 128, 20, 8),     # tiles of half as many rows as fit, for twice as many SMs
+    (9, 7, 1, 128, 34, 8),       # a candidate per tile
+    (133, 7, 1, 128, 300, 40),   # boxes of 8 rows, for a round of the SMs less
 ]
 
 
@@ -39,7 +42,7 @@ def test_forward_matches_the_oracle(shape):
     B, Hq, Hkv, d, P, S = shape
     w = Workload("tiles", 900 + sum(shape), B=B, Hq=Hq, Hkv=Hkv, d=d, P=P, S=S)
     assert pskv.pskv_kernel_family(0, B, Hq, Hkv, S, P, d) == 1
-    cand = None if B <= 64 else [0, 1, 2, 149, 150, 297, 298, 299]
+    cand = None if B <= 64 else [0, 1, 2, B // 2 - 1, B // 2, B - 3, B - 2, B - 1]
     parity.fwd_parity(w, cand=cand, strict_abs=(P + S >= 128))
 
 
