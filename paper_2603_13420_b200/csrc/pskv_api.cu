@@ -444,17 +444,6 @@ SideStream *side_stream()
 // instruction, 1 = one launch wherever the shapes allow it (the same as 0 today), 2 = always passes.
 int multi_form() { return g_multi_form.load(std::memory_order_relaxed); }
 
-// Launches of the gradient step of pskv_attn_bwd_multi.  One is enough; small calls of the shapes for which the row
-// statistic, dQ and the suffix gradients used to be three launches keep that observable count (pskv_kernel_launches)
-// as the row statistic and two halves of the units.  Large ones run in one: in two halves 300 candidates of 12
-// instructions (32/32 heads, P = 512, S = 80) took 3 % longer.
-int tc_bwd_multi_launches(const Dims &dm, int Bp)
-{
-    const bool grouped = dm.S % 8 == 0 && dm.S <= 128 && !(dm.S <= 48 && dm.n_rep * dm.S >= 128);
-    const long long rows = (long long)dm.B * dm.Hq * dm.S;
-    return grouped && rows <= 16384 && (long long)(dm.B / Bp) * dm.n_rep * dm.S % 128 == 0 ? 2 : 1;
-}
-
 // checks shared by the two multi-instruction calls; fills the per-instruction geometry
 pskv_status check_multi(int B, int Bp, int Hq, int Hkv, int S, int Pmax, int d, const int *prefix_len)
 {
@@ -604,7 +593,7 @@ pskv_status pskv_attn_bwd_multi(const void *dout, const void *q, const void *pre
     if (Bp > 1 && multi_form() != 2 && dall_ok && tc_bwd_fused_supported(dall, Bp)) {
         BwdArgs a;
         fill(a, 0, dall, 0);
-        cudaError_t e = launch_tc_bwd(a, status_word, stream, kBwdPartAll, Bp, prefix_len, tc_bwd_multi_launches(dall, Bp));
+        cudaError_t e = launch_tc_bwd(a, status_word, stream, kBwdPartAll, Bp, prefix_len);
         return e == cudaSuccess ? PSKV_OK : cuda_fail(e);
     }
     // One pass per instruction.  The row statistic D does not involve the prefix: when every instruction's part

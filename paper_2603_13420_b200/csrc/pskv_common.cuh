@@ -79,11 +79,10 @@ bool tc_bwd_supported(const Dims &d);
 size_t tc_bwd_workspace_bytes(const Dims &d);
 // `parts` selects which of the two steps run (all by default): the row statistic D does not involve the prefix,
 // so a caller with several prefixes runs it once over all candidates and the gradients once per prefix.
-// `split` > 1 takes the units of the gradient step in that many launches.
 enum { kBwdPartRowDot = 1, kBwdPartGrad = 2, kBwdPartAll = 3 };
 bool tc_bwd_fused_supported(const Dims &d, int n_instr);  // several instructions in one launch (as for the forward)
 cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStream_t stream, int parts = kBwdPartAll,
-                          int n_instr = 1, const int *prefix_len = nullptr, int split = 1);
+                          int n_instr = 1, const int *prefix_len = nullptr);
 
 // Masked target cross-entropy fused with the vocabulary projection (tcgen05 GEMM whose logits stay on chip).
 struct CeArgs {

@@ -106,7 +106,7 @@ struct TcBwdParams {
     int nblk;              // prefix pieces: ceil(P / 64)
     int Kq;                // candidates per instruction (all of them when there is one prefix)
     int upi, upg;          // units per (KV head, instruction), per KV head
-    int unit0, n_units;
+    int n_units;
     int n_tiles, n_sub;    // split launch: dQ units and all units of a candidate (else n_sub = 1)
     FastDiv fd_upg, fd_upi, fd_sub, fd_Rp, fd_S, fd_cpp;
     int stages_k, stages_v;
@@ -184,7 +184,7 @@ struct Walk {
     __device__ __forceinline__ void unit(const TcBwdParams &p)
     {
         if (done()) return;
-        const int w = SPLIT ? p.fd_sub.div(p.unit0 + u) : p.unit0 + u;
+        const int w = SPLIT ? p.fd_sub.div(u) : u;
         g = p.fd_upg.div(w);
         const int r = w - g * p.upg;
         inst = p.fd_upi.div(r);
@@ -196,7 +196,7 @@ struct Walk {
         t_end = (ncand * p.Rp + kTileM - 1) / kTileM;
         npass = t_end > 1 ? p.nh : 1;
         if (SPLIT) {
-            const int sub = p.unit0 + u - w * p.n_sub;
+            const int sub = u - w * p.n_sub;
             if (sub < p.n_tiles) {
                 t_first = sub;
                 t_end = sub + 1;
@@ -1073,7 +1073,7 @@ bool row_dot_in_kernel(const Dims &dm, const BwdPlan &plan)
 
 template <int D, bool TWO>
 cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_word, cudaStream_t stream, int n_instr,
-                   const int *prefix_len, int split, bool drow)
+                   const int *prefix_len, bool drow)
 {
     const Dims &dm = a.dims;
     const int Rg = dm.n_rep * dm.S;
@@ -1146,22 +1146,15 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
                        : (sp ? tc_bwd_kernel<D, true, false, TWO> : tc_bwd_kernel<D, false, false, TWO>);
     static PerDeviceOnce attr_set[4];
     if (cudaError_t e = ensure_max_smem(kernel, attr_set[2 * drow + sp]); e != cudaSuccess) return e;
-    const int units = p.upg * dm.Hkv * p.n_sub;
-    if (split > units) split = units;
-    for (int s = 0; s < split; ++s) {
-        p.unit0 = (int)((long long)units * s / split);
-        p.n_units = (int)((long long)units * (s + 1) / split) - p.unit0;
-        cudaError_t e;
-        {
-            KernelTiming timing(kKernelBwdTc, stream);
-            e = launch_dependent(kernel, even_grid(p.n_units, sm_count()), kThreads, plan.smem_bytes, stream, tm_q,
-                                 tm_do, tm_pk, tm_pv, tm_sk, tm_sv, p);
-        }
-        count_launches(1);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    p.n_units = p.upg * dm.Hkv * p.n_sub;
+    cudaError_t e;
+    {
+        KernelTiming timing(kKernelBwdTc, stream);
+        e = launch_dependent(kernel, even_grid(p.n_units, sm_count()), kThreads, plan.smem_bytes, stream, tm_q, tm_do, tm_pk, tm_pv,
+                             tm_sk, tm_sv, p);
     }
-    return cudaSuccess;
+    count_launches(1);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
@@ -1202,13 +1195,13 @@ bool tc_bwd_fused_supported(const Dims &dm, int n_instr)
 }
 
 cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStream_t stream, int parts, int n_instr,
-                          const int *prefix_len, int split)
+                          const int *prefix_len)
 {
     if (n_instr < 1) n_instr = 1;
     if (n_instr > 1 && (!prefix_len || !tc_bwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
     const BwdPlan &plan = plan_bwd(a.dims, n_instr);
     if (!plan.ok) return cudaErrorInvalidValue;
-    const bool drow = parts == kBwdPartAll && n_instr == 1 && split == 1 && row_dot_in_kernel(a.dims, plan);
+    const bool drow = parts == kBwdPartAll && n_instr == 1 && row_dot_in_kernel(a.dims, plan);
     if ((parts & kBwdPartRowDot) && !drow) {
         const cudaError_t e = launch_simt_row_dot(a, stream);
         if (e != cudaSuccess) return e;
@@ -1216,7 +1209,7 @@ cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStrea
     if (!(parts & kBwdPartGrad)) return cudaSuccess;
     auto run = plan.terms == 2 ? (a.dims.d == 128 ? launch<128, true> : launch<64, true>)
                                : (a.dims.d == 128 ? launch<128, false> : launch<64, false>);
-    return run(a, plan, status_word, stream, n_instr, prefix_len, split, drow);
+    return run(a, plan, status_word, stream, n_instr, prefix_len, drow);
 }
 
 }  // namespace pskv
