@@ -19,6 +19,8 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "pskv.h"
@@ -59,10 +61,16 @@ void *ptr(const at::Tensor &t)
 }
 void *ptr(PyObject *o) { return o == Py_None ? nullptr : ptr(tensor(o)); }
 
-// q, dout, ... [B, H, S, d] or the like
+// q [B, H, S, d], hidden [N, Lr, Dm]
 void want_dims(const at::Tensor &t, int n)
 {
     if (t.dim() != n) throw BadArgument{PyExc_ValueError, "a tensor has the wrong number of dimensions"};
+}
+// the other tensors are asked for the sizes the call needs and may have further dimensions, or merged ones, behind them
+int64_t size_at(const at::Tensor &t, int i)
+{
+    if (t.dim() <= i) throw BadArgument{PyExc_IndexError, "a tensor has too few dimensions"};
+    return t.size(i);
 }
 
 at::Tensor like(const at::Tensor &t) { return at::Tensor(at::detail::empty_cuda(t.sizes(), t.scalar_type(), t.device(), std::nullopt)); }
@@ -93,8 +101,10 @@ struct Scratch {
 
 float number(PyObject *o)
 {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw python_error();
+    PyObject *f = PyNumber_Float(o);  // float(o): also of a string
+    if (!f) throw python_error();
+    const double v = PyFloat_AsDouble(f);
+    Py_DECREF(f);
     return (float)v;
 }
 
@@ -103,10 +113,11 @@ void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 template <class Fn>
 pskv_status without_gil(Fn fn)
 {
-    PyThreadState *save = PyEval_SaveThread();
-    const pskv_status st = fn();
-    PyEval_RestoreThread(save);
-    return st;
+    struct Released {  // taken back however fn is left: what turns an exception into a Python one needs it
+        PyThreadState *save = PyEval_SaveThread();
+        ~Released() { PyEval_RestoreThread(save); }
+    } released;
+    return fn();
 }
 
 template <class... T>
@@ -141,26 +152,20 @@ PyObject *entry(PyObject *, PyObject *const *a, Py_ssize_t n)
 struct Dims {
     int B, Hq, Hkv, S, P, d;
 };
-// prefix [Hkv, P, d] or [Bp, Hkv, P, d]; the prefix length is its second-last size
-Dims dims_of(const at::Tensor &q, PyObject *prefix_k, const at::Tensor &suffix_k, int prefix_dims)
+// prefix [Hkv, P, d] (p_at = 1) or [Bp, Hkv, P, d] (p_at = 2)
+Dims dims_of(const at::Tensor &q, PyObject *prefix_k, const at::Tensor &suffix_k, int p_at)
 {
     want_dims(q, 4);
-    want_dims(suffix_k, 4);
+    const int64_t Hkv = size_at(suffix_k, 1), P = prefix_k == Py_None ? 0 : size_at(tensor(prefix_k), p_at);
     ptr(q);  // (before anything is allocated where q is)
-    int64_t P = 0;
-    if (prefix_k != Py_None) {
-        const at::Tensor &t = tensor(prefix_k);
-        want_dims(t, prefix_dims);
-        P = t.size(prefix_dims - 2);
-    }
-    return {(int)q.size(0), (int)q.size(1), (int)suffix_k.size(1), (int)q.size(2), (int)P, (int)q.size(3)};
+    return {(int)q.size(0), (int)q.size(1), (int)Hkv, (int)q.size(2), (int)P, (int)q.size(3)};
 }
 
 // (q, prefix_k, prefix_v, suffix_k, suffix_v, scale, out, lse, workspace)
 PyObject *fwd(PyObject *const *a)
 {
     const at::Tensor &q = tensor(a[0]), &sk = tensor(a[3]);
-    const Dims m = dims_of(q, a[1], sk, 3);
+    const Dims m = dims_of(q, a[1], sk, 1);
     const at::Tensor out = given_or_like(a[6], q), lse = floats(a[7], {m.B, m.Hq, m.S}, q);
     const Scratch ws(a[8], a[8] == Py_None ? api.fwd_ws(m.B, m.Hq, m.Hkv, m.S, m.P, m.d) : 0, q);
     void *qp = ptr(q), *pk = ptr(a[1]), *pv = ptr(a[2]), *skp = ptr(sk), *sv = ptr(a[4]), *op = ptr(out), *lp = ptr(lse), *s = stream();
@@ -174,7 +179,7 @@ PyObject *fwd(PyObject *const *a)
 PyObject *bwd(PyObject *const *a)
 {
     const at::Tensor &q = tensor(a[2]), &sk = tensor(a[5]), &sv = tensor(a[6]);
-    const Dims m = dims_of(q, a[3], sk, 3);
+    const Dims m = dims_of(q, a[3], sk, 1);
     const at::Tensor dq = given_or_like(a[10], q), dk = given_or_like(a[11], sk), dv = given_or_like(a[12], sv);
     const Scratch ws(a[13], a[13] == Py_None ? api.bwd_ws(m.B, m.Hq, m.Hkv, m.S, m.P, m.d) : 0, q);
     void *dop = ptr(a[0]), *dl = ptr(a[1]), *qp = ptr(q), *pk = ptr(a[3]), *pv = ptr(a[4]), *skp = ptr(sk), *svp = ptr(sv), *op = ptr(a[7]),
@@ -192,8 +197,8 @@ PyObject *bwd(PyObject *const *a)
 PyObject *fwd_decode(PyObject *const *a)
 {
     const at::Tensor &q = tensor(a[0]), &sk = tensor(a[3]);
-    const Dims m = dims_of(q, a[1], sk, 3);
-    const int Skv = (int)sk.size(2);
+    const Dims m = dims_of(q, a[1], sk, 1);
+    const int Skv = (int)size_at(sk, 2);
     if (a[5] != Py_None) {
         const at::Tensor &n = tensor(a[5]);
         if (n.scalar_type() != at::kInt || n.dim() != 1 || n.size(0) != m.B)
@@ -212,13 +217,14 @@ PyObject *fwd_decode(PyObject *const *a)
 
 std::vector<int> lengths(PyObject *o)
 {
+    if (PyObject_Size(o) < 0) throw python_error();  // (an iterator has no length)
     PyObject *seq = PySequence_Fast(o, "prefix_len must be a sequence of integers");
     if (!seq) throw python_error();
     std::vector<int> v;
     bool ok = true;
     for (Py_ssize_t i = 0; ok && i < PySequence_Fast_GET_SIZE(seq); ++i) {
         PyObject *n = PyNumber_Long(PySequence_Fast_GET_ITEM(seq, i));
-        const long x = n ? PyLong_AsLong(n) : -1;
+        const unsigned long x = n ? PyLong_AsUnsignedLongMask(n) : 0;  // the low bits, as a C int of ctypes takes them
         Py_XDECREF(n);
         ok = !PyErr_Occurred();
         v.push_back((int)x);
@@ -232,7 +238,7 @@ std::vector<int> lengths(PyObject *o)
 PyObject *fwd_multi(PyObject *const *a)
 {
     const at::Tensor &q = tensor(a[0]), &sk = tensor(a[4]);
-    const Dims m = dims_of(q, a[1], sk, 4);
+    const Dims m = dims_of(q, a[1], sk, 2);
     const std::vector<int> len = lengths(a[3]);
     const int Bp = (int)len.size();
     const at::Tensor out = given_or_like(a[7], q), lse = floats(a[8], {m.B, m.Hq, m.S}, q);
@@ -249,7 +255,7 @@ PyObject *fwd_multi(PyObject *const *a)
 PyObject *bwd_multi(PyObject *const *a)
 {
     const at::Tensor &q = tensor(a[1]), &sk = tensor(a[5]), &sv = tensor(a[6]);
-    const Dims m = dims_of(q, a[2], sk, 4);
+    const Dims m = dims_of(q, a[2], sk, 2);
     const std::vector<int> len = lengths(a[4]);
     const int Bp = (int)len.size();
     const at::Tensor dq = given_or_like(a[10], q), dk = given_or_like(a[11], sk), dv = given_or_like(a[12], sv);
@@ -269,11 +275,10 @@ PyObject *target_ce(PyObject *const *a)
     const at::Tensor &h = tensor(a[0]), &w = tensor(a[1]), &t = tensor(a[2]), &m = tensor(a[3]);
     want_dims(h, 3);
     ptr(h);
-    want_dims(w, 2);
     if (t.scalar_type() != at::kInt || m.scalar_type() != at::kFloat)
         throw BadArgument{PyExc_ValueError, "target must be int32 and mask float32"};
-    const int64_t N = h.size(0), Lr = h.size(1), Dm = h.size(2), V = w.size(0);
-    if (t.sizes() != at::IntArrayRef({N, Lr}) || m.sizes() != at::IntArrayRef({N, Lr}) || w.size(1) != Dm)
+    const int64_t N = h.size(0), Lr = h.size(1), Dm = h.size(2), V = size_at(w, 0);
+    if (t.sizes() != at::IntArrayRef({N, Lr}) || m.sizes() != at::IntArrayRef({N, Lr}) || size_at(w, 1) != Dm)
         throw BadArgument{PyExc_ValueError, "shape mismatch"};
     const at::Tensor nll = floats(a[4], {N, Lr}, h), lse = floats(a[5], {N, Lr}, h), loss = floats(a[6], {N}, h);
     const Scratch ws(a[7], a[7] == Py_None ? std::max<size_t>(256, api.ce_ws((int)N, (int)Lr, (int)Dm, (int)V)) : 0, h);
