@@ -12,6 +12,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 
 import torch
 
@@ -140,6 +141,10 @@ def native():
         except ImportError as e:
             raise RuntimeError("the extension module _native.so is missing or does not load: build it with `python -m "
                                "paper_2603_13420_b200.build` (there is no fallback)") from e
+        here = "%s torch %s" % (sys.implementation.cache_tag, torch.__version__)
+        if module.built_for != here:
+            raise RuntimeError("_native.so was built for %s, this is %s: build it again with `python -m paper_2603_13420_b200.build`"
+                               % (module.built_for, here))
         module.init(*[ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _NATIVE_ENTRIES])
         _native = module
     return _native

@@ -36,20 +36,40 @@ def _older(target, sources) -> bool:
     return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in sources)
 
 
+def _torch_dir() -> str:
+    import importlib.util
+
+    return os.path.dirname(importlib.util.find_spec("torch").origin)
+
+
+def built_for() -> str:
+    """The interpreter and torch that the extension module is built for (torch itself need not be imported)."""
+    version = {}
+    with open(os.path.join(_torch_dir(), "version.py")) as f:
+        exec(f.read(), version)
+    return "%s torch %s" % (sys.implementation.cache_tag, version["__version__"])
+
+
+def _native_stale() -> bool:
+    if _older(NATIVE_PATH, [NATIVE_SRC, _deps()[0]]):
+        return True
+    with open(NATIVE_PATH, "rb") as f:
+        return built_for().encode() + b"\0" not in f.read()
+
+
 def is_stale() -> bool:
-    return _older(LIB_PATH, _deps()) or _older(NATIVE_PATH, [NATIVE_SRC, _deps()[0]])
+    return _older(LIB_PATH, _deps()) or _native_stale()
 
 
 def _build_native() -> None:
     """The Python extension module; it needs torch's headers and libraries, not CUDA kernels."""
-    import importlib.util
     import sysconfig
 
-    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    torch_dir = _torch_dir()
     inc = os.path.join(torch_dir, "include")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = NATIVE_PATH + ".tmp.%d" % os.getpid()
-    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I", INCLUDE, "-I", inc,
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", '-DPSKV_BUILT_FOR="%s"' % built_for(), "-I", INCLUDE, "-I", inc,
                     "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", sysconfig.get_paths()["include"],
                     "-I", os.path.join(cuda, "include"), NATIVE_SRC, "-o", tmp, "-L", os.path.join(torch_dir, "lib"),
                     "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"], check=True)
@@ -59,7 +79,7 @@ def _build_native() -> None:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source into paper_2603_13420_b200/libpskv.so, and the extension module beside it; returns the
     library's path."""
-    if force or _older(NATIVE_PATH, [NATIVE_SRC, _deps()[0]]):
+    if force or _native_stale():
         _build_native()
     if not force and not _older(LIB_PATH, _deps()):
         return LIB_PATH

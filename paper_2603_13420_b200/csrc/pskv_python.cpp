@@ -318,4 +318,17 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native(void) { return PyModule_Create(&module); }
+#ifndef PSKV_BUILT_FOR
+#error "the build passes the interpreter and torch that this module is made for"
+#endif
+
+PyMODINIT_FUNC PyInit__native(void)
+{
+    PyObject *m = PyModule_Create(&module);
+    // binding.py refuses a module made for another torch: its C++ interface is not a stable one
+    if (m && PyModule_AddStringConstant(m, "built_for", PSKV_BUILT_FOR) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

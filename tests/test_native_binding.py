@@ -51,3 +51,16 @@ def test_host_tensors_are_refused():
     t = torch.zeros((1, 1, 1, 64), dtype=torch.bfloat16)
     with pytest.raises(ValueError):
         pskv.pskv_attn_fwd(t, None, None, t, t, 0.1)
+
+
+def test_a_module_built_for_another_torch_is_stale_and_refused(monkeypatch):
+    from paper_2603_13420_b200 import _native, binding, build
+
+    assert _native.built_for == build.built_for() and torch.__version__ in _native.built_for
+    assert not build._native_stale()
+    monkeypatch.setattr(build, "built_for", lambda: "cpython-312 torch 0.0.1")
+    assert build._native_stale() and build.is_stale()
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.raises(RuntimeError, match="built for"):
+        binding.native()
