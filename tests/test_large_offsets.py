@@ -23,8 +23,8 @@ def _device_randn(shape, seed):
     return x
 
 
-@pytest.mark.parametrize("S,B", [(48, 11000),     # tensor-core kernels
-                                  (47, 11200)])    # general kernels (S not a multiple of 8)
+@pytest.mark.parametrize("S,B", [(48, 11000),
+                                  (47, 11200)])    # candidates padded to 48 rows, gradients in two terms
 def test_forward_and_backward_with_more_than_2_to_31_elements(S, B):
     Hq, Hkv, P, d = 32, 8, 256, 128            # q, out, dout, dq: more than 2^31 elements each
     first_past = 2 ** 31 // (Hq * S * d) + 1   # first candidate that lies wholly past element 2^31
@@ -32,6 +32,7 @@ def test_forward_and_backward_with_more_than_2_to_31_elements(S, B):
     free, _ = torch.cuda.mem_get_info()
     if free < 30 * 2 ** 30:
         pytest.skip("needs about 24 GB of device memory")
+    assert pskv.pskv_kernel_family(0, B, Hq, Hkv, S, P, d) == 1 and pskv.pskv_kernel_family(1, B, Hq, Hkv, S, P, d) == 1
     scale = 1.0 / np.sqrt(d)
     q = _device_randn((B, Hq, S, d), 1)
     dout = _device_randn((B, Hq, S, d), 2)
@@ -90,6 +91,52 @@ def test_decode_shaped_call_with_a_suffix_cache_of_more_than_2_to_31_elements():
     nl = lens[cand].numpy()
     ref_out, ref_lse = oracle.attn_fwd_decode(f(q), fp(pk), fp(pv), f(sk), f(sv), scale, nl)
     parity.check_tensor("out", f(out), ref_out, strict_abs=True)
+    parity.check_lse(f(lse), ref_lse)
+    rq, rk, rv = oracle.attn_bwd_decode(f(dout), f(q), fp(pk), fp(pv), f(sk), f(sv), scale, nl)
+    parity.check_tensor("dq", f(dq), rq)
+    parity.check_tensor("dk_suffix", f(dk), rk)
+    parity.check_tensor("dv_suffix", f(dv), rv)
+
+
+def test_general_kernels_with_more_than_2_to_31_elements():
+    """Eleven heads per KV head and 13 query tokens are 143 rows, which no tile of 16 to 128 rows divides: the decode-shaped call
+    runs on the CUDA-core kernels in both directions."""
+    Hq, Hkv, Sq, Skv, P, d = 22, 2, 13, 16, 24, 128
+    B = 58700                                  # q, out, dout, dq: 2.15e9 elements each
+    assert B * Hq * Sq * d > 2 ** 31
+    free, _ = torch.cuda.mem_get_info()
+    if free < 30 * 2 ** 30:
+        pytest.skip("needs about 20 GB of device memory")
+    scale = 1.0 / np.sqrt(d)
+    q = _device_randn((B, Hq, Sq, d), 51)
+    dout = _device_randn((B, Hq, Sq, d), 52)
+    sk = _device_randn((B, Hkv, Skv, d), 53)
+    sv = _device_randn((B, Hkv, Skv, d), 54)
+    pk = _device_randn((Hkv, P, d), 55)
+    pv = _device_randn((Hkv, P, d), 56)
+    gen = torch.Generator(device="cpu")
+    gen.manual_seed(57)
+    lens = torch.randint(Sq, Skv + 1, (B,), generator=gen, dtype=torch.int32)
+    dlens = lens.cuda()
+    names = [pskv.pskv_kernel_timing_name(i) for i in range(pskv.pskv_kernel_timing_count())]
+    pskv.pskv_kernel_timing_enable(True)
+    try:
+        out, lse = pskv.pskv_attn_fwd_decode(q, pk, pv, sk, sv, dlens, scale)
+        dq, dk, dv = pskv.pskv_attn_bwd_decode(dout, q, pk, pv, sk, sv, dlens, out, lse, scale)
+        torch.cuda.synchronize()
+        ran = {n for i, n in enumerate(names) if pskv.pskv_kernel_timing_read(i)[1] > 0}
+    finally:
+        pskv.pskv_kernel_timing_enable(False)
+    assert {"simt_fwd_kernel", "simt_bwd_dq_kernel", "simt_bwd_dkv_kernel"} <= ran and not any(n.startswith("tc_") for n in ran), ran
+    assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
+    first_past = 2 ** 31 // (Hq * Sq * d) + 1
+    cand = [0, B // 3, first_past - 1, first_past, B - 2, B - 1]
+    idx = torch.tensor(cand, device="cuda")
+    f = lambda x: parity.to_f64(x.index_select(0, idx).cpu())
+    fp = lambda x: parity.to_f64(x.cpu())
+    nl = lens[cand].numpy()
+    ref_out, ref_lse = oracle.attn_fwd_decode(f(q), fp(pk), fp(pv), f(sk), f(sv), scale, nl)
+    parity.check_tensor("out", f(out), ref_out)
     parity.check_lse(f(lse), ref_lse)
     rq, rk, rv = oracle.attn_bwd_decode(f(dout), f(q), fp(pk), fp(pv), f(sk), f(sv), scale, nl)
     parity.check_tensor("dq", f(dq), rq)

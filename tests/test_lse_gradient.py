@@ -1,5 +1,5 @@
 """pskv_attn_bwd_lse: the backward with a gradient arriving on the log-sum-exp output, against the fp64
-oracle (L = sum(out * dout) + sum(lse * dlse)), on the tensor-core and the general kernel families."""
+oracle (L = sum(out * dout) + sum(lse * dlse)), with one and with two bf16 terms per dS."""
 import ctypes
 
 import numpy as np
@@ -13,10 +13,10 @@ from paper_2603_13420_b200.inputs import Workload, make_inputs
 
 SHAPES = [
     # B, Hq, Hkv, S, P, d
-    (24, 32, 8, 48, 256, 128),   # the GQA layer shape (tensor-core dQ and suffix-gradient kernels)
+    (24, 32, 8, 48, 256, 128),   # the GQA layer shape
     (16, 4, 4, 40, 160, 128),    # MHA
     (6, 8, 2, 16, 300, 64),      # head dim 64
-    (4, 4, 2, 5, 33, 128),       # general kernels (odd S)
+    (4, 4, 2, 5, 33, 128),       # odd S: two terms
 ]
 
 

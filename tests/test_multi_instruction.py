@@ -35,7 +35,7 @@ CASES = [
     (12, 3, 8, 2, 16, 300, 128, (300, 129, 40)),   # tensor-core path, ragged prefixes, GQA
     (8, 2, 4, 4, 40, 160, 128, (160, 96)),         # MHA, 40-token suffix
     (6, 3, 4, 2, 8, 64, 64, (0, 64, 17)),          # head dim 64, an empty prefix, odd length
-    (4, 4, 2, 1, 5, 33, 128, (33, 1, 20, 7)),      # general kernels (S not a multiple of 8)
+    (4, 4, 2, 1, 5, 33, 128, (33, 1, 20, 7)),      # a candidate per instruction, five rows each; passes only
     (64, 2, 32, 8, 48, 256, 128, (256, 200)),      # the GQA layer shape, two instructions
     (16, 4, 8, 2, 16, 600, 128, (600, 0, 130, 471)),  # one launch, prefix blocks streamed; an empty prefix and
                                                    # one whose padding covers three whole key blocks
@@ -43,8 +43,8 @@ CASES = [
     (40, 5, 8, 2, 32, 200, 128, (200, 199, 73, 128, 1)),  # one launch, five instructions, odd lengths
 ]
 
-# cases whose shape allows all instructions in one launch (every tile inside one instruction); the library takes
-# that form by itself only while the padding is a small share of the keys, so the tests name the form
+# cases whose shape allows all instructions in one forward launch (an instruction is a whole number of tiles, or at least four);
+# the backward takes one launch for all of them
 ONE_LAUNCH_SHAPES = {0, 4, 5, 6, 7}
 
 
@@ -83,7 +83,7 @@ def test_forward_and_backward_match_the_oracle(case, form):
     pskv.pskv_attn_bwd_multi(dev["dout"], dev["q"], dev["prefix_k"], dev["prefix_v"], lens, dev["suffix_k"],
                              dev["suffix_v"], out.view, lse.view, scale, dq=dq.view, dk_suffix=dk.view,
                              dv_suffix=dv.view)
-    if one:   # the row statistic, then one launch for the three gradients of all instructions
+    if form == "one":   # the row statistic, then one launch for the three gradients of all instructions
         assert pskv.pskv_kernel_launches() - n0 == 2
     assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
     dq.check("dq"); dk.check("dk_suffix"); dv.check("dv_suffix")
