@@ -201,13 +201,14 @@ __device__ __forceinline__ int sfx_long_rows(const Params &p, int j)
 }
 
 // MODE 1: all prefix blocks of a KV head stay in shared memory; MODE 0: they stream through rings,
-// and the suffix keys of a tile sit in one block with buffers of its own; MODE 2 (suffix-ring): a
-// tile is a run of whole candidates and their suffix keys follow the prefix through the same rings
-// in as many blocks as it takes -- the mode of the decode-shaped operator, where a 128-row tile
-// spans many candidates, and of full-suffix shapes the other two modes cannot tile; MODE 3: the same with tiles that
-// straddle candidates or lie inside a head whose rows are padded to whole tiles.  A compile-time
-// switch so that each launch carries only the code of its own mode (with MODE 3's decisions taken at run time in MODE 2, 729
-// beams, 32/32 heads, 4 tokens over 147 cached ones took 644 us instead of 572).
+// and the suffix keys of a tile sit in one block with buffers of its own; MODE 2 and 3 (suffix-ring): the suffix
+// keys follow the prefix through the same rings in as many blocks as it takes.  MODE 2: a tile lies inside one
+// candidate, whose rows the tiles divide (suffix caches beyond a block, prompts); MODE 3: any row list -- whole candidates
+// (the decode-shaped operator, where a 128-row tile spans many), tiles that straddle candidates, tiles inside a head
+// whose rows are padded to whole tiles.  A compile-time
+// switch so that each launch carries only the code of its own mode.  The last two are apart for what the compiler makes of
+// them: 729 beams, 32/32 heads, 4 tokens over 147 cached ones take 572 us in MODE 2 and 644 with MODE 3's decisions at run time,
+// 512 beams, 32/8 heads, one token over 48 23.8 us in MODE 3 and 25.6 with MODE 2's code.
 // MI 1: several instructions, each a whole number of tiles; 2: the last tile of each is short.  Apart because a tile's
 // place is worked out by every role (8 x 64 candidates, 32/8 heads, P = 256, S = 48: 139 us with the second's division, 132).
 //
@@ -902,8 +903,9 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     const int slot = item % kSlots;
                     const uint32_t s_tmem = tmem + lane_addr + slot * kBlockN + wg * kPiece;
                     // valid columns of this row: [lo, hi].  Padding rows of a tile take part in prefix
-                    // blocks like real rows (their scores are finite and never stored) and see no
-                    // suffix key.
+                    // blocks like real rows and see no suffix key.  They are never stored; where no copy wrote
+                    // them their scores are whatever shared memory held, NaN included, and the epilogue stages
+                    // zeros for such rows.
                     int n, lo, hi;
                     if (k < p.nblk_p) {
                         n = prefix_block_rows(p, k);
@@ -1028,7 +1030,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (lane == 0) mbar_arrive(bar(kBarMlFree));
             const bool row_ok = l >= kMinRowSum && l <= kMaxRowSum;  // false for overflow (inf, NaN), underflow
             // staged values must be finite (the buffer may double as suffix V, whose padding rows
-            // meet zero probabilities): rows that failed stage zeros, and are redone anyway
+            // meet zero probabilities): rows that failed stage zeros and are redone, and so do padding rows, whose
+            // sums may be NaN (they are not redone)
             const float inv = row_ok ? 1.f / l : 0.f;
             if (p.slab_stage) {
                 // One 64-column slab at a time through a staging buffer of one slab: load, hand O back after
@@ -1184,7 +1187,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 
 struct TilePlan {
     bool ok;
-    int mode;   // kernel template MODE: 0 rings, 1 resident prefix, 2 suffix-ring, 3 suffix-ring with any row list
+    int mode;   // kernel template MODE: 0 rings, 1 resident prefix, 2 / 3 suffix-ring (see there)
     int cbox, Spad, cpb;  // suffix-ring mode: candidates per tile, rows per candidate in a block, candidates per block
     int long_sfx;         // suffix-ring mode: tiles inside one candidate, its suffix keys in 128-key blocks
     int two_terms;        // suffix-ring mode: probabilities as two bf16 terms
@@ -1346,6 +1349,7 @@ TilePlan plan_suffix_ring(const Dims &dm)
                 pl.cbox = c;
             }
         }
+        pl.mode = 3;
         pl.Rp = Rg;
         pl.one_box = 1;
         pl.tile_rows = pl.seg_rows = Rg * pl.cbox;
