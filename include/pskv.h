@@ -171,9 +171,12 @@ long long pskv_attn_bwd_static_max_rows(void);
  * must be a multiple of Bp and each cache is reused by its B / Bp candidates.  Everything else (q,
  * suffix_k, suffix_v, out, lse, dout, dq, dk_suffix, dv_suffix; scale; causal rule; error codes) is as
  * in pskv_attn_fwd / pskv_attn_bwd, with P replaced per candidate by the true prefix length of its
- * instruction.  When (B / Bp) * (Hq / Hkv) * S is a multiple of the kernels' row tile (128 rows in the
- * usual case), Bp <= 64 and the shape runs on the tensor-core kernels, all instructions are served by one
- * launch per kernel (pskv_set_multi_form(2) turns this off).  Otherwise the work is one pass per instruction; the passes are independent, so every
+ * instruction.
+ * With Bp <= 64 one launch may serve all instructions (pskv_set_multi_form(2) turns this off); forward and
+ * backward decide by themselves.  The forward does where the suffix keys of a row tile fit one 128-key block
+ * and an instruction's rows, as the kernel pads them, are a whole number of tiles or at least four; the backward
+ * on every shape of the tensor-core kernel with Pmax >= 1 (one launch for the row statistic, one for the three
+ * gradients).  Otherwise the work is one pass per instruction; the passes are independent, so every
  * other one is enqueued on a stream of the library's own that forks from `cuda_stream` at the start of the
  * call and joins it again before the call returns (to the caller everything is ordered as if it had run on
  * `cuda_stream`, also under stream capture).
