@@ -26,7 +26,7 @@
 // Measured (whole forward + backward step, before: a dQ kernel and a suffix-gradient kernel that each read q and
 // dout, for S a multiple of 8 and up to 64, CUDA-core kernels for the rest): B = 512, 32/8 heads, P = 256, S = 48
 // 563 -> 519 us; B = 128, 32/32 heads, P = 160, S = 40 171 -> 142 us; B = 100, 32/32 heads, P = 78, S = 113 10.4 ms ->
-// 0.30 ms.  With a staging buffer for dQ instead of four K and three V stages (three and two fit): 529 us.
+// 0.30 ms (0.32 with two terms, below).  With a staging buffer for dQ instead of four K and three V stages (three and two fit): 529 us.
 //
 // Suffixes beyond 64 keys have several pieces per candidate but only one pair of accumulators (128 columns).
 // When the unit is one tile the pieces take turns; when it is several tiles, pass 0 accumulates piece 0 (and
@@ -35,7 +35,8 @@
 // Launches of few candidates (the gradient of a search's one current suffix) are split: every tile's dQ and every
 // suffix piece's dK / dV is a unit of its own, so that one candidate keeps up to tiles + pieces SMs per KV head
 // busy instead of one, at the price of forming the scores of the suffix pieces once more.  Whole steps: B = 1, 32/8
-// heads, P = 78, S = 113 45 -> 25 us; B = 4, 32/8, P = 1000, S = 100 96 -> 56; B = 20, 32/8, P = 200, S = 90 84 -> 77.
+// heads, P = 78, S = 113 45 -> 25 us; B = 4, 32/8, P = 1000, S = 100 96 -> 56; B = 20, 32/8, P = 200, S = 90 84 -> 77 (with
+// one term; with two 28, 59 and 80).
 //
 // Two terms (TWO): P and dS go to shared memory as sums of two bf16 values (16 bits of mantissa), and the contractions run over
 // both.  Taken where the suffix length is no multiple of 8 or exceeds 64 (multiples of 8 up to 128: for dK / dV alone):
@@ -979,7 +980,7 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
     const int sms = sm_count();
     double best = -1.0;
     // A candidate's rows may be padded further than to the next multiple of 8: 4 heads x 42 rows are two tiles, one of
-    // them a third full, or, as 176 rows, three tiles for two candidates (kernel alone, B = 250, P = 385 240 -> 203 us;
+    // them a third full, or, as 176 rows, three tiles for two candidates (kernel alone, one term, B = 250, P = 385 240 -> 203 us;
     // 4 x 67 rows, B = 100, P = 300 181 -> 169; 4 x 35, B = 144, P = 92 74 -> 66).
     for (int Rp = round_up(Rg, 8); Rp < Rg + 64; Rp += 8) {
         const int seg = gcd_int(Rp, kTileM);
@@ -1061,7 +1062,7 @@ const BwdPlan &plan_bwd(const Dims &dm, int n_instr)
 }
 
 // D in the kernel: the smallest launches, whose CTAs have one tile each.  Its loads then run under those of the tile's
-// operands, and a launch in the chain of three goes away.  Whole steps, with the pre-pass and with D in here: 8 candidates, 4/4
+// operands, and a launch in the chain of three goes away.  Whole steps, gradients in one term, with the pre-pass and with D in here: 8 candidates, 4/4
 // heads, d = 64, P = 32, S = 8 14.1 and 12.0 us; 9, 32/8 heads, P = 256, S = 30 21.8 and 18.2; 2, 32/32 heads, P = 200, S =
 // 128 24.3 and 21.6, P = 300, S = 50 21.7 and 21.2.  With several tiles per CTA every tile waits for its own D: 1
 // candidate, 32/8 heads, P = 78, S = 113 (four tiles in a unit) 25.3 and 28.8, 12 candidates, 32/32 heads, P = 90, S = 77

@@ -56,10 +56,10 @@ enum : unsigned int {
 };
 
 // MODE 3.  The compiler reads runs of the kernel's parameters in one instruction where they are aligned, and what that makes of the
-// walk over tiles differs: with the fields behind these moved by 12 bytes the kernel for several instructions took 140 us for 8
-// x 64 candidates, 32/8 heads, P = 256, S = 48, moved by 0 or 16 132; the others want the 12 (149 candidates, 4/4 heads, P =
-// 315, S = 8: 10.3 us, else 11.4).
-template <bool SEVERAL>
+// walk over tiles differs: with the fields behind these moved by 12 bytes the kernel for several instructions of whole tiles
+// took 140 us for 8 x 64 candidates, 32/8 heads, P = 256, S = 48, moved by 0 or 16 132; the others want the 12 (149 candidates,
+// 4/4 heads, P = 315, S = 8: 10.3 us, else 11.4; 6 x 90 candidates with short last tiles, 32/8, P = 300, S = 37 180, else 189).
+template <bool ALIGNED>
 struct BoxFields {
     int Sh;               // rows a query head takes in the row list: S, or S padded to whole tiles (head_box)
     int one_box;          // 1: a tile's Q is one box per slab (whole candidates, or rows of one head), else runs of seg_rows
@@ -80,7 +80,7 @@ struct TcFwdParams {
     int Rg;               // rows a candidate takes in the row list of a KV-head group (its n_rep * S real rows, padded)
     int Rr;               // its real rows: n_rep * S
     int Sp;               // key columns a candidate takes in a tile's suffix block: S rounded up to 8
-    BoxFields<(MI != 0)> box;
+    BoxFields<MI == 1> box;
     int tile_rows;        // rows of the flat row list per tile (<= 128, multiple of seg_rows)
     int seg_rows;         // rows per Q / out TMA box: gcd(Rg, tile_rows) (rows past Rr are zero-filled, never stored)
     int tiles_per_group;
@@ -1643,7 +1643,7 @@ size_t tc_fwd_workspace_bytes(const Dims &) { return 0; }
 // tiling).  An instruction starts a tile of its own, so its last tile may be short: taken where an instruction is a
 // whole number of tiles, or at least four, so that the short one costs at most a fifth (90 candidates of 6
 // instructions, 32/8 heads, P = 300, S = 37: one launch 107 us for forward + backward, six passes
-// on two streams 131).
+// on two streams 131, the gradients in one term both times).
 bool tc_fwd_fused_supported(const Dims &dm, int n_instr)
 {
     if (n_instr < 2 || n_instr > kMaxFusedInstructions || dm.B % n_instr != 0 || dm.P < 1 || dm.Pstride != dm.P ||
