@@ -126,7 +126,8 @@ struct Cfg {
 };
 
 enum {
-    kBarQFull = 0,   // Q and dO of a tile landed
+    kBarQFull = 0,   // Q of a tile landed (SPLIT: and dO)
+    kBarDoFull,      // dO of a tile landed
     kBarQFree,       // the last MMA of each issuer that reads them has completed (2 arrivals)
     kBarDqFull,      // dQ of a tile is final
     kBarDqFree,      // the epilogue has read it out (4 arrivals)
@@ -523,14 +524,22 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             ok = mbar_wait_warp(bar(kBarQFree), (tile & 1u) ^ 1u, abort_flag, p.status, kErrProdQ);
             if (!ok) break;
             PSKV_TRACE_EVENT(2, tile);
-            if (lane == 0) mbar_arrive_expect_tx(bar(kBarQFull), (uint32_t)(nb * 2 * C::kSlabs * step * 128));
+            const uint32_t tx = (uint32_t)(nb * C::kSlabs * step * 128);
+            if (lane == 0) {
+                if (!SPLIT) mbar_arrive_expect_tx(bar(kBarDoFull), tx);
+                mbar_arrive_expect_tx(bar(kBarQFull), SPLIT ? 2 * tx : tx);
+            }
             __syncwarp();
             if (lane < nb) {
 #pragma unroll
                 for (int sl = 0; sl < C::kSlabs; ++sl) {
                     const uint32_t off = (uint32_t)(sl * C::kSlabBytes + lane * step * 128);
+                    tma_load_4d(sbase + p.off_do + off, &tm_do, bar(SPLIT ? kBarQFull : kBarDoFull), sl * 64, r, g, b);
+                }
+#pragma unroll
+                for (int sl = 0; sl < C::kSlabs; ++sl) {
+                    const uint32_t off = (uint32_t)(sl * C::kSlabBytes + lane * step * 128);
                     tma_load_4d(sbase + p.off_q + off, &tm_q, bar(kBarQFull), sl * 64, r, g, b);
-                    tma_load_4d(sbase + p.off_do + off, &tm_do, bar(kBarQFull), sl * 64, r, g, b);
                 }
             }
             if (!DROW) {
@@ -562,12 +571,33 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             const uint32_t x = __shfl_sync(0xffffffffu, descs[item & 7u].x, 0);
             if (x & kDescEnd) break;
             const uint32_t idesc = make_idesc_bf16(kTileM, (int)(x & kDescN), 0);
-            if (x & kDescFirst) ok = mbar_wait_warp(bar(kBarQFull), descs[item & 7u].w & 1u, abort_flag, p.status, kErrMmaS);
+            const uint32_t tile_ph = descs[item & 7u].w & 1u;
+            if (x & kDescFirst) ok = mbar_wait_warp(bar(SPLIT ? kBarQFull : kBarDoFull), tile_ph, abort_flag, p.status, kErrMmaS);
             if (ok) ok = mbar_wait_warp(bar(kBarSFree + slot), ((item >> 1) & 1u) ^ 1u, abort_flag, p.status, kErrMmaS);
             if (ok) ok = mbar_wait_warp(bar(kBarVFull + vs), vph, abort_flag, p.status, kErrMmaS);
             if (!ok) break;
             PSKV_TRACE_EVENT(15, item);
             tc_fence_after();
+            // dP first: its V piece is handed back while S is under way (with two terms there is one V stage, and its next piece
+            // is what the following item waits for), and a tile's first dP starts when dO has landed, before Q.  Whole steps:
+            // 58 candidates, 32/32 heads, P = 1735, S = 66 601 -> 569 us, 61, 32/32, P = 1206, S = 54 314 -> 303, 14, 32/32, P = 417, S =
+            // 123 97 -> 94; in one term and on small launches no change.  (Split launches have few items to a tile; waiting for
+            // the two in turn costs them more: one candidate, 32/8, P = 78, S = 113 27.9 -> 28.8.)
+            if (elect_one_sync()) {
+#pragma unroll
+                for (int i = 0; i < D / 16; ++i) {
+                    const uint64_t aoff = (uint64_t)(((i >> 2) * C::kSlabBytes + (i & 3) * 32) >> 4);
+                    const uint64_t boff = (uint64_t)(((i >> 2) * C::kPieceSlab + (i & 3) * 32) >> 4);
+                    mma_ss(d_tmem + kColDp, do_desc + aoff, v_desc + boff, idesc, i > 0 ? 1u : 0u);
+                }
+                tc_commit(bar(kBarVFree + vs));
+            }
+            if (!SPLIT && (x & kDescFirst)) {
+                __syncwarp();
+                ok = mbar_wait_warp(bar(kBarQFull), tile_ph, abort_flag, p.status, kErrMmaS);
+                if (!ok) break;
+                tc_fence_after();
+            }
             if (elect_one_sync()) {
 #pragma unroll
                 for (int i = 0; i < D / 16; ++i) {
@@ -575,14 +605,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     const uint64_t boff = (uint64_t)(((i >> 2) * C::kPieceSlab + (i & 3) * 32) >> 4);
                     mma_ss(d_tmem, q_desc + aoff, k_desc + boff, idesc, i > 0 ? 1u : 0u);
                 }
-#pragma unroll
-                for (int i = 0; i < D / 16; ++i) {
-                    const uint64_t aoff = (uint64_t)(((i >> 2) * C::kSlabBytes + (i & 3) * 32) >> 4);
-                    const uint64_t boff = (uint64_t)(((i >> 2) * C::kPieceSlab + (i & 3) * 32) >> 4);
-                    mma_ss(d_tmem + kColDp, do_desc + aoff, v_desc + boff, idesc, i > 0 ? 1u : 0u);
-                }
                 tc_commit(bar(kBarSFull + slot));
-                tc_commit(bar(kBarVFree + vs));
                 if (x & kDescLast) tc_commit(bar(kBarQFree));
             }
             __syncwarp();
