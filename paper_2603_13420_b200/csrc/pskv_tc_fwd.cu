@@ -338,7 +338,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             prefetch_tensormap(&tm_sk);
             if (p.P > 0) { prefetch_tensormap(&tm_pk); prefetch_tensormap(&tm_pk_tail); }
         }
-        uint32_t kload = 0;  // streaming mode: prefix K blocks loaded so far
+        uint32_t ks = 0, kph = 1;  // ring of K blocks: stage, parity of its release
         bool ok = true;
 #pragma unroll 1
         for (int tl = 0; tl < n_tiles && ok; ++tl) {
@@ -395,9 +395,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             } else {
 #pragma unroll 1
                 for (int k = first_block(inst); k < p.nblk_p; ++k) {
-                    const uint32_t ks = kload % (uint32_t)p.stages;
-                    ok = mbar_wait_warp(bar(kBarKFree + ks), ((kload / (uint32_t)p.stages) & 1) ^ 1, abort_flag,
-                                        p.status, kErrProducerK);
+                    ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProducerK);
                     if (!ok) break;
                     const bool tail = k == p.nblk_p - 1;
                     const int slab = tail ? tail_slab : C::kSlabBytes;
@@ -409,7 +407,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                                         bar(kBarKFull + ks), sl * 64, k * kBlockN, ph);
                     }
                     __syncwarp();
-                    ++kload;
+                    if (++ks == (uint32_t)p.stages) { ks = 0; kph ^= 1u; }
                 }
                 if (!ok) break;
             }
@@ -419,9 +417,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 const int nbs = items_of(t) - p.nblk_p;
 #pragma unroll 1
                 for (int j = 0; j < nbs; ++j) {
-                    const uint32_t ks = kload % (uint32_t)p.stages;
-                    ok = mbar_wait_warp(bar(kBarKFree + ks), ((kload / (uint32_t)p.stages) & 1) ^ 1, abort_flag,
-                                        p.status, kErrProducerK);
+                    ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProducerK);
                     if (!ok) break;
                     if (p.long_sfx) {
                         // keys [128 j, 128 j + 128) of the tile's candidate; rows past the cache are zero-filled
@@ -446,7 +442,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         }
                     }
                     __syncwarp();
-                    ++kload;
+                    if (++ks == (uint32_t)p.stages) { ks = 0; kph ^= 1u; }
                 }
                 if (!ok) break;
             } else {
@@ -497,7 +493,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         // last value MMA has read suffix V, and suffix V of tile t+1 is then fetched only once the
         // stores of tile t have read the staging buffer.
         const uint32_t stage = sbase + p.off_stage;
-        uint32_t vload = 0;
+        uint32_t vs = 0, vph = 1;  // ring of V blocks: stage, parity of its release
         int store_slab = 0;  // slab_stage: slabs of the previous tile's output stored so far
         bool ok = true;
 #pragma unroll 1
@@ -543,9 +539,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             while (ok && (k < nk || pend_store || pend_sv)) {
                 const bool block = k >= nk;  // nothing else left to do for this tile: wait for the jobs
                 if (k < nk) {
-                    const uint32_t vs = vload % (uint32_t)p.stages;
-                    ok = mbar_wait_warp(bar(kBarVFree + vs), ((vload / (uint32_t)p.stages) & 1) ^ 1, abort_flag,
-                                        p.status, kErrProducerV);
+                    ok = mbar_wait_warp(bar(kBarVFree + vs), vph, abort_flag, p.status, kErrProducerV);
                     if (!ok) break;
                     if (SR && k >= p.nblk_p) {
                         // a suffix V block: one box of Skv rows per candidate, Spad rows apart
@@ -584,7 +578,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         }
                     }
                     __syncwarp();
-                    ++vload;
+                    if (++vs == (uint32_t)p.stages) { vs = 0; vph ^= 1u; }
                     ++k;
                 }
                 bool sv_ready = false;
@@ -659,20 +653,28 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         __syncwarp();
     } else if (role == 1) {
         // ------------------------------------------------------------------ score MMAs: S = Q K^T
+        // An MMA is issued about when the one a few places ahead of it starts, so what a warp does between two of them costs the
+        // tensor cores nothing, and what it does between items does.  The next item is therefore worked out in the middle of
+        // this one's MMAs.  (Between them, with the ring positions by division, it took this warp 700 to 1 100 cycles per item and
+        // the value issuer as long, against 1 024 of MMAs: 256 candidates, 32/8 heads, P = 2048, S = 32 267-274 us, now 254-260.  A tile's
+        // first item worked out behind the MMAs instead, so that a short last block is not held up: 262, the compiler spills.)
         int tl = 0;
-        uint32_t kuse = 0;  // streaming mode: K blocks consumed from the ring
+        uint32_t ks = 0, kph = 0;        // ring of K blocks: stage, parity of its loads
+        uint32_t slot = 0, slot_ph = 1;  // score slot, parity of its release
         TileInfo t = tile_info<MI == 2>(p, tile_at(0), t_begin);
         int nitems = items_of(t);
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint64_t q_desc = make_smem_desc(sbase + p.off_q, 0, 1024);
         bool ok = true;
-        for (int i = 0; tl < n_tiles && ok; ++i) {
-            const int slot = i % kSlots;
-            // everything that does not depend on a wait comes first, so that it is out of the way
-            // when the waits return
-            uint32_t kaddr, kbar, kpar;
+        // the coming item
+        uint64_t k_desc, k_slab;
+        uint32_t idesc, kbar, kpar;
+        bool kwait, ring;
+        auto prepare = [&]() {
+            uint32_t kaddr;
             int n, slab;
-            bool kwait = true;
+            kwait = true;
+            ring = (k < p.nblk_p || SR) && !RES;
             if (k < p.nblk_p || SR) {
                 n = k < p.nblk_p ? prefix_block_rows(p, k)
                     : p.long_sfx ? sfx_long_rows(p, k - p.nblk_p) : sfx_block_rows(p, t.nc, k - p.nblk_p);
@@ -684,9 +686,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     kpar = (uint32_t)(run_of(t, inst) - run_first) & 1u;
                     kaddr = sbase + p.off_pk + k * C::kTileBytes;
                 } else {
-                    const uint32_t ks = kuse % (uint32_t)p.stages;
                     kbar = bar(kBarKFull + ks);
-                    kpar = (kuse / (uint32_t)p.stages) & 1u;
+                    kpar = kph;
                     kaddr = sbase + p.off_pk + ks * C::kTileBytes;
                 }
             } else {
@@ -696,26 +697,28 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 kpar = (uint32_t)tl & 1u;
                 kaddr = sbase + p.off_sk;
             }
-            const uint32_t idesc = make_idesc_bf16(kTileM, n, 0);
-            const uint32_t d_tmem = tmem + slot * kBlockN;
-            const uint64_t k_desc = make_smem_desc(kaddr, 0, 1024);
-            const uint64_t k_slab = (uint64_t)(slab >> 4);
-            const bool last_of_tile = k == nitems - 1;
-            const bool free_stage = (k < p.nblk_p || SR) && !RES;
-            // the slot is free once the value MMAs of item i-3 (which read P from it) have completed
+            idesc = make_idesc_bf16(kTileM, n, 0);
+            k_desc = make_smem_desc(kaddr, 0, 1024);
+            k_slab = (uint64_t)(slab >> 4);
+        };
+        if (n_tiles > 0) prepare();
+#pragma unroll 1
+        for (int i = 0; tl < n_tiles; ++i) {
+            // The slot is free once the value MMAs of item i-3 (which read P from it) have completed.  As a rule everything
+            // is there: looked at together the barriers cost one vote.
             PSKV_TRACE_EVENT(16, i);
-            ok = mbar_wait_warp(bar(kBarPvDone + slot), ((i / kSlots) & 1) ^ 1, abort_flag, p.status, kErrMmaQk);
-            if (!ok) break;
-            PSKV_TRACE_EVENT(18, i);
-            if (k == kfirst) {
-                ok = mbar_wait_warp(bar(kBarQFull), tl & 1, abort_flag, p.status, kErrMmaQk);
+            const bool qwait = k == kfirst;
+            bool ready = mbar_test_wait(bar(kBarPvDone + slot), slot_ph);
+            if (kwait) ready &= mbar_test_wait(kbar, kpar);
+            if (qwait) ready &= mbar_test_wait(bar(kBarQFull), tl & 1);
+            if (!__all_sync(0xffffffffu, ready)) {
+                ok = mbar_wait_warp(bar(kBarPvDone + slot), slot_ph, abort_flag, p.status, kErrMmaQk);
+                PSKV_TRACE_EVENT(18, i);
+                if (ok && qwait) ok = mbar_wait_warp(bar(kBarQFull), tl & 1, abort_flag, p.status, kErrMmaQk);
+                if (ok && kwait) ok = mbar_wait_warp(kbar, kpar, abort_flag, p.status, kErrMmaQk);
                 if (!ok) break;
             }
-            if (kwait) {
-                ok = mbar_wait_warp(kbar, kpar, abort_flag, p.status, kErrMmaQk);
-                if (!ok) break;
-            }
-            if (MI && RES && k == kfirst && first_of_run(t, inst_of(t))) {
+            if (MI && RES && qwait && first_of_run(t, inst_of(t))) {
                 // The resident copy of a run always loads every prefix block, also those this run skips as
                 // padding.  Nobody multiplies them, so their loads are waited for here: a load must have
                 // landed before its buffer and barrier are armed again for the next run, and before the
@@ -727,20 +730,23 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             }
             PSKV_TRACE_EVENT(10, i);
             tc_fence_after();
+            const uint32_t d_tmem = tmem + slot * kBlockN, idesc_i = idesc;
+            const uint64_t kd = k_desc, kslab = k_slab;
+            auto issue = [&](int ks16) {
+                const uint64_t qoff = (uint64_t)(((ks16 >> 2) * C::kSlabBytes + (ks16 & 3) * 32) >> 4);
+                const uint64_t koff = (uint64_t)(ks16 >> 2) * kslab + (uint64_t)(((ks16 & 3) * 32) >> 4);
+                mma_ss(d_tmem, q_desc + qoff, kd + koff, idesc_i, ks16 > 0 ? 1u : 0u);
+            };
+            constexpr int kSteps = D / 16, kAhead = kSteps * 3 / 4;
             if (elect_one_sync()) {
 #pragma unroll
-                for (int ks16 = 0; ks16 < D / 16; ++ks16) {
-                    const uint64_t qoff = (uint64_t)(((ks16 >> 2) * C::kSlabBytes + (ks16 & 3) * 32) >> 4);
-                    const uint64_t koff = (uint64_t)(ks16 >> 2) * k_slab + (uint64_t)(((ks16 & 3) * 32) >> 4);
-                    mma_ss(d_tmem, q_desc + qoff, k_desc + koff, idesc, ks16 > 0 ? 1u : 0u);
-                }
-                tc_commit(bar(kBarSFull + slot));
-                if (free_stage) tc_commit(bar(kBarKFree + (kuse % (uint32_t)p.stages)));
-                if (last_of_tile) tc_commit(bar(kBarQkFree));  // the suffix block ends the tile's scores
+                for (int ks16 = 0; ks16 < kAhead; ++ks16) issue(ks16);
             }
             __syncwarp();
-            PSKV_TRACE_EVENT(12, i);
-            if (free_stage) ++kuse;
+            const uint32_t full = bar(kBarSFull + slot), freed = ring ? bar(kBarKFree + ks) : 0u;
+            const bool last_of_tile = k == nitems - 1;
+            if (ring && ++ks == (uint32_t)p.stages) { ks = 0; kph ^= 1u; }
+            if (++slot == kSlots) { slot = 0; slot_ph ^= 1u; }
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
@@ -749,22 +755,37 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     k = kfirst = first_block(inst_of(t));
                 }
             }
+            prepare();  // (of no item behind the last one: nothing is read)
+            if (elect_one_sync()) {
+#pragma unroll
+                for (int ks16 = kAhead; ks16 < kSteps; ++ks16) issue(ks16);
+                tc_commit(full);
+                if (freed) tc_commit(freed);
+                if (last_of_tile) tc_commit(bar(kBarQkFree));  // the suffix block ends the tile's scores
+            }
+            __syncwarp();
+            PSKV_TRACE_EVENT(12, i);
         }
     } else if (role == 2) {
         // ------------------------------------------------------------------ value MMAs: O += P V
         int tl = 0;
-        uint32_t vuse = 0;
+        uint32_t vs = 0, vph = 0;        // ring of V blocks: stage, parity of its loads
+        uint32_t slot = 0, slot_ph = 0;  // score slot, parity of its probabilities
         TileInfo t = tile_info<MI == 2>(p, tile_at(0), t_begin);
         int nitems = items_of(t);
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint32_t idesc_pv = make_idesc_bf16(kTileM, D, 1);
         bool ok = true;
-        for (int i = 0; tl < n_tiles && ok; ++i) {
-            const int slot = i % kSlots;
-            // everything that does not depend on a wait comes first
-            uint32_t vaddr, vbar, vpar;
+        // the coming item (worked out in the middle of this one's MMAs, as above)
+        uint64_t v_desc;
+        uint32_t vbar, vpar;
+        int nk;
+        bool vwait, ring;
+        auto prepare = [&]() {
+            uint32_t vaddr;
             int n, slab;
-            bool vwait = true;
+            vwait = true;
+            ring = (k < p.nblk_p || SR) && !RES;
             if (k < p.nblk_p || SR) {
                 n = k < p.nblk_p ? prefix_block_rows(p, k)
                     : p.long_sfx ? sfx_long_rows(p, k - p.nblk_p) : sfx_block_rows(p, t.nc, k - p.nblk_p);
@@ -776,9 +797,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     vpar = (uint32_t)(run_of(t, inst) - run_first) & 1u;
                     vaddr = sbase + p.off_pv + k * C::kTileBytes;
                 } else {
-                    const uint32_t vs = vuse % (uint32_t)p.stages;
                     vbar = bar(kBarVFull + vs);
-                    vpar = (vuse / (uint32_t)p.stages) & 1u;
+                    vpar = vph;
                     vaddr = sbase + p.off_pv + vs * C::kTileBytes;
                 }
             } else {
@@ -788,27 +808,27 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 vpar = (uint32_t)tl & 1u;
                 vaddr = sbase + p.off_sv;
             }
-            const uint32_t p_tmem = tmem + slot * kBlockN;  // bf16 pairs: 8 columns per 16 keys
-            const uint64_t v_desc = make_smem_desc(vaddr, (uint32_t)slab, 1024);
-            const int nk = n >> 4;
-            const bool last_of_tile = k == nitems - 1;
-            const bool free_stage = (k < p.nblk_p || SR) && !RES;
-            const uint32_t acc0 = k > kfirst ? 1u : 0u;
+            v_desc = make_smem_desc(vaddr, (uint32_t)slab, 1024);
+            nk = n >> 4;
+        };
+        if (n_tiles > 0) prepare();
+#pragma unroll 1
+        for (int i = 0; tl < n_tiles; ++i) {
             PSKV_TRACE_EVENT(17, i);
-            ok = mbar_wait_warp(bar(kBarPReady + slot), (i / kSlots) & 1, abort_flag, p.status, kErrMmaPv);
-            if (!ok) break;
-            if (k == kfirst && tl > 0) {
-                // O of the previous tile must have been read out by the epilogue warps
+            // (O of the previous tile must have been read out by the epilogue warps)
+            const bool first = k == kfirst, owait = first && tl > 0;
+            bool ready = mbar_test_wait(bar(kBarPReady + slot), slot_ph);
+            if (vwait) ready &= mbar_test_wait(vbar, vpar);
+            if (owait) ready &= mbar_test_wait(bar(kBarOFree), (tl - 1) & 1);
+            if (!__all_sync(0xffffffffu, ready)) {
+                ok = mbar_wait_warp(bar(kBarPReady + slot), slot_ph, abort_flag, p.status, kErrMmaPv);
                 PSKV_TRACE_EVENT(15, i);
-                ok = mbar_wait_warp(bar(kBarOFree), (tl - 1) & 1, abort_flag, p.status, kErrMmaPv);
-                if (!ok) break;
-            }
-            if (vwait) {
+                if (ok && owait) ok = mbar_wait_warp(bar(kBarOFree), (tl - 1) & 1, abort_flag, p.status, kErrMmaPv);
                 PSKV_TRACE_EVENT(14, i);
-                ok = mbar_wait_warp(vbar, vpar, abort_flag, p.status, kErrMmaPv);
+                if (ok && vwait) ok = mbar_wait_warp(vbar, vpar, abort_flag, p.status, kErrMmaPv);
                 if (!ok) break;
             }
-            if (MI && RES && k == kfirst && first_of_run(t, inst_of(t))) {  // (as for the K blocks above)
+            if (MI && RES && first && first_of_run(t, inst_of(t))) {  // (as for the K blocks above)
                 const uint32_t par = (uint32_t)(run_of(t, inst_of(t)) - run_first) & 1u;
                 for (int kk = 0; kk < kfirst && kk < p.nblk_p && ok; ++kk)
                     ok = mbar_wait_warp(bar(kBarVFull + kk), par, abort_flag, p.status, kErrMmaPv);
@@ -816,26 +836,27 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             }
             PSKV_TRACE_EVENT(11, i);
             tc_fence_after();
+            const uint32_t p_tmem = tmem + slot * kBlockN;  // bf16 pairs: 8 columns per 16 keys
+            const uint32_t acc0 = first ? 0u : 1u;
+            const uint64_t vd = v_desc;
+            const int steps = nk;
+            auto issue = [&](int ks16) {
+                if (ks16 >= steps) return;
+                const uint32_t p_cols = p_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8;
+                const uint64_t v_rows = vd + (uint64_t)(ks16 * (2048 >> 4));
+                mma_ts(tmem + kOCol, p_cols, v_rows, idesc_pv, ks16 > 0 ? 1u : acc0);
+                if (TWO) mma_ts(tmem + kOCol, p_cols + kPiece / 2, v_rows, idesc_pv, 1u);
+            };
+            constexpr int kSteps = kBlockN / 16, kAhead = kSteps * 3 / 4;
             if (elect_one_sync()) {
 #pragma unroll
-                for (int ks16 = 0; ks16 < kBlockN / 16; ++ks16) {
-                    if (ks16 < nk) {
-                        const uint32_t p_cols = p_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8;
-                        const uint64_t v_rows = v_desc + (uint64_t)(ks16 * (2048 >> 4));
-                        mma_ts(tmem + kOCol, p_cols, v_rows, idesc_pv, ks16 > 0 ? 1u : acc0);
-                        if (TWO) mma_ts(tmem + kOCol, p_cols + kPiece / 2, v_rows, idesc_pv, 1u);
-                    }
-                }
-                tc_commit(bar(kBarPvDone + slot));
-                if (free_stage) tc_commit(bar(kBarVFree + (vuse % (uint32_t)p.stages)));
-                if (last_of_tile) {
-                    tc_commit(bar(kBarSVFree));
-                    tc_commit(bar(kBarOFull));
-                }
+                for (int ks16 = 0; ks16 < kAhead; ++ks16) issue(ks16);
             }
             __syncwarp();
-            PSKV_TRACE_EVENT(13, i);
-            if (free_stage) ++vuse;
+            const uint32_t done = bar(kBarPvDone + slot), freed = ring ? bar(kBarVFree + vs) : 0u;
+            const bool last_of_tile = k == nitems - 1;
+            if (ring && ++vs == (uint32_t)p.stages) { vs = 0; vph ^= 1u; }
+            if (++slot == kSlots) { slot = 0; slot_ph ^= 1u; }
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
@@ -844,6 +865,19 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     k = kfirst = first_block(inst_of(t));
                 }
             }
+            prepare();
+            if (elect_one_sync()) {
+#pragma unroll
+                for (int ks16 = kAhead; ks16 < kSteps; ++ks16) issue(ks16);
+                tc_commit(done);
+                if (freed) tc_commit(freed);
+                if (last_of_tile) {
+                    tc_commit(bar(kBarSVFree));
+                    tc_commit(bar(kBarOFull));
+                }
+            }
+            __syncwarp();
+            PSKV_TRACE_EVENT(13, i);
         }
     } else if (warp < 4 + 4 * kGroups) {
         // ------------------------------------------------------------------ softmax warps (4..19)
