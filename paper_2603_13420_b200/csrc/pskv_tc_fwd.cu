@@ -1621,7 +1621,9 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
 
         static PerDeviceOnce attr_set[9];
         if (cudaError_t e = ensure_max_smem(kernel, attr_set[slot]); e != cudaSuccess) return e;
-        const int grid = even_grid(p.total_tiles, sm_count());
+        // Tiles dealt by cost go to every SM: the 512 tiles of a prompt of 2048 tokens, 32 heads, put 34 key blocks on the
+        // busiest of 128 CTAs of four tiles, 30 on the busiest of 148.
+        const int grid = p.deal_by_cost ? (p.total_tiles < sm_count() ? p.total_tiles : sm_count()) : even_grid(p.total_tiles, sm_count());
         cudaError_t launch_err;
         {
             KernelTiming timing(kKernelFwdTc, stream);
