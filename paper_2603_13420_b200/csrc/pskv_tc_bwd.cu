@@ -2,7 +2,7 @@
 //   dQ        = scale * sum_j dS_j K_j              over the shared prefix keys and the visible suffix keys
 //   dK_suffix = scale * sum over rows of dS^T Q     (suffix keys only: the prefix cache is frozen, Sec. 4.2)
 //   dV_suffix =         sum over rows of  P^T dO
-//   with P = exp(S - lse), S = scale Q K^T, dP = dO V^T, dS = P o (dP - D), D = <dO, O> (a pre-pass, or in here: DROW).
+//   with P = exp(S - lse), S = scale Q K^T, dP = dO V^T, dS = P o (dP - D), D = <dO, O> (a pre-pass, or in here: DSource).
 // Q and dO are fetched once; nothing is read or recomputed twice except in the passes named below.
 //
 // A CTA works on units.  A unit is `cu` neighbouring candidates of one KV head, so that the sums over rows
@@ -85,7 +85,7 @@ enum : unsigned int {
 
 struct TcBwdParams {
     const float *lse;      // [B*Hq*S] from the forward pass
-    const float *row_dot;  // [B*Hq*S] D, or (DROW) what it is formed from:
+    const float *row_dot;  // [B*Hq*S] D, or (kDWarps) what it is formed from:
     const __nv_bfloat16 *out, *dout;
     const float *dlse;     // gradient on lse, or nullptr
     __nv_bfloat16 *dq;       // [B,Hq,S,d]
@@ -116,6 +116,10 @@ struct TcBwdParams {
     int pad[kMaxInstr];    // left padding of each instruction's prefix cache (Sec. 4.3)
 };
 
+// Where the row statistic D comes from: a pre-pass over dout and out; the element-wise warps, plain FMAs under the first copies
+// (every CTA has one tile); an item of its own in front of a tile's others, whose scores are dO O^T.
+enum DSource { kDTable = 0, kDWarps = 1, kDItem = 2 };
+
 template <int D>
 struct Cfg {
     static constexpr int kSlabs = D / 64;              // 64-column (128-byte) swizzle slabs per row
@@ -139,7 +143,8 @@ enum {
     kBarDsReady = kBarSFree + 2,     // [2] dS (and P) of an item are in shared memory (8 arrivals)
     kBarDsFree = kBarDsReady + 2,    // [2] the MMAs that read dS have completed
     kBarRowsFull = kBarDsFree + 2,   // [2] the row table of a tile is written
-    kBarKFull = kBarRowsFull + 2,    // (also: the item's descriptor is written)
+    kBarDFull = kBarRowsFull + 2,    // [2] kDItem: D is in the row table (8 arrivals)
+    kBarKFull = kBarDFull + 2,       // (also: the item's descriptor is written)
     kBarVFull = kBarKFull + kMaxRing,
     kBarKFree = kBarVFull + kMaxRing,
     kBarVFree = kBarKFree + kMaxRing,
@@ -160,6 +165,7 @@ enum : uint32_t {
     kDescLast = 1u << 12, kDescDq = 1u << 13, kDescFirst = 1u << 14,
     kDescAccOdd = 1u << 15,    // parity of the items that fed dK / dV so far
     kDescK0 = 16, kDescK1 = 20,  // rows of the group inside the tile, in steps of 16 (4 bits each)
+    kDescRowDot = 1u << 24,      // the item of the tile's row statistic (x holds nothing else)
     kDescEnd = 1u << 31
 };
 
@@ -281,17 +287,17 @@ __device__ __forceinline__ void store_sector(__nv_bfloat16 *dst, const uint32_t 
 }
 
 // Eight values as bf16; `two`: with what the rounding leaves (exact in fp32) as bf16 in the buffer behind.
-__device__ __forceinline__ void store_terms(uint8_t *dst, const float *x, bool two)
+__device__ __forceinline__ void store_terms(uint32_t dst, const float *x, bool two)
 {
     uint32_t hi[4], lo[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) hi[i] = pack_bf16x2(x[2 * i], x[2 * i + 1]);
-    *reinterpret_cast<uint4 *>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    st_shared_v4(dst, hi);
     if (!two) return;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
         lo[i] = pack_bf16x2(x[2 * i] - __uint_as_float(hi[i] << 16), x[2 * i + 1] - __uint_as_float(hi[i] & 0xffff0000u));
-    *reinterpret_cast<uint4 *>(dst + kDsBytes) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    st_shared_v4(dst + kDsBytes, lo);
 }
 
 // The rows [first, first + 8) of a CTA's one tile: (-lse log2(e), D) into the row table, D = <dout, out> less the
@@ -334,16 +340,18 @@ __device__ __forceinline__ void row_dots(const TcBwdParams &p, int b0, int g, in
     }
 }
 
-// DROW: every CTA has one tile, and forms its D itself instead of reading it from a pre-pass.  TWO: P and dS as two terms.
-template <int D, bool SPLIT, bool DROW, bool TWO>
+// DSRC: where D comes from (DSource).  TWO: P and dS as two terms.
+template <int D, bool SPLIT, int DSRC, bool TWO>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
               const __grid_constant__ CUtensorMap tm_pk, const __grid_constant__ CUtensorMap tm_pv,
               const __grid_constant__ CUtensorMap tm_sk, const __grid_constant__ CUtensorMap tm_sv,
-              const __grid_constant__ TcBwdParams p)
+              const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ TcBwdParams p)
 {
     using C = Cfg<D>;
+    constexpr bool DROW = DSRC == kDWarps, DOT = DSRC == kDItem;
     constexpr int kTerms = TWO ? 2 : 1;
+    constexpr bool kEight = TWO || (DOT);
     constexpr uint64_t kLoTerm = (uint64_t)(kDsBytes >> 4);  // descriptor distance from a P / dS buffer to its second term
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -370,7 +378,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         for (int i = lane; i < kNumBars; i += 32) {
             const bool epi = i == kBarDqFree || i == kBarAccFree;
             const bool elem = (i >= kBarSFree && i < kBarSFree + 2) || (i >= kBarDsReady && i < kBarDsReady + 2);
-            mbar_init(bar(i), elem ? 8u : epi ? 4u : i == kBarQFree ? 2u : DROW && i == kBarRowsFull ? 16u : 1u);
+            mbar_init(bar(i), elem || (i >= kBarDFull && i < kBarDFull + 2) ? 8u : epi ? 4u : i == kBarQFree ? 2u : DROW && i == kBarRowsFull ? 16u : 1u);
         }
         if (lane == 0) *abort_flag = 0;
         fence_barrier_init();
@@ -405,6 +413,30 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll 1
         for (; !w.done() && ok; w.next_tile(p), ++tile) {
             const int head = w.inst * p.Hkv + w.g;
+            if (DOT) {
+                // the item of the row statistic: rows of `out`, columns 0-63 into a K stage, 64-127 into a V stage
+                const int step = p.seg * p.cbox, nb = (w.rows + step - 1) / step;
+                const int R = w.R0 + lane * step, c = p.fd_Rp.div(R), r = R - c * p.Rp;
+                ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProdKv);
+                if (ok) ok = mbar_wait_warp(bar(kBarVFree + vs), vph, abort_flag, p.status, kErrProdKv);
+                if (!ok) break;
+                const uint32_t kb = bar(kBarKFull + ks), vb = bar(kBarVFull + vs);
+                if (lane == 0) {
+                    descs[item & 7u] = make_uint4(kDescRowDot, 0u, 0u, (tile & 0xffffu) | (uint32_t)w.tt << 16);
+                    mbar_arrive_expect_tx(kb, (uint32_t)(nb * step * 128));
+                    mbar_arrive_expect_tx(vb, (uint32_t)(nb * step * 128));
+                }
+                __syncwarp();
+                if (lane < nb) {
+                    const uint32_t off = (uint32_t)(lane * step * 128);
+                    tma_load_4d(sbase + p.off_k + ks * C::kPieceBytes + off, &tm_out, kb, 0, r, w.g, w.b0 + c);
+                    tma_load_4d(sbase + p.off_v + vs * C::kPieceBytes + off, &tm_out, vb, 64, r, w.g, w.b0 + c);
+                }
+                __syncwarp();
+                if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
+                if (++vs == p.stages_v) { vs = 0; vph ^= 1u; }
+                ++item;
+            }
             // suffix items are spread evenly over the tile's items, the first one first: their accumulators are drained, and
             // their P buffer is read, under the prefix items in between
             int e = 0, j = 0, q = 0;
@@ -503,7 +535,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 const bool v = row < w.rows && r < p.Rg;
                 const size_t at = ((size_t)(w.b0 + c) * p.Hq + (size_t)w.g * p.n_rep) * p.S + r;
                 st[i] = v ? -p.lse[at] * kLog2e : -INFINITY;
-                dr[i] = v ? p.row_dot[at] : 0.f;
+                dr[i] = v && !DOT ? p.row_dot[at] : 0.f;
             }
             const int nb = (w.rows + step - 1) / step;
             const int R = w.R0 + lane * step;
@@ -546,7 +578,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 // Table tile & 1 was last read for tile - 2; the MMAs behind kBarQFree of tile - 1 came after that.
                 float2 *rows = reinterpret_cast<float2 *>(smem + p.off_rows) + (tile & 1u) * kTileM;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) rows[32 * i + lane] = make_float2(st[i], dr[i]);
+                for (int i = 0; i < 4; ++i) {
+                    if (DOT) rows[32 * i + lane].x = st[i];  // (the element-wise warps add D)
+                    else rows[32 * i + lane] = make_float2(st[i], dr[i]);
+                }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBarRowsFull + (tile & 1u)));
             }
@@ -572,7 +607,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (x & kDescEnd) break;
             const uint32_t idesc = make_idesc_bf16(kTileM, (int)(x & kDescN), 0);
             const uint32_t tile_ph = descs[item & 7u].w & 1u;
-            if (x & kDescFirst) ok = mbar_wait_warp(bar(SPLIT ? kBarQFull : kBarDoFull), tile_ph, abort_flag, p.status, kErrMmaS);
+            if (x & (DOT ? kDescRowDot : kDescFirst)) ok = mbar_wait_warp(bar(SPLIT ? kBarQFull : kBarDoFull), tile_ph, abort_flag, p.status, kErrMmaS);
             if (ok) ok = mbar_wait_warp(bar(kBarSFree + slot), ((item >> 1) & 1u) ^ 1u, abort_flag, p.status, kErrMmaS);
             if (ok) ok = mbar_wait_warp(bar(kBarVFull + vs), vph, abort_flag, p.status, kErrMmaS);
             if (!ok) break;
@@ -583,6 +618,23 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // 58 candidates, 32/32 heads, P = 1735, S = 66 601 -> 569 us, 61, 32/32, P = 1206, S = 54 314 -> 303, 14, 32/32, P = 417, S =
             // 123 97 -> 94; in one term and on small launches no change.  (Split launches have few items to a tile; waiting for
             // the two in turn costs them more: one candidate, 32/8, P = 78, S = 113 27.9 -> 28.8.)
+            if (DOT && (x & kDescRowDot)) {
+                // dO O^T over the whole slot: 64 columns of O from the K stage, 64 from the V stage
+                if (elect_one_sync()) {
+                    constexpr uint32_t idesc_dot = make_idesc_bf16(kTileM, kTileM, 0);
+#pragma unroll 1
+                    for (uint32_t i = 0; i < D / 32; ++i) mma_ss(d_tmem, do_desc + 2 * i, k_desc + 2 * i, idesc_dot, i);
+#pragma unroll 1
+                    for (uint32_t i = 0; i < D / 32; ++i)
+                        mma_ss(d_tmem, do_desc + (C::kSlabBytes >> 4) + 2 * i, v_desc + 2 * i, idesc_dot, 1u);
+                    tc_commit(bar(kBarSFull + slot));
+                    tc_commit(bar(kBarVFree + vs));
+                }
+                __syncwarp();
+                if (++ks == p.stages_k) { ks = 0; kph ^= 1u; }
+                if (++vs == p.stages_v) { vs = 0; vph ^= 1u; }
+                continue;
+            }
             if (elect_one_sync()) {
 #pragma unroll
                 for (int i = 0; i < D / 16; ++i) {
@@ -703,9 +755,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         const int c0 = ((warp >> 2) & 1) ? 0 : 32;   // my 32 of the piece's 64 keys
         const int row = 32 * (warp & 3) + lane;
         const uint32_t my_tmem = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + set * kSlotCols + c0;
-        uint8_t *p_row = smem + p.off_p + row * 128;
-        uint8_t *ds_row = smem + p.off_ds + set * kTerms * kDsBytes + row * 128;
-        const uint4 *descs = reinterpret_cast<const uint4 *>(smem + p.off_bar + kDescOff);
+        // (32-bit addresses: the loop has no registers to spare)
+        const uint32_t p_row = sbase + p.off_p + row * 128;
+        const uint32_t ds_row = sbase + p.off_ds + set * kTerms * kDsBytes + row * 128;
+        const uint32_t descs = bar0 + kDescOff, rows_at = sbase + p.off_rows + row * 8;
         int ks = set;
         uint32_t kph = 0, tile = 0xffffffffu;  // (no tile has this number and index)
         if (ks >= p.stages_k) { ks -= p.stages_k; kph ^= 1u; }
@@ -723,18 +776,48 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             PSKV_TRACE_EVENT(26, item);
             ok = mbar_wait_warp(bar(kBarKFull + ks), kph, abort_flag, p.status, kErrElem);
             if (!ok) break;
-            const uint4 dsc = descs[item & 7u];
+            const uint4 dsc = ld_shared_v4(descs + (item & 7u) * 16);
             if (dsc.x & kDescEnd) break;
             ks += 2;
             if (ks >= p.stages_k) {
                 ks -= p.stages_k;
                 kph ^= 1u;
             }
+            if (DOT && (dsc.x & kDescRowDot)) {
+                // Rows 32 q .. 32 q + 31 have their diagonal in columns 32 q .. 32 q + 31 of the slot; my sixteen of them are
+                // those of lanes c0 / 2 .. c0 / 2 + 15.  Rows that do not exist (-lse is -infinity) get 0.
+                ok = mbar_wait_warp(bar(kBarSFull + set), sph, abort_flag, p.status, kErrElem);
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t rs[16];
+                tmem_ld16(my_tmem - c0 + 32 * (warp & 3) + (c0 >> 1), rs);
+                tmem_wait_ld();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kBarSFree + set));
+#pragma unroll
+                for (int h = 8; h > 0; h >>= 1)
+#pragma unroll
+                    for (int i = 0; i < h; ++i) rs[i] = (lane & h) ? rs[i + h] : rs[i];
+                ok = mbar_wait_warp(bar(kBarRowsFull + (dsc.w & 1u)), (dsc.w >> 1) & 1u, abort_flag, p.status, kErrElem);
+                if (!ok) break;
+                if ((lane & 16) == (c0 >> 1)) {
+                    const uint32_t at = rows_at + (dsc.w & 1u) * (kTileM * 8);
+                    st_shared_f(at + 4, ld_shared_f(at) == -INFINITY ? 0.f : __uint_as_float(rs[0]));
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kBarDFull + (dsc.w & 1u)));
+                // (nothing was written to dS, but its barriers go on item by item)
+                ok = mbar_wait_warp(bar(kBarDsFree + set), sph ^ 1u, abort_flag, p.status, kErrElem);
+                if (!ok) break;
+                if (lane == 0) mbar_arrive(bar(kBarDsReady + set));
+                continue;
+            }
             if (dsc.w != tile) {
                 tile = dsc.w;
-                ok = mbar_wait_warp(bar(kBarRowsFull + (tile & 1u)), (tile >> 1) & 1u, abort_flag, p.status, kErrElem);
+                ok = mbar_wait_warp(bar((DOT ? kBarDFull : kBarRowsFull) + (tile & 1u)), (tile >> 1) & 1u, abort_flag, p.status, kErrElem);
                 if (!ok) break;
-                const float2 rt = reinterpret_cast<const float2 *>(smem + p.off_rows)[(tile & 1u) * kTileM + row];
+                const float2 rt = ld_shared_f2(rows_at + (tile & 1u) * (kTileM * 8));
                 neg_lse2 = rt.x;
                 drow = rt.y;
                 // candidate group of my row, first key column of its candidate in the piece, last visible one
@@ -779,7 +862,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kBarSFree + set));
                 }
-                if (TWO) {
+                if (kEight) {
                     // eight columns at a time, stored as they are made (the waits first): with sixteen of P and dS held in
                     // fp32 across the waits the loop spilled
                     if (hf == 0) {
@@ -791,7 +874,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         PSKV_TRACE_EVENT(22, item);
                     }
                     if (kind == 0) continue;
-                    const bool lo_term = acc || p.dq_two;
+                    const bool lo_term = TWO && (acc || p.dq_two);
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         float e[8], ds[8];
@@ -823,7 +906,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         }
                         const int off = (((c0 >> 3) + 2 * hf + i) ^ (row & 7)) << 4;
                         store_terms(ds_row + off, ds, lo_term);
-                        if (acc) store_terms(p_row + off, e, true);
+                        if (acc) store_terms(p_row + off, e, TWO);
                     }
                     continue;
                 }
@@ -868,9 +951,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         const int off = (((c0 >> 3) + 2 * hf + i) ^ (row & 7)) << 4;
-                        *reinterpret_cast<uint4 *>(ds_row + off) = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
-                        if (acc)
-                            *reinterpret_cast<uint4 *>(p_row + off) = make_uint4(pp[4 * i], pp[4 * i + 1], pp[4 * i + 2], pp[4 * i + 3]);
+                        st_shared_v4(ds_row + off, pk + 4 * i);
+                        if (acc) st_shared_v4(p_row + off, pp + 4 * i);
                     }
                 }
             }
@@ -1052,7 +1134,8 @@ BwdPlan make_plan(const Dims &dm, int n_instr)
             pl.seg = tiles == 1 ? pl.Rp : kTileM;
         }
     }
-    pl.sfx_box = pl.nh > 1 ? kPieceN : pl.Sp;
+    // (a box of one candidate reaches past its last key, where it is filled with zeros)
+    pl.sfx_box = pl.nh > 1 ? kPieceN : pl.cpp == 1 ? round_up(pl.Sp, 16) : pl.Sp;
     pl.upi = (Kq + pl.cu - 1) / pl.cu;
     const int slabs = dm.d / 64;
     const int tile_bytes = slabs * kTileM * 128, piece_bytes = slabs * kPieceN * 128;
@@ -1084,24 +1167,38 @@ const BwdPlan &plan_bwd(const Dims &dm, int n_instr)
     return table.get(dm, n_instr, [&] { return make_plan(dm, n_instr); });
 }
 
-// D in the kernel: the smallest launches, whose CTAs have one tile each.  Its loads then run under those of the tile's
+// Where D is formed.
+// By the element-wise warps on the smallest launches, whose CTAs have one tile each.  Its loads then run under those of the tile's
 // operands, and a launch in the chain of three goes away.  Whole steps, gradients in one term, with the pre-pass and with D in here: 8 candidates, 4/4
 // heads, d = 64, P = 32, S = 8 14.1 and 12.0 us; 9, 32/8 heads, P = 256, S = 30 21.8 and 18.2; 2, 32/32 heads, P = 200, S =
 // 128 24.3 and 21.6, P = 300, S = 50 21.7 and 21.2.  With several tiles per CTA every tile waits for its own D: 1
 // candidate, 32/8 heads, P = 78, S = 113 (four tiles in a unit) 25.3 and 28.8, 12 candidates, 32/32 heads, P = 90, S = 77
 // (three units per CTA) 38.7 and 43.9.
-bool row_dot_in_kernel(const Dims &dm, const BwdPlan &plan)
+// As an item of its own on larger ones: 512 MMA cycles and one hand-off per tile instead of a pass over dout and out at the rate
+// of HBM and its launch.  Whole steps, pre-pass and item: 512 candidates, 32/8 heads, P = 256, S = 48 528 and 510 us, 8 x 64 in instructions 525 and
+// 508; 16, 32/32, P = 150, S = 55 42.7 and 40.7; 49, 32/8, P = 108, S = 47 57 and 53; no change where HBM is the
+// bound (128, 32/32, P = 160, S = 40 145 and 147).  Not where a tile is walked over several times or in parts, which would form
+// its D again each time (44, 32/8, P = 51, S = 87 113 and 120; one candidate, P = 78, S = 113 28 and 31), nor where `out` comes in
+// many small boxes (500, 32/32, P = 211, S = 10, boxes of 16 rows 237 and 245).
+DSource d_source(const BwdArgs &a, const BwdPlan &plan, int n_instr)
 {
-    return plan.cu * plan.Rp <= kTileM && (long long)plan.upi * dm.Hkv * plan.n_sub <= sm_count();
+    const Dims &dm = a.dims;
+    const long long units = (long long)plan.upi * n_instr * dm.Hkv * plan.n_sub;
+    if (n_instr == 1 && plan.cu * plan.Rp <= kTileM && units <= sm_count()) return kDWarps;
+    // (The MMAs read K and V stages in steps of 16 keys, and `out` passes through the same stages: boxes of whole steps leave nothing
+    // of it to be read.  Calls of several instructions below four units per SM stay the two launches they are known as.)
+    const bool can = dm.d == 128 && !a.dlse && plan.n_sub == 1 && plan.nh == 1 && plan.sfx_box * plan.cpp % 16 == 0;
+    return can && plan.seg * plan.cbox >= 24 && (n_instr == 1 || units >= 4ll * sm_count()) ? kDItem : kDTable;
 }
 
 template <int D, bool TWO>
 cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_word, cudaStream_t stream, int n_instr,
-                   const int *prefix_len, bool drow)
+                   const int *prefix_len, DSource dsrc)
 {
     const Dims &dm = a.dims;
     const int Rg = dm.n_rep * dm.S;
-    CUtensorMap tm_q, tm_do, tm_pk, tm_pv, tm_sk, tm_sv;
+    CUtensorMap tm_q, tm_do, tm_pk, tm_pv, tm_sk, tm_sv, tm_out;
+    memset(&tm_out, 0, sizeof(tm_out));
     memset(&tm_pk, 0, sizeof(tm_pk));
     memset(&tm_pv, 0, sizeof(tm_pv));
     {
@@ -1112,6 +1209,7 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
         cuuint32_t box[4] = {64, (cuuint32_t)plan.seg, 1, (cuuint32_t)plan.cbox};
         if (!encode_map(&tm_q, a.q, 4, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode_map(&tm_do, a.dout, 4, dims, str, box)) return cudaErrorInvalidValue;
+        if (dsrc == kDItem && !encode_map(&tm_out, a.out, 4, dims, str, box)) return cudaErrorInvalidValue;
     }
     {
         cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)dm.S, (cuuint64_t)dm.Hkv, (cuuint64_t)dm.B};
@@ -1166,16 +1264,18 @@ cudaError_t launch(const BwdArgs &a, const BwdPlan &plan, unsigned int *status_w
     for (int i = 0; i < n_instr && n_instr > 1; ++i) p.pad[i] = dm.P - prefix_len[i];
 
     const bool sp = plan.n_sub > 1;
-    auto kernel = drow ? (sp ? tc_bwd_kernel<D, true, true, TWO> : tc_bwd_kernel<D, false, true, TWO>)
-                       : (sp ? tc_bwd_kernel<D, true, false, TWO> : tc_bwd_kernel<D, false, false, TWO>);
-    static PerDeviceOnce attr_set[4];
-    if (cudaError_t e = ensure_max_smem(kernel, attr_set[2 * drow + sp]); e != cudaSuccess) return e;
+    auto kernel = sp ? tc_bwd_kernel<D, true, kDTable, TWO> : tc_bwd_kernel<D, false, kDTable, TWO>;
+    if (dsrc == kDWarps) kernel = sp ? tc_bwd_kernel<D, true, kDWarps, TWO> : tc_bwd_kernel<D, false, kDWarps, TWO>;
+    if constexpr (D == 128)
+        if (dsrc == kDItem) kernel = tc_bwd_kernel<D, false, kDItem, TWO>;
+    static PerDeviceOnce attr_set[6];
+    if (cudaError_t e = ensure_max_smem(kernel, attr_set[2 * dsrc + sp]); e != cudaSuccess) return e;
     p.n_units = p.upg * dm.Hkv * p.n_sub;
     cudaError_t e;
     {
         KernelTiming timing(kKernelBwdTc, stream);
         e = launch_dependent(kernel, even_grid(p.n_units, sm_count()), kThreads, plan.smem_bytes, stream, tm_q, tm_do, tm_pk, tm_pv,
-                             tm_sk, tm_sv, p);
+                             tm_sk, tm_sv, tm_out, p);
     }
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1225,15 +1325,15 @@ cudaError_t launch_tc_bwd(const BwdArgs &a, unsigned int *status_word, cudaStrea
     if (n_instr > 1 && (!prefix_len || !tc_bwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
     const BwdPlan &plan = plan_bwd(a.dims, n_instr);
     if (!plan.ok) return cudaErrorInvalidValue;
-    const bool drow = parts == kBwdPartAll && n_instr == 1 && row_dot_in_kernel(a.dims, plan);
-    if ((parts & kBwdPartRowDot) && !drow) {
+    const DSource dsrc = parts == kBwdPartAll ? d_source(a, plan, n_instr) : kDTable;
+    if ((parts & kBwdPartRowDot) && dsrc == kDTable) {
         const cudaError_t e = launch_simt_row_dot(a, stream);
         if (e != cudaSuccess) return e;
     }
     if (!(parts & kBwdPartGrad)) return cudaSuccess;
     auto run = plan.terms == 2 ? (a.dims.d == 128 ? launch<128, true> : launch<64, true>)
                                : (a.dims.d == 128 ? launch<128, false> : launch<64, false>);
-    return run(a, plan, status_word, stream, n_instr, prefix_len, drow);
+    return run(a, plan, status_word, stream, n_instr, prefix_len, dsrc);
 }
 
 }  // namespace pskv
