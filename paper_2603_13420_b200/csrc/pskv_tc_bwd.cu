@@ -1176,8 +1176,10 @@ const BwdPlan &plan_bwd(const Dims &dm, int n_instr)
 // (three units per CTA) 38.7 and 43.9.
 // As an item of its own on larger ones: 512 MMA cycles and one hand-off per tile instead of a pass over dout and out at the rate
 // of HBM and its launch.  Whole steps, pre-pass and item: 512 candidates, 32/8 heads, P = 256, S = 48 528 and 510 us, 8 x 64 in instructions 525 and
-// 508; 16, 32/32, P = 150, S = 55 42.7 and 40.7; 49, 32/8, P = 108, S = 47 57 and 53; no change where HBM is the
-// bound (128, 32/32, P = 160, S = 40 145 and 147).  Not where a tile is walked over several times or in parts, which would form
+// 508; 49, 32/8, P = 108, S = 47 57 and 53; with one tile to a unit on launches of few units 16, 32/32, P = 150, S = 55 42.7 and 40.7; 60,
+// P = 128, S = 30 (480 units) 66.8 and 64.9.  Such units are short, and beyond about four per SM the hand-off costs as much
+// as the pass or more: 60, 32/32, P = 256, S = 47 (960) 122.6 and 123.7; 128, P = 160, S = 40 (1376) 145.7 and 148.0.  Not where a
+// tile is walked over several times or in parts, which would form
 // its D again each time (44, 32/8, P = 51, S = 87 113 and 120; one candidate, P = 78, S = 113 28 and 31), nor where `out` comes in
 // many small boxes (500, 32/32, P = 211, S = 10, boxes of 16 rows 237 and 245).
 DSource d_source(const BwdArgs &a, const BwdPlan &plan, int n_instr)
@@ -1188,7 +1190,8 @@ DSource d_source(const BwdArgs &a, const BwdPlan &plan, int n_instr)
     // (The MMAs read K and V stages in steps of 16 keys, and `out` passes through the same stages: boxes of whole steps leave nothing
     // of it to be read.  Calls of several instructions below four units per SM stay the two launches they are known as.)
     const bool can = dm.d == 128 && !a.dlse && plan.n_sub == 1 && plan.nh == 1 && plan.sfx_box * plan.cpp % 16 == 0;
-    return can && plan.seg * plan.cbox >= 24 && (n_instr == 1 || units >= 4ll * sm_count()) ? kDItem : kDTable;
+    const bool many = units >= 4ll * sm_count(), one_tile = plan.cu * plan.Rp <= kTileM;
+    return can && plan.seg * plan.cbox >= 24 && !(one_tile && many) && (n_instr == 1 || many) ? kDItem : kDTable;
 }
 
 template <int D, bool TWO>

@@ -14,10 +14,11 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("shape, launches", [
     # B, Hq, Hkv, d, P, S
-    ((300, 4, 4, 128, 40, 40), 1),     # three candidates in one box of 120 rows
+    ((300, 4, 4, 128, 40, 40), 1),     # three candidates in one box of 120 rows, 400 units
+    ((500, 4, 4, 128, 40, 40), 2),     # ... 668 units, more than four per SM: the pre-pass
     ((260, 8, 2, 128, 65, 48), 1),     # tiles straddle two candidates: boxes of 64 rows
     ((600, 3, 3, 128, 0, 24), 1),      # no prefix; two candidates to a key piece
-    ((333, 4, 2, 128, 17, 53), 1),     # two terms; padded rows and keys
+    ((250, 4, 2, 128, 17, 53), 1),     # two terms; padded rows and keys
     ((149, 1, 1, 128, 130, 64), 1),    # one unit more than SMs, half of each tile's rows do not exist
     ((300, 4, 4, 128, 40, 72), 2),     # two key pieces: the pre-pass
     ((300, 4, 4, 64, 40, 40), 2),      # head dim 64: the pre-pass
