@@ -175,8 +175,8 @@ long long pskv_attn_bwd_static_max_rows(void);
  * With Bp <= 64 one launch may serve all instructions (pskv_set_multi_form(2) turns this off); forward and
  * backward decide by themselves.  The forward does where the suffix keys of a row tile fit one 128-key block
  * and an instruction's rows, as the kernel pads them, are a whole number of tiles or at least four; the backward
- * on every shape of the tensor-core kernel with Pmax >= 1 (one launch for the row statistic, one for the three
- * gradients).  Otherwise the work is one pass per instruction; the passes are independent, so every
+ * on every shape of the tensor-core kernel with Pmax >= 1 (one launch for the three gradients, which on large calls
+ * forms the row statistic too; else one more for that).  Otherwise the work is one pass per instruction; the passes are independent, so every
  * other one is enqueued on a stream of the library's own that forks from `cuda_stream` at the start of the
  * call and joins it again before the call returns (to the caller everything is ordered as if it had run on
  * `cuda_stream`, also under stream capture).

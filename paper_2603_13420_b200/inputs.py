@@ -144,7 +144,8 @@ def kernel_work(w: Workload) -> dict:
     vis = (w.S + 1) / 2.0
     return {
         "tc_fwd_kernel": {"flops": fwd_flops(w), "bytes": fwd_bytes(w)},
-        # all three gradients: reads q, dout, lse, D, the prefix and the suffix K/V, writes dq, dk_suffix, dv_suffix
-        "tc_bwd_dq_kernel": {"flops": bwd_flops(w), "bytes": float(3 * q + 8 * rows + 2 * skv + pkv)},
+        # all three gradients: reads q, dout, lse, out (for D; 4 bytes a row of D where the pre-pass forms it), the prefix
+        # and the suffix K/V, writes dq, dk_suffix, dv_suffix
+        "tc_bwd_dq_kernel": {"flops": bwd_flops(w), "bytes": float(4 * q + 4 * rows + 2 * skv + pkv)},
         "simt_row_dot_kernel": {"flops": rows * 2.0 * w.d, "bytes": float(2 * q + 4 * rows)},
     }
