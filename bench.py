@@ -519,7 +519,7 @@ def roofline(w, kernels, peaks):
 # profiles/ (kernel, workload) -> bytes.
 TRAFFIC_BYTES_PER_LAUNCH = {
     ("tc_fwd_kernel", "C2"): 473.9e6,        # profiles/tc_fwd_kernel_C2.md
-    ("tc_bwd_dq_kernel", "C2"): 782.1e6,     # profiles/tc_bwd_kernel_C2.md
+    # (the backward was captured before it read `out` for the row statistic: profiles/tc_bwd_kernel_C2.md)
 }
 
 
