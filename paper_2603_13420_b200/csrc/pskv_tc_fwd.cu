@@ -290,6 +290,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int t_end = (int)((long long)(blockIdx.x + 1) * p.total_tiles / gridDim.x);
     const int G = (int)gridDim.x;
     const int Sh = ANY ? p.box.Sh : p.S;
+    // What MODE 2 knows of its plan: with these decided at run time it spilled 12 registers (396 bytes of loads; 20 candidates, 32/8
+    // heads, P = 64, S = 300 58 us, now 53).
+    const bool long_sfx = MODE == 2 || p.long_sfx;
+    const bool slab_stage = MODE != 2 && p.slab_stage, alias_stage = MODE != 2 && p.alias_stage;
     const int n_sp = (SR && p.deal_by_cost) ? Sh / p.tile_rows : 1;  // tiles per head
     const bool dealt = n_sp > 1;
     auto rank_at = [&](int tl) { return tl * G + ((tl & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
@@ -306,7 +310,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int n_tiles = !dealt ? t_end - t_begin : (n_rounds - 1) + (rank_at(n_rounds - 1) < p.total_tiles ? 1 : 0);
     // items of a tile: prefix blocks + the suffix block(s)
     auto items_of = [&](const TileInfo &t) {
-        return p.nblk_p + (!SR ? 1 : p.long_sfx ? sfx_blocks_long<ANY>(p, t) : p.fd_cpb.div(t.nc + p.cpb - 1));
+        return p.nblk_p + (!SR ? 1 : long_sfx ? sfx_blocks_long<ANY>(p, t) : p.fd_cpb.div(t.nc + p.cpb - 1));
     };
     // A run of tiles that shares one prefix: a KV head, or (several instructions) one instruction's
     // candidates inside a KV head.  Runs are numbered in tile order; the resident prefix is reloaded at the
@@ -419,7 +423,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 for (int j = 0; j < nbs; ++j) {
                     ok = mbar_wait_warp(bar(kBarKFree + ks), kph, abort_flag, p.status, kErrProducerK);
                     if (!ok) break;
-                    if (p.long_sfx) {
+                    if (long_sfx) {
                         // keys [128 j, 128 j + 128) of the tile's candidate; rows past the cache are zero-filled
                         if (elect_one_sync()) {
                             mbar_arrive_expect_tx(bar(kBarKFull + ks), (uint32_t)C::kTileBytes);
@@ -544,7 +548,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     if (SR && k >= p.nblk_p) {
                         // a suffix V block: one box of Skv rows per candidate, Spad rows apart
                         const int j = k - p.nblk_p;
-                        if (p.long_sfx) {
+                        if (long_sfx) {
                             if (elect_one_sync()) {
                                 mbar_arrive_expect_tx(bar(kBarVFull + vs), (uint32_t)C::kTileBytes);
 #pragma unroll 1
@@ -582,7 +586,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     ++k;
                 }
                 bool sv_ready = false;
-                if (pend_sv && !p.alias_stage) {
+                if (pend_sv && !alias_stage) {
                     if (tl == 0)
                         sv_ready = true;
                     else if (block)
@@ -593,7 +597,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 }
                 if (pend_store && !sv_ready) {
                     // the staging buffer holds the whole tile, or (slab_stage) one 64-column slab per round
-                    const uint32_t round = p.slab_stage ? (uint32_t)((tl - 1) * C::kSlabs + store_slab) : (uint32_t)(tl - 1);
+                    const uint32_t round = slab_stage ? (uint32_t)((tl - 1) * C::kSlabs + store_slab) : (uint32_t)(tl - 1);
                     bool ready;
                     if (block)
                         ready = ok = mbar_wait_warp(bar(kBarStageFull), round & 1, abort_flag, p.status, kErrEpilogue);
@@ -603,8 +607,8 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     if (ready) {
                         const TileInfo u = tile_info<MI == 2>(p, tile_at(tl - 1), t_begin);
                         const int nseg = (SR && (!ANY || p.box.one_box)) ? 1 : p.fd_seg.div(u.rows);
-                        const int sl_first = p.slab_stage ? store_slab : 0;
-                        const int sl_end = p.slab_stage ? store_slab + 1 : C::kSlabs;
+                        const int sl_first = slab_stage ? store_slab : 0;
+                        const int sl_end = slab_stage ? store_slab + 1 : C::kSlabs;
                         if (elect_one_sync()) {
 #pragma unroll 1
                             for (int sl = sl_first; sl < sl_end; ++sl)
@@ -615,7 +619,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                                     if (PAD && r >= p.Rr) continue;  // padding only
                                     int c1, c2;
                                     q_coords<ANY>(p, r, u.g, c1, c2);
-                                    tma_store_4d(&tm_out, stage + (p.slab_stage ? 0 : sl) * kStagingBytes + s * p.seg_rows * 128,
+                                    tma_store_4d(&tm_out, stage + (slab_stage ? 0 : sl) * kStagingBytes + s * p.seg_rows * 128,
                                                  sl * 64, c1, c2, b);
                                 }
                             tma_store_commit();
@@ -624,7 +628,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         }
                         __syncwarp();
                         PSKV_TRACE_EVENT(4, tl - 1);
-                        if (p.slab_stage && store_slab + 1 < C::kSlabs) {
+                        if (slab_stage && store_slab + 1 < C::kSlabs) {
                             ++store_slab;
                         } else {
                             store_slab = 0;
@@ -632,7 +636,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         }
                     }
                 }
-                if (pend_sv && p.alias_stage && !pend_store) sv_ready = true;
+                if (pend_sv && alias_stage && !pend_store) sv_ready = true;
                 if (sv_ready) {
                     if (elect_one_sync()) {
                         mbar_arrive_expect_tx(bar(kBarSVFull), (uint32_t)(t.nc * C::kSlabs * p.Sp * 128));
@@ -653,11 +657,13 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         __syncwarp();
     } else if (role == 1) {
         // ------------------------------------------------------------------ score MMAs: S = Q K^T
-        // An MMA is issued about when the one a few places ahead of it starts, so what a warp does between two of them costs the
-        // tensor cores nothing, and what it does between items does.  The next item is therefore worked out in the middle of
-        // this one's MMAs.  (Between them, with the ring positions by division, it took this warp 700 to 1 100 cycles per item and
-        // the value issuer as long, against 1 024 of MMAs: 256 candidates, 32/8 heads, P = 2048, S = 32 267-274 us, now 254-260.  A tile's
-        // first item worked out behind the MMAs instead, so that a short last block is not held up: 262, the compiler spills.)
+        // The two issuers.  An item is handed on as soon as its last MMA is issued, and the next one worked out behind that: working
+        // it out in the middle of this one's MMAs delayed every item that somebody waits for, as in tiles of few items (1000 beams,
+        // 32/32 heads, 2 tokens over 96 cached ones 303-318 us, now 296-302; 64 beams, P = 900, one over 120 19.1, now 18.6; 16 candidates, 32/8, P
+        // = 256, S = 48 11.9, now 11.6), and 256 candidates, 32/8, P = 2048, S = 32 take 254 us instead of 262 too.  With rings the
+        // positions are counters and the barriers are looked at together first, since as a rule everything is there (the last
+        // shape by division and one barrier after another: 287).  With the prefix resident nearly every item is waited for, and the
+        // compiler makes worse code of the counters (8 x 64 candidates, 32/8, P = 256, S = 48 172 us with them, else 153).
         int tl = 0;
         uint32_t ks = 0, kph = 0;        // ring of K blocks: stage, parity of its loads
         uint32_t slot = 0, slot_ph = 1;  // score slot, parity of its release
@@ -666,19 +672,21 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint64_t q_desc = make_smem_desc(sbase + p.off_q, 0, 1024);
         bool ok = true;
-        // the coming item
-        uint64_t k_desc, k_slab;
-        uint32_t idesc, kbar, kpar;
-        bool kwait, ring;
-        auto prepare = [&]() {
-            uint32_t kaddr;
+#pragma unroll 1
+        for (int i = 0; tl < n_tiles; ++i) {
+            // everything that does not depend on a wait comes first, so that it is out of the way
+            // when the waits return
+            if (RES) {
+                slot = (uint32_t)i % kSlots;
+                slot_ph = (((uint32_t)i / kSlots) & 1u) ^ 1u;
+            }
+            uint32_t kaddr, kbar, kpar;
             int n, slab;
-            kwait = true;
-            ring = (k < p.nblk_p || SR) && !RES;
+            bool kwait = true;
             if (k < p.nblk_p || SR) {
                 n = k < p.nblk_p ? prefix_block_rows(p, k)
-                    : p.long_sfx ? sfx_long_rows(p, k - p.nblk_p) : sfx_block_rows(p, t.nc, k - p.nblk_p);
-                slab = (SR && p.long_sfx && k >= p.nblk_p) ? C::kSlabBytes : n * 128;  // (full 128-row boxes)
+                    : long_sfx ? sfx_long_rows(p, k - p.nblk_p) : sfx_block_rows(p, t.nc, k - p.nblk_p);
+                slab = (SR && long_sfx && k >= p.nblk_p) ? C::kSlabBytes : n * 128;  // (full 128-row boxes)
                 if (RES) {
                     const int inst = inst_of(t);
                     kwait = first_of_run(t, inst);
@@ -697,28 +705,29 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 kpar = (uint32_t)tl & 1u;
                 kaddr = sbase + p.off_sk;
             }
-            idesc = make_idesc_bf16(kTileM, n, 0);
-            k_desc = make_smem_desc(kaddr, 0, 1024);
-            k_slab = (uint64_t)(slab >> 4);
-        };
-        if (n_tiles > 0) prepare();
-#pragma unroll 1
-        for (int i = 0; tl < n_tiles; ++i) {
-            // The slot is free once the value MMAs of item i-3 (which read P from it) have completed.  As a rule everything
-            // is there: looked at together the barriers cost one vote.
+            const uint32_t idesc = make_idesc_bf16(kTileM, n, 0);
+            const uint32_t d_tmem = tmem + slot * kBlockN;
+            const uint64_t k_desc = make_smem_desc(kaddr, 0, 1024);
+            const uint64_t k_slab = (uint64_t)(slab >> 4);
+            const bool last_of_tile = k == nitems - 1;
+            const bool free_stage = (k < p.nblk_p || SR) && !RES;
+            // the slot is free once the value MMAs of item i-3 (which read P from it) have completed
             PSKV_TRACE_EVENT(16, i);
             const bool qwait = k == kfirst;
-            bool ready = mbar_test_wait(bar(kBarPvDone + slot), slot_ph);
-            if (kwait) ready &= mbar_test_wait(kbar, kpar);
-            if (qwait) ready &= mbar_test_wait(bar(kBarQFull), tl & 1);
-            if (!__all_sync(0xffffffffu, ready)) {
+            bool ready = false;
+            if (!RES) {
+                ready = mbar_test_wait(bar(kBarPvDone + slot), slot_ph);
+                if (kwait) ready &= mbar_test_wait(kbar, kpar);
+                if (qwait) ready &= mbar_test_wait(bar(kBarQFull), tl & 1);
+            }
+            if (RES || !__all_sync(0xffffffffu, ready)) {
                 ok = mbar_wait_warp(bar(kBarPvDone + slot), slot_ph, abort_flag, p.status, kErrMmaQk);
                 PSKV_TRACE_EVENT(18, i);
                 if (ok && qwait) ok = mbar_wait_warp(bar(kBarQFull), tl & 1, abort_flag, p.status, kErrMmaQk);
                 if (ok && kwait) ok = mbar_wait_warp(kbar, kpar, abort_flag, p.status, kErrMmaQk);
                 if (!ok) break;
             }
-            if (MI && RES && qwait && first_of_run(t, inst_of(t))) {
+            if (MI && RES && k == kfirst && first_of_run(t, inst_of(t))) {
                 // The resident copy of a run always loads every prefix block, also those this run skips as
                 // padding.  Nobody multiplies them, so their loads are waited for here: a load must have
                 // landed before its buffer and barrier are armed again for the next run, and before the
@@ -730,23 +739,21 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             }
             PSKV_TRACE_EVENT(10, i);
             tc_fence_after();
-            const uint32_t d_tmem = tmem + slot * kBlockN, idesc_i = idesc;
-            const uint64_t kd = k_desc, kslab = k_slab;
-            auto issue = [&](int ks16) {
-                const uint64_t qoff = (uint64_t)(((ks16 >> 2) * C::kSlabBytes + (ks16 & 3) * 32) >> 4);
-                const uint64_t koff = (uint64_t)(ks16 >> 2) * kslab + (uint64_t)(((ks16 & 3) * 32) >> 4);
-                mma_ss(d_tmem, q_desc + qoff, kd + koff, idesc_i, ks16 > 0 ? 1u : 0u);
-            };
-            constexpr int kSteps = D / 16, kAhead = kSteps * 3 / 4;
             if (elect_one_sync()) {
 #pragma unroll
-                for (int ks16 = 0; ks16 < kAhead; ++ks16) issue(ks16);
+                for (int ks16 = 0; ks16 < D / 16; ++ks16) {
+                    const uint64_t qoff = (uint64_t)(((ks16 >> 2) * C::kSlabBytes + (ks16 & 3) * 32) >> 4);
+                    const uint64_t koff = (uint64_t)(ks16 >> 2) * k_slab + (uint64_t)(((ks16 & 3) * 32) >> 4);
+                    mma_ss(d_tmem, q_desc + qoff, k_desc + koff, idesc, ks16 > 0 ? 1u : 0u);
+                }
+                tc_commit(bar(kBarSFull + slot));
+                if (free_stage) tc_commit(bar(kBarKFree + ks));
+                if (last_of_tile) tc_commit(bar(kBarQkFree));  // the suffix block ends the tile's scores
             }
             __syncwarp();
-            const uint32_t full = bar(kBarSFull + slot), freed = ring ? bar(kBarKFree + ks) : 0u;
-            const bool last_of_tile = k == nitems - 1;
-            if (ring && ++ks == (uint32_t)p.stages) { ks = 0; kph ^= 1u; }
-            if (++slot == kSlots) { slot = 0; slot_ph ^= 1u; }
+            PSKV_TRACE_EVENT(12, i);
+            if (free_stage && ++ks == (uint32_t)p.stages) { ks = 0; kph ^= 1u; }
+            if (!RES && ++slot == kSlots) { slot = 0; slot_ph ^= 1u; }
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
@@ -755,16 +762,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     k = kfirst = first_block(inst_of(t));
                 }
             }
-            prepare();  // (of no item behind the last one: nothing is read)
-            if (elect_one_sync()) {
-#pragma unroll
-                for (int ks16 = kAhead; ks16 < kSteps; ++ks16) issue(ks16);
-                tc_commit(full);
-                if (freed) tc_commit(freed);
-                if (last_of_tile) tc_commit(bar(kBarQkFree));  // the suffix block ends the tile's scores
-            }
-            __syncwarp();
-            PSKV_TRACE_EVENT(12, i);
         }
     } else if (role == 2) {
         // ------------------------------------------------------------------ value MMAs: O += P V
@@ -776,20 +773,20 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int kfirst = first_block(inst_of(t)), k = kfirst;
         const uint32_t idesc_pv = make_idesc_bf16(kTileM, D, 1);
         bool ok = true;
-        // the coming item (worked out in the middle of this one's MMAs, as above)
-        uint64_t v_desc;
-        uint32_t vbar, vpar;
-        int nk;
-        bool vwait, ring;
-        auto prepare = [&]() {
-            uint32_t vaddr;
+#pragma unroll 1
+        for (int i = 0; tl < n_tiles; ++i) {
+            // everything that does not depend on a wait comes first
+            if (RES) {
+                slot = (uint32_t)i % kSlots;
+                slot_ph = ((uint32_t)i / kSlots) & 1u;
+            }
+            uint32_t vaddr, vbar, vpar;
             int n, slab;
-            vwait = true;
-            ring = (k < p.nblk_p || SR) && !RES;
+            bool vwait = true;
             if (k < p.nblk_p || SR) {
                 n = k < p.nblk_p ? prefix_block_rows(p, k)
-                    : p.long_sfx ? sfx_long_rows(p, k - p.nblk_p) : sfx_block_rows(p, t.nc, k - p.nblk_p);
-                slab = (SR && p.long_sfx && k >= p.nblk_p) ? C::kSlabBytes : n * 128;  // (full 128-row boxes)
+                    : long_sfx ? sfx_long_rows(p, k - p.nblk_p) : sfx_block_rows(p, t.nc, k - p.nblk_p);
+                slab = (SR && long_sfx && k >= p.nblk_p) ? C::kSlabBytes : n * 128;  // (full 128-row boxes)
                 if (RES) {
                     const int inst = inst_of(t);
                     vwait = first_of_run(t, inst);
@@ -808,19 +805,21 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 vpar = (uint32_t)tl & 1u;
                 vaddr = sbase + p.off_sv;
             }
-            v_desc = make_smem_desc(vaddr, (uint32_t)slab, 1024);
-            nk = n >> 4;
-        };
-        if (n_tiles > 0) prepare();
-#pragma unroll 1
-        for (int i = 0; tl < n_tiles; ++i) {
+            const uint32_t p_tmem = tmem + slot * kBlockN;  // bf16 pairs: 8 columns per 16 keys
+            const uint64_t v_desc = make_smem_desc(vaddr, (uint32_t)slab, 1024);
+            const int nk = n >> 4;
+            const bool last_of_tile = k == nitems - 1;
+            const bool free_stage = (k < p.nblk_p || SR) && !RES;
+            const uint32_t acc0 = k > kfirst ? 1u : 0u;
             PSKV_TRACE_EVENT(17, i);
-            // (O of the previous tile must have been read out by the epilogue warps)
-            const bool first = k == kfirst, owait = first && tl > 0;
-            bool ready = mbar_test_wait(bar(kBarPReady + slot), slot_ph);
-            if (vwait) ready &= mbar_test_wait(vbar, vpar);
-            if (owait) ready &= mbar_test_wait(bar(kBarOFree), (tl - 1) & 1);
-            if (!__all_sync(0xffffffffu, ready)) {
+            const bool owait = k == kfirst && tl > 0;  // (O of the previous tile must have been read out by the epilogue warps)
+            bool ready = false;
+            if (!RES) {
+                ready = mbar_test_wait(bar(kBarPReady + slot), slot_ph);
+                if (vwait) ready &= mbar_test_wait(vbar, vpar);
+                if (owait) ready &= mbar_test_wait(bar(kBarOFree), (tl - 1) & 1);
+            }
+            if (RES || !__all_sync(0xffffffffu, ready)) {
                 ok = mbar_wait_warp(bar(kBarPReady + slot), slot_ph, abort_flag, p.status, kErrMmaPv);
                 PSKV_TRACE_EVENT(15, i);
                 if (ok && owait) ok = mbar_wait_warp(bar(kBarOFree), (tl - 1) & 1, abort_flag, p.status, kErrMmaPv);
@@ -828,7 +827,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 if (ok && vwait) ok = mbar_wait_warp(vbar, vpar, abort_flag, p.status, kErrMmaPv);
                 if (!ok) break;
             }
-            if (MI && RES && first && first_of_run(t, inst_of(t))) {  // (as for the K blocks above)
+            if (MI && RES && k == kfirst && first_of_run(t, inst_of(t))) {  // (as for the K blocks above)
                 const uint32_t par = (uint32_t)(run_of(t, inst_of(t)) - run_first) & 1u;
                 for (int kk = 0; kk < kfirst && kk < p.nblk_p && ok; ++kk)
                     ok = mbar_wait_warp(bar(kBarVFull + kk), par, abort_flag, p.status, kErrMmaPv);
@@ -836,27 +835,27 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             }
             PSKV_TRACE_EVENT(11, i);
             tc_fence_after();
-            const uint32_t p_tmem = tmem + slot * kBlockN;  // bf16 pairs: 8 columns per 16 keys
-            const uint32_t acc0 = first ? 0u : 1u;
-            const uint64_t vd = v_desc;
-            const int steps = nk;
-            auto issue = [&](int ks16) {
-                if (ks16 >= steps) return;
-                const uint32_t p_cols = p_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8;
-                const uint64_t v_rows = vd + (uint64_t)(ks16 * (2048 >> 4));
-                mma_ts(tmem + kOCol, p_cols, v_rows, idesc_pv, ks16 > 0 ? 1u : acc0);
-                if (TWO) mma_ts(tmem + kOCol, p_cols + kPiece / 2, v_rows, idesc_pv, 1u);
-            };
-            constexpr int kSteps = kBlockN / 16, kAhead = kSteps * 3 / 4;
             if (elect_one_sync()) {
 #pragma unroll
-                for (int ks16 = 0; ks16 < kAhead; ++ks16) issue(ks16);
+                for (int ks16 = 0; ks16 < kBlockN / 16; ++ks16) {
+                    if (ks16 < nk) {
+                        const uint32_t p_cols = p_tmem + (ks16 >> 1) * kPiece + (ks16 & 1) * 8;
+                        const uint64_t v_rows = v_desc + (uint64_t)(ks16 * (2048 >> 4));
+                        mma_ts(tmem + kOCol, p_cols, v_rows, idesc_pv, ks16 > 0 ? 1u : acc0);
+                        if (TWO) mma_ts(tmem + kOCol, p_cols + kPiece / 2, v_rows, idesc_pv, 1u);
+                    }
+                }
+                tc_commit(bar(kBarPvDone + slot));
+                if (free_stage) tc_commit(bar(kBarVFree + vs));
+                if (last_of_tile) {
+                    tc_commit(bar(kBarSVFree));
+                    tc_commit(bar(kBarOFull));
+                }
             }
             __syncwarp();
-            const uint32_t done = bar(kBarPvDone + slot), freed = ring ? bar(kBarVFree + vs) : 0u;
-            const bool last_of_tile = k == nitems - 1;
-            if (ring && ++vs == (uint32_t)p.stages) { vs = 0; vph ^= 1u; }
-            if (++slot == kSlots) { slot = 0; slot_ph ^= 1u; }
+            PSKV_TRACE_EVENT(13, i);
+            if (free_stage && ++vs == (uint32_t)p.stages) { vs = 0; vph ^= 1u; }
+            if (!RES && ++slot == kSlots) { slot = 0; slot_ph ^= 1u; }
             if (++k == nitems) {
                 k = 0;
                 if (++tl < n_tiles) {
@@ -865,19 +864,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     k = kfirst = first_block(inst_of(t));
                 }
             }
-            prepare();
-            if (elect_one_sync()) {
-#pragma unroll
-                for (int ks16 = kAhead; ks16 < kSteps; ++ks16) issue(ks16);
-                tc_commit(done);
-                if (freed) tc_commit(freed);
-                if (last_of_tile) {
-                    tc_commit(bar(kBarSVFree));
-                    tc_commit(bar(kBarOFull));
-                }
-            }
-            __syncwarp();
-            PSKV_TRACE_EVENT(13, i);
         }
     } else if (warp < 4 + 4 * kGroups) {
         // ------------------------------------------------------------------ softmax warps (4..19)
@@ -914,7 +900,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 } else if (SR) {
                     // query i is suffix token L - S + i of its candidate: suffix keys 0 .. L - S + i
                     const int pos = suffix_tokens(p.suffix_len, b, p.S, p.Skv) - p.S + i;
-                    if (p.long_sfx) {
+                    if (long_sfx) {
                         lo_sfx = 0;
                         hi_sfx = pos;  // counted from the candidate's first key; block j starts at 128 j
                     } else {
@@ -945,7 +931,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         n = prefix_block_rows(p, k);
                         lo = max(0, pad - k * kBlockN);
                         hi = min(kBlockN, p.P - k * kBlockN) - 1;
-                    } else if (SR && p.long_sfx) {
+                    } else if (SR && long_sfx) {
                         n = sfx_long_rows(p, k - p.nblk_p);
                         lo = lo_sfx;  // 0 for a real row, 1 (with hi 0 - ...: nothing visible) for padding
                         hi = lo_sfx == 0 ? hi_sfx - (k - p.nblk_p) * kBlockN : 0;
@@ -1067,7 +1053,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // meet zero probabilities): rows that failed stage zeros and are redone, and so do padding rows, whose
             // sums may be NaN (they are not redone)
             const float inv = row_ok ? 1.f / l : 0.f;
-            if (p.slab_stage) {
+            if (slab_stage) {
                 // One 64-column slab at a time through a staging buffer of one slab: load, hand O back after
                 // the last load, wait for the previous slab's stores to have read the buffer, stage, tell
                 // the storing warp.  The buffer is this kernel's own: suffix V of the next tile is fetched
