@@ -531,7 +531,7 @@ pskv_status pskv_attn_fwd_multi(const void *q, const void *prefix_k, const void 
         a.suffix_len = nullptr;
         a.scale = scale;
         a.dims = dm;
-        cudaError_t e = tc_fwd_supported(dm) ? launch_tc_fwd(a, workspace, status_word, pass_stream)
+        cudaError_t e = tc_fwd_supported(dm) ? launch_tc_fwd(a, workspace, status_word, pass_stream, 1, nullptr, side ? Bp : 1)
                                              : launch_simt_fwd(a, pass_stream);
         if (e != cudaSuccess) result = cuda_fail(e);
     }

@@ -65,11 +65,12 @@ bool tc_fwd_supported(const Dims &d);
 size_t tc_fwd_workspace_bytes(const Dims &d);
 // Several instructions in one launch (Sec. 4.3): the B candidates fall into `n_instr` contiguous groups
 // of equal size, group i uses prefix cache i of prefix_k / prefix_v [n_instr][Hkv][P][d], whose last
-// prefix_len[i] rows (host array) are real tokens and whose first rows are left padding.
+// prefix_len[i] rows (host array) are real tokens and whose first rows are left padding.  `passes`: how many launches of
+// this size the call makes on two streams (one pass per instruction), this one among them.
 constexpr int kMaxFusedInstructions = 64;
 bool tc_fwd_fused_supported(const Dims &d, int n_instr);
 cudaError_t launch_tc_fwd(const FwdArgs &a, void *workspace, unsigned int *status_word,
-                          cudaStream_t stream, int n_instr = 1, const int *prefix_len = nullptr);
+                          cudaStream_t stream, int n_instr = 1, const int *prefix_len = nullptr, int passes = 1);
 // The forward on CTA pairs (cta_group::2), for the shapes it takes; launch_tc_fwd goes there by itself
 // unless pairs are switched off (pskv_enable_cta_pairs).
 bool tc_fwd_pair_supported(const Dims &d);

@@ -1504,9 +1504,23 @@ const TilePlan &plan_tiles(const Dims &dm, int n_instr = 1)
     return table.get(dm, n_instr, [&] { return make_plan(dm, n_instr); });
 }
 
+// CTAs for tiles that are dealt out by cost.  All SMs for a launch by itself: the 512 tiles of a prompt of 2048 tokens, 32 heads, put
+// 34 key blocks on the busiest of 128 CTAs of four tiles, 31 on the busiest of 148 (49.5 -> 45.5 us).  `passes` such launches on
+// two streams fill each other's free SMs, and a CTA's start is paid for each: counted in tiles in a row, the even grid
+// takes its CTAs in waves; on all SMs a pass takes something between its tiles per SM and the most that an SM gets.  Even and all: 4
+// passes of 192 tiles (2 candidates, 32/32 heads, P = 128, S = 384) 49.0 and 56.1 us, 8 of 192 (3, 32/8, P = 100, S = 256) 83 and 96, 5 of 192
+// (3, 32/8, P = 64, S = 200) 55.3 and 61.6; 3 of 320 (2, 32/8, P = 500, S = 640) 86 and 71, 4 of 512 (1, 32/8, P = 64, S = 2048) 191 and 175,
+// 2 of 320 (2, 32/32, P = 300, S = 520) 51.6 and 45.1; 4 of 288 (3, 32/8, P = 64, S = 384) 59.8 both.
+int dealt_grid(int tiles, int sms, int passes)
+{
+    const int even = even_grid(tiles, sms), in_a_row = (tiles + sms - 1) / sms;
+    const double waves = (double)(((long long)passes * even + sms - 1) / sms);
+    return passes * 0.5 * ((double)tiles / sms + in_a_row) < waves * in_a_row ? (tiles < sms ? tiles : sms) : even;
+}
+
 template <int D>
 cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsigned int *status_word,
-                   cudaStream_t stream, int n_instr, const int *prefix_len)
+                   cudaStream_t stream, int n_instr, const int *prefix_len, int passes)
 {
     const Dims &dm = a.dims;
     const int Rg = dm.n_rep * dm.S;
@@ -1607,9 +1621,7 @@ cudaError_t launch(const FwdArgs &a, const TilePlan &plan, void *workspace, unsi
 
         static PerDeviceOnce attr_set[9];
         if (cudaError_t e = ensure_max_smem(kernel, attr_set[slot]); e != cudaSuccess) return e;
-        // Tiles dealt by cost go to every SM: the 512 tiles of a prompt of 2048 tokens, 32 heads, put 34 key blocks on the
-        // busiest of 128 CTAs of four tiles, 30 on the busiest of 148.
-        const int grid = p.deal_by_cost ? (p.total_tiles < sm_count() ? p.total_tiles : sm_count()) : even_grid(p.total_tiles, sm_count());
+        const int grid = p.deal_by_cost ? dealt_grid(p.total_tiles, sm_count(), passes) : even_grid(p.total_tiles, sm_count());
         cudaError_t launch_err;
         {
             KernelTiming timing(kKernelFwdTc, stream);
@@ -1678,7 +1690,7 @@ bool tc_fwd_fused_supported(const Dims &dm, int n_instr)
 }
 
 cudaError_t launch_tc_fwd(const FwdArgs &a, void *workspace, unsigned int *status_word, cudaStream_t stream,
-                          int n_instr, const int *prefix_len)
+                          int n_instr, const int *prefix_len, int passes)
 {
     if (n_instr < 1) n_instr = 1;
     const TilePlan plan = plan_tiles(a.dims, n_instr);  // (a copy: the next look-up may replace the table's entry)
@@ -1686,8 +1698,8 @@ cudaError_t launch_tc_fwd(const FwdArgs &a, void *workspace, unsigned int *statu
     if (n_instr > 1 && (!prefix_len || !tc_fwd_fused_supported(a.dims, n_instr))) return cudaErrorInvalidValue;
     if (n_instr == 1 && cta_pairs_enabled() && tc_fwd_pair_supported(a.dims))
         return launch_tc_fwd_pair(a, status_word, stream);
-    return a.dims.d == 128 ? launch<128>(a, plan, workspace, status_word, stream, n_instr, prefix_len)
-                           : launch<64>(a, plan, workspace, status_word, stream, n_instr, prefix_len);
+    return a.dims.d == 128 ? launch<128>(a, plan, workspace, status_word, stream, n_instr, prefix_len, passes)
+                           : launch<64>(a, plan, workspace, status_word, stream, n_instr, prefix_len, passes);
 }
 
 }  // namespace pskv

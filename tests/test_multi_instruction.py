@@ -186,3 +186,25 @@ def test_back_to_back_one_launch_calls_with_prefixes_that_are_padding_only(monke
     assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
     for o, l in outs:
         assert torch.equal(o, ref_out) and torch.equal(l, ref_lse)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", [
+    # B, Bp, Hq, Hkv, S, Pmax, d, lens
+    (6, 3, 32, 32, 384, 100, 128, (100, 0, 37)),     # 192 tiles a pass, dealt by cost: the even grid beside other passes
+    (4, 2, 32, 32, 520, 130, 128, (130, 64)),        # 320: every SM
+    (3, 3, 32, 8, 640, 64, 128, (64, 64, 1)),        # 160: the even grid
+], ids=str)
+def test_passes_of_long_suffixes_equal_the_instructions_alone_bit_for_bit(case):
+    """Tiles dealt by cost take another grid beside other passes than in a call by itself; a tile's results do not depend on its CTA."""
+    pskv.pskv_set_multi_form("auto")
+    B, Bp, Hq, Hkv, S, Pmax, d, lens = case
+    dev = {k: v.cuda() for k, v in make(*case).items()}
+    out, lse = pskv.pskv_attn_fwd_multi(dev["q"], dev["prefix_k"], dev["prefix_v"], lens, dev["suffix_k"], dev["suffix_v"], 0.088)
+    K = B // Bp
+    for i, n in enumerate(lens):
+        part = slice(i * K, (i + 1) * K)
+        pk, pv = (dev[k][i, :, Pmax - n:].contiguous() if n else None for k in ("prefix_k", "prefix_v"))
+        o, l = pskv.pskv_attn_fwd(dev["q"][part], pk, pv, dev["suffix_k"][part], dev["suffix_v"][part], 0.088)
+        assert torch.equal(out[part], o) and torch.equal(lse[part], l)
+    assert pskv.pskv_poll_device_status() == pskv.PSKV_OK
