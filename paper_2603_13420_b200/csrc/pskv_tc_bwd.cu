@@ -130,7 +130,7 @@ struct Cfg {
 };
 
 enum {
-    kBarQFull = 0,   // Q of a tile landed (SPLIT: and dO)
+    kBarQFull = 0,   // Q of a tile landed (kJoint: and dO)
     kBarDoFull,      // dO of a tile landed
     kBarQFree,       // the last MMA of each issuer that reads them has completed (2 arrivals)
     kBarDqFull,      // dQ of a tile is final
@@ -351,7 +351,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     using C = Cfg<D>;
     constexpr bool DROW = DSRC == kDWarps, DOT = DSRC == kDItem;
     constexpr int kTerms = TWO ? 2 : 1;
-    constexpr bool kEight = TWO || (DOT);
+    constexpr bool kEight = TWO || DOT;
+    // Q and dO on one barrier: launches with few items to a tile, or with one tile to a CTA (see the S / dP issuer).
+    constexpr bool kJoint = SPLIT || DROW;
     constexpr uint64_t kLoTerm = (uint64_t)(kDsBytes >> 4);  // descriptor distance from a P / dS buffer to its second term
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -558,15 +560,15 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             PSKV_TRACE_EVENT(2, tile);
             const uint32_t tx = (uint32_t)(nb * C::kSlabs * step * 128);
             if (lane == 0) {
-                if (!SPLIT) mbar_arrive_expect_tx(bar(kBarDoFull), tx);
-                mbar_arrive_expect_tx(bar(kBarQFull), SPLIT ? 2 * tx : tx);
+                if (!kJoint) mbar_arrive_expect_tx(bar(kBarDoFull), tx);
+                mbar_arrive_expect_tx(bar(kBarQFull), kJoint ? 2 * tx : tx);
             }
             __syncwarp();
             if (lane < nb) {
 #pragma unroll
                 for (int sl = 0; sl < C::kSlabs; ++sl) {
                     const uint32_t off = (uint32_t)(sl * C::kSlabBytes + lane * step * 128);
-                    tma_load_4d(sbase + p.off_do + off, &tm_do, bar(SPLIT ? kBarQFull : kBarDoFull), sl * 64, r, g, b);
+                    tma_load_4d(sbase + p.off_do + off, &tm_do, bar(kJoint ? kBarQFull : kBarDoFull), sl * 64, r, g, b);
                 }
 #pragma unroll
                 for (int sl = 0; sl < C::kSlabs; ++sl) {
@@ -607,7 +609,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (x & kDescEnd) break;
             const uint32_t idesc = make_idesc_bf16(kTileM, (int)(x & kDescN), 0);
             const uint32_t tile_ph = descs[item & 7u].w & 1u;
-            if (x & (DOT ? kDescRowDot : kDescFirst)) ok = mbar_wait_warp(bar(SPLIT ? kBarQFull : kBarDoFull), tile_ph, abort_flag, p.status, kErrMmaS);
+            if (x & (DOT ? kDescRowDot : kDescFirst)) ok = mbar_wait_warp(bar(kJoint ? kBarQFull : kBarDoFull), tile_ph, abort_flag, p.status, kErrMmaS);
             if (ok) ok = mbar_wait_warp(bar(kBarSFree + slot), ((item >> 1) & 1u) ^ 1u, abort_flag, p.status, kErrMmaS);
             if (ok) ok = mbar_wait_warp(bar(kBarVFull + vs), vph, abort_flag, p.status, kErrMmaS);
             if (!ok) break;
@@ -616,8 +618,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // dP first: its V piece is handed back while S is under way (with two terms there is one V stage, and its next piece
             // is what the following item waits for), and a tile's first dP starts when dO has landed, before Q.  Whole steps:
             // 58 candidates, 32/32 heads, P = 1735, S = 66 601 -> 569 us, 61, 32/32, P = 1206, S = 54 314 -> 303, 14, 32/32, P = 417, S =
-            // 123 97 -> 94; in one term and on small launches no change.  (Split launches have few items to a tile; waiting for
-            // the two in turn costs them more: one candidate, 32/8, P = 78, S = 113 27.9 -> 28.8.)
+            // 123 97 -> 94; in one term no change.  (Split launches have few items to a tile, and where a CTA has one tile nothing runs
+            // before it; waiting for the two in turn costs them more: one candidate, 32/8, P = 78, S = 113 27.9 -> 28.8; the
+            // backward of 64, 4/4, d = 64, P = 256, S = 40 12.70 -> 12.86, of 40 12.18 -> 12.35.)
             if (DOT && (x & kDescRowDot)) {
                 // dO O^T over the whole slot: 64 columns of O from the K stage, 64 from the V stage
                 if (elect_one_sync()) {
@@ -644,7 +647,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 }
                 tc_commit(bar(kBarVFree + vs));
             }
-            if (!SPLIT && (x & kDescFirst)) {
+            if (!kJoint && (x & kDescFirst)) {
                 __syncwarp();
                 ok = mbar_wait_warp(bar(kBarQFull), tile_ph, abort_flag, p.status, kErrMmaS);
                 if (!ok) break;
