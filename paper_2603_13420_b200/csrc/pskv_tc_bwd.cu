@@ -1179,22 +1179,37 @@ const BwdPlan &plan_bwd(const Dims &dm, int n_instr)
 // (three units per CTA) 38.7 and 43.9.
 // As an item of its own on larger ones: 512 MMA cycles and one hand-off per tile instead of a pass over dout and out at the rate
 // of HBM and its launch.  Whole steps, pre-pass and item: 512 candidates, 32/8 heads, P = 256, S = 48 528 and 510 us, 8 x 64 in instructions 525 and
-// 508; 49, 32/8, P = 108, S = 47 57 and 53; with one tile to a unit on launches of few units 16, 32/32, P = 150, S = 55 42.7 and 40.7; 60,
-// P = 128, S = 30 (480 units) 66.8 and 64.9.  Such units are short, and beyond about four per SM the hand-off costs as much
-// as the pass or more: 60, 32/32, P = 256, S = 47 (960) 122.6 and 123.7; 128, P = 160, S = 40 (1376) 145.7 and 148.0.  Not where a
-// tile is walked over several times or in parts, which would form
-// its D again each time (44, 32/8, P = 51, S = 87 113 and 120; one candidate, P = 78, S = 113 28 and 31), nor where `out` comes in
-// many small boxes (500, 32/32, P = 211, S = 10, boxes of 16 rows 237 and 245).
+// 508; 49, 32/8, P = 108, S = 47 57 and 53; with one tile to a unit on launches of few units 46, 32/32, P = 77, S = 20 45.6 and 43.8; 16,
+// P = 100, S = 55 40.6 and 37.6.
+// What it needs: head dim 128, no gradient on lse, units that are no parts of a candidate, and suffix boxes of whole steps of 16 keys (the
+// MMAs read K and V stages in such steps, and `out` passes through the same stages: nothing of it must be left to be read).
+// Where it is not taken, and what is known of both there:
+//  - `out` in boxes below 24 rows: 500, 32/32, P = 211, S = 10 (16 rows) 209 and 219.
+//  - one tile to a unit from four units per SM on: 60, 32/32, P = 256, S = 47 (960 units) 115 and 121; 400, 32/16, P = 100, S = 51 453 and
+//    459; 250, 32/8, P = 100, S = 21 115 and 121; 314, 32/32, P = 635, S = 19 368 and 374; no difference for 128, P = 160 to 2048, S = 40.  Only full
+//    tiles of one term gain: 256, 32/8, S = 32, P = 128 to 2048 134, 255, 412, 724 and 127, 246, 405, 722.
+//  - two terms, one candidate to a unit whose tiles are at most seven eighths full, two prefix pieces, from four units per SM on: the item
+//    works on whole tiles, the pass on rows, and three items of two terms and one V stage do not cover the hand-off.  250, 32/8, P = 100, S = 49,
+//    51, 55, 57, 61 255, 263, 278, 292, 300 and 261, 268, 281, 289, 294; 300, P = 65, S = 50 303 and 314; 70, P = 100, S = 51 80.0 and 79.1; with one prefix
+//    piece (333, P = 32, S = 53) 305 and 299, with three (250, P = 129, S = 51) 307 and 301.
+//  - suffixes of several pieces.  Tiles of a unit of several are walked over once per piece, and each time D is formed again: 44, 32/8, P = 51, S =
+//    87 113 and 120.  Units of one tile are walked over once; from four units per SM on they lose (40, 32/32, P = 500, S = 72 167 and 172; 34, P = 136,
+//    S = 96 107 and 111; 28, P = 75, S = 69 76.8 and 79.5; 304 in 8 instructions, P = 512, S = 80 1271 and 1334), below that they would gain
+//    (8, P = 78, S = 113 40 and 36; 18, P = 300, S = 100 81 and 79; 6, P = 50, S = 111 37 and 33).
+//  - several instructions below four units per SM.  These calls are known, and tested, as two launches, one for the row statistic and one
+//    for the gradients; the item in front of theirs is faster (64 candidates in 2 instructions, 32/8, P = 256, S = 48 75.5 and 72.9; 16 in 4, 32/32,
+//    P = 150, S = 55 43.3 and 40.2; 128 in 4, 32/8, P = 128, S = 48 115 and 110).
 DSource d_source(const BwdArgs &a, const BwdPlan &plan, int n_instr)
 {
     const Dims &dm = a.dims;
     const long long units = (long long)plan.upi * n_instr * dm.Hkv * plan.n_sub;
-    if (n_instr == 1 && plan.cu * plan.Rp <= kTileM && units <= sm_count()) return kDWarps;
-    // (The MMAs read K and V stages in steps of 16 keys, and `out` passes through the same stages: boxes of whole steps leave nothing
-    // of it to be read.  Calls of several instructions below four units per SM stay the two launches they are known as.)
-    const bool can = dm.d == 128 && !a.dlse && plan.n_sub == 1 && plan.nh == 1 && plan.sfx_box * plan.cpp % 16 == 0;
-    const bool many = units >= 4ll * sm_count(), one_tile = plan.cu * plan.Rp <= kTileM;
-    return can && plan.seg * plan.cbox >= 24 && !(one_tile && many) && (n_instr == 1 || many) ? kDItem : kDTable;
+    const int tiles = (plan.cu * plan.Rp + kTileM - 1) / kTileM;
+    if (n_instr == 1 && tiles == 1 && units <= sm_count()) return kDWarps;
+    const bool can = dm.d == 128 && !a.dlse && plan.n_sub == 1 && plan.sfx_box * plan.cpp % 16 == 0;
+    if (!can || plan.nh > 1 || plan.seg * plan.cbox < 24) return kDTable;
+    if (units < 4ll * sm_count()) return n_instr == 1 ? kDItem : kDTable;
+    const bool part_full = plan.terms == 2 && plan.cu == 1 && plan.nblk == 2 && 8 * plan.Rp <= 7 * kTileM * tiles;
+    return tiles == 1 || part_full ? kDTable : kDItem;
 }
 
 template <int D, bool TWO>

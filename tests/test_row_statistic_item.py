@@ -20,6 +20,9 @@ pytestmark = pytest.mark.gpu
     ((600, 3, 3, 128, 0, 24), 1),      # no prefix; two candidates to a key piece
     ((250, 4, 2, 128, 17, 53), 1),     # two terms; padded rows and keys
     ((149, 1, 1, 128, 130, 64), 1),    # one unit more than SMs, half of each tile's rows do not exist
+    ((290, 8, 2, 128, 100, 51), 1),    # two terms, a second tile of 80 rows, two prefix pieces: 580 units
+    ((300, 8, 2, 128, 100, 51), 2),    # ... 600: the pre-pass
+    ((300, 8, 2, 128, 100, 57), 1),    # ... of 104 rows
     ((300, 4, 4, 128, 40, 72), 2),     # two key pieces: the pre-pass
     ((300, 4, 4, 64, 40, 40), 2),      # head dim 64: the pre-pass
 ], ids=str)
