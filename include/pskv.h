@@ -17,6 +17,10 @@
  *     Appendix E; Table 8 lists the head counts).
  *   - Suffix row i of a candidate sees all P prefix keys and suffix keys 0..i
  *     (causal, diagonal included: the K_{<=t} of Eq. 2).  P = 0 is legal.
+ *   - Input tensors must hold finite numbers.  The query rows of neighbouring candidates share tiles of 128
+ *     rows, and in a tile another candidate's rows, keys and values meet probabilities of zero: a NaN or an
+ *     infinity of one candidate reaches that candidate's results, and can reach those of the candidates in the
+ *     same tiles too, all but their lse.  Which candidates those are depends on the tiling.
  *   - Work is enqueued on `cuda_stream` (a cudaStream_t passed as void*, NULL =
  *     the default stream) and the call returns without synchronising.
  *   - Arguments are validated on the host before anything is launched; a call
@@ -175,8 +179,8 @@ long long pskv_attn_bwd_static_max_rows(void);
  * With Bp <= 64 one launch may serve all instructions (pskv_set_multi_form(2) turns this off); forward and
  * backward decide by themselves.  The forward does where the suffix keys of a row tile fit one 128-key block
  * and an instruction's rows, as the kernel pads them, are a whole number of tiles or at least four; the backward
- * on every shape of the tensor-core kernel with Pmax >= 1 (one launch for the three gradients, which on large calls
- * forms the row statistic too; else one more for that).  Otherwise the work is one pass per instruction; the passes are independent, so every
+ * on every shape of the tensor-core kernel with Pmax >= 1: one launch for the three gradients, and one before it for the
+ * row statistic, which some large calls form in the first (d = 128, S <= 64, units of several row tiles).  Otherwise the work is one pass per instruction; the passes are independent, so every
  * other one is enqueued on a stream of the library's own that forks from `cuda_stream` at the start of the
  * call and joins it again before the call returns (to the caller everything is ordered as if it had run on
  * `cuda_stream`, also under stream capture).

@@ -722,7 +722,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 }
                 PSKV_TRACE_EVENT(11, item);
                 const uint32_t idesc_acc = make_idesc_bf16_ab(128, n, 1, 1);
-                // rows of the tile that belong to the group (the others are zero in P and dS)
+                // rows of the tile that belong to the group, in steps of 16 (the others among them are zero in P and dS, for finite inputs)
                 const int k0 = (int)((x >> kDescK0) & 15u), k1 = (int)((x >> kDescK1) & 15u);
                 if (elect_one_sync()) {
                     uint32_t a = (x & kDescAccFirst) ? 0u : 1u;
