@@ -492,7 +492,7 @@ def roofline(w, kernels, peaks):
     in the timed region (CUDA events around each launch, on the launch stream).  Algorithmic bytes
     and flops per launch come from inputs.kernel_work; the binding roof is the slower of
     bytes / measured HBM peak and flops / measured bf16 peak."""
-    work = wl.kernel_work(w)
+    work = wl.kernel_work(w, "simt_row_dot_kernel" in kernels)
     cands = {k: v for k, v in kernels.items() if k in work}
     if not cands:
         return None
@@ -519,7 +519,7 @@ def roofline(w, kernels, peaks):
 # profiles/ (kernel, workload) -> bytes.
 TRAFFIC_BYTES_PER_LAUNCH = {
     ("tc_fwd_kernel", "C2"): 473.9e6,        # profiles/tc_fwd_kernel_C2.md
-    # (the backward was captured before it read `out` for the row statistic: profiles/tc_bwd_kernel_C2.md)
+    ("tc_bwd_dq_kernel", "C2"): 1004.0e6,    # profiles/tc_bwd_kernel_C2.md
 }
 
 

@@ -134,9 +134,11 @@ def bwd_bytes(w: Workload) -> float:
     return float(3 * q + lse + skv + pkv + q + skv)
 
 
-def kernel_work(w: Workload) -> dict:
+def kernel_work(w: Workload, row_dot_kernel: bool = False) -> dict:
     """Algorithmic flops and HBM bytes per launch of each kernel of the tensor-core path
-    (every input read once, every output written once; recomputed scores are not counted)."""
+    (every input read once, every output written once; recomputed scores are not counted).
+    `row_dot_kernel`: a launch of its own forms the backward's row statistic D, and the gradient kernel
+    reads that (4 bytes a row) instead of `out`."""
     rows = w.B * w.Hq * w.S
     q = rows * w.d * 2
     skv = 2 * w.B * w.Hkv * w.S * w.d * 2
@@ -144,8 +146,8 @@ def kernel_work(w: Workload) -> dict:
     vis = (w.S + 1) / 2.0
     return {
         "tc_fwd_kernel": {"flops": fwd_flops(w), "bytes": fwd_bytes(w)},
-        # all three gradients: reads q, dout, lse, out (for D; 4 bytes a row of D where the pre-pass forms it), the prefix
-        # and the suffix K/V, writes dq, dk_suffix, dv_suffix
-        "tc_bwd_dq_kernel": {"flops": bwd_flops(w), "bytes": float(4 * q + 4 * rows + 2 * skv + pkv)},
+        # all three gradients: reads q, dout, lse, out or D, the prefix and the suffix K/V, writes dq, dk_suffix, dv_suffix
+        "tc_bwd_dq_kernel": {"flops": bwd_flops(w),
+                             "bytes": float(3 * q + (4 * rows if row_dot_kernel else q) + 4 * rows + 2 * skv + pkv)},
         "simt_row_dot_kernel": {"flops": rows * 2.0 * w.d, "bytes": float(2 * q + 4 * rows)},
     }

@@ -38,3 +38,15 @@ def test_one_rank_needs_no_process_group():
 def test_gpus_flag_must_match_an_outer_launcher():
     r = _run(["--gpus", "4", "--stub-step-ms", "1"], env={"WORLD_SIZE": "2", "RANK": "0", "LOCAL_RANK": "0"})
     assert r.returncode != 0 and "does not match" in (r.stderr + r.stdout)
+
+
+def test_bytes_of_the_gradient_kernel_count_out_only_where_it_reads_it():
+    sys.path.insert(0, ROOT)
+    from paper_2603_13420_b200.inputs import WORKLOADS, bwd_bytes, kernel_work
+
+    for w in WORKLOADS.values():
+        rows = w.B * w.Hq * w.S
+        alone, behind = kernel_work(w), kernel_work(w, row_dot_kernel=True)
+        assert alone["tc_bwd_dq_kernel"]["bytes"] == bwd_bytes(w)                  # every tensor of the call once
+        pair = behind["tc_bwd_dq_kernel"]["bytes"] + behind["simt_row_dot_kernel"]["bytes"]
+        assert pair == bwd_bytes(w) + 2 * rows * w.d + 8 * rows                    # dout twice, D written and read
