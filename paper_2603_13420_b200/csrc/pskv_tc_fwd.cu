@@ -56,9 +56,9 @@ enum : unsigned int {
 };
 
 // MODE 3.  The compiler reads runs of the kernel's parameters in one instruction where they are aligned, and what that makes of the
-// walk over tiles differs: with the fields behind these moved by 12 bytes the kernel for several instructions of whole tiles
-// took 140 us for 8 x 64 candidates, 32/8 heads, P = 256, S = 48, moved by 0 or 16 132; the others want the 12 (149 candidates,
-// 4/4 heads, P = 315, S = 8: 10.3 us, else 11.4; 6 x 90 candidates with short last tiles, 32/8, P = 300, S = 37 180, else 189).
+// walk over tiles differs.  The fields behind these moved by 12 bytes and by 16: several instructions of whole tiles, prefix resident, 8 x 64
+// candidates, 32/8 heads, P = 256, S = 48 178 and 160 us, 4 x 32, P = 128 38.5 and 35.3; streamed, 6 x 60, P = 300, S = 40 130 and 136; short last
+// tiles, 6 x 90, P = 300, S = 37 196 and 198; one prefix, 333, P = 217, S = 53 119 and 116, 149, 4/4, P = 315, S = 8 10.4 both.
 template <bool ALIGNED>
 struct BoxFields {
     int Sh;               // rows a query head takes in the row list: S, or S padded to whole tiles (head_box)
@@ -663,7 +663,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         // = 256, S = 48 11.9, now 11.6), and 256 candidates, 32/8, P = 2048, S = 32 take 254 us instead of 262 too.  With rings the
         // positions are counters and the barriers are looked at together first, since as a rule everything is there (the last
         // shape by division and one barrier after another: 287).  With the prefix resident nearly every item is waited for, and the
-        // compiler makes worse code of the counters (8 x 64 candidates, 32/8, P = 256, S = 48 172 us with them, else 153).
+        // compiler makes worse code of the counters (8 x 64 candidates, 32/8, P = 256, S = 48 172 us with them, else 153).  There the
+        // order in which the two issuers' MMAs meet decides: working ahead took some calls from 203 to 187 us (509 candidates, 32/32,
+        // P = 180, S = 38; 199 now) or 121 to 115 (150, P = 150, S = 96) and others from 94 to 99 (200, P = 200, S = 64; 97 now) or 57.5 to
+        // 59.5 (300, 32/8, P = 200, S = 30), with no rule in the sizes; most lost.
         int tl = 0;
         uint32_t ks = 0, kph = 0;        // ring of K blocks: stage, parity of its loads
         uint32_t slot = 0, slot_ph = 1;  // score slot, parity of its release
